@@ -22,11 +22,17 @@ LIB = os.path.join(HERE, "libcello_gpu.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
           "-I", INCLUDE, "-I", CSRC]
+# float32 bulk path: hardware-approximate division and square root
+F32 = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]
 UNITS = {
-    # float32 bulk path: hardware-approximate division and square root
-    "k_f32.cu": ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"],
+    "k_f32.cu": F32,
+    "k_f32_n8.cu": F32,
+    "k_f32_n16.cu": F32,
+    "k_f32_n32.cu": F32,
     "k_f64.cu": ["-fmad=false"],
-    "k_de_f32.cu": ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"],
+    "k_de_f32_n8.cu": F32,
+    "k_de_f32_n16.cu": F32,
+    "k_de_f32_n32.cu": F32,
     "k_de_f64.cu": ["-fmad=false"],
     "table.cu": [],
     "mesh.cu": [],

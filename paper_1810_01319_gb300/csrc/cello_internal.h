@@ -26,8 +26,6 @@ struct SweepVariant {
 };
 int sweep_variant_count_f32();
 int sweep_variant_count_f64();
-SweepVariant sweep_variant_f32(int v);
-SweepVariant sweep_variant_f64(int v);
 
 // Neighbour kinds of the 27-entry table.
 enum NbKind : int8_t { kSame = 0, kCoarse = 1, kFine = 2, kBoundary = 3 };
@@ -82,18 +80,81 @@ struct FastDiv {
   __device__ __forceinline__ unsigned div(unsigned x) const { return (__umulhi(x, m) + x) >> s; }
 };
 
+// Transverse pencils of one work item's leaf: cb pencils along transverse axis
+// B times count / cb along A, from (a0, b0).  Region 0 of a sweep is a
+// rectangle of every leaf; regions 1 and 2 belong to listed faces (leaf * 6 +
+// face), the ghost rows behind one face, shifted by (da, db) on its + side.
+struct SweepRegion {
+  int a0, b0, da, db;
+  int cb, count;
+  int tiles;               // work items per leaf or face, set by the launcher from the pencils per CTA
+  int items;               // set by the launcher
+  FastDiv div_cb, div_tiles;
+  const int* faces;        // null in region 0
+  int nfaces;
+};
+
+// Where a pencil of a work item lies.
+struct PencilAt {
+  int leaf;
+  int q;                   // first pencil of the item within its region
+  int r;                   // region
+  int a0, b0;
+};
+
 struct SweepParams {
   void* U;
   int leaf0, nleaf;        // leaves [leaf0, leaf0 + nleaf)
   int axis;
-  int a0, a1, b0, b1;      // transverse ranges (padded coordinates)
-  int tiles_per_leaf;      // set by the launcher from the variant's pencils per CTA
+  SweepRegion reg3[3];
+  int push;                // transverse axis across whose same-level faces the updated rows are also stored, or -1
   const double* dt;        // device scalar
   double* reg;             // flux registers (may be null)
   unsigned* work;          // work counter for persistent variants (device, 4 bytes)
   int n_items;             // set by the launcher
   int variant;             // index into the sweep variants of the precision
-  FastDiv div_tiles, div_cb;   // set by the launcher: by tiles_per_leaf and by the B-range length
+
+  // The items of the three regions for per_cta pencils per item.
+  void plan(int per_cta) {
+    n_items = 0;
+    for (int r = 0; r < 3; ++r) {
+      SweepRegion& g = reg3[r];
+      const int owners = r == 0 ? nleaf : g.nfaces;
+      g.tiles = owners > 0 ? (g.count + per_cta - 1) / per_cta : 0;
+      g.items = owners * g.tiles;
+      if (g.items > 0) {
+        g.div_cb = FastDiv::make((unsigned)g.cb);
+        g.div_tiles = FastDiv::make((unsigned)g.tiles);
+      }
+      n_items += g.items;
+    }
+  }
+
+  __device__ __forceinline__ PencilAt locate(int item, int per_cta) const {
+    PencilAt w;
+    w.r = 0;
+    if (item >= reg3[0].items) {
+      item -= reg3[0].items;
+      w.r = item < reg3[1].items ? 1 : 2;
+      if (w.r == 2) item -= reg3[1].items;
+    }
+    const SweepRegion& g = reg3[w.r];
+    const int owner = (int)g.div_tiles.div((unsigned)item);
+    w.q = (item - owner * g.tiles) * per_cta;
+    w.a0 = g.a0;
+    w.b0 = g.b0;
+    if (w.r == 0) {
+      w.leaf = leaf0 + owner;
+    } else {
+      const int f = g.faces[owner];
+      w.leaf = f / 6;
+      if (f & 1) {
+        w.a0 += g.da;
+        w.b0 += g.db;
+      }
+    }
+    return w;
+  }
 };
 
 struct AdjSweepParams {
@@ -140,14 +201,30 @@ void launch_neighbour_table(const DevMesh& m, const unsigned long long* keys, in
 // reads the margins the earlier ones filled in the face neighbours).
 // `phases` selects a subset; a phase must have run on every leaf before the
 // next one starts.
-enum RefreshPhase : int { kRefreshSlow = 1, kRefreshX = 2, kRefreshY = 4, kRefreshZ = 8, kRefreshAll = 15 };
+//
+// The two forms a step needs, whose sweeps fill the ghost rows behind
+// same-level faces themselves (see push_offset in kernels.cuh): an x, y, z step
+// reads the x margins of the interior rows and the slow regions (kRefreshXFirst);
+// a z, y, x step the z ghosts of the interior columns (kRefreshZRows, whole rows
+// of interior y) and then the slow regions nested the other way round
+// (kRefreshSlowZFirst: the interior columns behind a z face, all z behind a y
+// face, all y and z behind an x face).
+enum RefreshPhase : int {
+  kRefreshSlow = 1, kRefreshX = 2, kRefreshY = 4, kRefreshZ = 8, kRefreshAll = 15,
+  kRefreshZRows = 16, kRefreshSlowZFirst = 32,
+  kRefreshXFirst = kRefreshSlow | kRefreshX, kRefreshZFirst = kRefreshZRows | kRefreshSlowZFirst
+};
 void launch_refresh_f32(const DevMesh& m, float* U, int leaf0, int nleaf, const int* slow, int nslow,
                         int phases, cudaStream_t s);
 void launch_refresh_f64(const DevMesh& m, double* U, int leaf0, int nleaf, const int* slow, int nslow,
                         int phases, cudaStream_t s);
-void launch_sweep_f32(const DevMesh& m, const SweepParams& p, int pencils, cudaStream_t s);
-void launch_sweep_f64(const DevMesh& m, const SweepParams& p, int pencils, cudaStream_t s);
-// Dual-energy sweeps (both float32 forms, k_de_f32.cu; float64, k_de_f64.cu),
+void launch_sweep_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s);
+void launch_sweep_f64(const DevMesh& m, const SweepParams& p, cudaStream_t s);
+template <int NB>
+void prepare_sweep_f32(int sms);
+template <int NB>
+void launch_sweep_f32_nb(const DevMesh& m, const SweepParams& p, cudaStream_t s);
+// Dual-energy sweeps (both float32 forms, sweep_de_f32.cuh; float64, k_de_f64.cu),
 // launched by the planners above with the grid they computed.
 template <int NB, int P, int MINB>
 void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
@@ -155,7 +232,8 @@ template <int NB, int CT, int MINB, int VEC>
 void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
 template <int NB>
 void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
-void prepare_kernels_de_f32();
+template <int NB>
+void prepare_sweep_de_f32();
 void prepare_kernels_de_f64();
 void launch_fluxcorr(const DevMesh& m, void* U, int precision, const CoarseFace* faces,
                      const int* group_start, int ngroups, const double* reg, const double* dt,

@@ -1,0 +1,9 @@
+// Float32 PPM sweep of 8^3-cell blocks.
+#include "sweep_f32.cuh"
+
+namespace cello {
+template void prepare_sweep_f32<8>(int sms);
+template void launch_sweep_f32_nb<8>(const DevMesh& m, const SweepParams& p, cudaStream_t s);
+
+int sweep_variant_count_f32() { return kNV; }
+}  // namespace cello

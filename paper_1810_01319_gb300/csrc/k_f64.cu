@@ -39,14 +39,11 @@ static void prepare_nb64(int sms) {
 }
 
 template <int NB>
-static void launch_nb64(const DevMesh& m, SweepParams p, int pencils, cudaStream_t s) {
+static void launch_nb64(const DevMesh& m, SweepParams p, cudaStream_t s) {
   constexpr int N = NB + 2 * kGhosts;
   const int v = (p.variant >= 0 && p.variant < kNV64) ? p.variant : 0;
-  p.tiles_per_leaf = (pencils + 7) / 8;
-  p.n_items = p.nleaf * p.tiles_per_leaf;
+  p.plan(8);
   if (p.n_items <= 0) return;
-  p.div_tiles = FastDiv::make((unsigned)p.tiles_per_leaf);
-  p.div_cb = FastDiv::make((unsigned)(p.b1 - p.b0));
   int grid = p.n_items;
   if (kVariants64[v].persistent && p.work) {
     cudaMemsetAsync(p.work, 0, sizeof(unsigned), s);
@@ -64,13 +61,12 @@ static void launch_nb64(const DevMesh& m, SweepParams p, int pencils, cudaStream
 }
 
 int sweep_variant_count_f64() { return kNV64; }
-SweepVariant sweep_variant_f64(int v) { return kVariants64[v]; }
 
-void launch_sweep_f64(const DevMesh& m, const SweepParams& p, int pencils, cudaStream_t s) {
+void launch_sweep_f64(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
   switch (m.n) {
-    case 8: launch_nb64<8>(m, p, pencils, s); break;
-    case 16: launch_nb64<16>(m, p, pencils, s); break;
-    case 32: launch_nb64<32>(m, p, pencils, s); break;
+    case 8: launch_nb64<8>(m, p, s); break;
+    case 16: launch_nb64<16>(m, p, s); break;
+    case 32: launch_nb64<32>(m, p, s); break;
   }
 }
 
@@ -119,7 +115,8 @@ static void refresh_nf(const DevMesh& m, T* U, int leaf0, int nleaf, const int* 
                        cudaStream_t s) {
   constexpr int G = kGhosts, N = NB + 2 * G;
   auto blocks = [](long threads, int per) { return (unsigned)((threads + per - 1) / per); };
-  if ((phases & kRefreshSlow) && nslow > 0) refresh_slow_kernel<T, NB, NF><<<nslow, 128, 0, s>>>(m, U, slow, nslow);
+  if ((phases & kRefreshSlow) && nslow > 0)
+    refresh_slow_kernel<T, NB, NF, false><<<nslow, 128, 0, s>>>(m, U, slow, nslow);
   if (nleaf <= 0) return;
   if (phases & kRefreshX)   // float32: one thread per row pair (see refresh_x_kernel)
     refresh_x_kernel<T, NB, NF><<<blocks((long)nleaf * NB * (sizeof(T) == 4 ? NB / 2 : NB), 256), 256, 0, s>>>(
@@ -129,8 +126,13 @@ static void refresh_nf(const DevMesh& m, T* U, int leaf0, int nleaf, const int* 
     refresh_y_kernel<T, NB, NF><<<blocks((long)nleaf * 2 * NF * NB * (G * N / S), 256), 256, 0, s>>>(m, U, leaf0,
                                                                                                    nleaf);
   if (phases & kRefreshZ)
-    refresh_z_kernel<T, NB, NF><<<blocks((long)nleaf * 2 * NF * (G * N * N / S), 256), 256, 0, s>>>(m, U, leaf0,
-                                                                                                    nleaf);
+    refresh_z_kernel<T, NB, NF, false><<<blocks((long)nleaf * 2 * NF * (G * N * N / S), 256), 256, 0, s>>>(
+        m, U, leaf0, nleaf);
+  if (phases & kRefreshZRows)
+    refresh_z_kernel<T, NB, NF, true><<<blocks((long)nleaf * 2 * NF * (G * NB * N / S), 256), 256, 0, s>>>(
+        m, U, leaf0, nleaf);
+  if ((phases & kRefreshSlowZFirst) && nslow > 0)
+    refresh_slow_kernel<T, NB, NF, true><<<nslow, 128, 0, s>>>(m, U, slow, nslow);
 }
 
 template <typename T, int NB>

@@ -124,7 +124,9 @@ void prepare_kernels() {
   std::call_once(once, [] {
     prepare_kernels_f32();
     prepare_kernels_f64();
-    prepare_kernels_de_f32();
+    prepare_sweep_de_f32<8>();
+    prepare_sweep_de_f32<16>();
+    prepare_sweep_de_f32<32>();
     prepare_kernels_de_f64();
   });
   // L2 fetch granularity of this process's context on the current device, set
@@ -179,6 +181,8 @@ struct cello_mesh {
   double* d_partials = nullptr;
   int* d_slow = nullptr;           // faces the refresh computes (leaf * 6 + face): neighbour not same-level
   std::vector<int> slow_start;     // per-leaf offsets into d_slow, B + 1 entries
+  int* d_slow_ax[3] = {nullptr, nullptr, nullptr};   // the same faces by axis, and their per-leaf offsets
+  std::vector<int> slow_ax_start[3];
   int exec_mode = CELLO_EXEC_BATCHED;
   int sweep_variant[3] = {0, 0, 0};   // per sweep axis; chosen by cello_autotune or set by the caller
   unsigned* d_work = nullptr;      // work counter of the persistent sweep variants
@@ -244,6 +248,10 @@ struct cello_mesh {
     d_zero = nullptr;
     if (d_slow) cudaFree(d_slow);
     d_slow = nullptr;
+    for (int*& p : d_slow_ax) {
+      if (p) cudaFree(p);
+      p = nullptr;
+    }
     void* ptrs[] = {d_leaf, d_keys, d_kind, d_idx, d_fine8, d_face_slot, d_cfaces, d_group_start, d_reg, d_partials};
     for (void* p : ptrs)
       if (p) cudaFree(p);
@@ -450,14 +458,20 @@ cello_status finish_build(cello_mesh* M) {
   // faces whose phase region the refresh computes instead of copying: those
   // whose neighbour is not a same-level leaf (coarser, finer, boundary)
   {
-    std::vector<int> slow;
+    std::vector<int> slow, by_axis[3];
     M->slow_start.assign((size_t)B + 1, 0);
+    for (int a = 0; a < 3; ++a) M->slow_ax_start[a].assign((size_t)B + 1, 0);
     for (int b = 0; b < B; ++b) {
       for (int f = 0; f < 6; ++f)
-        if (M->kind[(size_t)b * 27 + face_dir(f >> 1, (f & 1) ? 1 : -1)] != kSame) slow.push_back(b * 6 + f);
+        if (M->kind[(size_t)b * 27 + face_dir(f >> 1, (f & 1) ? 1 : -1)] != kSame) {
+          slow.push_back(b * 6 + f);
+          by_axis[f >> 1].push_back(b * 6 + f);
+        }
       M->slow_start[b + 1] = (int)slow.size();
+      for (int a = 0; a < 3; ++a) M->slow_ax_start[a][b + 1] = (int)by_axis[a].size();
     }
     CELLO_TRY(upload(&M->d_slow, slow));
+    for (int a = 0; a < 3; ++a) CELLO_TRY(upload(&M->d_slow_ax[a], by_axis[a]));
   }
   CELLO_CUDA(cudaMalloc((void**)&M->d_work, sizeof(unsigned)));
   CELLO_CUDA(cudaMalloc((void**)&M->d_err, sizeof(unsigned)));
@@ -488,45 +502,90 @@ void sweep_ranges(const cello_mesh* M, int axis, const bool swept[3], int& a0, i
   b1 = swept[tb] ? g + n : N;
 }
 
-// The launch sequence of one step on stream s.
+// The pencils of the step's oi-th sweep over leaves [leaf0, leaf0 + nleaf).
+// whole: the sweep of a whole step, in which each leaf sweeps its interior rows
+// and the ghost rows behind its faces that are not same-level, and stores the
+// rows its same-level neighbours read behind the next sweep's faces into their
+// ghost rows (push_offset in kernels.cuh); the ghost rows behind the last
+// sweep's faces are needed by the second sweep only.  Otherwise (a leaf range, or
+// a state whose ghost rows are read afterwards): every row a later sweep of the
+// same leaf reads, nothing stored elsewhere.
+void set_regions(const cello_mesh* M, SweepParams& p, const int order[3], int oi, int leaf0, int nleaf, bool whole) {
+  const int n = M->desc.n, g = M->desc.ghosts, N = M->N;
+  p.axis = order[oi];
+  p.leaf0 = leaf0;
+  p.nleaf = nleaf;
+  p.push = -1;
+  SweepRegion& r0 = p.reg3[0];
+  if (!whole) {
+    bool swept[3] = {false, false, false};
+    for (int k = 0; k < oi; ++k) swept[order[k]] = true;
+    int a1, b1;
+    sweep_ranges(M, p.axis, swept, r0.a0, a1, r0.b0, b1);
+    r0.cb = b1 - r0.b0;
+    r0.count = (a1 - r0.a0) * r0.cb;
+    return;
+  }
+  r0.a0 = r0.b0 = g;
+  r0.cb = n;
+  r0.count = n * n;
+  if (oi < 2) p.push = order[oi + 1];
+  const int ta = p.axis == 2 ? 1 : 2;
+  for (int k = 1; oi + k < 3; ++k) {   // faces of the next sweep's axis, then (first sweep) of the last one's
+    const int f = order[oi + k];
+    const bool full = k == 2;          // behind those, the second sweep reads all rows of its own axis
+    SweepRegion& r = p.reg3[k];
+    const int along = full ? N : n, from = full ? 0 : g;
+    if (f == ta) {
+      r.a0 = 0; r.da = g + n;
+      r.b0 = from; r.cb = along;
+    } else {
+      r.a0 = from;
+      r.b0 = 0; r.db = g + n; r.cb = g;
+    }
+    r.count = g * along;
+    const int s0 = M->slow_ax_start[f][leaf0];
+    r.faces = M->d_slow_ax[f] ? M->d_slow_ax[f] + s0 : nullptr;
+    r.nfaces = M->slow_ax_start[f][leaf0 + nleaf] - s0;
+  }
+}
+
+void launch_sweep(const cello_mesh* M, const DevMesh& dm, const SweepParams& p, cudaStream_t s) {
+  if (M->desc.precision == 4) launch_sweep_f32(dm, p, s);
+  else launch_sweep_f64(dm, p, s);
+}
+
 // The three split sweeps of leaves [leaf0, leaf0 + nleaf) (x, y, z on even
 // cycles, z, y, x on odd ones), face fluxes of coarse-fine faces into the
-// registers; plain: one launch per leaf and sweep; ev (nullable): events
-// after each sweep at ev[2 ..].
+// registers; whole: see set_regions; plain: one launch per leaf and sweep; ev
+// (nullable): events after each sweep at ev[2 ..].
 void enqueue_sweeps(const cello_mesh* M, const DevMesh& dm, void* U, const double* dt, int cycle, int leaf0,
-                    int nleaf, bool plain, cudaStream_t s, cudaEvent_t* ev) {
-  const cello_mesh_desc& d = M->desc;
+                    int nleaf, bool whole, bool plain, cudaStream_t s, cudaEvent_t* ev) {
   const int order[3] = {cycle % 2 == 0 ? 0 : 2, 1, cycle % 2 == 0 ? 2 : 0};
-  bool swept[3] = {false, false, false};
   for (int oi = 0; oi < 3; ++oi) {
-    const int axis = order[oi];
     SweepParams p{};
     p.U = U;
-    p.axis = axis;
-    sweep_ranges(M, axis, swept, p.a0, p.a1, p.b0, p.b1);
-    const int pencils = (p.a1 - p.a0) * (p.b1 - p.b0);
     p.dt = dt;
     p.reg = M->d_reg;
     p.work = M->d_work;
-    p.variant = M->sweep_variant[axis];
+    p.variant = M->sweep_variant[order[oi]];
     if (plain) {
       for (int b = leaf0; b < leaf0 + nleaf; ++b) {
-        p.leaf0 = b;
-        p.nleaf = 1;
-        if (d.precision == 4) launch_sweep_f32(dm, p, pencils, s);
-        else launch_sweep_f64(dm, p, pencils, s);
+        set_regions(M, p, order, oi, b, 1, whole);
+        launch_sweep(M, dm, p, s);
       }
     } else if (nleaf > 0) {
-      p.leaf0 = leaf0;
-      p.nleaf = nleaf;
-      if (d.precision == 4) launch_sweep_f32(dm, p, pencils, s);
-      else launch_sweep_f64(dm, p, pencils, s);
+      set_regions(M, p, order, oi, leaf0, nleaf, whole);
+      launch_sweep(M, dm, p, s);
     }
-    swept[axis] = true;
     if (ev) cudaEventRecord(ev[2 + oi], s);
   }
 }
 
+// The ghost cells that the sweeps of a whole step read before writing them.
+int step_refresh(int cycle) { return cycle % 2 == 0 ? kRefreshXFirst : kRefreshZFirst; }
+
+// The launch sequence of one step on stream s.
 void enqueue_step(const cello_mesh* M, void* U, const double* dt, int cycle, double cfl, double* dt_next,
                   double* totals, cudaStream_t s, cudaEvent_t* ev = nullptr) {
   const cello_mesh_desc& d = M->desc;
@@ -534,13 +593,15 @@ void enqueue_step(const cello_mesh* M, void* U, const double* dt, int cycle, dou
   const int B = M->B;
   const bool plain = M->exec_mode == CELLO_EXEC_PLAIN && !ev;
   if (ev) cudaEventRecord(ev[0], s);
-  if (plain)   // one launch per leaf and phase; each phase over every leaf before the next
-    for (int ph : {kRefreshSlow, kRefreshX, kRefreshY, kRefreshZ})
+  if (plain) {   // one launch per leaf and phase; each phase over every leaf before the next
+    const int even[2] = {kRefreshSlow, kRefreshX}, odd[2] = {kRefreshZRows, kRefreshSlowZFirst};
+    for (int ph : cycle % 2 == 0 ? even : odd)
       for (int b = 0; b < B; ++b) launch_refresh(M, dm, U, b, 1, s, ph);
-  else
-    launch_refresh(M, dm, U, 0, B, s);
+  } else {
+    launch_refresh(M, dm, U, 0, B, s, step_refresh(cycle));
+  }
   if (ev) cudaEventRecord(ev[1], s);
-  enqueue_sweeps(M, dm, U, dt, cycle, 0, B, plain, s, ev);
+  enqueue_sweeps(M, dm, U, dt, cycle, 0, B, true, plain, s, ev);
   if (!M->cfaces.empty())
     launch_fluxcorr(dm, U, d.precision, M->d_cfaces, M->d_group_start, (int)M->group_start.size() - 1, M->d_reg,
                     dt, s);
@@ -568,9 +629,9 @@ void enqueue_step_cfl(const cello_mesh* M, void* U, int cycle, double cfl, doubl
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   launch_reduce(dm, U, d.precision, cfl, M->d_partials, dt_used, totals, M->side_stream, kSideReduceCtasPerSm * sms);
   cudaEventRecord(M->join_ev, M->side_stream);
-  launch_refresh(M, dm, U, 0, M->B, s);
+  launch_refresh(M, dm, U, 0, M->B, s, step_refresh(cycle));
   cudaStreamWaitEvent(s, M->join_ev, 0);
-  enqueue_sweeps(M, dm, U, dt_used, cycle, 0, M->B, false, s, nullptr);
+  enqueue_sweeps(M, dm, U, dt_used, cycle, 0, M->B, true, false, s, nullptr);
   if (!M->cfaces.empty())
     launch_fluxcorr(dm, U, d.precision, M->d_cfaces, M->d_group_start, (int)M->group_start.size() - 1, M->d_reg,
                     dt_used, s);
@@ -610,17 +671,12 @@ cello_status adjoint_step(cello_mesh* M, const void* Un, void* lam, const double
       CELLO_CUDA(cudaMemcpyAsync(entry[oi + 1], entry[oi], state, cudaMemcpyDeviceToDevice, s));
       SweepParams p{};
       p.U = entry[oi + 1];
-      p.axis = axis;
-      p.a0 = rng[oi][0]; p.a1 = rng[oi][1]; p.b0 = rng[oi][2]; p.b1 = rng[oi][3];
-      const int pencils = (p.a1 - p.a0) * (p.b1 - p.b0);
       p.dt = dt;
       p.reg = nullptr;
       p.work = M->d_work;
       p.variant = M->sweep_variant[axis];
-      p.leaf0 = 0;
-      p.nleaf = B;
-      if (d.precision == 4) launch_sweep_f32(dm, p, pencils, s);
-      else launch_sweep_f64(dm, p, pencils, s);
+      set_regions(M, p, order, oi, 0, B, false);   // the adjoint sweeps read every ghost row
+      launch_sweep(M, dm, p, s);
     }
     swept[axis] = true;
   }
@@ -902,7 +958,7 @@ cello_status cello_hydro_step_part(cello_mesh* M, void* U, const double* dt, int
   const DevMesh dm = M->dev();
   if (part == 0) {
     launch_refresh(M, dm, U, 0, M->B, s);
-    enqueue_sweeps(M, dm, U, dt, cycle, (int)leaf0, (int)nleaf, false, s, nullptr);
+    enqueue_sweeps(M, dm, U, dt, cycle, (int)leaf0, (int)nleaf, false, false, s, nullptr);
   } else if (!M->cfaces.empty()) {
     // the groups (one per coarse leaf, in leaf order) whose leaf is in the range
     const int ng = (int)M->group_start.size() - 1;
@@ -1118,24 +1174,17 @@ cello_status cello_autotune(cello_mesh* M, void* U, int* variants_out, float* ms
       // each axis is timed in both of its positions
       for (int parity = 0; parity < 2 && err == cudaSuccess; ++parity) {
         const int order[3] = {parity == 0 ? 0 : 2, 1, parity == 0 ? 2 : 0};
-        bool swept[3] = {false, false, false};
         cudaEventRecord(ev[0], s);
         for (int oi = 0; oi < 3; ++oi) {
-          const int axis = order[oi];
           SweepParams p{};
           p.U = U;
-          p.axis = axis;
-          sweep_ranges(M, axis, swept, p.a0, p.a1, p.b0, p.b1);
-          const int pencils = (p.a1 - p.a0) * (p.b1 - p.b0);
           p.dt = M->d_zero;
           p.reg = nullptr;
           p.work = M->d_work;
           p.variant = v;
-          p.leaf0 = 0;
-          p.nleaf = nleaf;
-          if (d.precision == 4) launch_sweep_f32(dm, p, pencils, s);
-          else launch_sweep_f64(dm, p, pencils, s);
-          swept[axis] = true;
+          set_regions(M, p, order, oi, 0, nleaf, true);
+          p.push = -1;   // the sample's neighbours keep their ghost rows
+          launch_sweep(M, dm, p, s);
           cudaEventRecord(ev[oi + 1], s);
         }
         err = cudaEventSynchronize(ev[3]);

@@ -1,7 +1,10 @@
 // Float32 dual-energy sweeps (both forms with a sixth field rho e; method
-// code RS | 4).  Compiled with the float32 sweep's flags; the planners in
-// k_f32.cu compute the grid and call launch_sweep_de_f32 (shared-memory
+// code RS | 4) for blocks of CELLO_DE_NB cells per edge, one translation unit
+// per block size.  Compiled with the float32 sweep's flags; the planners in
+// sweep_f32.cuh compute the grid and call launch_sweep_de_f32 (shared-memory
 // form) or launch_stream_de_f32 (register streaming).
+#pragma once
+
 #include "kernels.cuh"
 
 namespace cello {
@@ -40,9 +43,7 @@ void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cuda
   X(NB, 64, 6, 3)
 #define CELLO_DE_SINST(NB, CT, MINB, VEC) \
   template void launch_stream_de_f32<NB, CT, MINB, VEC>(const DevMesh&, const SweepParams&, int, cudaStream_t);
-CELLO_DE_STREAM(CELLO_DE_SINST, 8)
-CELLO_DE_STREAM(CELLO_DE_SINST, 16)
-CELLO_DE_STREAM(CELLO_DE_SINST, 32)
+CELLO_DE_STREAM(CELLO_DE_SINST, CELLO_DE_NB)
 #undef CELLO_DE_SINST
 #undef CELLO_DE_STREAM
 
@@ -62,16 +63,13 @@ static void prepare_de() {
 #define CELLO_DE_VARIANTS(X, NB) X(NB, 8, 3) X(NB, 8, 4) X(NB, 4, 6) X(NB, 16, 1) X(NB, 4, 8) X(NB, 16, 2)
 #define CELLO_DE_INST(NB, P, MINB) \
   template void launch_sweep_de_f32<NB, P, MINB>(const DevMesh&, const SweepParams&, int, cudaStream_t);
-CELLO_DE_VARIANTS(CELLO_DE_INST, 8)
-CELLO_DE_VARIANTS(CELLO_DE_INST, 16)
-CELLO_DE_VARIANTS(CELLO_DE_INST, 32)
+CELLO_DE_VARIANTS(CELLO_DE_INST, CELLO_DE_NB)
 #undef CELLO_DE_INST
 
-void prepare_kernels_de_f32() {
+template <>
+void prepare_sweep_de_f32<CELLO_DE_NB>() {
 #define CELLO_DE_PREP(NB, P, MINB) prepare_de<NB, P, MINB>();
-  CELLO_DE_VARIANTS(CELLO_DE_PREP, 8)
-  CELLO_DE_VARIANTS(CELLO_DE_PREP, 16)
-  CELLO_DE_VARIANTS(CELLO_DE_PREP, 32)
+  CELLO_DE_VARIANTS(CELLO_DE_PREP, CELLO_DE_NB)
 #undef CELLO_DE_PREP
 }
 #undef CELLO_DE_VARIANTS
