@@ -228,7 +228,7 @@ void launch_sweep_f32_nb(const DevMesh& m, const SweepParams& p, cudaStream_t s)
 // launched by the planners above with the grid they computed.
 template <int NB, int P, int MINB>
 void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
-template <int NB, int CT, int MINB, int VEC>
+template <int NB, int CT, int VEC>
 void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
 template <int NB>
 void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);

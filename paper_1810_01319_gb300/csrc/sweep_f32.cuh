@@ -100,7 +100,7 @@ static void launch_stream_variant(const DevMesh& m, SweepParams p, int v, cudaSt
   if (!plan_launch<NB>(p, CT, v, grid, s)) return;
   constexpr size_t sh = stream_smem<CT, VEC>();
   if (m.nf == 6) {   // dual energy (sweep_de_f32.cuh)
-    launch_stream_de_f32<NB, CT, MINB, VEC>(m, p, grid, s);
+    launch_stream_de_f32<NB, CT, VEC>(m, p, grid, s);
     return;
   }
   switch (method_code(m.riemann, m.steepen)) {
