@@ -2,33 +2,38 @@
 // the hydro Method of Sec. II.C with dt held fixed).  Each *_bwd function
 // recomputes what it needs of its forward counterpart in ppm.cuh and
 // accumulates the adjoints of its inputs (+=).  At a kink (min, max, a
-// branch) the derivative of the branch the forward pass took is used.
+// branch) the derivative of the branch the forward pass took is used: every
+// value that decides a branch is the forward expression, in its order.  What
+// only scales an adjoint is written for GB300's float64 pipe, which bounds the
+// float64 adjoint and takes ~10 instructions for a division: one reciprocal per
+// divisor, fused multiply-adds.
 #pragma once
 
 #include "ppm.cuh"
 
 namespace cello {
 
+CELLO_HD float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+CELLO_HD double vfma(double a, double b, double c) { return fma(a, b, c); }
+
+// W = to_primitive(U); rho = max(U_0, floor) and p = max(p of U, floor).
 template <typename T>
-CELLO_HD void to_primitive_bwd(const T U[5], const Gas<T>& gs, const T Wb[5], T Ub[5]) {
-  const T rho = vmax(U[0], T(kRhoFloor));
-  const T un = U[1] / rho, ut1 = U[2] / rho, ut2 = U[3] / rho;
-  const T s = un * un + (ut1 * ut1 + ut2 * ut2);
-  const T h = T(0.5) * rho;
-  const T praw = gs.gm1 * (U[4] - h * s);
-  const T prawb = (praw > T(kPFloor)) ? Wb[4] : T(0);
-  Ub[4] += gs.gm1 * prawb;
+CELLO_HD void to_primitive_bwd(const T W[5], const Gas<T>& gs, const T Wb[5], T Ub[5]) {
+  const T rho = W[0], un = W[1], ut1 = W[2], ut2 = W[3];
+  const T ir = T(1) / rho;
+  const T s = vfma(un, un, vfma(ut1, ut1, ut2 * ut2));
+  const T prawb = (W[4] > T(kPFloor)) ? Wb[4] : T(0);
   const T keb = -gs.gm1 * prawb;
-  T rhob = Wb[0] + T(0.5) * (keb * s);
-  const T sb = keb * h;
-  const T unb = Wb[1] + T(2) * un * sb;
-  const T t1b = Wb[2] + T(2) * ut1 * sb;
-  const T t2b = Wb[3] + T(2) * ut2 * sb;
-  Ub[1] += unb / rho;
-  Ub[2] += t1b / rho;
-  Ub[3] += t2b / rho;
-  rhob -= (unb * un + t1b * ut1 + t2b * ut2) / rho;
-  if (U[0] > T(kRhoFloor)) Ub[0] += rhob;
+  Ub[4] -= keb;
+  const T sb2 = keb * rho;   // twice the adjoint of s
+  const T unb = vfma(un, sb2, Wb[1]), t1b = vfma(ut1, sb2, Wb[2]), t2b = vfma(ut2, sb2, Wb[3]);
+  Ub[1] = vfma(unb, ir, Ub[1]);
+  Ub[2] = vfma(t1b, ir, Ub[2]);
+  Ub[3] = vfma(t2b, ir, Ub[3]);
+  if (rho > T(kRhoFloor)) {
+    const T rhob = vfma(T(0.5) * keb, s, Wb[0]);
+    Ub[0] += vfma(-vfma(unb, un, vfma(t1b, ut1, t2b * ut2)), ir, rhob);
+  }
 }
 
 template <typename T>
@@ -111,21 +116,23 @@ CELLO_HD void flatten_monotone_bwd(T a, T f, T aL, T aR, T oLb, T oRb, T& ab, T&
 template <typename T>
 CELLO_HD void avg_right_bwd(T aL, T aR, T a6, T s, T ob, T& aLb, T& aRb, T& a6b, T& sb) {
   const T h = T(0.5) * s, g = T(1) - T(2.0 / 3.0) * s;
-  const T inner = (aR - aL) - g * a6;
-  aRb += ob * (T(1) - h);
-  aLb += ob * h;
-  a6b += ob * (h * g);
-  sb -= ob * (T(0.5) * inner + h * (T(2.0 / 3.0) * a6));
+  const T inner = vfma(-g, a6, aR - aL);
+  const T oh = ob * h;
+  aRb += ob - oh;
+  aLb += oh;
+  a6b = vfma(oh, g, a6b);
+  sb = vfma(-ob, vfma(h * T(2.0 / 3.0), a6, T(0.5) * inner), sb);
 }
 
 template <typename T>
 CELLO_HD void avg_left_bwd(T aL, T aR, T a6, T s, T ob, T& aLb, T& aRb, T& a6b, T& sb) {
   const T h = T(0.5) * s, g = T(1) - T(2.0 / 3.0) * s;
-  const T inner = (aR - aL) + g * a6;
-  aLb += ob * (T(1) - h);
-  aRb += ob * h;
-  a6b += ob * (h * g);
-  sb += ob * (T(0.5) * inner - h * (T(2.0 / 3.0) * a6));
+  const T inner = vfma(g, a6, aR - aL);
+  const T oh = ob * h;
+  aLb += ob - oh;
+  aRb += oh;
+  a6b = vfma(oh, g, a6b);
+  sb = vfma(ob, vfma(-h * T(2.0 / 3.0), a6, T(0.5) * inner), sb);
 }
 
 // Reverse of trace(): adjoints of the two edge states -> adjoints of the
@@ -142,9 +149,10 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
     a6b[q] = T(0);
   }
   const T lm = un - c, l0 = un, lp = un + c;
-  const T hrc = (T(0.5) * rho) / c;
-  const T hic = T(0.5) / csq;
-  const T cr = c / rho;
+  const T ic = T(1) / c, ir = T(1) / rho, icsq = ic * ic;
+  const T hrc = (T(0.5) * rho) * ic;
+  const T hic = T(0.5) * icsq;
+  const T cr = c * ir;
   T lmb = 0, l0b = 0, lpb = 0, csqb = 0, cb = 0, rhob = 0, hrcb = 0, hicb = 0, crb = 0;
 
   {  // right edge
@@ -163,7 +171,7 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
     if (l0 > T(0)) {
       A0 = avg_right(aL[0], aR[0], a6[0], s0);
       A4 = avg_right(aL[4], aR[4], a6[4], s0);
-      b0 = (ref[0] - A0) - (ref[4] - A4) / csq;
+      b0 = (ref[0] - A0) - (ref[4] - A4) * icsq;
     }
     T bmb = 0, b0b = 0, spb = 0, s0b = 0, smb = 0;
     // transverse components
@@ -194,8 +202,8 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
       refb[0] += b0b;
       const T A0b = -b0b;
       const T D4 = ref[4] - A4;
-      const T D4b = -b0b / csq;
-      csqb += b0b * D4 / (csq * csq);
+      const T D4b = -b0b * icsq;
+      csqb = vfma(-D4b * icsq, D4, csqb);
       refb[4] += D4b;
       const T A4b = -D4b;
       avg_right_bwd(aL[0], aR[0], a6[0], s0, A0b, aLb[0], aRb[0], a6b[0], s0b);
@@ -233,7 +241,7 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
     if (l0 < T(0)) {
       A0 = avg_left(aL[0], aR[0], a6[0], t0);
       A4 = avg_left(aL[4], aR[4], a6[4], t0);
-      b0 = (ref[0] - A0) - (ref[4] - A4) / csq;
+      b0 = (ref[0] - A0) - (ref[4] - A4) * icsq;
     }
     T bpb = 0, b0b = 0, tpb = 0, t0b = 0, tmb = 0;
     for (int q = 2; q < 4; ++q) {
@@ -263,8 +271,8 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
       refb[0] += b0b;
       const T A0b = -b0b;
       const T D4 = ref[4] - A4;
-      const T D4b = -b0b / csq;
-      csqb += b0b * D4 / (csq * csq);
+      const T D4b = -b0b * icsq;
+      csqb = vfma(-D4b * icsq, D4, csqb);
       refb[4] += D4b;
       const T A4b = -D4b;
       avg_left_bwd(aL[0], aR[0], a6[0], t0, A0b, aLb[0], aRb[0], a6b[0], t0b);
@@ -289,61 +297,48 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
   // shared coefficients
   T unb = lmb + l0b + lpb;
   cb += lpb - lmb;
-  rhob += T(0.5) * hrcb / c;
-  cb -= hrcb * hrc / c;
-  csqb -= hicb * hic / csq;
-  cb += crb / rho;
-  rhob -= crb * cr / rho;
+  rhob = vfma(T(0.5) * hrcb, ic, rhob);
+  cb = vfma(-hrcb * hrc, ic, cb);
+  csqb = vfma(-hicb * hic, icsq, csqb);
+  cb = vfma(crb, ir, cb);
+  rhob = vfma(-crb * cr, ir, rhob);
   for (int q = 0; q < 5; ++q) {
     Wb[q] += T(6) * a6b[q];
     aLb[q] -= T(3) * a6b[q];
     aRb[q] -= T(3) * a6b[q];
   }
-  csqb += cb / (T(2) * c);
-  T pb = csqb * gs.gamma / rho;
-  rhob -= csqb * csq / rho;
+  csqb = vfma(T(0.5) * cb, ic, csqb);
+  const T pb = csqb * gs.gamma * ir;
+  rhob = vfma(-csqb * csq, ir, rhob);
   Wb[0] += rhob;
   Wb[1] += unb;
   Wb[4] += pb;
 }
 
-// Shock-curve quantities of one side at pressure ps (as in riemann_flux).
+// One side of the two-shock solver in reverse: its pressure, wave impedance C,
+// their reciprocals, the sign of its velocity jump, and the adjoints of its
+// pressure, C and velocity.
 template <typename T>
-struct Curve {
-  T x, W, us, Z;
+struct ShockSide {
+  T p, C, ip, iC, sgn;
+  T pb, Cb, ub;
 };
 
+// Adjoints of (us, Z, W) of the shock curve at pressure ps -> (ps, p, C, u):
+// x = 1 + g1 (ps/p - 1), W = C sqrt(x), us = u -/+ (ps - p)/W,
+// Z = 2 W^3/(W^2 + C^2).  Returns the adjoint of ps.
 template <typename T>
-CELLO_HD Curve<T> curve(T ps, T pK, T CK, T uK, T sgn, const Gas<T>& gs) {
-  Curve<T> c;
-  c.x = T(1) + gs.g1 * (ps / pK - T(1));
-  c.W = CK * vsqrt(c.x);
-  c.us = (sgn < T(0)) ? uK - (ps - pK) / c.W : uK + (ps - pK) / c.W;
-  c.Z = ((T(2) * c.W) * c.W) * c.W / (c.W * c.W + CK * CK);
-  return c;
-}
-
-// Reverse of curve(): adjoints of (us, Z, W) -> (ps, pK, CK, uK).
-template <typename T>
-CELLO_HD void curve_bwd(T ps, T pK, T CK, T sgn, const Gas<T>& gs, const Curve<T>& c, T usb, T Zb, T Wb,
-                        T& psb, T& pKb, T& CKb, T& uKb) {
-  const T W = c.W;
-  const T den = W * W + CK * CK;
-  T Wbar = Wb + Zb * ((T(2) * W * W * W * W + T(6) * W * W * CK * CK) / (den * den));
-  CKb += Zb * (-(T(4) * W * W * W * CK) / (den * den));
-  uKb += usb;
-  // us = uK -/+ (ps - pK)/W
-  const T q = (ps - pK) / W;
-  const T qb = (sgn < T(0)) ? -usb : usb;
-  psb += qb / W;
-  pKb -= qb / W;
-  Wbar -= qb * q / W;
-  // W = CK*sqrt(x), x = 1 + g1*(ps/pK - 1)
-  const T sx = vsqrt(c.x);
-  CKb += Wbar * sx;
-  const T xb = Wbar * CK / (T(2) * sx);
-  psb += xb * gs.g1 / pK;
-  pKb -= xb * gs.g1 * ps / (pK * pK);
+CELLO_HD T shock_side_bwd(ShockSide<T>& k, T ps, T W, T usb, T Zb, T Wb, const Gas<T>& gs) {
+  const T W2 = W * W, C2 = k.C * k.C;
+  const T iW = T(1) / W, iden = T(1) / (W2 + C2);
+  const T z = T(2) * W2 * (iden * iden) * Zb;
+  const T q = (ps - k.p) * iW, qb = k.sgn * usb * iW;
+  const T Wbar = vfma(-qb, q, vfma(z, vfma(T(3), C2, W2), Wb));
+  const T xb = T(0.5) * Wbar * C2 * iW * gs.g1 * k.ip;   // adjoint of ps/p, over p
+  k.ub += usb;
+  k.Cb = vfma(Wbar, W * k.iC, vfma(T(-2) * z * W, k.C, k.Cb));
+  k.pb -= vfma(xb * ps, k.ip, qb);
+  return qb + xb;
 }
 
 // Reverse of riemann_flux(): flux adjoints -> adjoints of the two states.
@@ -353,150 +348,166 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
   const T rR = R[0], uR = R[1], pR = R[4];
   const T CL = vsqrt((gs.gamma * pL) * rL);
   const T CR = vsqrt((gs.gamma * pR) * rR);
-  T ps_hist[kRiemannIters + 1];
-  bool floor_hit[kRiemannIters + 1];
+  // the forward iteration with its exit at a fixed point; pressures and W kept
+  T hp[kRiemannIters + 1], hL[kRiemannIters + 1], hR[kRiemannIters + 1];
+  unsigned floored = 0;   // bit k: the pressure of evaluation k was floored
   const T ps_raw0 = ((CR * pL + CL * pR) + (CL * CR) * (uL - uR)) / (CL + CR);
   T ps = vmax(ps_raw0, T(kPFloor));
-  floor_hit[0] = !(ps_raw0 > T(kPFloor));
-  ps_hist[0] = ps;
-  for (int it = 0; it < kRiemannIters; ++it) {
-    const Curve<T> cl = curve(ps, pL, CL, uL, T(-1), gs), cr = curve(ps, pR, CR, uR, T(1), gs);
-    const T raw = ps - ((cl.Z * cr.Z) * (cr.us - cl.us)) / (cl.Z + cr.Z);
-    ps = vmax(raw, T(kPFloor));
-    floor_hit[it + 1] = !(raw > T(kPFloor));
-    ps_hist[it + 1] = ps;
+  if (!(ps_raw0 > T(kPFloor))) floored |= 1u;
+  T WLs, WRs, uLs, uRs, ZL, ZR;
+  int last = 0;
+#pragma unroll 1
+  for (;; ++last) {
+    WLs = CL * vsqrt(T(1) + gs.g1 * (ps / pL - T(1)));
+    WRs = CR * vsqrt(T(1) + gs.g1 * (ps / pR - T(1)));
+    uLs = uL - (ps - pL) / WLs;
+    uRs = uR + (ps - pR) / WRs;
+    ZL = ((T(2) * WLs) * WLs) * WLs / (WLs * WLs + CL * CL);
+    ZR = ((T(2) * WRs) * WRs) * WRs / (WRs * WRs + CR * CR);
+    hp[last] = ps;
+    hL[last] = WLs;
+    hR[last] = WRs;
+    if (last == kRiemannIters) break;
+    const T raw = ps - ((ZL * ZR) * (uRs - uLs)) / (ZL + ZR);
+    const T pn = vmax(raw, T(kPFloor));
+    if (!(raw > T(kPFloor))) floored |= 2u << last;
+    if (pn == ps) break;
+    ps = pn;
   }
-  const Curve<T> cl = curve(ps, pL, CL, uL, T(-1), gs), cr = curve(ps, pR, CR, uR, T(1), gs);
-  const T Dz = cl.Z + cr.Z;
-  const T us = (cl.Z * cl.us + cr.Z * cr.us) / Dz;
+  const T iD = T(1) / (ZL + ZR);
+  const T us = (ZL * uLs + ZR * uRs) / (ZL + ZR);
   const bool left = us >= T(0);
-  const T rs = left ? rL : rR, u_s = left ? uL : uR, p_s = left ? pL : pR, W_s = left ? cl.W : cr.W;
+  const T rs = left ? rL : rR, u_s = left ? uL : uR, p_s = left ? pL : pR, W_s = left ? WLs : WRs;
   const T t1 = left ? L[2] : R[2], t2 = left ? L[3] : R[3];
   const T v_s = left ? -uL : uR, v_star = left ? -us : us;
   const T tau = T(1) / rs - (ps - p_s) / (W_s * W_s);
   const T rstar_raw = (tau > T(0)) ? T(1) / tau : T(kRhoFloor);
   const T rstar = vmax(rstar_raw, T(kRhoFloor));
-  const T c_s = vsqrt((gs.gamma * p_s) / rs);
-  const T c_star = vsqrt((gs.gamma * ps) / rstar);
   const bool shock = ps > p_s;
-  const T head = shock ? v_s + W_s / rs : v_s + c_s;
-  const T tail = shock ? head : v_star + c_star;
+  T c_s = T(0), c_star = T(0), head, tail;
+  if (shock) {
+    head = tail = v_s + W_s / rs;
+  } else {
+    c_s = vsqrt((gs.gamma * p_s) / rs);
+    c_star = vsqrt((gs.gamma * ps) / rstar);
+    head = v_s + c_s;
+    tail = v_star + c_star;
+  }
   const bool orig = head <= T(0);
   const bool star = !orig && (tail > T(0));
-  T r, u, p, w = T(0);
+  const bool fan = !orig && !star;
+  T r, u, p, w = T(0), iht = T(0);
   if (orig) {
     r = rs; u = u_s; p = p_s;
   } else if (star) {
     r = rstar; u = us; p = ps;
   } else {
-    w = head / (head - tail);
-    r = rs + w * (rstar - rs);
-    u = u_s + w * (us - u_s);
-    p = p_s + w * (ps - p_s);
+    iht = T(1) / (head - tail);
+    w = head * iht;
+    r = vfma(w, rstar - rs, rs);
+    u = vfma(w, us - u_s, u_s);
+    p = vfma(w, ps - p_s, p_s);
   }
   // flux
   const T f0 = r * u;
-  const T E = p * gs.inv_gm1 + (T(0.5) * r) * (u * u + (t1 * t1 + t2 * t2));
+  const T tt = vfma(t1, t1, t2 * t2);
+  const T k2 = vfma(u, u, tt);
+  const T E = vfma(p, gs.inv_gm1, (T(0.5) * r) * k2);
   const T Eb = Fb[4] * u;
-  const T f0b = Fb[0] + Fb[1] * u + Fb[2] * t1 + Fb[3] * t2;
-  T ub = Fb[1] * f0 + Fb[4] * (E + p) + f0b * r + Eb * (T(0.5) * r) * (T(2) * u);
-  T pb = Fb[1] + Fb[4] * u + Eb * gs.inv_gm1;
-  T rb = f0b * u + Eb * (T(0.5) * (u * u + (t1 * t1 + t2 * t2)));
-  const T t1b = Fb[2] * f0 + Eb * (T(0.5) * r) * (T(2) * t1);
-  const T t2b = Fb[3] * f0 + Eb * (T(0.5) * r) * (T(2) * t2);
+  const T Er = Eb * r;
+  const T f0b = vfma(Fb[1], u, vfma(Fb[2], t1, vfma(Fb[3], t2, Fb[0])));
+  const T ub = vfma(Fb[1], f0, vfma(Fb[4], E + p, vfma(f0b, r, Er * u)));
+  const T pb = vfma(Fb[4], u, vfma(Eb, gs.inv_gm1, Fb[1]));
+  const T rb = vfma(f0b, u, T(0.5) * Eb * k2);
+  const T t1b = vfma(Fb[2], f0, Er * t1);
+  const T t2b = vfma(Fb[3], f0, Er * t2);
   // sampling
-  T rsb = 0, u_sb = 0, p_sb = 0, W_sb = 0, rstarb = 0, usb = 0, psb = 0, v_sb = 0, v_starb = 0, c_sb = 0,
-    c_starb = 0;
+  T rsb = 0, u_sb = 0, p_sb = 0, W_sb = 0, rstarb = 0, usb = 0, psb = 0, v_sb = 0, v_starb = 0;
   if (orig) {
-    rsb += rb; u_sb += ub; p_sb += pb;
+    rsb = rb; u_sb = ub; p_sb = pb;
   } else if (star) {
-    rstarb += rb; usb += ub; psb += pb;
-  } else {
-    const T wb = rb * (rstar - rs) + ub * (us - u_s) + pb * (ps - p_s);
-    rsb += rb * (T(1) - w); rstarb += rb * w;
-    u_sb += ub * (T(1) - w); usb += ub * w;
-    p_sb += pb * (T(1) - w); psb += pb * w;
-    const T den = head - tail;
-    const T headb = wb * (-tail) / (den * den);
-    const T tailb = wb * head / (den * den);
-    v_sb += headb; c_sb += headb;          // rarefaction: head = v_s + c_s
-    v_starb += tailb; c_starb += tailb;    //              tail = v* + c*
+    rstarb = rb; usb = ub; psb = pb;
   }
-  {  // c_star = sqrt(gamma*ps/rstar)
-    const T x = (gs.gamma * ps) / rstar;
-    const T xb = c_starb / (T(2) * c_star);
-    psb += xb * gs.gamma / rstar;
-    rstarb -= xb * x / rstar;
-  }
-  {  // c_s = sqrt(gamma*p_s/rs)
-    const T x = (gs.gamma * p_s) / rs;
-    const T xb = c_sb / (T(2) * c_s);
-    p_sb += xb * gs.gamma / rs;
-    rsb -= xb * x / rs;
+  const T irs = T(1) / rs;
+  if (fan) {   // rarefaction: head = v_s + c_s, tail = v* + c*, c = sqrt(gamma p / rho)
+    const T wb = vfma(rb, rstar - rs, vfma(ub, us - u_s, pb * (ps - p_s)));
+    rstarb = rb * w; rsb = rb - rstarb;
+    usb = ub * w; u_sb = ub - usb;
+    psb = pb * w; p_sb = pb - psb;
+    v_sb = -wb * tail * (iht * iht);
+    v_starb = wb * w * iht;
+    const T sb = T(0.5) * v_sb / c_s, xb = T(0.5) * v_starb / c_star, irst = T(1) / rstar;
+    p_sb = vfma(sb * gs.gamma, irs, p_sb);
+    rsb = vfma(-sb * gs.gamma * p_s, irs * irs, rsb);
+    psb = vfma(xb * gs.gamma, irst, psb);
+    rstarb = vfma(-xb * gs.gamma * ps, irst * irst, rstarb);
   }
   if (rstar_raw > T(kRhoFloor) && tau > T(0)) {  // rstar = 1/tau
     const T taub = -rstarb * rstar * rstar;
-    rsb -= taub / (rs * rs);
-    const T w2 = W_s * W_s;
-    psb -= taub / w2;
-    p_sb += taub / w2;
-    W_sb += taub * T(2) * (ps - p_s) / (w2 * W_s);
+    rsb = vfma(-taub, irs * irs, rsb);
+    const T iW = T(1) / W_s, tw = taub * iW * iW;
+    psb -= tw;
+    p_sb += tw;
+    W_sb = T(2) * tw * (ps - p_s) * iW;
   }
-  T Lb_[5] = {0, 0, 0, 0, 0}, Rb_[5] = {0, 0, 0, 0, 0};
-  if (left) {
-    Lb_[0] += rsb; Lb_[1] += u_sb - v_sb; Lb_[4] += p_sb; Lb_[2] += t1b; Lb_[3] += t2b;
-    usb -= v_starb;
-  } else {
-    Rb_[0] += rsb; Rb_[1] += u_sb + v_sb; Rb_[4] += p_sb; Rb_[2] += t1b; Rb_[3] += t2b;
-    usb += v_starb;
-  }
-  // us = (ZL*usL + ZR*usR)/Dz
-  T ZLb = usb * (cl.us - us) / Dz, ZRb = usb * (cr.us - us) / Dz;
-  T usLb = usb * cl.Z / Dz, usRb = usb * cr.Z / Dz;
-  T WLb = left ? W_sb : T(0), WRb = left ? T(0) : W_sb;
-  T CLb = 0, CRb = 0;
-  curve_bwd(ps, pL, CL, T(-1), gs, cl, usLb, ZLb, WLb, psb, Lb_[4], CLb, Lb_[1]);
-  curve_bwd(ps, pR, CR, T(1), gs, cr, usRb, ZRb, WRb, psb, Rb_[4], CRb, Rb_[1]);
-  // Newton iterations in reverse: ps_{k+1} = max(ps_k - q(ps_k), floor)
-  for (int it = kRiemannIters - 1; it >= 0; --it) {
-    if (floor_hit[it + 1]) {
+  usb += left ? -v_starb : v_starb;
+  ShockSide<T> a, b;
+  a.p = pL; a.C = CL; a.ip = T(1) / pL; a.iC = T(1) / CL; a.sgn = T(-1);
+  b.p = pR; b.C = CR; b.ip = T(1) / pR; b.iC = T(1) / CR; b.sgn = T(1);
+  a.pb = a.Cb = a.ub = b.pb = b.Cb = b.ub = T(0);
+  // us = (ZL*usL + ZR*usR)/D
+  psb += shock_side_bwd(a, ps, WLs, usb * ZL * iD, usb * (uLs - us) * iD, left ? W_sb : T(0), gs);
+  psb += shock_side_bwd(b, ps, WRs, usb * ZR * iD, usb * (uRs - us) * iD, left ? T(0) : W_sb, gs);
+  // Newton iterations in reverse, p_{k+1} = max(p_k - q(p_k), floor): those
+  // after a fixed point all have its derivative m = 1 - q', so n of them pass
+  // psb m^n on and add (1 + m + ... + m^(n-1)) times one iteration's adjoints
+  int reps = kRiemannIters - last;
+#pragma unroll 1
+  for (int it = reps > 0 ? last : last - 1; it >= 0; --it, reps = 1) {
+    if (reps == 0) reps = 1;
+    if (floored & (2u << it)) {
       psb = T(0);
       continue;
     }
-    const T pk = ps_hist[it];
-    const Curve<T> a = curve(pk, pL, CL, uL, T(-1), gs), b = curve(pk, pR, CR, uR, T(1), gs);
-    const T D = a.Z + b.Z, du = b.us - a.us;
-    const T q = ((a.Z * b.Z) * du) / D;
-    const T qb = -psb;   // psb of ps_k accumulates the direct term below
-    const T aZb = qb * (b.Z * du - q) / D;
-    const T bZb = qb * (a.Z * du - q) / D;
-    const T dub = qb * (a.Z * b.Z) / D;
-    T pkb = psb;
-    curve_bwd(pk, pL, CL, T(-1), gs, a, -dub, aZb, T(0), pkb, Lb_[4], CLb, Lb_[1]);
-    curve_bwd(pk, pR, CR, T(1), gs, b, dub, bZb, T(0), pkb, Rb_[4], CRb, Rb_[1]);
-    psb = pkb;
+    const T pk = hp[it], WA = hL[it], WB = hR[it];
+    const T ZA = T(2) * WA * WA * WA / vfma(WA, WA, CL * CL), ZB = T(2) * WB * WB * WB / vfma(WB, WB, CR * CR);
+    const T iZ = T(1) / (ZA + ZB);
+    const T du = (uR + (pk - pR) / WB) - (uL - (pk - pL) / WA);
+    const T zz = ZA * ZB * iZ, q = zz * du;
+    ShockSide<T> x = a, y = b;   // one iteration's adjoints for psb = 1
+    x.pb = x.Cb = x.ub = y.pb = y.Cb = y.ub = T(0);
+    T m = T(1);
+    m += shock_side_bwd(x, pk, WA, zz, -vfma(ZB, du, -q) * iZ, T(0), gs);
+    m += shock_side_bwd(y, pk, WB, -zz, -vfma(ZA, du, -q) * iZ, T(0), gs);
+    T sum = T(0);
+    for (int k = 0; k < reps; ++k) {
+      sum += psb;
+      psb *= m;
+    }
+    a.pb = vfma(sum, x.pb, a.pb); a.Cb = vfma(sum, x.Cb, a.Cb); a.ub = vfma(sum, x.ub, a.ub);
+    b.pb = vfma(sum, y.pb, b.pb); b.Cb = vfma(sum, y.Cb, b.Cb); b.ub = vfma(sum, y.ub, b.ub);
   }
-  if (!floor_hit[0]) {  // ps0 = ((CR pL + CL pR) + (CL CR)(uL - uR)) / (CL + CR)
-    const T Dn = CL + CR;
-    const T num = (CR * pL + CL * pR) + (CL * CR) * (uL - uR);
-    const T nb = psb / Dn;
-    const T Dnb = -psb * num / (Dn * Dn);
-    Lb_[4] += nb * CR;
-    Rb_[4] += nb * CL;
-    CLb += nb * (pR + CR * (uL - uR)) + Dnb;
-    CRb += nb * (pL + CL * (uL - uR)) + Dnb;
-    Lb_[1] += nb * (CL * CR);
-    Rb_[1] -= nb * (CL * CR);
+  if (!(floored & 1u)) {  // p_0 = ((CR pL + CL pR) + (CL CR)(uL - uR)) / (CL + CR)
+    const T nb = psb / (CL + CR), du = uL - uR, cc = nb * CL * CR;
+    a.pb = vfma(nb, CR, a.pb);
+    b.pb = vfma(nb, CL, b.pb);
+    a.Cb = vfma(nb, vfma(CR, du, pR) - ps_raw0, a.Cb);
+    b.Cb = vfma(nb, vfma(CL, du, pL) - ps_raw0, b.Cb);
+    a.ub += cc;
+    b.ub -= cc;
   }
-  // CK = sqrt(gamma*pK*rK)
-  Lb_[4] += CLb * (gs.gamma * rL) / (T(2) * CL);
-  Lb_[0] += CLb * (gs.gamma * pL) / (T(2) * CL);
-  Rb_[4] += CRb * (gs.gamma * rR) / (T(2) * CR);
-  Rb_[0] += CRb * (gs.gamma * pR) / (T(2) * CR);
-  for (int q2 = 0; q2 < 5; ++q2) {
-    Lb[q2] += Lb_[q2];
-    Rb[q2] += Rb_[q2];
-  }
+  // C = sqrt(gamma p rho)
+  const T ga = T(0.5) * gs.gamma * a.Cb * a.iC, gb = T(0.5) * gs.gamma * b.Cb * b.iC;
+  Lb[0] += vfma(ga, pL, left ? rsb : T(0));
+  Lb[1] += a.ub + (left ? u_sb - v_sb : T(0));
+  Lb[2] += left ? t1b : T(0);
+  Lb[3] += left ? t2b : T(0);
+  Lb[4] += vfma(ga, rL, a.pb + (left ? p_sb : T(0)));
+  Rb[0] += vfma(gb, pR, left ? T(0) : rsb);
+  Rb[1] += b.ub + (left ? T(0) : u_sb + v_sb);
+  Rb[2] += left ? T(0) : t1b;
+  Rb[3] += left ? T(0) : t2b;
+  Rb[4] += vfma(gb, rR, b.pb + (left ? T(0) : p_sb));
 }
 
 // The flux at the interface between cells 3 and 4 of an 8-cell window of
@@ -599,7 +610,7 @@ CELLO_HD void window_flux_vjp(const T U[8][5], T dtdx, const Gas<T>& gs, const T
   for (int c = 6; c >= 1; --c)
     for (int q = 0; q < 5; ++q) limited_slope_bwd(W[c - 1][q], W[c][q], W[c + 1][q], dmb[c][q], Wb[c - 1][q], Wb[c][q],
                                                   Wb[c + 1][q]);
-  for (int c = 0; c < 8; ++c) to_primitive_bwd(U[c], gs, Wb[c], Ub[c]);
+  for (int c = 0; c < 8; ++c) to_primitive_bwd(W[c], gs, Wb[c], Ub[c]);
 }
 
 }  // namespace cello

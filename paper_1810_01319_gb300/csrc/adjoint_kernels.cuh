@@ -9,23 +9,48 @@ namespace cello {
 
 // ---------------------------------------------------------------------
 // Adjoint sweep.  The forward sweep maps U to U' with
-//   U'_j = U_j - (dt/dx) (F_{j+1/2} - F_{j-1/2})  for updated cells j,
-// F_{c+1/2} a function of cells c-3..c+4.  Given lam' (adjoint of U'), the
-// adjoint of U is lam_j = lam'_j + sum_c (dF_c/dU_j)^T mu_c with
-// mu_c = (dt/dx)(m_{c+1} lam'_{c+1} - m_c lam'_c), m = 1 on updated cells.
-// One CTA item = P pencils; phase 1 stages U and lam', phase 2 computes
-// each interface's vector-Jacobian product into shared memory, phase 3
-// gathers the eight contributions of each cell in a fixed order.
+//   U'_j = U_j - (dt/dx) (F_{j+1/2} - F_{j-1/2})  for updated cells j.
+// Given lam' (adjoint of U'), the flux at interface c|c+1 gets the adjoint
+// mu_c = (dt/dx)(m_{c+1} lam'_{c+1} - m_c lam'_c), m = 1 on updated cells, and
+// lam = lam' + (dF/dU)^T mu is the sweep in reverse.  One CTA item = P
+// pencils, one thread per cell and pencil, the pencils of a cell in one warp;
+// the sweep's phases run forward (primitives, slopes and shock detector,
+// interface values, edge values and tracing) and then backward (Riemann
+// problem, tracing and edge values, interface values, slopes and shock
+// detector, primitives), each quantity and its adjoint evaluated once per cell
+// or interface and handed to the neighbours through shared memory.
+//
+// The float64 kernel is bound by the float64 pipe (1.6 lanes per SM and clock
+// measured).  Evaluating each interface's whole eight-cell stencil in its own
+// thread ran every primitive, slope and edge value up to eight times: three
+// steps of a gradient on 64 leaves of 16^3 took 99.9 ms; with reciprocals shared
+// per divisor and the Newton reverse from the stored history 69.1 ms; each
+// quantity once, as here, 38.2 ms.
+// P: enough pencils that the cells without an edge state (three at each end)
+// leave whole warps idle rather than lanes, within the registers of one CTA.
 // ---------------------------------------------------------------------
-template <typename T, int NB, int P>
-__global__ void __launch_bounds__((NB + 8) * P)
+template <typename T, int NB>
+constexpr size_t adjoint_smem() {
+  constexpr int A = (NB + 2 * kGhosts) * adj_pencils(NB);
+  return (sizeof(T) * 33 + sizeof(int)) * A;
+}
+
+template <typename T, int NB>
+__global__ void __launch_bounds__((NB + 8) * adj_pencils(NB))
 adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
-  constexpr int G = kGhosts, N = NB + 2 * G, S = P + 1, A = N * S, NI = NB + 1;
+  constexpr int G = kGhosts, N = NB + 2 * G, P = adj_pencils(NB), A = N * P;
   constexpr long SLAB = (long)N * N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sU = reinterpret_cast<T*>(smem_raw);
-  T* sL = sU + 5 * A;
-  T* sC = sL + 5 * A;   // [NI][8][5][P]
+  T* sW = reinterpret_cast<T*>(smem_raw);   // primitives
+  T* sLam = sW + 5 * A;                      // lam', then lam
+  T* sD = sLam + 5 * A;                      // slopes, then adjoints they give cell j-1
+  T* sI = sD + 5 * A;                        // interface values j+1/2, then slope adjoints for cell j+1
+  T* sL = sI + 5 * A;                        // left edge states, their adjoints, adjoints of interface j-1/2
+  T* sR = sL + 5 * A;                        // right edge states, their adjoints, adjoints of interface j+1/2
+  T* sFT = sR + 5 * A;                       // shock detector, then its adjoint for p of cells j+-1
+  T* sF2 = sFT + A;                          // its adjoint for p of cells j+-2
+  T* sFb = sF2 + A;                          // adjoint of the flattening coefficient
+  int* sSel = reinterpret_cast<int*>(sFb + A);   // which detector it was taken from (-1, 0, 1)
 
   const Gas<T> gs = Gas<T>::make(m.gamma);
   const T* U = static_cast<const T*>(prm.U);
@@ -40,8 +65,9 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
   comp[2] = axis == 0 ? 2 : 1;
   comp[3] = axis == 2 ? 2 : 3;
   const int t = threadIdx.x;
-  const int lc = axis == 0 ? t % N : t / P;
-  const int lp = axis == 0 ? t / N : t % P;
+  // cell and pencil moved to and from memory (along x first on the x sweep), and computed
+  const int mc = axis == 0 ? t % N : t / P, mp = axis == 0 ? t / N : t % P;
+  const int j = t / P, at = t, p = t % P;
   __shared__ T s_dtdx[16];
   if (t <= m.max_level) s_dtdx[t] = T(*prm.dt / ldexp(m.dx0, -t));
   __syncthreads();
@@ -50,32 +76,84 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
     const int leaf = prm.leaf0 + item / prm.tiles_per_leaf;
     const int tile = item % prm.tiles_per_leaf;
     const T dtdx = s_dtdx[m.leaf[leaf].x];
-    const int q = tile * P + lp;
-    const bool valid = q < cA * cB;
-    const int pa = prm.a0 + (valid ? q / cB : 0), pb = prm.b0 + (valid ? q % cB : 0);
-    const long off = (long)leaf * 5 * SLAB + pa * sTA + pb * sTB + lc * sAx;
-    if (valid) {
+    const int mq = tile * P + mp;
+    const bool moves = mq < cA * cB;
+    const int ma = prm.a0 + (moves ? mq / cB : 0), mb = prm.b0 + (moves ? mq % cB : 0);
+    const long off = (long)leaf * 5 * SLAB + ma * sTA + mb * sTB + mc * sAx;
+    {
+      T Us[5], W[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) Us[k] = moves ? U[off + comp[k] * SLAB] : T(1);
+      to_primitive(Us, gs, W);
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
-        sU[k * A + lc * S + lp] = U[off + comp[k] * SLAB];
-        sL[k * A + lc * S + lp] = lam[off + comp[k] * SLAB];
+        sW[k * A + mc * P + mp] = W[k];
+        sLam[k * A + mc * P + mp] = moves ? lam[off + comp[k] * SLAB] : T(0);
       }
     }
     __syncthreads();
-    if (t < NI * P) {
-      const int p = t % P, ci = t / P, c = 3 + ci;
-      const T m0 = (c >= G && c < G + NB) ? T(1) : T(0);
-      const T m1 = (c + 1 >= G && c + 1 < G + NB) ? T(1) : T(0);
-      T mu[5];
+    // ---- forward: slopes and shock detector, interface values, edge states
+    T ft = T(0);
+    if (j >= 2 && j <= N - 3) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const T* a = sW + k * A + at;
+        sD[k * A + at] = limited_slope(a[-P], a[0], a[P]);
+      }
+      const T *pr = sW + 4 * A + at, *un = sW + A + at;
+      ft = flatten_tilde(pr[-2 * P], pr[-P], pr[P], pr[2 * P], un[-P], un[P]);
+    }
+    sFT[at] = ft;
+    __syncthreads();
+    if (j >= 2 && j <= N - 4) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k)
+        sI[k * A + at] = interface_value(sW[k * A + at], sW[k * A + at + P], sD[k * A + at], sD[k * A + at + P]);
+    }
+    __syncthreads();
+    const bool traced = j >= 3 && j <= N - 4;
+    T f = T(0), aL[5], aR[5];
+    int sel = 0;
+    if (traced) {
+      const T* pr = sW + 4 * A + at;
+      const T s = pr[P] - pr[-P];
+      const T fm = sFT[at - P], fp = sFT[at + P];
+      f = ft;
+      if (s > T(0)) {
+        if (!(ft > fm)) { f = fm; sel = -1; }
+      } else if (s < T(0)) {
+        if (!(ft > fp)) { f = fp; sel = 1; }
+      }
+      T W[5], Wm[5], Wp[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        W[k] = sW[k * A + at];
+        aL[k] = sI[k * A + at - P];
+        aR[k] = sI[k * A + at];
+        flatten_monotone(W[k], f, aL[k], aR[k]);
+      }
+      trace(W, aL, aR, dtdx, gs, Wm, Wp);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        sL[k * A + at] = Wm[k];
+        sR[k * A + at] = Wp[k];
+      }
+    }
+    __syncthreads();
+    // ---- backward: the Riemann problem at j+1/2 turns the states beside it into their adjoints
+    if (j >= 3 && j <= N - 5) {
+      const T m0 = (j >= G) ? T(1) : T(0);
+      const T m1 = (j + 1 < G + NB) ? T(1) : T(0);
+      T mu[5], Lb[5], Rb[5];
       bool any = false;
 #pragma unroll
-      for (int k = 0; k < 5; ++k) mu[k] = dtdx * (m1 * sL[k * A + (c + 1) * S + p] - m0 * sL[k * A + c * S + p]);
-      if (prm.regb && (c == G - 1 || c == G + NB - 1)) {   // flux kept for the coarse-fine correction
-        const int qq = tile * P + p;
-        if (qq < cA * cB) {
-          const int ca = prm.a0 + qq / cB, cb = prm.b0 + qq % cB;
+      for (int k = 0; k < 5; ++k) mu[k] = dtdx * (m1 * sLam[k * A + at + P] - m0 * sLam[k * A + at]);
+      if (prm.regb && (j == G - 1 || j == G + NB - 1)) {   // flux kept for the coarse-fine correction
+        const int q = tile * P + p;
+        if (q < cA * cB) {
+          const int ca = prm.a0 + q / cB, cb = prm.b0 + q % cB;
           if (ca >= G && ca < G + NB && cb >= G && cb < G + NB) {
-            const int slot = m.face_slot[leaf * 6 + 2 * axis + (c == G - 1 ? 0 : 1)];
+            const int slot = m.face_slot[leaf * 6 + 2 * axis + (j == G - 1 ? 0 : 1)];
             if (slot >= 0) {
               const double* r = prm.regb + (long)slot * 5 * NB * NB + (ca - G) * NB + (cb - G);
 #pragma unroll
@@ -85,35 +163,114 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
         }
       }
 #pragma unroll
-      for (int k = 0; k < 5; ++k) any = any || (mu[k] != T(0));
-      T Ub[8][5];
-#pragma unroll
-      for (int c8 = 0; c8 < 8; ++c8)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) Ub[c8][k] = T(0);
-      if (any) {
-        T W8[8][5];
-#pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8)
-#pragma unroll
-          for (int k = 0; k < 5; ++k) W8[c8][k] = sU[k * A + (c - 3 + c8) * S + p];
-        window_flux_vjp(W8, dtdx, gs, mu, Ub);
+      for (int k = 0; k < 5; ++k) {
+        any = any || (mu[k] != T(0));
+        Lb[k] = Rb[k] = T(0);
       }
+      if (any) {
+        T L[5], R[5];
 #pragma unroll
-      for (int c8 = 0; c8 < 8; ++c8)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) sC[((ci * 8 + c8) * 5 + k) * P + p] = Ub[c8][k];
-    }
-    __syncthreads();
-    if (valid) {
-      const int ci0 = lc - 7 > 0 ? lc - 7 : 0;
-      const int ci1 = lc < NI - 1 ? lc : NI - 1;
+        for (int k = 0; k < 5; ++k) {
+          L[k] = sR[k * A + at];
+          R[k] = sL[k * A + at + P];
+        }
+        riemann_flux_bwd(L, R, gs, mu, Lb, Rb);
+      }
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
-        T v = sL[k * A + lc * S + lp];
-        for (int ci = ci0; ci <= ci1; ++ci) v += sC[((ci * 8 + (lc - ci)) * 5 + k) * P + lp];
-        lam[off + comp[k] * SLAB] = v;
+        sR[k * A + at] = Lb[k];
+        sL[k * A + at + P] = Rb[k];
       }
+    }
+    // the first traced cell has no interface on its left, the last none on its right
+    if (j == 3)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sL[k * A + at] = T(0);
+    if (j == N - 4)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sR[k * A + at] = T(0);
+    __syncthreads();
+    // ---- tracing and the edge values
+    T Wb[5] = {0, 0, 0, 0, 0};
+    T fb = T(0);
+    if (traced) {
+      T Wmb[5], Wpb[5];
+      bool any = false;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        Wmb[k] = sL[k * A + at];
+        Wpb[k] = sR[k * A + at];
+        any = any || Wmb[k] != T(0) || Wpb[k] != T(0);
+      }
+      if (any) {
+        T W[5], aLb[5] = {0, 0, 0, 0, 0}, aRb[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+        for (int k = 0; k < 5; ++k) W[k] = sW[k * A + at];
+        trace_bwd(W, aL, aR, dtdx, gs, Wmb, Wpb, Wb, aLb, aRb);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          T lb = T(0), rb = T(0);
+          flatten_monotone_bwd(W[k], f, sI[k * A + at - P], sI[k * A + at], aLb[k], aRb[k], Wb[k], fb, lb, rb);
+          sL[k * A + at] = lb;
+          sR[k * A + at] = rb;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sL[k * A + at] = sR[k * A + at] = T(0);
+    }
+    sFb[at] = fb;
+    sSel[at] = sel;
+    __syncthreads();
+    // ---- interface values, slopes, shock detector: cell j's share, the neighbours' left in shared memory
+    T d1 = T(0), d2 = T(0);
+    if (j >= 2 && j <= N - 3) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const T im = sR[k * A + at - P] + sL[k * A + at], ip = sR[k * A + at] + sL[k * A + at + P];
+        const T* a = sW + k * A + at;
+        T lo = T(0), own = T(0.5) * (im + ip), hi = T(0);
+        limited_slope_bwd(a[-P], a[0], a[P], (ip - im) * T(1.0 / 6.0), lo, own, hi);
+        Wb[k] += own;
+        sD[k * A + at] = lo;
+        sI[k * A + at] = hi;
+      }
+      T ftb = (sSel[at] == 0) ? fb : T(0);
+      if (sSel[at - P] == 1) ftb += sFb[at - P];
+      if (sSel[at + P] == -1) ftb += sFb[at + P];
+      if (ftb != T(0)) {
+        const T *pr = sW + 4 * A + at, *un = sW + A + at;
+        T m2 = T(0), m1 = T(0);
+        flatten_tilde_bwd(pr[-2 * P], pr[-P], pr[P], pr[2 * P], un[-P], un[P], ftb, m2, m1, d1, d2);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sD[k * A + at] = sI[k * A + at] = T(0);
+    }
+    sFT[at] = d1;
+    sF2[at] = d2;
+    __syncthreads();
+    // ---- primitives
+    {
+      T W[5], Ub[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        W[k] = sW[k * A + at];
+        if (j >= 1) Wb[k] += sI[k * A + at - P];
+        if (j <= N - 2) Wb[k] += sD[k * A + at + P];
+      }
+      if (j >= 1) Wb[4] += sFT[at - P];
+      if (j <= N - 2) Wb[4] -= sFT[at + P];
+      if (j >= 2) Wb[4] += sF2[at - 2 * P];
+      if (j <= N - 3) Wb[4] -= sF2[at + 2 * P];
+      to_primitive_bwd(W, gs, Wb, Ub);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sLam[k * A + at] += Ub[k];
+    }
+    __syncthreads();
+    if (moves) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) lam[off + comp[k] * SLAB] = sLam[k * A + mc * P + mp];
     }
     __syncthreads();
   }

@@ -11,7 +11,8 @@ namespace cello {
 
 constexpr int kGhosts = 4;
 constexpr int kFields = 5;
-constexpr int kAdjPencils = 4;       // pencils per adjoint-sweep CTA
+// Pencils per adjoint-sweep CTA for blocks of n cells per edge.
+constexpr int adj_pencils(int n) { return n == 32 ? 8 : 16; }
 
 // Launch variants of the PPM sweep: pencils per CTA, the minimum number of
 // resident CTAs per SM the register allocation is bounded for, and the

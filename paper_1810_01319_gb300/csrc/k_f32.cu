@@ -32,22 +32,16 @@ void launch_sweep_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
   }
 }
 
-template <int NB, int P>
-static size_t adj_smem() {
-  constexpr int N = NB + 2 * kGhosts;
-  return sizeof(float) * (10 * N * (P + 1) + (NB + 1) * 40 * P);
-}
-
 template <int NB>
 static void prepare_adj() {
-  cudaFuncSetAttribute(adjoint_sweep_kernel<float, NB, kAdjPencils>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)adj_smem<NB, kAdjPencils>());
+  cudaFuncSetAttribute(adjoint_sweep_kernel<float, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)adjoint_smem<float, NB>());
 }
 
 template <int NB>
 static void adj_sweep_n(const DevMesh& m, const AdjSweepParams& p, cudaStream_t s) {
-  constexpr int N = NB + 2 * kGhosts;
-  adjoint_sweep_kernel<float, NB, kAdjPencils><<<p.n_items, N * kAdjPencils, adj_smem<NB, kAdjPencils>(), s>>>(m, p);
+  constexpr int threads = (NB + 2 * kGhosts) * adj_pencils(NB);
+  adjoint_sweep_kernel<float, NB><<<p.n_items, threads, adjoint_smem<float, NB>(), s>>>(m, p);
 }
 
 void launch_adjoint_sweep_f32(const DevMesh& m, const AdjSweepParams& p, cudaStream_t s) {
