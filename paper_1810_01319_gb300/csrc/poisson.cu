@@ -3,28 +3,35 @@
 // block table of a uniform periodic mesh.
 //
 // Each leaf block carries its own grid on every level where a block still
-// has at least 4 cells per edge (n, n/2, ..., 4), as an array of padded
-// blocks [B][(n_l + 2)^3] with a one-cell ghost layer.  Before every stencil
-// the ghost layer is refreshed from the same-level neighbour blocks through
-// the 27-entry neighbour table of the hydro refresh (every ghost cell takes
-// the interior cell of the neighbour leaf in its direction; the periodic
-// wrap is in the table).  Below the last block level the restricted
-// residual of the blocks forms one grid of 2 cells per block edge, and the
-// remaining coarse levels are single arrays with periodic indexing (a block
-// of one or two cells has nothing left to exchange that the index wrap does
-// not already give).  float64, no contraction.
+// has at least 4 cells per edge (n, n/2, ..., 4), stored without ghost layers
+// ([B][n_l^3]; on the finest level the layout of the caller's f and phi): a
+// kernel stages a tile of a block with its halo in shared memory and reads the
+// halo from the same-level neighbour blocks through the 27-entry neighbour
+// table of the hydro refresh (the periodic wrap is in the table).  Below the
+// last block level the restricted residual of the blocks forms one grid of 2
+// cells per block edge with periodic indexing: tiles while the edge is a
+// multiple of 4, then every remaining level in one CTA.  float64, no
+// contraction.
+//
+// What bounds it: float32 cycles on large grids, HBM and L2 traffic, hence one
+// kernel per leg and level (two sweeps, residual and restriction read f once and
+// write phi once; interpolation and two sweeps read phi and f once and write
+// once); float64 cycles and the float64 residual of mixed ones, the float64 pipe;
+// small grids, the number of dependent launches (8 per mixed cycle on 64^3).
 //
 // V-cycle (spacing h): two damped Jacobi sweeps (w = 6/7), the residual of
 // the 8 children of each coarse cell restricted by their mean, a V-cycle for
 // the coarse error from zero with spacing 2h, its trilinear prolongation
 // added, two more sweeps; a 1-cell grid gives 0, an odd grid above 1 takes
 // 50 sweeps.  Mean of f removed first, mean of phi removed last.  Every value
-// is the oracle's expression in its order on the same grid values (the
-// block layout only changes where they are stored); the Laplacian's 1/h^2
-// and the Jacobi 1/6 are multiplications by reciprocals computed once.
+// is the plain expression in its order on the same grid values (the block
+// layout only changes where they are stored), with 1/h^2 and 1/6 as
+// multiplications by reciprocals computed once and the multiply-adds fused.
+#include <mutex>
 #include <vector>
 
 #include "cello_internal.h"
+#include "widen.cuh"
 
 namespace cello {
 namespace {
@@ -40,6 +47,31 @@ __device__ __forceinline__ unsigned gidx(int x, int y, int z, int M) {
   return ((unsigned)z * (unsigned)M + (unsigned)y) * (unsigned)M + (unsigned)x;
 }
 __device__ __forceinline__ int wrapm(int v, int M) { return v < 0 ? v + M : (v >= M ? v - M : v); }
+
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+
+// Damped Jacobi value of a cell from its value c, neighbour sum s and
+// right-hand side f: (1 - w) c + (w / 6) (s - h^2 f), 3 instructions.
+template <typename T>
+__device__ __forceinline__ T relax(T c, T s, T f, T h2) {
+  return mad(T(kOmega / 6.0), mad(-h2, f, s), T(1.0 - kOmega) * c);
+}
+// The same from a zero field (neighbour sum and cell 0).
+template <typename T>
+__device__ __forceinline__ T relax_zero(T f, T h2) {
+  return T(kOmega / 6.0) * (-h2 * f);
+}
+// f - lap(phi).
+template <typename T>
+__device__ __forceinline__ T residual_of(T c, T s, T f, T ih2) {
+  return mad(-ih2, mad(T(-6), c, s), f);
+}
+// Linear interpolation a quarter of the way from p to q.
+template <typename T>
+__device__ __forceinline__ T quarter(T p, T q) {
+  return mad(T(0.75), p, T(0.25) * q);
+}
 
 template <typename T>
 __device__ __forceinline__ T nbsum(const T* p, int x, int y, int z, int M) {
@@ -86,7 +118,7 @@ __global__ void jacobi_kernel(const T* __restrict__ in, T* __restrict__ out, con
     // the neighbour sum in the order of nbsum: x-1, x+1, y-1, y+1, z-1, z+1
     const T s = ((((in[zb + row + xm] + in[zb + row + xp]) + in[zb + rym + x]) + in[zb + ryp + x]) + cm) + cp;
     const unsigned i = zb + row + x;
-    out[i] = T(1.0 - kOmega) * cc + T(kOmega) * ((s - h2 * f[i]) * T(1.0 / 6.0));
+    out[i] = relax(cc, s, f[i], h2);
     cm = cc;
     cc = cp;
     zb += P;
@@ -109,31 +141,32 @@ __global__ void residual_restrict_kernel(const T* __restrict__ phi, const T* __r
       for (int dx = 0; dx < 2; ++dx) {
         const int x = 2 * X + dx, y = 2 * Y + dy, z = 2 * Z + dz;
         const unsigned o = gidx(x, y, z, M);
-        const T r = f[o] - (nbsum(phi, x, y, z, M) - T(6) * phi[o]) * ih2;
+        const T r = residual_of(phi[o], nbsum(phi, x, y, z, M), f[o], ih2);
         s = first ? r : s + r;
         first = false;
       }
   fc[i] = s * T(0.125);
 }
 
-// phi += trilinear prolongation of the coarse error ec.
+// Trilinear prolongation of the coarse error ec (Mc cells per edge) at a fine cell.
 template <typename T>
-__global__ void prolong_add_kernel(const T* __restrict__ ec, T* __restrict__ phi, int M) {
-  const int Mc = M / 2;
-  int x, y, z;
-  if (!cell3(M, x, y, z)) return;
-  const unsigned i = gidx(x, y, z, M);
+__device__ __forceinline__ T prolonged(const T* ec, int x, int y, int z, int Mc) {
   const int X = x >> 1, Y = y >> 1, Z = z >> 1;
   const int sx = (x & 1) ? 1 : -1, sy = (y & 1) ? 1 : -1, sz = (z & 1) ? 1 : -1;
   const int X1 = wrapm(X + sx, Mc), Y1 = wrapm(Y + sy, Mc), Z1 = wrapm(Z + sz, Mc);
-  const T a = T(0.75), q = T(0.25);
-  const T c00 = a * ec[gidx(X, Y, Z, Mc)] + q * ec[gidx(X1, Y, Z, Mc)];
-  const T c10 = a * ec[gidx(X, Y1, Z, Mc)] + q * ec[gidx(X1, Y1, Z, Mc)];
-  const T c01 = a * ec[gidx(X, Y, Z1, Mc)] + q * ec[gidx(X1, Y, Z1, Mc)];
-  const T c11 = a * ec[gidx(X, Y1, Z1, Mc)] + q * ec[gidx(X1, Y1, Z1, Mc)];
-  const T c0 = a * c00 + q * c10;
-  const T c1 = a * c01 + q * c11;
-  phi[i] = phi[i] + (a * c0 + q * c1);
+  const T c00 = quarter(ec[gidx(X, Y, Z, Mc)], ec[gidx(X1, Y, Z, Mc)]);
+  const T c10 = quarter(ec[gidx(X, Y1, Z, Mc)], ec[gidx(X1, Y1, Z, Mc)]);
+  const T c01 = quarter(ec[gidx(X, Y, Z1, Mc)], ec[gidx(X1, Y, Z1, Mc)]);
+  const T c11 = quarter(ec[gidx(X, Y1, Z1, Mc)], ec[gidx(X1, Y1, Z1, Mc)]);
+  return quarter(quarter(c00, c10), quarter(c01, c11));
+}
+
+template <typename T>
+__global__ void prolong_add_kernel(const T* __restrict__ ec, T* __restrict__ phi, int M) {
+  int x, y, z;
+  if (!cell3(M, x, y, z)) return;
+  const unsigned i = gidx(x, y, z, M);
+  phi[i] = phi[i] + prolonged(ec, x, y, z, M / 2);
 }
 
 template <typename T>
@@ -147,37 +180,24 @@ __global__ void add_kernel(double* p, long count, const double* shift, double sc
   if (i < count) p[i] = p[i] - *shift * scale;
 }
 
-// Partial sums (op 0) or max |residual| (op 1) per CTA, then one CTA folds them.
-__global__ void reduce_kernel(const double* __restrict__ a, const double* __restrict__ f, long count, int M,
-                              double ih2, int op, double* __restrict__ partial) {
+// Partial sums per CTA; one CTA folds them (or maxima: op 1).
+__global__ void reduce_kernel(const double* __restrict__ a, long count, double* __restrict__ partial) {
   __shared__ double sh[kRedThreads];
   double acc = 0.0;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x) {
-    if (op == 0) {
-      acc += a[i];
-    } else {
-      const unsigned u = (unsigned)i, uM = (unsigned)M;   // M^3 <= 2^30: 32-bit index arithmetic
-      const int x = (int)(u % uM), y = (int)((u / uM) % uM), z = (int)(u / (uM * uM));
-      const double r = fabs(f[i] - (nbsum(a, x, y, z, M) - 6.0 * a[i]) * ih2);
-      acc = r > acc ? r : acc;
-    }
-  }
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x) acc += a[i];
   sh[threadIdx.x] = acc;
   __syncthreads();
   for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      const double o = sh[threadIdx.x + s];
-      sh[threadIdx.x] = op == 0 ? sh[threadIdx.x] + o : (o > sh[threadIdx.x] ? o : sh[threadIdx.x]);
-    }
+    if (threadIdx.x < s) sh[threadIdx.x] = sh[threadIdx.x] + sh[threadIdx.x + s];
     __syncthreads();
   }
   if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
 }
 
-__global__ void fold_kernel(const double* __restrict__ partial, int n, int op, double scale, double* out) {
+__global__ void fold_kernel(const double* __restrict__ partial, long n, int op, double scale, double* out) {
   __shared__ double sh[kRedThreads];
   double acc = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) acc = op == 0 ? acc + partial[i] : fmax(acc, partial[i]);
+  for (long i = threadIdx.x; i < n; i += blockDim.x) acc = op == 0 ? acc + partial[i] : fmax(acc, partial[i]);
   sh[threadIdx.x] = acc;
   __syncthreads();
   for (int s = kRedThreads / 2; s > 0; s >>= 1) {
@@ -189,323 +209,555 @@ __global__ void fold_kernel(const double* __restrict__ partial, int n, int op, d
 }
 
 // ---------------------------------------------------------------------------
-// Block levels: arrays of padded blocks [B][P^3], P = n + 2 (one ghost cell),
-// interior cells at padded coordinates 1 .. n.
-__device__ __forceinline__ long bidx(int b, int x, int y, int z, int P) {
-  return (((long)b * P + z) * P + y) * P + x;
-}
+// Tile levels: arrays [B][n^3] of blocks without ghost layers; a CTA stages one
+// E^3 tile of a block and a halo of one or two cells in shared memory, the halo
+// cells read from the neighbour blocks through the 27-entry table (a periodic
+// single array is one block that is its own neighbour in all 27 directions).
+// Two cells of halo let one kernel run two sweeps and a residual, or an
+// interpolation and two sweeps, on values that never leave the SM.
+struct TileLevel {
+  int n;                 // cells per block edge
+  const int* idx;        // [B][27] neighbour blocks, or null: one periodic block
+};
 
-// Block edges are powers of two (n, n/2, ..., 4): global cell gid of a
-// level -> block b and padded coordinates of its interior cell (x fastest),
-// by shifts and masks.
-__device__ __forceinline__ int blk_cell(long gid, int n, int& x, int& y, int& z) {
-  const int ln = __ffs(n) - 1;
-  const int c = (int)(gid & (((long)1 << (3 * ln)) - 1));
-  x = (c & (n - 1)) + 1;
-  y = ((c >> ln) & (n - 1)) + 1;
-  z = (c >> (2 * ln)) + 1;
-  return (int)(gid >> (3 * ln));
-}
+// A CTA's tile: block b, its 27 neighbours in shared memory, origin (x, y, z).
+template <int E>
+struct Tile {
+  int b, x, y, z;
+};
 
-// Ghost layer of every block: each ghost cell takes the interior cell of the
-// same-level neighbour leaf in its direction (the 27-entry table; the mesh
-// is uniform and periodic, so every entry is a same-level leaf).  Ghost cell
-// q of a block: the z planes 0 and P-1, then the y rows 0 and P-1 of the
-// interior z planes, then the x columns 0 and P-1 of the interior rows.
-template <typename T>
-__global__ void blk_refresh_kernel(DevMesh m, T* a, int n, int B) {
-  const int P = n + 2;
-  const long per = (long)P * P * P - (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * per) return;
-  const int b = (int)(gid / per);
-  int q = (int)(gid - (long)b * per);
-  int x, y, z;
-  if (q < 2 * P * P) {
-    z = q < P * P ? 0 : P - 1;
-    q %= P * P;
-    y = q / P;
-    x = q % P;
-  } else if (q < 2 * P * P + 2 * n * P) {
-    q -= 2 * P * P;
-    z = 1 + q / (2 * P);
-    const int r = q % (2 * P);
-    y = r < P ? 0 : P - 1;
-    x = r % P;
-  } else {
-    q -= 2 * P * P + 2 * n * P;
-    z = 1 + q / (2 * n);
-    const int r = q % (2 * n);
-    y = 1 + r / 2;
-    x = (r & 1) ? P - 1 : 0;
-  }
-  const int d0 = x == 0 ? -1 : (x == P - 1 ? 1 : 0);
-  const int d1 = y == 0 ? -1 : (y == P - 1 ? 1 : 0);
-  const int d2 = z == 0 ? -1 : (z == P - 1 ? 1 : 0);
-  const int src = m.idx[b * 27 + (d2 + 1) * 9 + (d1 + 1) * 3 + (d0 + 1)];
-  a[bidx(b, x, y, z, P)] = a[bidx(src, x - d0 * n, y - d1 * n, z - d2 * n, P)];
-}
-
-template <typename T>
-__device__ __forceinline__ T bnbsum(const T* p, long i, int P) {
-  const long PP = (long)P * P;
-  return ((((p[i - 1] + p[i + 1]) + p[i - P]) + p[i + P]) + p[i - PP]) + p[i + PP];
-}
-
-// Damped Jacobi sweep over every block's interior (ghosts of `in` refreshed).
-template <typename T>
-__global__ void blk_jacobi_kernel(const T* __restrict__ in, T* __restrict__ out, const T* __restrict__ f, int n,
-                                  int B, T h2) {
-  const long n3 = (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * n3) return;
-  int x, y, z;
-  const int b = blk_cell(gid, n, x, y, z);
-  const int P = n + 2;
-  const long i = bidx(b, x, y, z, P);
-  out[i] = T(1.0 - kOmega) * in[i] + T(kOmega) * ((bnbsum(in, i, P) - h2 * f[i]) * T(1.0 / 6.0));
-}
-
-// Residual f - lap(phi) of the 8 children of each coarse cell, their mean in
-// (dz, dy, dx) order: into the next block level (g == nullptr) or into the
-// global grid of Mg cells per axis (coarse cell of block b at global
-// (i n/2 + X, j n/2 + Y, k n/2 + Z)).
-template <typename T>
-__global__ void blk_residual_restrict_kernel(DevMesh m, const T* __restrict__ phi, const T* __restrict__ f,
-                                             T* __restrict__ fc, T* __restrict__ g, int Mg, int n, int B, T ih2) {
-  const int nc = n / 2, P = n + 2, Pc = nc + 2;
-  const long nc3 = (long)nc * nc * nc;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * nc3) return;
-  int X, Y, Z;
-  const int b = blk_cell(gid, nc, X, Y, Z);   // padded: 1 .. nc
-  T s = T(0);
-  bool first = true;
-  for (int dz = 0; dz < 2; ++dz)
-    for (int dy = 0; dy < 2; ++dy)
-      for (int dx = 0; dx < 2; ++dx) {
-        const long o = bidx(b, 2 * X - 1 + dx, 2 * Y - 1 + dy, 2 * Z - 1 + dz, P);
-        const T r = f[o] - (bnbsum(phi, o, P) - T(6) * phi[o]) * ih2;
-        s = first ? r : s + r;
-        first = false;
-      }
-  if (g) {
-    const int4 lf = m.leaf[b];
-    g[gidx(lf.y * nc + X - 1, lf.z * nc + Y - 1, lf.w * nc + Z - 1, Mg)] = s * T(0.125);
-  } else {
-    fc[bidx(b, X, Y, Z, Pc)] = s * T(0.125);
-  }
-}
-
-// phi += trilinear prolongation of the coarse error: from the next block
-// level ec (its ghosts refreshed, edges and corners included), or from the
-// global grid g of Mc cells per axis (periodic indexing).
-template <typename T>
-__global__ void blk_prolong_add_kernel(DevMesh m, const T* __restrict__ ec, const T* __restrict__ g, int Mc,
-                                       T* __restrict__ phi, int n, int B) {
-  const long n3 = (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * n3) return;
-  int x, y, z;
-  const int b = blk_cell(gid, n, x, y, z);
-  const int P = n + 2, nc = n / 2, Pc = nc + 2;
-  // interior offsets 0 .. n-1; the parent and the nearer coarse neighbour
-  const int ix = x - 1, iy = y - 1, iz = z - 1;
-  const int sx = (ix & 1) ? 1 : -1, sy = (iy & 1) ? 1 : -1, sz = (iz & 1) ? 1 : -1;
-  const T a = T(0.75), q = T(0.25);
-  T e000, e100, e010, e110, e001, e101, e011, e111;
-  if (g) {
-    const int4 lf = m.leaf[b];
-    const int X = (lf.y * n + ix) >> 1, Y = (lf.z * n + iy) >> 1, Z = (lf.w * n + iz) >> 1;
-    const int X1 = wrapm(X + sx, Mc), Y1 = wrapm(Y + sy, Mc), Z1 = wrapm(Z + sz, Mc);
-    e000 = g[gidx(X, Y, Z, Mc)]; e100 = g[gidx(X1, Y, Z, Mc)];
-    e010 = g[gidx(X, Y1, Z, Mc)]; e110 = g[gidx(X1, Y1, Z, Mc)];
-    e001 = g[gidx(X, Y, Z1, Mc)]; e101 = g[gidx(X1, Y, Z1, Mc)];
-    e011 = g[gidx(X, Y1, Z1, Mc)]; e111 = g[gidx(X1, Y1, Z1, Mc)];
-  } else {
-    const int X = (ix >> 1) + 1, Y = (iy >> 1) + 1, Z = (iz >> 1) + 1;   // padded coarse coordinates
-    const int X1 = X + sx, Y1 = Y + sy, Z1 = Z + sz;
-    e000 = ec[bidx(b, X, Y, Z, Pc)]; e100 = ec[bidx(b, X1, Y, Z, Pc)];
-    e010 = ec[bidx(b, X, Y1, Z, Pc)]; e110 = ec[bidx(b, X1, Y1, Z, Pc)];
-    e001 = ec[bidx(b, X, Y, Z1, Pc)]; e101 = ec[bidx(b, X1, Y, Z1, Pc)];
-    e011 = ec[bidx(b, X, Y1, Z1, Pc)]; e111 = ec[bidx(b, X1, Y1, Z1, Pc)];
-  }
-  const T c00 = a * e000 + q * e100;
-  const T c10 = a * e010 + q * e110;
-  const T c01 = a * e001 + q * e101;
-  const T c11 = a * e011 + q * e111;
-  const T c0 = a * c00 + q * c10;
-  const T c1 = a * c01 + q * c11;
-  const long i = bidx(b, x, y, z, P);
-  phi[i] = phi[i] + (a * c0 + q * c1);
-}
-
-// Level 0 in and out: compact leaf interiors [B][n^3] <-> padded blocks.
-// in: dst = src - *shift (the mean of f); out: dst = src.
-__global__ void blk_from_leaves_kernel(const double* __restrict__ src, double* __restrict__ dst, int n, int B,
-                                       const double* shift) {
-  const long n3 = (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * n3) return;
-  int x, y, z;
-  const int b = blk_cell(gid, n, x, y, z);
-  dst[bidx(b, x, y, z, n + 2)] = src[gid] - *shift;
-}
-
-__global__ void blk_to_leaves_kernel(const double* __restrict__ src, double* __restrict__ dst, int n, int B) {
-  const long n3 = (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * n3) return;
-  int x, y, z;
-  const int b = blk_cell(gid, n, x, y, z);
-  dst[gid] = src[bidx(b, x, y, z, n + 2)];
-}
-
-// Mixed precision on level 0: the float64 residual rounded to float32 (the
-// right-hand side of a float32 V-cycle), and the float32 correction added.
-__global__ void blk_residual_f32_kernel(const double* __restrict__ phi, const double* __restrict__ f,
-                                        float* __restrict__ r, int n, int B, double ih2) {
-  const long n3 = (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * n3) return;
-  int x, y, z;
-  const int b = blk_cell(gid, n, x, y, z);
-  const long i = bidx(b, x, y, z, n + 2);
-  r[i] = (float)(f[i] - (bnbsum(phi, i, n + 2) - 6.0 * phi[i]) * ih2);
-}
-
-__global__ void blk_correct_kernel(double* __restrict__ phi, const float* __restrict__ e, int n, int B) {
-  const long n3 = (long)n * n * n;
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (long)B * n3) return;
-  int x, y, z;
-  const int b = blk_cell(gid, n, x, y, z);
-  const long i = bidx(b, x, y, z, n + 2);
-  phi[i] = phi[i] + (double)e[i];
-}
-
-// max |f - lap(phi)| over the interiors (ghosts of phi refreshed): one
-// partial per CTA.
-__global__ void blk_resmax_kernel(const double* __restrict__ phi, const double* __restrict__ f, int n, int B,
-                                  double ih2, double* __restrict__ partial) {
-  __shared__ double sh[kRedThreads];
-  const long n3 = (long)n * n * n, count = (long)B * n3;
-  double acc = 0.0;
-  for (long gid = (long)blockIdx.x * blockDim.x + threadIdx.x; gid < count; gid += (long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    const int b = blk_cell(gid, n, x, y, z);
-    const long i = bidx(b, x, y, z, n + 2);
-    const double r = fabs(f[i] - (bnbsum(phi, i, n + 2) - 6.0 * phi[i]) * ih2);
-    acc = r > acc ? r : acc;
-  }
-  sh[threadIdx.x] = acc;
+template <int E>
+__device__ __forceinline__ Tile<E> tile_of(const TileLevel& L, int* s_nb) {
+  const int per = L.n / E;
+  unsigned t = blockIdx.x;
+  Tile<E> w;
+  w.x = (int)(t % per) * E; t /= per;
+  w.y = (int)(t % per) * E; t /= per;
+  w.z = (int)(t % per) * E; t /= per;
+  w.b = (int)t;
+  if (threadIdx.x < 27) s_nb[threadIdx.x] = L.idx ? L.idx[(long)w.b * 27 + threadIdx.x] : 0;
   __syncthreads();
-  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
+  return w;
+}
+
+// Offset of the cell (x, y, z) of a block of n cells per edge, each coordinate
+// in [-n, 2n), in the array of its level.
+__device__ __forceinline__ long cell_at(int n, const int* s_nb, int x, int y, int z) {
+  int e = 13;
+  if (x < 0) { e -= 1; x += n; } else if (x >= n) { e += 1; x -= n; }
+  if (y < 0) { e -= 3; y += n; } else if (y >= n) { e += 3; y -= n; }
+  if (z < 0) { e -= 9; z += n; } else if (z >= n) { e += 9; z -= n; }
+  return (((long)s_nb[e] * n + z) * n + y) * n + x;
+}
+
+// Cell i of a cube of E + 2 H cells per edge around the tile: offsets from the
+// tile's origin, -H .. E + H - 1.
+template <int E, int H>
+__device__ __forceinline__ void cube_cell(int i, int& x, int& y, int& z) {
+  constexpr int W = E + 2 * H;
+  x = i % W - H;
+  y = (i / W) % W - H;
+  z = i / (W * W) - H;
+}
+template <int E, int H>
+__device__ __forceinline__ int cube_at(int x, int y, int z) {
+  constexpr int W = E + 2 * H;
+  return ((z + H) * W + (y + H)) * W + x + H;
+}
+template <int E, int H> constexpr int kCube = (E + 2 * H) * (E + 2 * H) * (E + 2 * H);
+template <int E> constexpr int kTileThreads = E == 16 ? 512 : (E == 8 ? 256 : 64);
+
+template <typename T, int W>
+__device__ __forceinline__ T cube_sum(const T* p) {
+  return ((((p[-1] + p[1]) + p[-W]) + p[W]) + p[-W * W]) + p[W * W];
+}
+// Where the restricted residual goes: the blocks of the next level ([B][(n/2)^3]),
+// or, leaf given, one periodic array of Mg cells per edge.
+struct Coarse {
+  const int4* leaf;
+  int Mg;
+};
+__device__ __forceinline__ long coarse_at(const Coarse& c, int nc, int b, int X, int Y, int Z) {
+  if (c.leaf) {
+    const int4 lf = c.leaf[b];
+    return gidx(lf.y * nc + X, lf.z * nc + Y, lf.w * nc + Z, c.Mg);
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
+  return (((long)b * nc + Z) * nc + Y) * nc + X;
+}
+
+// Mean of the 8 children of each coarse cell of the tile, in (dz, dy, dx)
+// order; r: residuals in a cube with halo H.
+template <typename T, int E, int H>
+__device__ __forceinline__ void restrict_tile(const T* r, const TileLevel& L, const Tile<E>& w, const Coarse& to,
+                                              T* fc) {
+  constexpr int W = E + 2 * H, EC = E / 2;
+  for (int i = threadIdx.x; i < EC * EC * EC; i += blockDim.x) {
+    const int X = i % EC, Y = (i / EC) % EC, Z = i / (EC * EC);
+    const T* p = r + cube_at<E, H>(2 * X, 2 * Y, 2 * Z);
+    T s = p[0];
+    s = s + p[1];
+    s = s + p[W];
+    s = s + p[W + 1];
+    s = s + p[W * W];
+    s = s + p[W * W + 1];
+    s = s + p[W * W + W];
+    s = s + p[W * W + W + 1];
+    fc[coarse_at(to, L.n / 2, w.b, w.x / 2 + X, w.y / 2 + Y, w.z / 2 + Z)] = s * T(0.125);
+  }
+}
+
+// Down leg of a cycle in float32: two sweeps from zero, the residual and its
+// restriction, reading f once and writing phi once.
+template <typename T, int E>
+__global__ void __launch_bounds__(kTileThreads<E>)
+tile_down_kernel(TileLevel L, const T* __restrict__ f, T* __restrict__ phi, Coarse to, T* __restrict__ fc, T h2,
+                 T ih2) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  T* sF = reinterpret_cast<T*>(tile_raw);         // f, halo 2; then the residuals of the tile
+  T* sP = sF + kCube<E, 2>;                        // phi after two sweeps, halo 1
+  __shared__ int s_nb[27];
+  const Tile<E> w = tile_of<E>(L, s_nb);
+  int x, y, z;
+  for (int i = threadIdx.x; i < kCube<E, 2>; i += blockDim.x) {
+    cube_cell<E, 2>(i, x, y, z);
+    sF[i] = f[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)];
+  }
+  __syncthreads();
+  constexpr int W2 = E + 4, W1 = E + 2;
+  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
+    cube_cell<E, 1>(i, x, y, z);
+    const T* p = sF + cube_at<E, 2>(x, y, z);
+    const T s = ((((relax_zero(p[-1], h2) + relax_zero(p[1], h2)) + relax_zero(p[-W2], h2)) + relax_zero(p[W2], h2)) +
+                 relax_zero(p[-W2 * W2], h2)) + relax_zero(p[W2 * W2], h2);
+    sP[i] = relax(relax_zero(p[0], h2), s, p[0], h2);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
+    cube_cell<E, 0>(i, x, y, z);
+    const T* p = sP + cube_at<E, 1>(x, y, z);
+    T* q = sF + cube_at<E, 2>(x, y, z);
+    phi[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)] = p[0];
+    *q = residual_of(p[0], cube_sum<T, W1>(p), *q, ih2);
+  }
+  __syncthreads();
+  restrict_tile<T, E, 2>(sF, L, w, to, fc);
+}
+
+// The coarse error around a tile (halo 2 in coarse cells) into shared memory:
+// from the next level's blocks, or from one periodic array of Mg cells per edge.
+template <typename T, int E>
+__device__ __forceinline__ void load_coarse(const TileLevel& L, const Tile<E>& w, const int* s_nb, const Coarse& from,
+                                            const T* __restrict__ ec, T* sC) {
+  constexpr int EC = E / 2;
+  const int nc = L.n / 2;
+  int x, y, z;
+  for (int i = threadIdx.x; i < kCube<EC, 2>; i += blockDim.x) {
+    cube_cell<EC, 2>(i, x, y, z);
+    x += w.x / 2;
+    y += w.y / 2;
+    z += w.z / 2;
+    if (from.leaf) {
+      const int4 lf = from.leaf[w.b];
+      const int M = from.Mg;   // >= 2: an offset of two cells wraps at most once
+      sC[i] = ec[gidx(wrapm(lf.y * nc + x, M), wrapm(lf.z * nc + y, M), wrapm(lf.w * nc + z, M), M)];
+    } else {
+      sC[i] = ec[cell_at(nc, s_nb, x, y, z)];
+    }
+  }
+}
+
+// Trilinear interpolation of the coarse error to the fine cells of the tile and
+// its halo of H cells, one axis at a time through shared memory, so that each
+// one-axis value is formed once (2 instructions) instead of once per fine cell
+// that uses it (14 a cell): x for the coarse rows, y for the coarse planes, z
+// by the caller.
+template <int E, int H> constexpr int kInterpX = (E + 2 * H) * (E / 2 + 4) * (E / 2 + 4);
+template <int E, int H> constexpr int kInterpXY = (E + 2 * H) * (E + 2 * H) * (E / 2 + 4);
+
+template <typename T, int E, int H>
+__device__ __forceinline__ void interpolate_xy(const T* sC, T* sX, T* sXY) {
+  constexpr int W = E + 2 * H, WC = E / 2 + 4;
+  for (int i = threadIdx.x; i < kInterpX<E, H>; i += blockDim.x) {
+    const int x = i % W - H, row = i / W;
+    const T* p = sC + row * WC + (x >> 1) + 2;   // arithmetic shift: floor for the halo
+    sX[i] = quarter(p[0], p[(x & 1) ? 1 : -1]);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kInterpXY<E, H>; i += blockDim.x) {
+    const int ix = i % W, y = (i / W) % W - H, cz = i / (W * W);
+    const T* p = sX + (cz * WC + (y >> 1) + 2) * W + ix;
+    sXY[i] = quarter(p[0], p[(y & 1) ? W : -W]);
+  }
+  __syncthreads();
+}
+template <typename T, int E, int H>
+__device__ __forceinline__ T interpolate_z(const T* sXY, int x, int y, int z) {
+  constexpr int W = E + 2 * H;
+  const T* p = sXY + (((z >> 1) + 2) * W + y + H) * W + x + H;
+  return quarter(p[0], p[(z & 1) ? W * W : -W * W]);
+}
+
+// Up leg in float32: the interpolated coarse error added to phi, then two
+// sweeps.  OUT: 0 the result to out; on the finest level of a mixed-precision
+// cycle it goes straight to the float64 potential, 1 added, 2 as its first value.
+template <typename T, int E, int OUT>
+__global__ void __launch_bounds__(kTileThreads<E>)
+tile_up_kernel(TileLevel L, const T* __restrict__ f, const T* __restrict__ phi, Coarse from,
+               const T* __restrict__ ec, T* __restrict__ out, double* __restrict__ phi64, T h2) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  T* sQ = reinterpret_cast<T*>(tile_raw);         // phi plus the interpolated error, halo 2
+  T* sC = sQ + kCube<E, 2>;                        // the coarse error, halo 2
+  T* sX = sC + kCube<E / 2, 2>;                    // its interpolation along x, and along x and y
+  T* sXY = sX + kInterpX<E, 2>;
+  T* sR = sX;                                      // then the field after the first sweep, halo 1
+  __shared__ int s_nb[27];
+  const Tile<E> w = tile_of<E>(L, s_nb);
+  int x, y, z;
+  load_coarse<T, E>(L, w, s_nb, from, ec, sC);
+  __syncthreads();
+  interpolate_xy<T, E, 2>(sC, sX, sXY);
+  for (int i = threadIdx.x; i < kCube<E, 2>; i += blockDim.x) {
+    cube_cell<E, 2>(i, x, y, z);
+    sQ[i] = phi[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)] + interpolate_z<T, E, 2>(sXY, x, y, z);
+  }
+  __syncthreads();
+  constexpr int W2 = E + 4, W1 = E + 2;
+  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
+    cube_cell<E, 1>(i, x, y, z);
+    const T* p = sQ + cube_at<E, 2>(x, y, z);
+    sR[i] = relax(p[0], cube_sum<T, W2>(p), f[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)], h2);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
+    cube_cell<E, 0>(i, x, y, z);
+    const T* p = sR + cube_at<E, 1>(x, y, z);
+    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
+    const T v = relax(p[0], cube_sum<T, W1>(p), f[o], h2);
+    if (OUT == 0) out[o] = v;
+    else if (OUT == 1) phi64[o] = phi64[o] + widen(v);
+    else phi64[o] = widen(v);
+  }
+}
+
+// Float64 cycles are bound by the float64 pipe (two lanes per SM and clock), so
+// nothing is evaluated twice that costs more than a pointwise product: the legs
+// are split into passes with a halo of one cell.
+enum TilePass : int { kSmoothZero = 0, kSweep = 1, kUpSweep = 2, kRestrict = 3 };
+
+// kSmoothZero: out = two sweeps from zero.  kSweep: out = one sweep of phi.
+// kUpSweep: out = one sweep of phi plus the interpolated coarse error.
+// kRestrict: fc = restricted residual of phi.
+template <typename T, int E, int PASS>
+__global__ void __launch_bounds__(kTileThreads<E>)
+tile_pass_kernel(TileLevel L, const T* __restrict__ f, const T* __restrict__ phi, Coarse other,
+                 const T* __restrict__ ec, T* __restrict__ out, T* __restrict__ fc, T h2, T ih2) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  T* sP = reinterpret_cast<T*>(tile_raw);          // the field being swept, halo 1
+  T* sC = sP + kCube<E, 1>;                         // kUpSweep: the coarse error; kRestrict: the residuals
+  T* sX = sC + kCube<E / 2, 2>;                     // kUpSweep: its interpolation along x, and along x and y
+  T* sXY = sX + kInterpX<E, 1>;
+  __shared__ int s_nb[27];
+  const Tile<E> w = tile_of<E>(L, s_nb);
+  int x, y, z;
+  if (PASS == kUpSweep) {
+    load_coarse<T, E>(L, w, s_nb, other, ec, sC);
+    __syncthreads();
+    interpolate_xy<T, E, 1>(sC, sX, sXY);
+  }
+  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
+    cube_cell<E, 1>(i, x, y, z);
+    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
+    if (PASS == kSmoothZero) sP[i] = relax_zero(f[o], h2);
+    else if (PASS == kUpSweep) sP[i] = phi[o] + interpolate_z<T, E, 1>(sXY, x, y, z);
+    else sP[i] = phi[o];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
+    cube_cell<E, 0>(i, x, y, z);
+    const T* p = sP + cube_at<E, 1>(x, y, z);
+    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
+    const T s = cube_sum<T, E + 2>(p);
+    if (PASS == kRestrict) sC[i] = residual_of(p[0], s, f[o], ih2);
+    else out[o] = relax(p[0], s, f[o], h2);
+  }
+  if (PASS == kRestrict) {
+    __syncthreads();
+    restrict_tile<T, E, 0>(sC, L, w, other, fc);
+  }
+}
+
+// Float64 residual on the finest level: rounded to float32 (the right-hand side
+// of a mixed-precision cycle), or its largest magnitude per CTA.
+template <int E, bool MAX>
+__global__ void __launch_bounds__(kTileThreads<E>)
+tile_residual_kernel(TileLevel L, const double* __restrict__ f, const double* __restrict__ phi,
+                     float* __restrict__ r, double* __restrict__ partial, double ih2) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  double* sP = reinterpret_cast<double*>(tile_raw);
+  __shared__ int s_nb[27];
+  const Tile<E> w = tile_of<E>(L, s_nb);
+  int x, y, z;
+  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
+    cube_cell<E, 1>(i, x, y, z);
+    sP[i] = phi[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)];
+  }
+  __syncthreads();
+  double worst = 0.0;
+  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
+    cube_cell<E, 0>(i, x, y, z);
+    const double* p = sP + cube_at<E, 1>(x, y, z);
+    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
+    const double v = residual_of(p[0], cube_sum<double, E + 2>(p), f[o], ih2);
+    if (MAX) worst = fabs(v) > worst ? fabs(v) : worst;
+    else r[o] = (float)v;
+  }
+  if (MAX) {
+    for (int k = 16; k > 0; k >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, k));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sP[threadIdx.x >> 5] = worst;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int k = 1; k < (int)(blockDim.x >> 5); ++k) worst = fmax(worst, sP[k]);
+      partial[blockIdx.x] = worst;
+    }
+  }
+}
+
+// f without its mean, in float64 and, for a mixed-precision solve, rounded to
+// float32: the residual of phi = 0 is f itself.
+__global__ void shift_kernel(const double* __restrict__ src, double* __restrict__ dst, float* __restrict__ r,
+                             long count, const double* shift) {
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const double v = src[i] - *shift;
+  dst[i] = v;
+  if (r) r[i] = (float)v;
+}
+
+// ---------------------------------------------------------------------------
+// The bottom of the cycle in one CTA: every level from M cells per edge down,
+// phi, a second field and f of each in shared memory.
+__host__ __device__ inline long bottom_cells(int M) {
+  long c = 0;
+  for (int m = M;; m /= 2) {
+    c += (long)m * m * m;
+    if (m == 1 || m % 2 == 1) break;
+  }
+  return c;
+}
+
+template <typename T>
+__device__ void bottom_sweep(const T* in, T* out, const T* f, int M, T h2) {
+  for (int i = threadIdx.x; i < M * M * M; i += blockDim.x) {
+    const int x = i % M, y = (i / M) % M, z = i / (M * M);
+    out[i] = relax(in[i], nbsum(in, x, y, z, M), f[i], h2);
+  }
+  __syncthreads();
+}
+
+constexpr int kBottomThreads = 512;
+
+template <typename T>
+__global__ void __launch_bounds__(kBottomThreads)
+bottom_kernel(const T* __restrict__ f, T* __restrict__ out, int M0, double h0) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  T* base = reinterpret_cast<T*>(tile_raw);
+  for (int i = threadIdx.x; i < M0 * M0 * M0; i += blockDim.x) base[2 * M0 * M0 * M0 + i] = f[i];
+  __syncthreads();
+  // level of M cells: [phi, second field, f]; the coarser levels follow it
+  int M = M0, depth = 0;
+  double h = h0;
+  T* lv = base;
+  while (M > 1 && M % 2 == 0) {
+    const int c = M * M * M, Mc = M / 2, cc = Mc * Mc * Mc;
+    T *phi = lv, *tmp = lv + c, *g = lv + 2 * c, *gc = lv + 3 * c + 2 * cc;
+    const T h2 = T(h * h), ih2 = T(1.0 / (h * h));
+    for (int i = threadIdx.x; i < c; i += blockDim.x) tmp[i] = relax_zero(g[i], h2);
+    __syncthreads();
+    bottom_sweep(tmp, phi, g, M, h2);
+    for (int i = threadIdx.x; i < c; i += blockDim.x) {
+      const int x = i % M, y = (i / M) % M, z = i / (M * M);
+      tmp[i] = residual_of(phi[i], nbsum(phi, x, y, z, M), g[i], ih2);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < cc; i += blockDim.x) {
+      const T* p = tmp + gidx(2 * (i % Mc), 2 * ((i / Mc) % Mc), 2 * (i / (Mc * Mc)), M);
+      T s = p[0];
+      s = s + p[1];
+      s = s + p[M];
+      s = s + p[M + 1];
+      s = s + p[M * M];
+      s = s + p[M * M + 1];
+      s = s + p[M * M + M];
+      s = s + p[M * M + M + 1];
+      gc[i] = s * T(0.125);
+    }
+    __syncthreads();
+    lv += 3 * c;
+    M = Mc;
+    h *= 2.0;
+    ++depth;
+  }
+  {
+    const int c = M * M * M;
+    for (int i = threadIdx.x; i < c; i += blockDim.x) lv[i] = T(0);
+    __syncthreads();
+    if (M > 1) {   // odd coarsest grid (an even number of sweeps: the result is in phi)
+      const T h2 = T(h * h);
+      for (int k = 0; k < kCoarseSweeps; k += 2) {
+        bottom_sweep(lv, lv + c, lv + 2 * c, M, h2);
+        bottom_sweep(lv + c, lv, lv + 2 * c, M, h2);
+      }
+    }
+  }
+  while (depth > 0) {
+    const int Mc = M;
+    const T* ec = lv;
+    M *= 2;
+    h *= 0.5;
+    --depth;
+    const int c = M * M * M;
+    lv -= 3 * c;
+    T *phi = lv, *tmp = lv + c, *g = lv + 2 * c;
+    const T h2 = T(h * h);
+    for (int i = threadIdx.x; i < c; i += blockDim.x) {
+      const int x = i % M, y = (i / M) % M, z = i / (M * M);
+      phi[i] = phi[i] + prolonged(ec, x, y, z, Mc);
+    }
+    __syncthreads();
+    bottom_sweep(phi, tmp, g, M, h2);
+    bottom_sweep(tmp, phi, g, M, h2);
+  }
+  for (int i = threadIdx.x; i < M0 * M0 * M0; i += blockDim.x) out[i] = base[i];
 }
 
 unsigned blocks_for(long count) { return (unsigned)((count + 255) / 256); }
 
+// How a level runs: on tiles, in the one-CTA bottom (with every level below it),
+// or on the single-array kernels (an edge that is no multiple of 4, too large
+// for the bottom).
+enum LevelKind { kTiles, kBottom, kArray };
+
 template <typename T>
 struct Level {
-  int M;
+  LevelKind kind;
+  int n;             // cells per block edge, or per edge of the single array
+  int blocks;
+  const int* idx;    // neighbour blocks, null for a single array
   double h;
   T *phi, *tmp, *f;
+
+  long cells() const { return (long)blocks * n * n * n; }
 };
 
-// The single-array coarse levels.
+// Largest edge of a grid the one-CTA bottom takes.  Float32: 16 (16^3 cells and
+// the levels below take 56 KB and ~10 us; two tile launches per level cost as
+// much).  Float64: 10, one SM's float64 pipe (two lanes a clock) needs 13 us for
+// 10^3 cells and 52 us for 16^3, where the launches of a tile level take ~10.
+template <typename T> constexpr int kBottomMax = sizeof(T) == 4 ? 16 : 10;
+
+// Tile edge of a level: 16 where that leaves at least two CTAs per SM, else 8, 4
+// where the edge asks for it.
+inline int tile_edge(int n, int blocks) {
+  if (n % 16 == 0 && (long)blocks * (n / 16) * (n / 16) * (n / 16) >= 304) return 16;
+  return n % 8 == 0 ? 8 : 4;
+}
+
+// Shared memory of the up leg: the float32 kernel reuses the interpolation's
+// arrays for its second field.
+template <typename T, int E>
+constexpr size_t up_smem() {
+  constexpr int H = sizeof(T) == 4 ? 2 : 1;
+  constexpr int interp = kInterpX<E, H> + kInterpXY<E, H>;
+  constexpr int second = sizeof(T) == 4 ? kCube<E, 1> : 0;
+  return sizeof(T) * (kCube<E, H> + kCube<E / 2, 2> + (interp > second ? interp : second));
+}
+
 template <typename T>
 struct Cycle {
   std::vector<Level<T>> lv;
+  const int4* leaf;     // of the mesh: where a block's cells lie in the first single array
   cudaStream_t s;
 
+  // ---- single arrays, one pass per launch
   void sweeps(Level<T>& L, int count) {
     for (int k = 0; k < count; ++k) {
-      jacobi_kernel<T><<<grid_zc(L.M), kBlock3, 0, s>>>(L.phi, L.tmp, L.f, L.M, T(L.h * L.h));
+      jacobi_kernel<T><<<grid_zc(L.n), kBlock3, 0, s>>>(L.phi, L.tmp, L.f, L.n, T(L.h * L.h));
       std::swap(L.phi, L.tmp);
     }
   }
-
-  void vcycle(int l) {
+  void array_level(int l) {
     Level<T>& L = lv[l];
-    if (L.M == 1) {
-      fill_kernel<T><<<1, 32, 0, s>>>(L.phi, 1, T(0));
-      return;
-    }
-    if (L.M % 2 == 1) {
+    fill_kernel<T><<<blocks_for(L.cells()), 256, 0, s>>>(L.phi, L.cells(), T(0));
+    if (L.n % 2 == 1) {
       sweeps(L, kCoarseSweeps);
       return;
     }
     sweeps(L, kNu);
     Level<T>& C = lv[l + 1];
-    const long cc = (long)C.M * C.M * C.M;
-    residual_restrict_kernel<T><<<grid3(C.M), kBlock3, 0, s>>>(L.phi, L.f, C.f, L.M, T(1.0 / (L.h * L.h)));
-    fill_kernel<T><<<blocks_for(cc), 256, 0, s>>>(C.phi, cc, T(0));
-    vcycle(l + 1);
-    prolong_add_kernel<T><<<grid3(L.M), kBlock3, 0, s>>>(C.phi, L.phi, L.M);
+    residual_restrict_kernel<T><<<grid3(C.n), kBlock3, 0, s>>>(L.phi, L.f, C.f, L.n, T(1.0 / (L.h * L.h)));
+    solve(l + 1);
+    prolong_add_kernel<T><<<grid3(L.n), kBlock3, 0, s>>>(C.phi, L.phi, L.n);
     sweeps(L, kNu);
   }
-};
 
-// A block level: n cells per block edge, spacing h, padded arrays.
-template <typename T>
-struct BLevel {
-  int n;
-  double h;
-  T *phi, *tmp, *f;
-};
-
-// The V-cycle over the block levels, then the single-array tail.
-template <typename T>
-struct BlockCycle {
-  DevMesh m;
-  int B;
-  std::vector<BLevel<T>> blk;
-  Cycle<T> tail;
-  cudaStream_t s;
-
-  void refresh(const BLevel<T>& L, T* a) {
-    const long g = (long)B * ((long)(L.n + 2) * (L.n + 2) * (L.n + 2) - (long)L.n * L.n * L.n);
-    blk_refresh_kernel<T><<<blocks_for(g), 256, 0, s>>>(m, a, L.n, B);
-  }
-
-  void sweeps(BLevel<T>& L, int count) {
-    const long c = (long)B * L.n * L.n * L.n;
-    for (int k = 0; k < count; ++k) {
-      refresh(L, L.phi);
-      blk_jacobi_kernel<T><<<blocks_for(c), 256, 0, s>>>(L.phi, L.tmp, L.f, L.n, B, T(L.h * L.h));
-      std::swap(L.phi, L.tmp);
-    }
-  }
-
-  void vcycle(int l) {
-    BLevel<T>& L = blk[l];
-    sweeps(L, kNu);
-    refresh(L, L.phi);
-    const long cc = (long)B * (L.n / 2) * (L.n / 2) * (L.n / 2);
-    const T ih2 = T(1.0 / (L.h * L.h));
-    if (l + 1 < (int)blk.size()) {
-      BLevel<T>& C = blk[l + 1];
-      const long pc = (long)B * (C.n + 2) * (C.n + 2) * (C.n + 2);
-      blk_residual_restrict_kernel<T><<<blocks_for(cc), 256, 0, s>>>(m, L.phi, L.f, C.f, nullptr, 0, L.n, B, ih2);
-      fill_kernel<T><<<blocks_for(pc), 256, 0, s>>>(C.phi, pc, T(0));
-      vcycle(l + 1);
-      refresh(C, C.phi);
-      blk_prolong_add_kernel<T><<<blocks_for((long)B * L.n * L.n * L.n), 256, 0, s>>>(m, C.phi, nullptr, 0, L.phi,
-                                                                                    L.n, B);
+  // ---- tiles
+  template <int E>
+  void tile_level(int l, double* phi64, bool add, bool zero) {
+    Level<T>& L = lv[l];
+    Level<T>& C = lv[l + 1];
+    const unsigned grid = (unsigned)((long)L.blocks * (L.n / E) * (L.n / E) * (L.n / E));
+    constexpr int TH = kTileThreads<E>;
+    const TileLevel t{L.n, L.idx};
+    const Coarse c{L.idx && !C.idx ? leaf : nullptr, C.n};   // blocks above a single array
+    const T h2 = T(L.h * L.h), ih2 = T(1.0 / (L.h * L.h));
+    if constexpr (sizeof(T) == 4) {
+      constexpr size_t down = sizeof(T) * (kCube<E, 2> + kCube<E, 1>);
+      constexpr size_t up = up_smem<T, E>();
+      tile_down_kernel<T, E><<<grid, TH, down, s>>>(t, L.f, L.phi, c, C.f, h2, ih2);
+      solve(l + 1);
+      if (!phi64) {
+        tile_up_kernel<T, E, 0><<<grid, TH, up, s>>>(t, L.f, L.phi, c, C.phi, L.tmp, nullptr, h2);
+        std::swap(L.phi, L.tmp);
+      } else if (add) {
+        tile_up_kernel<T, E, 1><<<grid, TH, up, s>>>(t, L.f, L.phi, c, C.phi, nullptr, phi64, h2);
+      } else {
+        tile_up_kernel<T, E, 2><<<grid, TH, up, s>>>(t, L.f, L.phi, c, C.phi, nullptr, phi64, h2);
+      }
     } else {
-      Level<T>& G = tail.lv[0];
-      const long gc = (long)G.M * G.M * G.M;
-      blk_residual_restrict_kernel<T><<<blocks_for(cc), 256, 0, s>>>(m, L.phi, L.f, nullptr, G.f, G.M, L.n, B, ih2);
-      fill_kernel<T><<<blocks_for(gc), 256, 0, s>>>(G.phi, gc, T(0));
-      tail.vcycle(0);
-      blk_prolong_add_kernel<T><<<blocks_for((long)B * L.n * L.n * L.n), 256, 0, s>>>(m, nullptr, G.phi, G.M,
-                                                                                    L.phi, L.n, B);
+      constexpr size_t one = sizeof(T) * kCube<E, 1>;
+      constexpr size_t up = up_smem<T, E>(), rr = one + sizeof(T) * E * E * E;
+      if (zero) {
+        tile_pass_kernel<T, E, kSmoothZero><<<grid, TH, one, s>>>(t, L.f, nullptr, c, nullptr, L.phi, nullptr, h2,
+                                                                  ih2);
+      } else {
+        tile_pass_kernel<T, E, kSweep><<<grid, TH, one, s>>>(t, L.f, L.phi, c, nullptr, L.tmp, nullptr, h2, ih2);
+        tile_pass_kernel<T, E, kSweep><<<grid, TH, one, s>>>(t, L.f, L.tmp, c, nullptr, L.phi, nullptr, h2, ih2);
+      }
+      tile_pass_kernel<T, E, kRestrict><<<grid, TH, rr, s>>>(t, L.f, L.phi, c, nullptr, nullptr, C.f, h2, ih2);
+      solve(l + 1);
+      tile_pass_kernel<T, E, kUpSweep><<<grid, TH, up, s>>>(t, L.f, L.phi, c, C.phi, L.tmp, nullptr, h2, ih2);
+      tile_pass_kernel<T, E, kSweep><<<grid, TH, one, s>>>(t, L.f, L.tmp, c, nullptr, L.phi, nullptr, h2, ih2);
     }
-    sweeps(L, kNu);
+  }
+
+  // One V-cycle on level l, its result in lv[l].phi, or (finest level of a
+  // mixed-precision cycle) in, or added to, phi64.  It starts from zero, or
+  // (finest level of a float64 cycle) from lv[l].phi.
+  void solve(int l, double* phi64 = nullptr, bool add = false, bool zero = true) {
+    Level<T>& L = lv[l];
+    if (L.kind == kBottom) {
+      const size_t sh = sizeof(T) * 3 * bottom_cells(L.n);
+      bottom_kernel<T><<<1, kBottomThreads, sh, s>>>(L.f, L.phi, L.n, L.h);
+    } else if (L.kind == kArray) {
+      array_level(l);
+    } else {
+      switch (tile_edge(L.n, L.blocks)) {
+        case 16: tile_level<16>(l, phi64, add, zero); break;
+        case 8: tile_level<8>(l, phi64, add, zero); break;
+        default: tile_level<4>(l, phi64, add, zero); break;
+      }
+    }
   }
 };
 
@@ -516,11 +768,15 @@ struct BlockCycle {
 // first solve of each kind, freed with the mesh.
 struct PoissonScratch {
   std::vector<void*> d64, d32;
+  double* f64 = nullptr;   // mixed precision: f without its mean
   double* red = nullptr;   // 1024 partials + 2 scalars
+  double* top = nullptr;   // residual maxima per tile of the finest level
   ~PoissonScratch() {
     for (void* p : d64) cudaFree(p);
     for (void* p : d32) cudaFree(p);
+    if (f64) cudaFree(f64);
     if (red) cudaFree(red);
+    if (top) cudaFree(top);
   }
 };
 
@@ -535,7 +791,13 @@ cudaError_t alloc_levels(std::vector<void*>& bufs, const std::vector<long>& cell
     for (int k = 0; k < 3; ++k) {
       void* d = nullptr;
       cudaError_t e = cudaMalloc(&d, elem * (size_t)cells[l]);
-      if (e != cudaSuccess) return e;
+      if (e != cudaSuccess) {
+        for (; k > 0; --k) {   // a level has all three arrays or none
+          cudaFree(bufs.back());
+          bufs.pop_back();
+        }
+        return e;
+      }
       bufs.push_back(d);
     }
   return cudaSuccess;
@@ -543,47 +805,86 @@ cudaError_t alloc_levels(std::vector<void*>& bufs, const std::vector<long>& cell
 
 // The level structure: block levels n, n/2, ..., 4, then single arrays of
 // M = root 2^L 2 cells per axis, halved while even and above 1.
-struct Plan {
-  std::vector<int> bn;      // cells per block edge of the block levels
-  std::vector<int> gm;      // cells per axis of the single-array levels
-  std::vector<long> cells;  // cells of each level's arrays, block levels first
-};
-
-Plan plan_levels(int B, int n, int Mblocks) {
-  Plan p;
-  for (int nl = n; nl >= 4; nl /= 2) {
-    p.bn.push_back(nl);
-    p.cells.push_back((long)B * (nl + 2) * (nl + 2) * (nl + 2));
+template <typename T>
+std::vector<Level<T>> plan_levels(const DevMesh& m, int Mblocks, double h) {
+  std::vector<Level<T>> lv;
+  for (int nl = m.n; nl >= 4; nl /= 2, h *= 2.0) lv.push_back(Level<T>{kTiles, nl, m.B, m.idx, h, nullptr, nullptr, nullptr});
+  for (int Ml = Mblocks * 2;; Ml /= 2, h *= 2.0) {
+    const LevelKind k = Ml <= kBottomMax<T> ? kBottom : (Ml % 4 == 0 ? kTiles : kArray);
+    lv.push_back(Level<T>{k, Ml, 1, nullptr, h, nullptr, nullptr, nullptr});
+    if (k == kBottom || Ml % 2 == 1) break;
   }
-  for (int Ml = Mblocks * 2;; Ml /= 2) {
-    p.gm.push_back(Ml);
-    p.cells.push_back((long)Ml * Ml * Ml);
-    if (Ml == 1 || Ml % 2 == 1) break;
-  }
-  return p;
+  return lv;
 }
 
 template <typename T>
-BlockCycle<T> make_cycle(const DevMesh& m, const std::vector<void*>& bufs, const Plan& P, double h, cudaStream_t s) {
-  BlockCycle<T> C;
-  C.m = m;
-  C.B = m.B;
+cudaError_t make_cycle(Cycle<T>& C, const DevMesh& m, int Mblocks, double h, std::vector<void*>& bufs,
+                       cudaStream_t s) {
+  C.lv = plan_levels<T>(m, Mblocks, h);
+  C.leaf = m.leaf;
   C.s = s;
-  C.tail.s = s;
-  size_t k = 0;
-  for (size_t l = 0; l < P.bn.size(); ++l, ++k)
-    C.blk.push_back(BLevel<T>{P.bn[l], h * (double)(1L << l), static_cast<T*>(bufs[3 * k]),
-                              static_cast<T*>(bufs[3 * k + 1]), static_cast<T*>(bufs[3 * k + 2])});
-  for (size_t l = 0; l < P.gm.size(); ++l, ++k)
-    C.tail.lv.push_back(Level<T>{P.gm[l], h * (double)(1L << k), static_cast<T*>(bufs[3 * k]),
-                                 static_cast<T*>(bufs[3 * k + 1]), static_cast<T*>(bufs[3 * k + 2])});
-  return C;
+  std::vector<long> cells;
+  for (const Level<T>& L : C.lv) cells.push_back(L.cells());
+  const cudaError_t e = alloc_levels(bufs, cells, sizeof(T));
+  if (e != cudaSuccess) return e;
+  for (size_t k = 0; k < C.lv.size(); ++k) {
+    C.lv[k].phi = static_cast<T*>(bufs[3 * k]);
+    C.lv[k].tmp = static_cast<T*>(bufs[3 * k + 1]);
+    C.lv[k].f = static_cast<T*>(bufs[3 * k + 2]);
+  }
+  return cudaSuccess;
+}
+
+template <typename K>
+void allow_smem(K kernel, size_t bytes) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <int E>
+void prepare_tiles() {
+  constexpr size_t f2 = sizeof(float) * (kCube<E, 2> + kCube<E, 1>), fu = up_smem<float, E>();
+  allow_smem(tile_down_kernel<float, E>, f2);
+  allow_smem(tile_up_kernel<float, E, 0>, fu);
+  allow_smem(tile_up_kernel<float, E, 1>, fu);
+  allow_smem(tile_up_kernel<float, E, 2>, fu);
+  constexpr size_t d1 = sizeof(double) * kCube<E, 1>;
+  allow_smem(tile_pass_kernel<double, E, kSmoothZero>, d1);
+  allow_smem(tile_pass_kernel<double, E, kSweep>, d1);
+  allow_smem(tile_pass_kernel<double, E, kUpSweep>, up_smem<double, E>());
+  allow_smem(tile_pass_kernel<double, E, kRestrict>, d1 + sizeof(double) * E * E * E);
+  allow_smem(tile_residual_kernel<E, false>, d1);
+  allow_smem(tile_residual_kernel<E, true>, d1);
+}
+
+void prepare_poisson() {
+  prepare_tiles<16>();
+  prepare_tiles<8>();
+  prepare_tiles<4>();
+  allow_smem(bottom_kernel<float>, sizeof(float) * 3 * bottom_cells(kBottomMax<float>));
+  allow_smem(bottom_kernel<double>, sizeof(double) * 3 * bottom_cells(kBottomMax<double>));
 }
 
 // mean of a compact array (count doubles) into *out
 void mean_of(const double* a, long count, double* red, double* out, cudaStream_t s) {
-  reduce_kernel<<<1024, kRedThreads, 0, s>>>(a, nullptr, count, 0, 0.0, 0, red);
+  reduce_kernel<<<1024, kRedThreads, 0, s>>>(a, count, red);
   fold_kernel<<<1, kRedThreads, 0, s>>>(red, 1024, 0, 1.0 / (double)count, out);
+}
+
+template <int E>
+void residual_pass(const DevMesh& m, const double* f, const double* phi, float* r, double* partial, double ih2,
+                   cudaStream_t s) {
+  const unsigned grid = (unsigned)((long)m.B * (m.n / E) * (m.n / E) * (m.n / E));
+  const TileLevel t{m.n, m.idx};
+  constexpr size_t sh = sizeof(double) * kCube<E, 1>;
+  if (r) tile_residual_kernel<E, false><<<grid, kTileThreads<E>, sh, s>>>(t, f, phi, r, nullptr, ih2);
+  else tile_residual_kernel<E, true><<<grid, kTileThreads<E>, sh, s>>>(t, f, phi, nullptr, partial, ih2);
+}
+
+// The finest level's float64 residual: rounded into r, or its maxima per tile.
+void residual(const DevMesh& m, const double* f, const double* phi, float* r, double* partial, double ih2,
+              cudaStream_t s) {
+  if (tile_edge(m.n, m.B) == 16) residual_pass<16>(m, f, phi, r, partial, ih2, s);
+  else residual_pass<8>(m, f, phi, r, partial, ih2, s);
 }
 
 }  // namespace
@@ -591,62 +892,45 @@ void mean_of(const double* a, long count, double* red, double* out, cudaStream_t
 cudaError_t poisson_solve(PoissonScratch** scratch, const DevMesh& m, int M, double h, const double* f_leaves,
                           double* phi_leaves, int cycles, int inner, double* resid_host, cudaStream_t s) {
   const int n = m.n, B = m.B;
-  const Plan P = plan_levels(B, n, M / n);
+  static std::once_flag once;
+  std::call_once(once, prepare_poisson);
   if (!*scratch) *scratch = new PoissonScratch();
   PoissonScratch* S = *scratch;
-  // float64 level 0 always; the float64 hierarchy for float64 cycles, the
-  // float32 hierarchy for mixed precision
-  cudaError_t e = alloc_levels(S->d64, inner == 8 ? P.cells : std::vector<long>{P.cells[0]}, sizeof(double));
-  if (e == cudaSuccess && inner == 4) e = alloc_levels(S->d32, P.cells, sizeof(float));
+  const long nl = (long)B * n * n * n;
+  Cycle<double> C64;
+  Cycle<float> C32;
+  cudaError_t e = inner == 8 ? make_cycle(C64, m, M / n, h, S->d64, s) : make_cycle(C32, m, M / n, h, S->d32, s);
+  if (e == cudaSuccess && inner == 4 && !S->f64) e = cudaMalloc(&S->f64, sizeof(double) * (size_t)nl);
   if (e == cudaSuccess && !S->red) e = cudaMalloc(&S->red, sizeof(double) * (1024 + 2));
+  const int edge = tile_edge(n, B);
+  const long tiles = (long)B * (n / edge) * (n / edge) * (n / edge);
+  if (e == cudaSuccess && resid_host && !S->top) e = cudaMalloc(&S->top, sizeof(double) * (size_t)tiles);
   if (e != cudaSuccess) return e;
   double* scalar = S->red + 1024;
-  const long nl = (long)B * n * n * n;
-  const long p0 = P.cells[0];
   const double ih2 = 1.0 / (h * h);
-  BlockCycle<double> C64;
-  BlockCycle<float> C32;
-  // level 0 in float64: f without its mean, phi = 0
-  BLevel<double> L0{n, h, static_cast<double*>(S->d64[0]), static_cast<double*>(S->d64[1]),
-                    static_cast<double*>(S->d64[2])};
-  if (inner == 8) {
-    C64 = make_cycle<double>(m, S->d64, P, h, s);
-    L0 = C64.blk[0];
-  } else {
-    C32 = make_cycle<float>(m, S->d32, P, h, s);
-    C64.m = m;
-    C64.B = B;
-    C64.s = s;
-  }
+  // f without its mean; phi starts at 0
+  double* f0 = inner == 8 ? C64.lv[0].f : S->f64;
   mean_of(f_leaves, nl, S->red, scalar, s);
-  blk_from_leaves_kernel<<<blocks_for(nl), 256, 0, s>>>(f_leaves, L0.f, n, B, scalar);
-  fill_kernel<double><<<blocks_for(p0), 256, 0, s>>>(L0.phi, p0, 0.0);
+  shift_kernel<<<blocks_for(nl), 256, 0, s>>>(f_leaves, f0, inner == 4 ? C32.lv[0].f : nullptr, nl, scalar);
+  double* phi = inner == 4 ? phi_leaves : nullptr;
   for (int k = 0; k < cycles; ++k) {
-    if (inner == 8) {
-      C64.blk[0].phi = L0.phi;
-      C64.blk[0].tmp = L0.tmp;
-      C64.vcycle(0);
-      L0.phi = C64.blk[0].phi;
-      L0.tmp = C64.blk[0].tmp;
+    if (inner == 4) {
+      if (k > 0) residual(m, f0, phi, C32.lv[0].f, nullptr, ih2, s);   // of phi = 0: f, already there
+      C32.solve(0, phi, k > 0);
     } else {
-      BLevel<float>& F = C32.blk[0];
-      C64.refresh(L0, L0.phi);
-      blk_residual_f32_kernel<<<blocks_for(nl), 256, 0, s>>>(L0.phi, L0.f, F.f, n, B, ih2);
-      fill_kernel<float><<<blocks_for(p0), 256, 0, s>>>(F.phi, p0, 0.0f);
-      C32.vcycle(0);
-      blk_correct_kernel<<<blocks_for(nl), 256, 0, s>>>(L0.phi, F.phi, n, B);
+      C64.solve(0, nullptr, false, k == 0);
+      phi = C64.lv[0].phi;
     }
     if (resid_host) {
-      C64.refresh(L0, L0.phi);
-      blk_resmax_kernel<<<1024, kRedThreads, 0, s>>>(L0.phi, L0.f, n, B, ih2, S->red);
-      fold_kernel<<<1, kRedThreads, 0, s>>>(S->red, 1024, 1, 1.0, scalar + 1);
+      residual(m, f0, phi, nullptr, S->top, ih2, s);
+      fold_kernel<<<1, kRedThreads, 0, s>>>(S->top, tiles, 1, 1.0, scalar + 1);
       e = cudaMemcpyAsync(resid_host + k, scalar + 1, sizeof(double), cudaMemcpyDeviceToHost, s);
       if (e != cudaSuccess) return e;
     }
   }
-  blk_to_leaves_kernel<<<blocks_for(nl), 256, 0, s>>>(L0.phi, phi_leaves, n, B);
-  mean_of(phi_leaves, nl, S->red, scalar, s);
-  add_kernel<<<blocks_for(nl), 256, 0, s>>>(phi_leaves, nl, scalar, 1.0);
+  mean_of(phi, nl, S->red, scalar, s);
+  if (inner == 8) shift_kernel<<<blocks_for(nl), 256, 0, s>>>(phi, phi_leaves, nullptr, nl, scalar);
+  else add_kernel<<<blocks_for(nl), 256, 0, s>>>(phi_leaves, nl, scalar, 1.0);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (resid_host) e = cudaStreamSynchronize(s);
