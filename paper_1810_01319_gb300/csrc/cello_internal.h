@@ -178,8 +178,13 @@ struct RemapEntry {
   int k;
   int src[8];
 };
-void launch_remap(const DevMesh& neu, const DevMesh& old, const void* Uold, void* Unew, const RemapEntry* map,
+// The entries of every new leaf into map, then the cells; where a new leaf has
+// no source, *bad is set and no cell is written.
+void launch_remap(const DevMesh& neu, const unsigned long long* nkeys, const DevMesh& old,
+                  const unsigned long long* okeys, const void* Uold, void* Unew, RemapEntry* map, int* bad,
                   int precision, cudaStream_t s);
+void launch_remap_map(const DevMesh& neu, const unsigned long long* nkeys, const DevMesh& old,
+                      const unsigned long long* okeys, RemapEntry* map, int* bad, cudaStream_t s);
 
 // Accessors for translation units that see cello_mesh only as an opaque type.
 DevMesh mesh_dev(const cello_mesh* mesh);
@@ -194,7 +199,8 @@ void prepare_kernels_f64();
 
 // Launchers (defined in the kernel translation units).
 void launch_neighbour_table(const DevMesh& m, const unsigned long long* keys, int8_t* kind, int* idx,
-                            int* fine8, cudaStream_t s);
+                            int* fine8, int8_t* face, int* bad, cudaStream_t s);
+void launch_fine_slots(const DevMesh& m, CoarseFace* faces, int count, cudaStream_t s);
 // Ghost refresh of leaves [leaf0, leaf0+nleaf) in phases, in this order: the
 // listed slow faces (leaf * 6 + face of the faces of these leaves whose
 // neighbour is not a same-level leaf: their phase regions computed from leaf

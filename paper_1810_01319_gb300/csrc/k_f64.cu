@@ -267,16 +267,18 @@ void launch_zero_ghosts(const DevMesh& m, void* lam, int precision, cudaStream_t
 #undef CELLO_ZG
 }
 
-void launch_remap(const DevMesh& neu, const DevMesh& old, const void* Uold, void* Unew, const RemapEntry* map,
+void launch_remap(const DevMesh& neu, const unsigned long long* nkeys, const DevMesh& old,
+                  const unsigned long long* okeys, const void* Uold, void* Unew, RemapEntry* map, int* bad,
                   int precision, cudaStream_t s) {
   const long threads = (long)neu.B * neu.n * neu.n * neu.n;
   if (threads <= 0) return;
+  launch_remap_map(neu, nkeys, old, okeys, map, bad, s);
   const unsigned grid = (unsigned)((threads + 255) / 256);
 #define CELLO_RM(T, NB)                                                                                      \
   if (neu.nf == 6)                                                                                          \
-    remap_kernel<T, NB, 6><<<grid, 256, 0, s>>>(neu, old, static_cast<const T*>(Uold), static_cast<T*>(Unew), map); \
+    remap_kernel<T, NB, 6><<<grid, 256, 0, s>>>(neu, old, static_cast<const T*>(Uold), static_cast<T*>(Unew), map, bad); \
   else                                                                                                      \
-    remap_kernel<T, NB><<<grid, 256, 0, s>>>(neu, old, static_cast<const T*>(Uold), static_cast<T*>(Unew), map)
+    remap_kernel<T, NB><<<grid, 256, 0, s>>>(neu, old, static_cast<const T*>(Uold), static_cast<T*>(Unew), map, bad)
 #define CELLO_RM_T(T)                       \
   switch (neu.n) {                          \
     case 8: CELLO_RM(T, 8); break;          \
@@ -292,11 +294,13 @@ void launch_flags(const DevMesh& m, const void* U, int precision, int field, dou
                   int8_t* flags, cudaStream_t s) {
   if (m.B <= 0) return;
   const double thr = 2.0 * tau, thr_c = 2.0 * tau_c;
+  auto plain = [](double v) { return v == 0.0 || (std::abs(v) >= 1e-20 && std::abs(v) <= 1e20); };
+  const bool filter = plain(thr) && plain(thr_c);   // float32 holds the thresholds to its rounding
 #define CELLO_FLG(T, NB)                                                                                     \
   if (m.nf == 6)                                                                                            \
-    flags_kernel<T, NB, 6><<<m.B, 256, 0, s>>>(m, static_cast<const T*>(U), field, thr, thr_c, flags);     \
+    flags_kernel<T, NB, 6><<<m.B, 256, 0, s>>>(m, static_cast<const T*>(U), field, thr, thr_c, filter, flags); \
   else                                                                                                      \
-    flags_kernel<T, NB><<<m.B, 256, 0, s>>>(m, static_cast<const T*>(U), field, thr, thr_c, flags)
+    flags_kernel<T, NB><<<m.B, 256, 0, s>>>(m, static_cast<const T*>(U), field, thr, thr_c, filter, flags)
 #define CELLO_FLG_T(T)                        \
   switch (m.n) {                              \
     case 8: CELLO_FLG(T, 8); break;           \

@@ -7,7 +7,6 @@
 #include <cstring>
 #include <mutex>
 #include <string>
-#include <unordered_map>
 #include <unordered_set>
 #include <vector>
 
@@ -57,29 +56,67 @@ inline Node child(const Node& t, int o) {
   return Node{t.L + 1, 2 * t.i + (o & 1), 2 * t.j + ((o >> 1) & 1), 2 * t.k + (o >> 2)};
 }
 
-// Leaf set with its internal (refined) ancestors, for balance queries.
-struct Tree {
-  const cello_mesh_desc& d;
-  std::unordered_set<unsigned long long> leaves, internal;
-  explicit Tree(const cello_mesh_desc& desc) : d(desc) {}
+// Set of packed nodes: open addressing, linear probing.
+class NodeSet {
+ public:
+  explicit NodeSet(size_t expected) {
+    size_t cap = 64;
+    while (cap < 2 * expected) cap *= 2;
+    resize(cap);
+  }
+  bool insert(unsigned long long key) {   // false if it is there already
+    if (2 * (count_ + 1) > slots_.size()) grow();
+    const size_t i = find(key);
+    if (slots_[i] == key + 1) return false;
+    slots_[i] = key + 1;
+    ++count_;
+    return true;
+  }
+  bool contains(unsigned long long key) const { return slots_[find(key)] == key + 1; }
 
-  void index(const std::vector<Node>& ls) {
-    leaves.clear();
-    internal.clear();
-    for (const Node& t : ls) {
-      leaves.insert(pack(t));
-      Node p = t;
-      while (p.L > 0) {
-        p = Node{p.L - 1, p.i >> 1, p.j >> 1, p.k >> 1};
-        if (!internal.insert(pack(p)).second) break;
-      }
+ private:
+  std::vector<unsigned long long> slots_;   // key + 1, 0: empty (no packed node is all ones)
+  size_t count_ = 0;
+  int shift_ = 0;
+  size_t find(unsigned long long key) const {
+    size_t i = (size_t)((key * 0x9E3779B97F4A7C15ull) >> shift_);
+    while (slots_[i] != 0 && slots_[i] != key + 1) i = (i + 1) & (slots_.size() - 1);
+    return i;
+  }
+  void resize(size_t cap) {
+    slots_.assign(cap, 0);
+    shift_ = 64;
+    for (size_t c = cap; c > 1; c /= 2) --shift_;
+  }
+  void grow() {
+    std::vector<unsigned long long> old;
+    old.swap(slots_);
+    resize(old.size() * 2);
+    for (unsigned long long v : old)
+      if (v) slots_[find(v - 1)] = v;
+  }
+};
+
+// The refined nodes of a mesh, by level; its leaves are their children that are
+// not refined (and the roots that are not).
+struct Tree {
+  const cello_mesh_desc* d;
+  NodeSet internal;
+  std::vector<Node> level[12];
+  Tree(const cello_mesh_desc& desc, size_t expected) : d(&desc), internal(expected) {}
+
+  void refine(Node t) {   // the node and its ancestors
+    while (internal.insert(pack(t))) {
+      level[t.L].push_back(t);
+      if (t.L == 0) break;
+      t = Node{t.L - 1, t.i >> 1, t.j >> 1, t.k >> 1};
     }
   }
 
   bool wrap(int L, int a, int& v) const {
-    const int nb = d.root[a] << L;
+    const int nb = d->root[a] << L;
     if (v >= 0 && v < nb) return true;
-    if (d.bc[a] != CELLO_PERIODIC) return false;
+    if (d->bc[a] != CELLO_PERIODIC) return false;
     v = ((v % nb) + nb) % nb;
     return true;
   }
@@ -88,7 +125,7 @@ struct Tree {
   // same-level neighbour node is refined and one of its children that
   // touches t is refined too.
   bool touches_deeper(const Node& t) const {
-    if (t.L + 2 > d.max_level) return false;
+    if (t.L + 2 > d->max_level) return false;
     for (int dz = -1; dz <= 1; ++dz)
       for (int dy = -1; dy <= 1; ++dy)
         for (int dx = -1; dx <= 1; ++dx) {
@@ -98,16 +135,48 @@ struct Tree {
           for (int a = 0; a < 3; ++a) in = in && wrap(t.L, a, v[a]);
           if (!in) continue;
           const Node nb{t.L, v[0], v[1], v[2]};
-          if (!internal.count(pack(nb))) continue;
+          if (!internal.contains(pack(nb))) continue;
           for (int o = 0; o < 8; ++o) {
             const int ox = o & 1, oy = (o >> 1) & 1, oz = o >> 2;
             if ((dx == 1 && ox) || (dx == -1 && !ox) || (dy == 1 && oy) || (dy == -1 && !oy) || (dz == 1 && oz) ||
                 (dz == -1 && !oz))
               continue;
-            if (internal.count(pack(child(nb, o)))) return true;
+            if (internal.contains(pack(child(nb, o)))) return true;
           }
         }
     return false;
+  }
+
+  // 2:1 balance: a leaf that touches a leaf two levels finer is refined, until
+  // there is none.  A refined node c asks for exactly the nodes one level
+  // coarser that touch it, its parent's neighbours on the side of its octant (the
+  // others are its parent), so one pass over the refined nodes from the finest
+  // level up, 7 neighbours each, is the whole closure.
+  void balance() {
+    for (int L = d->max_level - 1; L >= 1; --L)
+      for (size_t n = 0; n < level[L].size(); ++n) {
+        const Node c = level[L][n];
+        const int at[3] = {c.i, c.j, c.k};
+        for (int mask = 1; mask < 8; ++mask) {
+          int v[3];
+          bool in = true;
+          for (int a = 0; a < 3; ++a) {
+            v[a] = at[a];
+            if (mask >> a & 1) v[a] += (at[a] & 1) ? 1 : -1;
+            in = in && wrap(L, a, v[a]);
+          }
+          if (in) refine(Node{L - 1, v[0] >> 1, v[1] >> 1, v[2] >> 1});
+        }
+      }
+  }
+
+  // The leaves under a node in Morton order.
+  void emit(const Node& t, std::vector<Node>& out) const {
+    if (!internal.contains(pack(t))) {
+      out.push_back(t);
+      return;
+    }
+    for (int o = 0; o < 8; ++o) emit(child(t, o), out);
   }
 };
 
@@ -164,11 +233,14 @@ struct cello_mesh {
   int B = 0, N = 0;
   std::vector<int4> leaves;
   std::vector<unsigned long long> keys;
-  std::vector<int8_t> kind;
-  std::vector<int> idx, fine8, face_slot;
-  std::vector<CoarseFace> cfaces;
+  std::vector<int> face_slot;
+  std::vector<CoarseFace> cfaces;   // fslot filled on the device only
   std::vector<int> group_start;
   int nslots = 0;
+  // device tables: two allocations, d_table (sized by the leaves) and d_lists
+  // (by the faces that are not same-level); the pointers below lie in them
+  char* d_table = nullptr;
+  char* d_lists = nullptr;
   int4* d_leaf = nullptr;
   unsigned long long* d_keys = nullptr;
   int8_t* d_kind = nullptr;
@@ -187,6 +259,8 @@ struct cello_mesh {
   int sweep_variant[3] = {0, 0, 0};   // per sweep axis; chosen by cello_autotune or set by the caller
   unsigned* d_work = nullptr;      // work counter of the persistent sweep variants
   unsigned* d_err = nullptr;       // error word set by the reduction
+  int* d_flag = nullptr;           // result word of the table and remap-map kernels
+  RemapEntry* d_map = nullptr;     // remap entries of this mesh as the new one
   PoissonScratch* poisson = nullptr;   // multigrid levels, allocated by the first Poisson solve
   double* d_zero = nullptr;        // dt = 0, for timing sweeps without changing the state
   void* adj_scratch = nullptr;   // three states for the adjoint's forward recomputation
@@ -240,23 +314,11 @@ struct cello_mesh {
     if (d_xlist) cudaFree(d_xlist);
     d_xlist = nullptr;
     xlist_cap = 0;
-    if (d_work) cudaFree(d_work);
-    if (d_zero) cudaFree(d_zero);
-    if (d_err) cudaFree(d_err);
-    d_err = nullptr;
-    d_work = nullptr;
-    d_zero = nullptr;
-    if (d_slow) cudaFree(d_slow);
-    d_slow = nullptr;
-    for (int*& p : d_slow_ax) {
-      if (p) cudaFree(p);
-      p = nullptr;
-    }
-    void* ptrs[] = {d_leaf, d_keys, d_kind, d_idx, d_fine8, d_face_slot, d_cfaces, d_group_start, d_reg, d_partials};
-    for (void* p : ptrs)
-      if (p) cudaFree(p);
-    d_leaf = nullptr; d_keys = nullptr; d_kind = nullptr; d_idx = nullptr; d_fine8 = nullptr;
-    d_face_slot = nullptr; d_cfaces = nullptr; d_group_start = nullptr; d_reg = nullptr; d_partials = nullptr;
+    if (d_reg) cudaFree(d_reg);
+    if (d_lists) cudaFree(d_lists);
+    if (d_table) cudaFree(d_table);
+    d_reg = nullptr;
+    d_lists = d_table = nullptr;
   }
   ~cello_mesh() { release(); }
 };
@@ -286,88 +348,77 @@ cello_status check_desc(const cello_mesh_desc* d) {
   return CELLO_OK;
 }
 
-// New leaf list from the previous one and flags (see cello_octree_build).
+// New leaf list, in Morton order, from the previous one and flags (see
+// cello_octree_build).
 std::vector<Node> build_leaves(const cello_mesh_desc& d, const cello_mesh* prev, const int8_t* flags) {
-  std::vector<Node> cur;
+  std::vector<Node> out;
   if (!prev) {
+    std::vector<std::pair<unsigned long long, Node>> roots;
+    roots.reserve((size_t)d.root[0] * d.root[1] * d.root[2]);
     for (int k = 0; k < d.root[2]; ++k)
       for (int j = 0; j < d.root[1]; ++j)
-        for (int i = 0; i < d.root[0]; ++i) cur.push_back(Node{0, i, j, k});
-    return cur;
+        for (int i = 0; i < d.root[0]; ++i) roots.emplace_back(leaf_key(d, Node{0, i, j, k}), Node{0, i, j, k});
+    std::sort(roots.begin(), roots.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
+    out.reserve(roots.size());
+    for (const auto& r : roots) out.push_back(r.second);
+    return out;
   }
   const int B = prev->B;
-  std::vector<Node> old(B);
-  for (int b = 0; b < B; ++b) {
+  auto leaf = [&](int b) {
     const int4 l = prev->leaves[b];
-    old[b] = Node{l.x, l.y, l.z, l.w};
-  }
-  std::unordered_map<unsigned long long, int> flag_of;
-  std::unordered_set<unsigned long long> refine;
-  for (int b = 0; b < B; ++b) {
-    const int f = flags ? flags[b] : 0;
-    flag_of[pack(old[b])] = f;
-    if (f > 0 && old[b].L < d.max_level) refine.insert(pack(old[b]));
-  }
-  for (const Node& t : old) {
-    if (refine.count(pack(t)))
-      for (int o = 0; o < 8; ++o) cur.push_back(child(t, o));
-    else
-      cur.push_back(t);
-  }
-  Tree tree(d);
-  tree.index(cur);
-  // coarsening candidates: complete octets of unrefined -1 leaves
-  std::unordered_map<unsigned long long, int> kids;
-  for (const Node& t : old)
-    if (t.L > 0) kids[pack(Node{t.L - 1, t.i >> 1, t.j >> 1, t.k >> 1})]++;
-  std::vector<Node> coarsen;
-  for (const auto& kv : kids) {
-    if (kv.second != 8) continue;
-    const unsigned long long pk = kv.first;
-    const Node p{(int)(pk >> 60), (int)((pk >> 40) & 0xfffff), (int)((pk >> 20) & 0xfffff), (int)(pk & 0xfffff)};
-    bool ok = true;
-    for (int o = 0; o < 8 && ok; ++o) {
-      const unsigned long long c = pack(child(p, o));
-      auto it = flag_of.find(c);
-      ok = it != flag_of.end() && it->second < 0 && !refine.count(c);
-    }
-    if (ok && !tree.touches_deeper(p)) coarsen.push_back(p);
-  }
-  if (!coarsen.empty()) {
-    std::unordered_set<unsigned long long> gone;
-    for (const Node& p : coarsen)
-      for (int o = 0; o < 8; ++o) gone.insert(pack(child(p, o)));
-    std::vector<Node> next;
-    for (const Node& t : cur)
-      if (!gone.count(pack(t))) next.push_back(t);
-    for (const Node& p : coarsen) next.push_back(p);
-    cur.swap(next);
-  }
-  // 2:1 balance: refine every leaf touching a leaf two levels finer
-  for (;;) {
-    tree.index(cur);
-    std::vector<Node> next;
-    bool changed = false;
-    for (const Node& t : cur) {
-      if (tree.touches_deeper(t)) {
-        changed = true;
-        for (int o = 0; o < 8; ++o) next.push_back(child(t, o));
-      } else {
-        next.push_back(t);
+    return Node{l.x, l.y, l.z, l.w};
+  };
+  // the previous mesh and the leaves to be refined
+  auto mesh_tree = [&](const NodeSet* gone) {
+    Tree t(d, (size_t)B / 4 + 64);
+    for (int b = 0; b < B; ++b) {
+      const Node n = leaf(b);
+      if (flags && flags[b] > 0 && n.L < d.max_level) {
+        t.refine(n);
+      } else if (n.L > 0) {
+        Node p{n.L - 1, n.i >> 1, n.j >> 1, n.k >> 1};
+        if (gone && gone->contains(pack(p))) {   // the parent becomes a leaf
+          if (p.L == 0) continue;
+          p = Node{p.L - 1, p.i >> 1, p.j >> 1, p.k >> 1};
+        }
+        t.refine(p);
       }
     }
-    cur.swap(next);
-    if (!changed) break;
+    return t;
+  };
+  Tree tree = mesh_tree(nullptr);
+  // coarsening: octets of leaves (consecutive in Morton order) that are all -1
+  // and whose parent would touch no leaf two levels finer
+  std::vector<Node> coarsen;
+  if (flags)
+    for (int b = 0; b + 7 < B; ++b) {
+      const Node t = leaf(b);
+      if (flags[b] >= 0 || t.L == 0 || ((t.i | t.j | t.k) & 1)) continue;
+      bool ok = true;
+      for (int o = 1; o < 8 && ok; ++o) {
+        const Node c = leaf(b + o);
+        ok = flags[b + o] < 0 && c.L == t.L && (c.i >> 1) == (t.i >> 1) && (c.j >> 1) == (t.j >> 1) &&
+             (c.k >> 1) == (t.k >> 1);
+      }
+      const Node p{t.L - 1, t.i >> 1, t.j >> 1, t.k >> 1};
+      if (ok && !tree.touches_deeper(p)) coarsen.push_back(p);
+    }
+  if (!coarsen.empty()) {
+    NodeSet gone(coarsen.size());
+    for (const Node& p : coarsen) gone.insert(pack(p));
+    tree = mesh_tree(&gone);
   }
-  return cur;
-}
-
-template <typename V>
-cello_status upload(V** dptr, const std::vector<V>& h) {
-  if (h.empty()) return CELLO_OK;
-  CELLO_CUDA(cudaMalloc((void**)dptr, h.size() * sizeof(V)));
-  CELLO_CUDA(cudaMemcpy(*dptr, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice));
-  return CELLO_OK;
+  tree.balance();
+  out.reserve((size_t)B);
+  Node last{-1, 0, 0, 0};
+  for (int b = 0; b < B; ++b) {   // the roots in the order of the leaves
+    const Node t = leaf(b);
+    const Node r{0, t.i >> t.L, t.j >> t.L, t.k >> t.L};
+    if (last.L == 0 && r.i == last.i && r.j == last.j && r.k == last.k) continue;
+    last = r;
+    tree.emit(r, out);
+  }
+  return out;
 }
 
 #define CELLO_TRY(expr)               \
@@ -376,109 +427,125 @@ cello_status upload(V** dptr, const std::vector<V>& h) {
     if (st_ != CELLO_OK) return st_;  \
   } while (0)
 
+// Parts of one allocation, each on a 256-byte boundary.
+struct Layout {
+  size_t bytes = 0;
+  template <typename V>
+  size_t add(size_t count) {
+    const size_t at = bytes;
+    bytes += (count * sizeof(V) + 255) / 256 * 256;
+    return at;
+  }
+};
+
+template <typename V>
+V* part(char* base, size_t at) { return reinterpret_cast<V*>(base + at); }
+
+// The device tables of M->leaves.  The neighbour table stays on the device: what
+// the host needs of it, whether the mesh is balanced and the kinds of each leaf's
+// six faces, comes back in one copy, and the lists made from those go up in one
+// (the whole table, 1 KB a leaf, walked on the host was a third of the build).
 cello_status finish_build(cello_mesh* M) {
   const cello_mesh_desc& d = M->desc;
-  const int B = M->B;
-  CELLO_TRY(upload(&M->d_leaf, M->leaves));
-  CELLO_TRY(upload(&M->d_keys, M->keys));
-  CELLO_CUDA(cudaMalloc((void**)&M->d_kind, (size_t)B * 27));
-  CELLO_CUDA(cudaMalloc((void**)&M->d_idx, (size_t)B * 27 * sizeof(int)));
-  CELLO_CUDA(cudaMalloc((void**)&M->d_fine8, (size_t)B * 27 * 8 * sizeof(int)));
-  DevMesh dm = M->dev();
-  launch_neighbour_table(dm, M->d_keys, M->d_kind, M->d_idx, M->d_fine8, 0);
+  const size_t B = (size_t)M->B;
+  cudaStream_t s = cudaStreamPerThread;
+  Layout t;
+  const size_t o_leaf = t.add<int4>(B), o_keys = t.add<unsigned long long>(B), o_word = t.add<double>(32);
+  const size_t head = t.bytes;   // uploaded: leaves, keys, the cleared words
+  const size_t o_flag = t.add<int>(1), o_face = t.add<int8_t>(B * 6);
+  const size_t tail = t.bytes - o_flag;   // downloaded
+  const size_t o_kind = t.add<int8_t>(B * 27), o_idx = t.add<int>(B * 27), o_fine8 = t.add<int>(B * 27 * 8);
+  const size_t o_part = t.add<double>(B * 6), o_map = t.add<RemapEntry>(B);
+  CELLO_CUDA(cudaMalloc((void**)&M->d_table, t.bytes));
+  M->d_leaf = part<int4>(M->d_table, o_leaf);
+  M->d_keys = part<unsigned long long>(M->d_table, o_keys);
+  M->d_err = part<unsigned>(M->d_table, o_word);
+  M->d_work = M->d_err + 8;
+  M->d_zero = part<double>(M->d_table, o_word) + 16;
+  M->d_flag = part<int>(M->d_table, o_flag);
+  M->d_kind = part<int8_t>(M->d_table, o_kind);
+  M->d_idx = part<int>(M->d_table, o_idx);
+  M->d_fine8 = part<int>(M->d_table, o_fine8);
+  M->d_partials = part<double>(M->d_table, o_part);
+  M->d_map = part<RemapEntry>(M->d_table, o_map);
+  std::vector<char> buf(std::max(head, tail), 0);
+  std::memcpy(buf.data() + o_leaf, M->leaves.data(), B * sizeof(int4));
+  std::memcpy(buf.data() + o_keys, M->keys.data(), B * sizeof(unsigned long long));
+  CELLO_CUDA(cudaMemcpyAsync(M->d_table, buf.data(), head, cudaMemcpyHostToDevice, s));
+  CELLO_CUDA(cudaMemsetAsync(M->d_flag, 0, sizeof(int), s));
+  const DevMesh dm = M->dev();
+  int8_t* d_face = part<int8_t>(M->d_table, o_face);
+  launch_neighbour_table(dm, M->d_keys, M->d_kind, M->d_idx, M->d_fine8, d_face, M->d_flag, s);
   CELLO_CUDA(cudaGetLastError());
-  M->kind.resize((size_t)B * 27);
-  M->idx.resize((size_t)B * 27);
-  M->fine8.resize((size_t)B * 27 * 8);
-  CELLO_CUDA(cudaMemcpy(M->kind.data(), M->d_kind, M->kind.size(), cudaMemcpyDeviceToHost));
-  CELLO_CUDA(cudaMemcpy(M->idx.data(), M->d_idx, M->idx.size() * sizeof(int), cudaMemcpyDeviceToHost));
-  CELLO_CUDA(cudaMemcpy(M->fine8.data(), M->d_fine8, M->fine8.size() * sizeof(int), cudaMemcpyDeviceToHost));
-  for (int8_t k : M->kind)
-    if (k < 0) return fail(CELLO_EINTERNAL, "2:1 balance violated: a neighbour is two levels coarser");
-  // every child of a refined neighbour node that touches the leaf must be a
-  // leaf (balance); the refresh and the slope lookups index only those
-  for (int b = 0; b < B; ++b)
-    for (int e = 0; e < 27; ++e) {
-      if (M->kind[(size_t)b * 27 + e] != kFine) continue;
-      const int dd[3] = {e % 3 - 1, (e / 3) % 3 - 1, e / 9 - 1};
-      for (int o = 0; o < 8; ++o) {
-        const int oo[3] = {o & 1, (o >> 1) & 1, o >> 2};
-        bool touch = true;
-        for (int a = 0; a < 3; ++a) touch = touch && !((dd[a] == 1 && oo[a]) || (dd[a] == -1 && !oo[a]));
-        if (touch && M->fine8[((size_t)b * 27 + e) * 8 + o] < 0)
-          return fail(CELLO_EINTERNAL, "2:1 balance violated: a touching neighbour is two levels finer");
-      }
-    }
-  // flux-register slots: faces whose neighbour is finer (coarse side) or coarser (fine side)
-  M->face_slot.assign((size_t)B * 6, -1);
+  CELLO_CUDA(cudaStreamSynchronize(s));   // buf is reused
+  CELLO_CUDA(cudaMemcpyAsync(buf.data(), M->d_flag, tail, cudaMemcpyDeviceToHost, s));
+  CELLO_CUDA(cudaStreamSynchronize(s));
+  int flag;
+  std::memcpy(&flag, buf.data(), sizeof(int));
+  if (flag & 1) return fail(CELLO_EINTERNAL, "2:1 balance violated: a neighbour is two levels coarser");
+  if (flag & 2) return fail(CELLO_EINTERNAL, "2:1 balance violated: a touching neighbour is two levels finer");
+  const int8_t* face = reinterpret_cast<const int8_t*>(buf.data() + (o_face - o_flag));
+  // flux-register slots: faces whose neighbour is finer (coarse side) or coarser
+  // (fine side); the coarse sides, grouped by leaf; the faces whose phase region
+  // the refresh computes instead of copying, those whose neighbour is not a
+  // same-level leaf (coarser, finer, boundary), in leaf order and by axis
+  M->face_slot.assign(B * 6, -1);
+  std::vector<int> slow, by_axis[3];
+  M->slow_start.assign(B + 1, 0);
+  for (int a = 0; a < 3; ++a) M->slow_ax_start[a].assign(B + 1, 0);
   int ns = 0;
-  for (int b = 0; b < B; ++b)
-    for (int f = 0; f < 6; ++f) {
-      const int k = M->kind[b * 27 + face_dir(f / 2, (f & 1) ? 1 : -1)];
-      if (k == kFine || k == kCoarse) M->face_slot[b * 6 + f] = ns++;
-    }
-  M->nslots = ns;
-  M->cfaces.clear();
-  M->group_start.clear();
-  for (int b = 0; b < B; ++b) {
+  for (size_t b = 0; b < B; ++b) {
     bool first = true;
     for (int f = 0; f < 6; ++f) {
-      const int axis = f / 2, side = (f & 1) ? 1 : -1;
-      const int e = b * 27 + face_dir(axis, side);
-      if (M->kind[e] != kFine) continue;
-      CoarseFace cf;
-      cf.leaf = b;
-      cf.axis = axis;
-      cf.side = side;
-      cf.cslot = M->face_slot[b * 6 + f];
-      const int t1 = axis == 0 ? 1 : 0, t2 = axis == 2 ? 1 : 2;
-      for (int o2 = 0; o2 < 2; ++o2)
-        for (int o1 = 0; o1 < 2; ++o1) {
-          int o[3];
-          o[axis] = side < 0 ? 1 : 0;
-          o[t1] = o1;
-          o[t2] = o2;
-          const int c = M->fine8[(size_t)e * 8 + o[2] * 4 + o[1] * 2 + o[0]];
-          if (c < 0) return fail(CELLO_EINTERNAL, "refined neighbour face without leaf children");
-          const int fs = M->face_slot[c * 6 + 2 * axis + (side < 0 ? 1 : 0)];
-          if (fs < 0) return fail(CELLO_EINTERNAL, "fine face without a register slot");
-          cf.fslot[o2 * 2 + o1] = fs;
-        }
+      const int at = (int)b * 6 + f, k = face[at];
+      if (k == kSame) continue;
+      slow.push_back(at);
+      by_axis[f >> 1].push_back(at);
+      if (k == kBoundary) continue;
+      M->face_slot[at] = ns++;
+      if (k != kFine) continue;
+      CoarseFace cf{};
+      cf.leaf = (int)b;
+      cf.axis = f >> 1;
+      cf.side = (f & 1) ? 1 : -1;
+      cf.cslot = M->face_slot[at];
       if (first) M->group_start.push_back((int)M->cfaces.size());
       first = false;
       M->cfaces.push_back(cf);
     }
+    M->slow_start[b + 1] = (int)slow.size();
+    for (int a = 0; a < 3; ++a) M->slow_ax_start[a][b + 1] = (int)by_axis[a].size();
   }
+  M->nslots = ns;
   if (!M->cfaces.empty()) M->group_start.push_back((int)M->cfaces.size());
-  CELLO_TRY(upload(&M->d_face_slot, M->face_slot));
-  CELLO_TRY(upload(&M->d_cfaces, M->cfaces));
-  CELLO_TRY(upload(&M->d_group_start, M->group_start));
-  if (ns > 0) CELLO_CUDA(cudaMalloc((void**)&M->d_reg, (size_t)ns * nfields(d) * d.n * d.n * sizeof(double)));
-  CELLO_CUDA(cudaMalloc((void**)&M->d_partials, (size_t)std::max(B, 1) * 6 * sizeof(double)));
-  // faces whose phase region the refresh computes instead of copying: those
-  // whose neighbour is not a same-level leaf (coarser, finer, boundary)
-  {
-    std::vector<int> slow, by_axis[3];
-    M->slow_start.assign((size_t)B + 1, 0);
-    for (int a = 0; a < 3; ++a) M->slow_ax_start[a].assign((size_t)B + 1, 0);
-    for (int b = 0; b < B; ++b) {
-      for (int f = 0; f < 6; ++f)
-        if (M->kind[(size_t)b * 27 + face_dir(f >> 1, (f & 1) ? 1 : -1)] != kSame) {
-          slow.push_back(b * 6 + f);
-          by_axis[f >> 1].push_back(b * 6 + f);
-        }
-      M->slow_start[b + 1] = (int)slow.size();
-      for (int a = 0; a < 3; ++a) M->slow_ax_start[a][b + 1] = (int)by_axis[a].size();
-    }
-    CELLO_TRY(upload(&M->d_slow, slow));
-    for (int a = 0; a < 3; ++a) CELLO_TRY(upload(&M->d_slow_ax[a], by_axis[a]));
+  Layout l;
+  const size_t o_slot = l.add<int>(B * 6), o_cf = l.add<CoarseFace>(M->cfaces.size()),
+               o_gs = l.add<int>(M->group_start.size()), o_slow = l.add<int>(slow.size());
+  size_t o_ax[3];
+  for (int a = 0; a < 3; ++a) o_ax[a] = l.add<int>(by_axis[a].size());
+  CELLO_CUDA(cudaMalloc((void**)&M->d_lists, l.bytes));
+  buf.resize(l.bytes);
+  auto put = [&](size_t at, const auto& v) {
+    if (!v.empty()) std::memcpy(buf.data() + at, v.data(), v.size() * sizeof(v[0]));
+  };
+  put(o_slot, M->face_slot);
+  put(o_cf, M->cfaces);
+  put(o_gs, M->group_start);
+  put(o_slow, slow);
+  for (int a = 0; a < 3; ++a) put(o_ax[a], by_axis[a]);
+  CELLO_CUDA(cudaMemcpyAsync(M->d_lists, buf.data(), l.bytes, cudaMemcpyHostToDevice, s));
+  M->d_face_slot = part<int>(M->d_lists, o_slot);
+  if (!M->cfaces.empty()) {
+    M->d_cfaces = part<CoarseFace>(M->d_lists, o_cf);
+    M->d_group_start = part<int>(M->d_lists, o_gs);
+    launch_fine_slots(M->dev(), M->d_cfaces, (int)M->cfaces.size(), s);
+    CELLO_CUDA(cudaGetLastError());
   }
-  CELLO_CUDA(cudaMalloc((void**)&M->d_work, sizeof(unsigned)));
-  CELLO_CUDA(cudaMalloc((void**)&M->d_err, sizeof(unsigned)));
-  CELLO_CUDA(cudaMemset(M->d_err, 0, sizeof(unsigned)));
-  CELLO_CUDA(cudaMalloc((void**)&M->d_zero, sizeof(double)));
-  CELLO_CUDA(cudaMemset(M->d_zero, 0, sizeof(double)));
-  CELLO_CUDA(cudaDeviceSynchronize());
+  if (!slow.empty()) M->d_slow = part<int>(M->d_lists, o_slow);
+  for (int a = 0; a < 3; ++a)
+    if (!by_axis[a].empty()) M->d_slow_ax[a] = part<int>(M->d_lists, o_ax[a]);
+  if (ns > 0) CELLO_CUDA(cudaMalloc((void**)&M->d_reg, (size_t)ns * nfields(d) * d.n * d.n * sizeof(double)));
+  CELLO_CUDA(cudaStreamSynchronize(s));   // the tables are read on any stream from here on
   return CELLO_OK;
 }
 
@@ -735,15 +802,13 @@ cello_status cello_octree_build(const cello_mesh_desc* desc, const cello_mesh* p
   if (!M) return fail(CELLO_ENOMEM, "host allocation failed");
   M->desc = *desc;
   M->N = desc->n + 2 * desc->ghosts;
-  std::vector<Node> ls = build_leaves(*desc, prev, flags_host);
-  std::vector<std::pair<unsigned long long, Node>> keyed;
-  keyed.reserve(ls.size());
-  for (const Node& t : ls) keyed.emplace_back(leaf_key(*desc, t), t);
-  std::sort(keyed.begin(), keyed.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
-  M->B = (int)keyed.size();
-  for (const auto& kv : keyed) {
-    M->keys.push_back(kv.first);
-    M->leaves.push_back(make_int4(kv.second.L, kv.second.i, kv.second.j, kv.second.k));
+  const std::vector<Node> ls = build_leaves(*desc, prev, flags_host);
+  M->B = (int)ls.size();
+  M->keys.reserve(ls.size());
+  M->leaves.reserve(ls.size());
+  for (const Node& t : ls) {
+    M->keys.push_back(leaf_key(*desc, t));
+    M->leaves.push_back(make_int4(t.L, t.i, t.j, t.k));
   }
   cello_status st = finish_build(M);
   if (st != CELLO_OK) {
@@ -836,9 +901,10 @@ cello_status cello_mesh_leaves(const cello_mesh* M, int32_t* out) {
 
 cello_status cello_neighbour_table(const cello_mesh* M, int8_t* kind, int32_t* idx, int32_t* fine8) {
   if (!M) return fail(CELLO_EINVAL, "mesh is NULL");
-  if (kind) std::memcpy(kind, M->kind.data(), M->kind.size());
-  if (idx) std::memcpy(idx, M->idx.data(), M->idx.size() * sizeof(int));
-  if (fine8) std::memcpy(fine8, M->fine8.data(), M->fine8.size() * sizeof(int));
+  const size_t entries = (size_t)M->B * 27;
+  if (kind) CELLO_CUDA(cudaMemcpy(kind, M->d_kind, entries, cudaMemcpyDeviceToHost));
+  if (idx) CELLO_CUDA(cudaMemcpy(idx, M->d_idx, entries * sizeof(int), cudaMemcpyDeviceToHost));
+  if (fine8) CELLO_CUDA(cudaMemcpy(fine8, M->d_fine8, entries * 8 * sizeof(int), cudaMemcpyDeviceToHost));
   return CELLO_OK;
 }
 
@@ -1075,53 +1141,17 @@ cello_status cello_remap(const cello_mesh* old, const void* U_old, const cello_m
   CELLO_REQUIRE_ALIGNED(U_new);
   if (std::memcmp(&old->desc, &neu->desc, sizeof(cello_mesh_desc)) != 0)
     return fail(CELLO_EINVAL, "meshes built from different descriptions");
-  std::unordered_map<unsigned long long, int> where;
-  for (int b = 0; b < old->B; ++b) {
-    const int4 l = old->leaves[b];
-    where[pack(Node{l.x, l.y, l.z, l.w})] = b;
-  }
-  std::vector<RemapEntry> map(neu->B);
-  for (int b = 0; b < neu->B; ++b) {
-    const int4 l = neu->leaves[b];
-    const Node t{l.x, l.y, l.z, l.w};
-    RemapEntry e{};
-    auto it = where.find(pack(t));
-    if (it != where.end()) {
-      e.kind = 0;
-      e.src[0] = it->second;
-    } else {
-      bool found = false;
-      for (int k = 1; k <= t.L && !found; ++k) {
-        auto a = where.find(pack(Node{t.L - k, t.i >> k, t.j >> k, t.k >> k}));
-        if (a != where.end()) {
-          e.kind = 1;
-          e.k = k;
-          e.src[0] = a->second;
-          found = true;
-        }
-      }
-      if (!found) {
-        e.kind = 2;
-        for (int o = 0; o < 8; ++o) {
-          auto c = where.find(pack(child(t, o)));
-          if (c == where.end()) return fail(CELLO_EINVAL, "meshes are not one adaptation apart");
-          e.src[o] = c->second;
-        }
-      }
-    }
-    map[b] = e;
-  }
-  RemapEntry* d_map = nullptr;
-  CELLO_CUDA(cudaMalloc((void**)&d_map, map.size() * sizeof(RemapEntry)));
+  // the entries by binary search of the sorted keys on the device; if a new leaf
+  // has no source there, nothing is written and the call says so
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = cudaMemcpyAsync(d_map, map.data(), map.size() * sizeof(RemapEntry), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) {
-    launch_remap(neu->dev(), old->dev(), U_old, U_new, d_map, neu->desc.precision, s);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the map is freed below
-  cudaFree(d_map);
-  CELLO_CUDA(e);
+  CELLO_CUDA(cudaMemsetAsync(neu->d_flag, 0, sizeof(int), s));
+  launch_remap(neu->dev(), neu->d_keys, old->dev(), old->d_keys, U_old, U_new, neu->d_map, neu->d_flag,
+               neu->desc.precision, s);
+  CELLO_CUDA(cudaGetLastError());
+  int flag = 0;
+  CELLO_CUDA(cudaMemcpyAsync(&flag, neu->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CELLO_CUDA(cudaStreamSynchronize(s));
+  if (flag) return fail(CELLO_EINVAL, "meshes are not one adaptation apart");
   return CELLO_OK;
 }
 
