@@ -113,7 +113,7 @@ struct SweepParams {
   double* reg;             // flux registers (may be null)
   unsigned* work;          // work counter for persistent variants (device, 4 bytes)
   int n_items;             // set by the launcher
-  int variant;             // index into the sweep variants of the precision
+  int variant;             // index into the sweep variants of the precision; -1: the launcher's rule
 
   // The items of the three regions for per_cta pencils per item.
   void plan(int per_cta) {
@@ -239,9 +239,12 @@ template <int NB, int CT, int VEC>
 void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
 template <int NB>
 void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
+constexpr int kSweepKernels = 12;   // float32 sweep kernel instantiations per method code
+// Attributes of the dual-energy kernels and their resident CTAs, rows 4 to 7 of the table.
 template <int NB>
-void prepare_sweep_de_f32();
-void prepare_kernels_de_f64();
+void prepare_sweep_de_f32(int (*resident)[kSweepKernels], int sms);
+// Attributes of the float64 dual-energy kernels and their resident CTAs, by block size and method code.
+void prepare_kernels_de_f64(int (*resident)[8], int sms);
 void launch_fluxcorr(const DevMesh& m, void* U, int precision, const CoarseFace* faces,
                      const int* group_start, int ngroups, const double* reg, const double* dt,
                      cudaStream_t s);

@@ -10,7 +10,7 @@ namespace cello {
 // Float64 sweep variants: {pencils per CTA, min resident CTAs per SM, persistent}.
 static const SweepVariant kVariants64[] = {{8, 2, false}, {8, 2, true}};
 constexpr int kNV64 = 2;
-static int g_resident64[3];
+static int g_resident64[3][8];   // resident CTAs per GPU by block size and method code
 
 static int nb_index64(int n) { return n == 8 ? 0 : (n == 16 ? 1 : 2); }
 
@@ -21,33 +21,35 @@ static constexpr size_t sweep_smem64() {
 }
 
 template <int NB, int RS>
-static void set_smem_attr64() {
-  cudaFuncSetAttribute(sweep_kernel<double, NB, 8, 2, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sweep_smem64<NB, RS>());
+static void prepare_method64(int sms) {
+  constexpr int T = (NB + 2 * kGhosts) * 8;
+  constexpr size_t sh = sweep_smem64<NB, RS>();
+  int nb = 0;
+  cudaFuncSetAttribute(sweep_kernel<double, NB, 8, 2, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<double, NB, 8, 2, RS>, T, sh);
+  g_resident64[nb_index64(NB)][RS] = (nb > 0 ? nb : 1) * sms;
 }
 
 template <int NB>
 static void prepare_nb64(int sms) {
-  constexpr int N = NB + 2 * kGhosts;
-  set_smem_attr64<NB, 0>();
-  set_smem_attr64<NB, 1>();
-  set_smem_attr64<NB, 2>();
-  set_smem_attr64<NB, 3>();
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<double, NB, 8, 2, 0>, N * 8, sweep_smem64<NB, 0>());
-  g_resident64[nb_index64(NB)] = (nb > 0 ? nb : 1) * sms;
+  prepare_method64<NB, 0>(sms);
+  prepare_method64<NB, 1>(sms);
+  prepare_method64<NB, 2>(sms);
+  prepare_method64<NB, 3>(sms);
 }
 
 template <int NB>
 static void launch_nb64(const DevMesh& m, SweepParams p, cudaStream_t s) {
   constexpr int N = NB + 2 * kGhosts;
-  const int v = (p.variant >= 0 && p.variant < kNV64) ? p.variant : 0;
+  // not chosen by the caller: the persistent schedule, never slower (939 leaves of
+  // 16^3, two steps: 57.4 -> 55.8 ms)
+  const int v = (p.variant >= 0 && p.variant < kNV64) ? p.variant : 1;
   p.plan(8);
   if (p.n_items <= 0) return;
   int grid = p.n_items;
   if (kVariants64[v].persistent && p.work) {
-    cudaMemsetAsync(p.work, 0, sizeof(unsigned), s);
-    grid = g_resident64[nb_index64(NB)] < grid ? g_resident64[nb_index64(NB)] : grid;
+    const int resident = g_resident64[nb_index64(NB)][method_code(m.riemann, m.steepen, m.nf == 6)];
+    grid = resident < grid ? resident : grid;
   } else {
     p.work = nullptr;
   }
@@ -99,6 +101,7 @@ void prepare_kernels_f64() {
   prepare_nb64<8>(sms);
   prepare_nb64<16>(sms);
   prepare_nb64<32>(sms);
+  prepare_kernels_de_f64(g_resident64, sms);
   prepare_adj<8>();
   prepare_adj<16>();
   prepare_adj<32>();
@@ -181,7 +184,7 @@ void launch_reduce_range(const DevMesh& m, const void* U, int precision, double 
     CELLO_RED(double)
   }
 #undef CELLO_RED
-  reduce_finish_kernel<<<1, 1024, 0, s>>>(partials + (long)leaf0 * 6, nleaf, cfl, dt_next, totals);
+  reduce_finish_kernel<<<1, kFinishThreads, 0, s>>>(partials + (long)leaf0 * 6, nleaf, cfl, dt_next, totals);
 }
 
 void launch_reduce(const DevMesh& m, const void* U, int precision, double cfl, double* partials,

@@ -83,6 +83,17 @@ __device__ __forceinline__ long push_offset(const DevMesh& m, const SweepParams&
   return ((long)m.idx[e] - at.leaf) * NQ * SLAB - side * NB * stride;
 }
 
+// The item after the one a CTA of the persistent schedule is about to work on
+// (its first is its block index): drawn from the counter before the work, so that
+// the atomic's latency lies under it.  Every item draws once, n_items draws in
+// all, so the draw of n_items - 1 is the last and leaves the counter at 0 for
+// the next launch.
+__device__ __forceinline__ int next_item(const SweepParams& prm) {
+  const unsigned v = atomicAdd(prm.work, 1u);
+  if (v == (unsigned)prm.n_items - 1u) *prm.work = 0u;
+  return (int)(gridDim.x + v);
+}
+
 template <typename T, int NB, int P, int MINB, int RS>
 __global__ void __launch_bounds__((NB + 8) * P, MINB)
 sweep_kernel(DevMesh m, SweepParams prm) {
@@ -126,12 +137,9 @@ sweep_kernel(DevMesh m, SweepParams prm) {
   __syncthreads();
 
   int item = blockIdx.x;
-  if (prm.work) {
-    if (t == 0) s_item = (int)atomicAdd(prm.work, 1u);
-    __syncthreads();
-    item = s_item;
-  }
   while (item < prm.n_items) {
+    int next = item + gridDim.x;
+    if (prm.work && t == 0) next = next_item(prm);
     const PencilAt at = prm.locate(item, P);
     const SweepRegion& rg = prm.reg3[at.r];
     const int leaf = at.leaf;
@@ -326,14 +334,14 @@ sweep_kernel(DevMesh m, SweepParams prm) {
         for (int k = 0; k < NQ; ++k) base[push + comp[k] * SLAB] = Un[k];
       }
     }
-    __syncthreads();
     if (prm.work) {
-      if (t == 0) s_item = (int)atomicAdd(prm.work, 1u);
+      if (t == 0) s_item = next;
       __syncthreads();
       item = s_item;
     } else {
-      item += gridDim.x;
+      item = next;
     }
+    __syncthreads();
   }
 }
 
@@ -608,12 +616,9 @@ sweep_stream_kernel(DevMesh m, SweepParams prm) {
   __syncthreads();
 
   int item = blockIdx.x;
-  if (prm.work) {
-    if (t == 0) s_item = (int)atomicAdd(prm.work, 1u);
-    __syncthreads();
-    item = s_item;
-  }
   while (item < prm.n_items) {
+    int next = item + gridDim.x;
+    if (prm.work && t == 0) next = next_item(prm);
     const PencilAt at = prm.locate(item, CT);
     const SweepRegion& rg = prm.reg3[at.r];
     const int leaf = at.leaf;
@@ -729,11 +734,11 @@ sweep_stream_kernel(DevMesh m, SweepParams prm) {
     }
     if (prm.work) {
       __syncthreads();
-      if (t == 0) s_item = (int)atomicAdd(prm.work, 1u);
+      if (t == 0) s_item = next;
       __syncthreads();
       item = s_item;
     } else {
-      item += gridDim.x;
+      item = next;
     }
   }
 }
@@ -1444,30 +1449,33 @@ __global__ void __launch_bounds__(256) remap_kernel(DevMesh neu, DevMesh old, co
 // then a single-CTA fixed-order finish.  Deterministic.
 // =====================================================================
 constexpr int kReduceThreads = 256;
+constexpr int kFinishThreads = 512;
 
-__device__ __forceinline__ void block_reduce6(double v[6], double* sh) {
-  // v[0] min, v[1..5] sums; fixed tree: xor shuffles, then warp 0 over warps.
+// Minimum of v[0] and sums of v[1..5] over the first `used` threads of the CTA,
+// in thread 0: each quantity by one warp, its lanes over the threads' values in
+// steps of 32 and then a fixed tree.  (Trees of shuffles in every warp run 30
+// float64 instructions per warp; the float64 pipe takes two lanes a clock.)
+template <int THREADS>
+__device__ __forceinline__ void block_reduce6(double v[6], double* sh, int used = THREADS) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v[0] = fmin(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
-#pragma unroll
-    for (int k = 1; k < 6; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (l == 0)
-#pragma unroll
-    for (int k = 0; k < 6; ++k) sh[w * 6 + k] = v[k];
+  for (int k = 0; k < 6; ++k) sh[k * THREADS + threadIdx.x] = v[k];
   __syncthreads();
-  if (w == 0) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) v[k] = (l < nw) ? sh[l * 6 + k] : (k == 0 ? INFINITY : 0.0);
+  const int k = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (k < 6) {
+    double* q = sh + k * THREADS;
+    double a = q[l];
+    for (int i = 32; i < used; i += 32) a = k == 0 ? fmin(a, q[i + l]) : a + q[i + l];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      v[0] = fmin(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
-#pragma unroll
-      for (int k = 1; k < 6; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+      const double b = __shfl_xor_sync(0xffffffffu, a, o);
+      a = k == 0 ? fmin(a, b) : a + b;
     }
+    if (l == 0) q[0] = a;
   }
+  __syncthreads();
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int k2 = 0; k2 < 6; ++k2) v[k2] = sh[k2 * THREADS];
 }
 
 // NF = 6 (dual energy): the pressure for the sound speed and the health
@@ -1477,7 +1485,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_kernel(DevMesh
                                                                          int leaf0, int nleaf) {
   constexpr int G = kGhosts, N = NB + 2 * G;
   constexpr long SLAB = (long)N * N * N;
-  __shared__ double sh[6 * 32];
+  __shared__ double sh[6 * kReduceThreads];
   for (int lr = blockIdx.x; lr < nleaf; lr += gridDim.x) {
   const int leaf = leaf0 + lr;
   const int4 lf = m.leaf[leaf];
@@ -1504,7 +1512,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_kernel(DevMesh
     v[1] += double(r0); v[2] += double(m1); v[3] += double(m2); v[4] += double(m3); v[5] += double(E);
   }
   bad = __syncthreads_or(bad);
-  block_reduce6(v, sh);
+  block_reduce6<kReduceThreads>(v, sh);
   if (threadIdx.x == 0) {
     const double dxd = ldexp(m.dx0, -lf.x);
     const double vol = dxd * dxd * dxd;
@@ -1533,7 +1541,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_f32_kernel(Dev
                                                                              double* partials, int leaf0, int nleaf) {
   constexpr int G = kGhosts, N = NB + 2 * G;
   constexpr long SLAB = (long)N * N * N;
-  __shared__ double sh[6 * 32];
+  __shared__ double sh[6 * kReduceThreads];
   for (int lr = blockIdx.x; lr < nleaf; lr += gridDim.x) {
   const int leaf = leaf0 + lr;
   const int4 lf = m.leaf[leaf];
@@ -1578,7 +1586,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_f32_kernel(Dev
 #pragma unroll
   for (int k = 0; k < 5; ++k) v[k + 1] = double(hi[k]) + double(lo[k]);
   bad = __syncthreads_or(bad);
-  block_reduce6(v, sh);
+  block_reduce6<kReduceThreads>(v, sh);
   if (threadIdx.x == 0) {
     const double dxd = ldexp(m.dx0, -lf.x);
     const double vol = dxd * dxd * dxd;
@@ -1591,15 +1599,15 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_f32_kernel(Dev
 }
 
 #ifdef CELLO_DEFINE_FINISH_KERNEL
-__global__ void __launch_bounds__(1024) reduce_finish_kernel(const double* partials, int B, double cfl,
+__global__ void __launch_bounds__(kFinishThreads) reduce_finish_kernel(const double* partials, int B, double cfl,
                                                              double* dt_next, double* totals) {
-  __shared__ double sh[6 * 32];
+  __shared__ double sh[6 * kFinishThreads];
   double v[6] = {INFINITY, 0, 0, 0, 0, 0};
   for (int i = threadIdx.x; i < B; i += blockDim.x) {
     v[0] = fmin(v[0], partials[i * 6]);
     for (int k = 1; k < 6; ++k) v[k] += partials[i * 6 + k];
   }
-  block_reduce6(v, sh);
+  block_reduce6<kFinishThreads>(v, sh, B < kFinishThreads ? B : kFinishThreads);
   if (threadIdx.x == 0) {
     if (dt_next) *dt_next = cfl * v[0];
     if (totals)

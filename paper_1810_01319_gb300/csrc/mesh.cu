@@ -193,10 +193,6 @@ void prepare_kernels() {
   std::call_once(once, [] {
     prepare_kernels_f32();
     prepare_kernels_f64();
-    prepare_sweep_de_f32<8>();
-    prepare_sweep_de_f32<16>();
-    prepare_sweep_de_f32<32>();
-    prepare_kernels_de_f64();
   });
   // L2 fetch granularity of this process's context on the current device, set
   // once per device: 64 bytes.  The ghost refresh reads 32-byte margin
@@ -256,7 +252,7 @@ struct cello_mesh {
   int* d_slow_ax[3] = {nullptr, nullptr, nullptr};   // the same faces by axis, and their per-leaf offsets
   std::vector<int> slow_ax_start[3];
   int exec_mode = CELLO_EXEC_BATCHED;
-  int sweep_variant[3] = {0, 0, 0};   // per sweep axis; chosen by cello_autotune or set by the caller
+  int sweep_variant[3] = {-1, -1, -1};   // per sweep axis; chosen by cello_autotune or set by the caller, -1: by rule
   unsigned* d_work = nullptr;      // work counter of the persistent sweep variants
   unsigned* d_err = nullptr;       // error word set by the reduction
   int* d_flag = nullptr;           // result word of the table and remap-map kernels

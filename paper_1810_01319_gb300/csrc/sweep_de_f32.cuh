@@ -31,9 +31,7 @@ void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaS
 // threads per SM): every variant is bounded for 384 threads per SM (168
 // registers), where nothing spills.  At 128 registers the spills (100 to 670
 // bytes a thread) cost more than the extra warps give: 183 leaves of 32^3 with
-// HLLC and steepening, two steps of variants 22, 21, 21, 2.06 -> 1.72 ms.  The
-// resident grid of the persistent schedule is the five-field kernel's: the CTAs
-// beyond 384 threads per SM start as others find the counter run out.
+// HLLC and steepening, two steps of variants 22, 21, 21, 2.06 -> 1.72 ms.
 template <int NB, int CT, int VEC>
 void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s) {
   constexpr int MINB = 384 / CT;
@@ -54,16 +52,31 @@ CELLO_DE_STREAM(CELLO_DE_SINST, CELLO_DE_NB)
 #undef CELLO_DE_SINST
 #undef CELLO_DE_STREAM
 
+template <typename K>
+static int resident_de(K kernel, int threads, size_t smem, int sms) {
+  int nb = 0;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem);
+  return (nb > 0 ? nb : 1) * sms;
+}
+
 template <int NB, int P, int MINB>
-static void prepare_de() {
-#define CELLO_DE_ATTR(RS)                                                                          \
-  cudaFuncSetAttribute(sweep_kernel<float, NB, P, MINB, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                       (int)de_smem<NB, P, RS>())
-  CELLO_DE_ATTR(4);
-  CELLO_DE_ATTR(5);
-  CELLO_DE_ATTR(6);
-  CELLO_DE_ATTR(7);
-#undef CELLO_DE_ATTR
+static void prepare_de(int (*resident)[kSweepKernels], int v, int sms) {
+  constexpr int T = (NB + 2 * kGhosts) * P;
+  resident[4][v] = resident_de(sweep_kernel<float, NB, P, MINB, 4>, T, de_smem<NB, P, 4>(), sms);
+  resident[5][v] = resident_de(sweep_kernel<float, NB, P, MINB, 5>, T, de_smem<NB, P, 5>(), sms);
+  resident[6][v] = resident_de(sweep_kernel<float, NB, P, MINB, 6>, T, de_smem<NB, P, 6>(), sms);
+  resident[7][v] = resident_de(sweep_kernel<float, NB, P, MINB, 7>, T, de_smem<NB, P, 7>(), sms);
+}
+
+template <int NB, int CT, int VEC>
+static void prepare_stream_de(int (*resident)[kSweepKernels], int v, int sms) {
+  constexpr int MINB = 384 / CT;
+  constexpr size_t sh = VEC == 3 ? sizeof(float4) * 4 * 6 * CT : 0;
+  resident[4][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 4>, CT, sh, sms);
+  resident[5][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 5>, CT, sh, sms);
+  resident[6][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 6>, CT, sh, sms);
+  resident[7][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 7>, CT, sh, sms);
 }
 
 // The shared-memory variants of the float32 table: {pencils, min CTAs per SM}.
@@ -73,12 +86,23 @@ static void prepare_de() {
 CELLO_DE_VARIANTS(CELLO_DE_INST, CELLO_DE_NB)
 #undef CELLO_DE_INST
 
-template <>
-void prepare_sweep_de_f32<CELLO_DE_NB>() {
-#define CELLO_DE_PREP(NB, P, MINB) prepare_de<NB, P, MINB>();
-  CELLO_DE_VARIANTS(CELLO_DE_PREP, CELLO_DE_NB)
-#undef CELLO_DE_PREP
-}
 #undef CELLO_DE_VARIANTS
+
+template <>
+void prepare_sweep_de_f32<CELLO_DE_NB>(int (*resident)[kSweepKernels], int sms) {
+  constexpr int NB = CELLO_DE_NB;
+  prepare_de<NB, 8, 3>(resident, 0, sms);
+  prepare_de<NB, 8, 4>(resident, 1, sms);
+  prepare_de<NB, 4, 6>(resident, 2, sms);
+  prepare_de<NB, 16, 1>(resident, 3, sms);
+  prepare_de<NB, 4, 8>(resident, 4, sms);
+  prepare_de<NB, 16, 2>(resident, 5, sms);
+  prepare_stream_de<NB, 64, 0>(resident, 6, sms);
+  prepare_stream_de<NB, 128, 0>(resident, 7, sms);
+  prepare_stream_de<NB, 64, 0>(resident, 8, sms);
+  prepare_stream_de<NB, 32, 0>(resident, 9, sms);
+  prepare_stream_de<NB, 64, 3>(resident, 10, sms);
+  prepare_stream_de<NB, 64, 3>(resident, 11, sms);
+}
 
 }  // namespace cello

@@ -19,9 +19,20 @@ static const SweepVariant kVariants[] = {
     {4, 8, true, false},   {16, 2, true, false},  {64, 8, true, true},  {128, 4, true, true},
     {64, 6, true, true},   {32, 16, true, true},  {64, 8, true, true, 3},  {64, 6, true, true, 3},
 };
-constexpr int kNT = 12;  // distinct kernel instantiations; variant v uses template v % kNT
+constexpr int kNT = kSweepKernels;  // variant v uses template v % kNT
 constexpr int kNV = sizeof(kVariants) / sizeof(kVariants[0]);
-template <int NB> inline int g_resident[kNV];   // resident CTAs per GPU by variant, from the occupancy API
+// Resident CTAs per GPU by method code and kernel instantiation, from the
+// occupancy API: a persistent launch of more would leave the rest waiting with
+// their first items.
+template <int NB> inline int g_resident[8][kNT];
+
+template <int NB, typename K>
+static void set_resident(int rs, int v, K kernel, int threads, size_t smem, int sms) {
+  int nb = 0;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem);
+  g_resident<NB>[rs][v] = (nb > 0 ? nb : 1) * sms;
+}
 
 // Shared memory of the shared-memory form: sweep_arrays(RS) arrays of N x P
 // values (21; 24 with contact steepening).
@@ -31,23 +42,13 @@ static constexpr size_t sweep_smem() {
   return sizeof(float) * sweep_arrays(RS) * N * P;
 }
 
-template <int NB, int P, int MINB, int RS>
-static void set_smem_attr() {
-  cudaFuncSetAttribute(sweep_kernel<float, NB, P, MINB, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sweep_smem<NB, P, RS>());
-}
-
 template <int NB, int P, int MINB>
 static void prepare_variant(int v, int sms) {
-  constexpr int N = NB + 2 * kGhosts;
-  set_smem_attr<NB, P, MINB, 0>();
-  set_smem_attr<NB, P, MINB, 1>();
-  set_smem_attr<NB, P, MINB, 2>();
-  set_smem_attr<NB, P, MINB, 3>();
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<float, NB, P, MINB, 0>, N * P,
-                                                sweep_smem<NB, P, 0>());
-  g_resident<NB>[v] = (nb > 0 ? nb : 1) * sms;
+  constexpr int T = (NB + 2 * kGhosts) * P;
+  set_resident<NB>(0, v, sweep_kernel<float, NB, P, MINB, 0>, T, sweep_smem<NB, P, 0>(), sms);
+  set_resident<NB>(1, v, sweep_kernel<float, NB, P, MINB, 1>, T, sweep_smem<NB, P, 1>(), sms);
+  set_resident<NB>(2, v, sweep_kernel<float, NB, P, MINB, 2>, T, sweep_smem<NB, P, 2>(), sms);
+  set_resident<NB>(3, v, sweep_kernel<float, NB, P, MINB, 3>, T, sweep_smem<NB, P, 3>(), sms);
 }
 
 // Dynamic shared memory of the streaming form: the staged form keeps three
@@ -59,21 +60,22 @@ static constexpr size_t stream_smem() {
 
 template <int NB, int CT, int MINB, int VEC>
 static void prepare_stream_variant(int v, int sms) {
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_stream_kernel<float, NB, CT, MINB, VEC, 0>, CT,
-                                                stream_smem<CT, VEC>());
-  g_resident<NB>[v] = (nb > 0 ? nb : 1) * sms;
+  constexpr size_t sh = stream_smem<CT, VEC>();
+  set_resident<NB>(0, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 0>, CT, sh, sms);
+  set_resident<NB>(1, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 1>, CT, sh, sms);
+  set_resident<NB>(2, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 2>, CT, sh, sms);
+  set_resident<NB>(3, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 3>, CT, sh, sms);
 }
 
 // Work items, grid and schedule of one launch; false if there is no work.
 template <int NB>
-static bool plan_launch(SweepParams& p, int per_cta, int v, int& grid, cudaStream_t s) {
+static bool plan_launch(const DevMesh& m, SweepParams& p, int per_cta, int v, int& grid) {
   p.plan(per_cta);
   if (p.n_items <= 0) return false;
   grid = p.n_items;
   if (kVariants[v].persistent && p.work) {
-    cudaMemsetAsync(p.work, 0, sizeof(unsigned), s);
-    grid = g_resident<NB>[v] < grid ? g_resident<NB>[v] : grid;
+    const int resident = g_resident<NB>[method_code(m.riemann, m.steepen, m.nf == 6)][v % kNT];
+    grid = resident < grid ? resident : grid;
   } else {
     p.work = nullptr;
   }
@@ -84,7 +86,7 @@ template <int NB, int P, int MINB>
 static void launch_variant(const DevMesh& m, SweepParams p, int v, cudaStream_t s) {
   constexpr int N = NB + 2 * kGhosts;
   int grid = 0;
-  if (!plan_launch<NB>(p, P, v, grid, s)) return;
+  if (!plan_launch<NB>(m, p, P, v, grid)) return;
   switch (method_code(m.riemann, m.steepen, m.nf == 6)) {
     case 0: sweep_kernel<float, NB, P, MINB, 0><<<grid, N * P, sweep_smem<NB, P, 0>(), s>>>(m, p); break;
     case 1: sweep_kernel<float, NB, P, MINB, 1><<<grid, N * P, sweep_smem<NB, P, 1>(), s>>>(m, p); break;
@@ -97,7 +99,7 @@ static void launch_variant(const DevMesh& m, SweepParams p, int v, cudaStream_t 
 template <int NB, int CT, int MINB, int VEC>
 static void launch_stream_variant(const DevMesh& m, SweepParams p, int v, cudaStream_t s) {
   int grid = 0;
-  if (!plan_launch<NB>(p, CT, v, grid, s)) return;
+  if (!plan_launch<NB>(m, p, CT, v, grid)) return;
   constexpr size_t sh = stream_smem<CT, VEC>();
   if (m.nf == 6) {   // dual energy (sweep_de_f32.cuh)
     launch_stream_de_f32<NB, CT, VEC>(m, p, grid, s);
@@ -125,12 +127,29 @@ void prepare_sweep_f32(int sms) {
   prepare_stream_variant<NB, 32, 16, 0>(9, sms);
   prepare_stream_variant<NB, 64, 8, 3>(10, sms);
   prepare_stream_variant<NB, 64, 6, 3>(11, sms);
-  for (int v = kNT; v < kNV; ++v) g_resident<NB>[v] = g_resident<NB>[v - kNT];
+  prepare_sweep_de_f32<NB>(g_resident<NB>, sms);
+}
+
+// The variant of a sweep that the caller has not chosen one for.  The streaming
+// form takes the time of one pencil's walk however few there are (18, 24 and 37
+// us for n = 8, 16 and 32), the shared-memory form, a thread per cell, less while
+// its CTAs fill one wave: 16.7, 22.8 and 36 us at 14, 16 and 18 thousand pencils,
+// 27, 39 and 75 against 22, 31 and 59 us at 33, 37 and 49 thousand.  The
+// persistent schedule is never slower than one CTA per item (64 leaves of 16^3:
+// 23 against 39 us).  On x the staged form bounded for 6 CTAs per SM is ahead up
+// to some hundred thousand pencils (512 leaves of 16^3: 73 against 80 us), for 8
+// beyond (4,096 leaves of 32^3: 3.7 against 4.0 ms).
+template <int NB>
+static int default_variant(const SweepParams& p) {
+  long pencils = (long)p.nleaf * p.reg3[0].count;
+  for (int r = 1; r < 3; ++r) pencils += (long)p.reg3[r].nfaces * p.reg3[r].count;
+  if (pencils < 20000) return 12;
+  return p.axis != 0 ? 18 : (pencils < 400000 ? 23 : 22);
 }
 
 template <int NB>
 void launch_sweep_f32_nb(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
-  const int v = (p.variant >= 0 && p.variant < kNV) ? p.variant : 0;
+  const int v = (p.variant >= 0 && p.variant < kNV) ? p.variant : default_variant<NB>(p);
   switch (v % kNT) {
     case 0: launch_variant<NB, 8, 3>(m, p, v, s); break;
     case 1: launch_variant<NB, 8, 4>(m, p, v, s); break;
