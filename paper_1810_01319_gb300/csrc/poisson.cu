@@ -250,27 +250,46 @@ __device__ __forceinline__ long cell_at(int n, const int* s_nb, int x, int y, in
   return (((long)s_nb[e] * n + z) * n + y) * n + x;
 }
 
-// Cell i of a cube of E + 2 H cells per edge around the tile: offsets from the
-// tile's origin, -H .. E + H - 1.
+// A thread works on columns along z of the cube of E + 2 H cells per edge around
+// a tile: where a column lies is found once (the neighbour lookup and the index
+// divisions took two thirds of the instructions of a cell-by-cell form), its
+// loads are independent, and a stencil keeps the column's own values in registers.
+template <int E, int H> constexpr int kColumns = (E + 2 * H) * (E + 2 * H);
+template <int E, int H> constexpr int kCube = kColumns<E, H> * (E + 2 * H);
+// Threads per CTA: one column each at the widest halo.
+template <int E> constexpr int kTileThreads = E == 16 ? 416 : (E == 8 ? 160 : 64);
+
+template <int E>
+struct Column {
+  long lo, mid, hi, plane;   // of the cells below, in and above the tile
+
+  // (x, y): offsets from the tile's origin
+  __device__ __forceinline__ Column(int n, const int* s_nb, const Tile<E>& w, int x, int y) {
+    plane = (long)n * n;
+    mid = cell_at(n, s_nb, w.x + x, w.y + y, w.z);
+    lo = w.z == 0 ? cell_at(n, s_nb, w.x + x, w.y + y, -1) + plane : mid;
+    hi = w.z + E == n ? cell_at(n, s_nb, w.x + x, w.y + y, n) - E * plane : mid;
+  }
+  __device__ __forceinline__ long at(int z) const { return (z < 0 ? lo : (z < E ? mid : hi)) + z * plane; }
+};
+
 template <int E, int H>
-__device__ __forceinline__ void cube_cell(int i, int& x, int& y, int& z) {
-  constexpr int W = E + 2 * H;
-  x = i % W - H;
-  y = (i / W) % W - H;
-  z = i / (W * W) - H;
+__device__ __forceinline__ void column_xy(int c, int& x, int& y) {
+  x = c % (E + 2 * H) - H;
+  y = c / (E + 2 * H) - H;
 }
 template <int E, int H>
 __device__ __forceinline__ int cube_at(int x, int y, int z) {
   constexpr int W = E + 2 * H;
   return ((z + H) * W + (y + H)) * W + x + H;
 }
-template <int E, int H> constexpr int kCube = (E + 2 * H) * (E + 2 * H) * (E + 2 * H);
-template <int E> constexpr int kTileThreads = E == 16 ? 512 : (E == 8 ? 256 : 64);
 
+// The neighbour sum of the cell at p, its column's neighbours in registers.
 template <typename T, int W>
-__device__ __forceinline__ T cube_sum(const T* p) {
-  return ((((p[-1] + p[1]) + p[-W]) + p[W]) + p[-W * W]) + p[W * W];
+__device__ __forceinline__ T cross_sum(const T* p, T below, T above) {
+  return ((((p[-1] + p[1]) + p[-W]) + p[W]) + below) + above;
 }
+
 // Where the restricted residual goes: the blocks of the next level ([B][(n/2)^3]),
 // or, leaf given, one periodic array of Mg cells per edge.
 struct Coarse {
@@ -291,7 +310,7 @@ template <typename T, int E, int H>
 __device__ __forceinline__ void restrict_tile(const T* r, const TileLevel& L, const Tile<E>& w, const Coarse& to,
                                               T* fc) {
   constexpr int W = E + 2 * H, EC = E / 2;
-  for (int i = threadIdx.x; i < EC * EC * EC; i += blockDim.x) {
+  for (int i = threadIdx.x; i < EC * EC * EC; i += kTileThreads<E>) {
     const int X = i % EC, Y = (i / EC) % EC, Z = i / (EC * EC);
     const T* p = r + cube_at<E, H>(2 * X, 2 * Y, 2 * Z);
     T s = p[0];
@@ -317,27 +336,46 @@ tile_down_kernel(TileLevel L, const T* __restrict__ f, T* __restrict__ phi, Coar
   T* sP = sF + kCube<E, 2>;                        // phi after two sweeps, halo 1
   __shared__ int s_nb[27];
   const Tile<E> w = tile_of<E>(L, s_nb);
-  int x, y, z;
-  for (int i = threadIdx.x; i < kCube<E, 2>; i += blockDim.x) {
-    cube_cell<E, 2>(i, x, y, z);
-    sF[i] = f[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)];
-  }
-  __syncthreads();
   constexpr int W2 = E + 4, W1 = E + 2;
-  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
-    cube_cell<E, 1>(i, x, y, z);
-    const T* p = sF + cube_at<E, 2>(x, y, z);
-    const T s = ((((relax_zero(p[-1], h2) + relax_zero(p[1], h2)) + relax_zero(p[-W2], h2)) + relax_zero(p[W2], h2)) +
-                 relax_zero(p[-W2 * W2], h2)) + relax_zero(p[W2 * W2], h2);
-    sP[i] = relax(relax_zero(p[0], h2), s, p[0], h2);
+  int x, y;
+  for (int c = threadIdx.x; c < kColumns<E, 2>; c += kTileThreads<E>) {
+    column_xy<E, 2>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+#pragma unroll
+    for (int z = -2; z < E + 2; ++z) sF[(z + 2) * W2 * W2 + c] = f[col.at(z)];
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
-    cube_cell<E, 0>(i, x, y, z);
-    const T* p = sP + cube_at<E, 1>(x, y, z);
-    T* q = sF + cube_at<E, 2>(x, y, z);
-    phi[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)] = p[0];
-    *q = residual_of(p[0], cube_sum<T, W1>(p), *q, ih2);
+  for (int c = threadIdx.x; c < kColumns<E, 1>; c += kTileThreads<E>) {
+    column_xy<E, 1>(c, x, y);
+    const T* p = sF + cube_at<E, 2>(x, y, -1);
+    T g = p[0];
+    T below = relax_zero(p[-W2 * W2], h2), own = relax_zero(g, h2);
+#pragma unroll
+    for (int z = -1; z < E + 1; ++z, p += W2 * W2) {
+      const T gn = p[W2 * W2], above = relax_zero(gn, h2);
+      const T s = ((((relax_zero(p[-1], h2) + relax_zero(p[1], h2)) + relax_zero(p[-W2], h2)) +
+                    relax_zero(p[W2], h2)) + below) + above;
+      sP[(z + 1) * W1 * W1 + c] = relax(own, s, g, h2);
+      below = own;
+      own = above;
+      g = gn;
+    }
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < kColumns<E, 0>; c += kTileThreads<E>) {
+    column_xy<E, 0>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    const T* p = sP + cube_at<E, 1>(x, y, 0);
+    T* q = sF + cube_at<E, 2>(x, y, 0);
+    T below = p[-W1 * W1], own = p[0];
+#pragma unroll
+    for (int z = 0; z < E; ++z, p += W1 * W1, q += W2 * W2) {
+      const T above = p[W1 * W1];
+      phi[col.at(z)] = own;
+      *q = residual_of(own, cross_sum<T, W1>(p, below, above), *q, ih2);
+      below = own;
+      own = above;
+    }
   }
   __syncthreads();
   restrict_tile<T, E, 2>(sF, L, w, to, fc);
@@ -348,11 +386,10 @@ tile_down_kernel(TileLevel L, const T* __restrict__ f, T* __restrict__ phi, Coar
 template <typename T, int E>
 __device__ __forceinline__ void load_coarse(const TileLevel& L, const Tile<E>& w, const int* s_nb, const Coarse& from,
                                             const T* __restrict__ ec, T* sC) {
-  constexpr int EC = E / 2;
+  constexpr int EC = E / 2, WC = EC + 4;
   const int nc = L.n / 2;
-  int x, y, z;
-  for (int i = threadIdx.x; i < kCube<EC, 2>; i += blockDim.x) {
-    cube_cell<EC, 2>(i, x, y, z);
+  for (int i = threadIdx.x; i < kCube<EC, 2>; i += kTileThreads<E>) {
+    int x = i % WC - 2, y = (i / WC) % WC - 2, z = i / (WC * WC) - 2;
     x += w.x / 2;
     y += w.y / 2;
     z += w.z / 2;
@@ -367,34 +404,35 @@ __device__ __forceinline__ void load_coarse(const TileLevel& L, const Tile<E>& w
 }
 
 // Trilinear interpolation of the coarse error to the fine cells of the tile and
-// its halo of H cells, one axis at a time through shared memory, so that each
-// one-axis value is formed once (2 instructions) instead of once per fine cell
-// that uses it (14 a cell): x for the coarse rows, y for the coarse planes, z
-// by the caller.
+// its halo of H cells, one axis at a time, so that each one-axis value is formed
+// once (2 instructions) instead of once per fine cell that uses it (14 a cell):
+// along x for the coarse rows into shared memory, along y for the coarse planes
+// into a column's registers, along z as the column is walked.
 template <int E, int H> constexpr int kInterpX = (E + 2 * H) * (E / 2 + 4) * (E / 2 + 4);
-template <int E, int H> constexpr int kInterpXY = (E + 2 * H) * (E + 2 * H) * (E / 2 + 4);
 
 template <typename T, int E, int H>
-__device__ __forceinline__ void interpolate_xy(const T* sC, T* sX, T* sXY) {
+__device__ __forceinline__ void interpolate_x(const T* sC, T* sX) {
   constexpr int W = E + 2 * H, WC = E / 2 + 4;
-  for (int i = threadIdx.x; i < kInterpX<E, H>; i += blockDim.x) {
+  for (int i = threadIdx.x; i < kInterpX<E, H>; i += kTileThreads<E>) {
     const int x = i % W - H, row = i / W;
     const T* p = sC + row * WC + (x >> 1) + 2;   // arithmetic shift: floor for the halo
     sX[i] = quarter(p[0], p[(x & 1) ? 1 : -1]);
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kInterpXY<E, H>; i += blockDim.x) {
-    const int ix = i % W, y = (i / W) % W - H, cz = i / (W * W);
-    const T* p = sX + (cz * WC + (y >> 1) + 2) * W + ix;
-    sXY[i] = quarter(p[0], p[(y & 1) ? W : -W]);
-  }
-  __syncthreads();
 }
-template <typename T, int E, int H>
-__device__ __forceinline__ T interpolate_z(const T* sXY, int x, int y, int z) {
-  constexpr int W = E + 2 * H;
-  const T* p = sXY + (((z >> 1) + 2) * W + y + H) * W + x + H;
-  return quarter(p[0], p[(z & 1) ? W * W : -W * W]);
+// The fine values of the column (x, y) from below the tile up: out(z, value).
+template <typename T, int E, int H, typename Out>
+__device__ __forceinline__ void interpolate_column(const T* sX, int x, int y, Out out) {
+  constexpr int W = E + 2 * H, WC = E / 2 + 4;
+  const T* p = sX + ((y >> 1) + 2) * W + x + H;
+  const int dy = (y & 1) ? W : -W;
+  T v[WC];
+#pragma unroll
+  for (int k = 0; k < WC; ++k) v[k] = quarter(p[k * WC * W], p[k * WC * W + dy]);
+#pragma unroll
+  for (int z = -H; z < E + H; ++z) {
+    const int k = (z + 4) / 2;   // floor(z / 2) + 2
+    out(z, quarter(v[k], v[(z & 1) ? k + 1 : k - 1]));
+  }
 }
 
 // Up leg in float32: the interpolated coarse error added to phi, then two
@@ -407,41 +445,58 @@ tile_up_kernel(TileLevel L, const T* __restrict__ f, const T* __restrict__ phi, 
   extern __shared__ __align__(16) unsigned char tile_raw[];
   T* sQ = reinterpret_cast<T*>(tile_raw);         // phi plus the interpolated error, halo 2
   T* sC = sQ + kCube<E, 2>;                        // the coarse error, halo 2
-  T* sX = sC + kCube<E / 2, 2>;                    // its interpolation along x, and along x and y
-  T* sXY = sX + kInterpX<E, 2>;
-  T* sR = sX;                                      // then the field after the first sweep, halo 1
+  T* sX = sC + kCube<E / 2, 2>;                    // its interpolation along x
+  T* sR = sC;                                      // then the field after the first sweep, halo 1
   __shared__ int s_nb[27];
   const Tile<E> w = tile_of<E>(L, s_nb);
-  int x, y, z;
+  constexpr int W2 = E + 4, W1 = E + 2;
+  int x, y;
   load_coarse<T, E>(L, w, s_nb, from, ec, sC);
   __syncthreads();
-  interpolate_xy<T, E, 2>(sC, sX, sXY);
-  for (int i = threadIdx.x; i < kCube<E, 2>; i += blockDim.x) {
-    cube_cell<E, 2>(i, x, y, z);
-    sQ[i] = phi[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)] + interpolate_z<T, E, 2>(sXY, x, y, z);
+  interpolate_x<T, E, 2>(sC, sX);
+  __syncthreads();
+  for (int c = threadIdx.x; c < kColumns<E, 2>; c += kTileThreads<E>) {
+    column_xy<E, 2>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    interpolate_column<T, E, 2>(sX, x, y, [&](int z, T e) { sQ[(z + 2) * W2 * W2 + c] = phi[col.at(z)] + e; });
   }
   __syncthreads();
-  constexpr int W2 = E + 4, W1 = E + 2;
-  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
-    cube_cell<E, 1>(i, x, y, z);
-    const T* p = sQ + cube_at<E, 2>(x, y, z);
-    sR[i] = relax(p[0], cube_sum<T, W2>(p), f[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)], h2);
+  for (int c = threadIdx.x; c < kColumns<E, 1>; c += kTileThreads<E>) {
+    column_xy<E, 1>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    const T* p = sQ + cube_at<E, 2>(x, y, -1);
+    T below = p[-W2 * W2], own = p[0];
+#pragma unroll
+    for (int z = -1; z < E + 1; ++z, p += W2 * W2) {
+      const T above = p[W2 * W2];
+      sR[(z + 1) * W1 * W1 + c] = relax(own, cross_sum<T, W2>(p, below, above), f[col.at(z)], h2);
+      below = own;
+      own = above;
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
-    cube_cell<E, 0>(i, x, y, z);
-    const T* p = sR + cube_at<E, 1>(x, y, z);
-    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
-    const T v = relax(p[0], cube_sum<T, W1>(p), f[o], h2);
-    if (OUT == 0) out[o] = v;
-    else if (OUT == 1) phi64[o] = phi64[o] + widen(v);
-    else phi64[o] = widen(v);
+  for (int c = threadIdx.x; c < kColumns<E, 0>; c += kTileThreads<E>) {
+    column_xy<E, 0>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    const T* p = sR + cube_at<E, 1>(x, y, 0);
+    T below = p[-W1 * W1], own = p[0];
+#pragma unroll
+    for (int z = 0; z < E; ++z, p += W1 * W1) {
+      const T above = p[W1 * W1];
+      const long o = col.at(z);
+      const T v = relax(own, cross_sum<T, W1>(p, below, above), f[o], h2);
+      if (OUT == 0) out[o] = v;
+      else if (OUT == 1) phi64[o] = phi64[o] + widen(v);
+      else phi64[o] = widen(v);
+      below = own;
+      own = above;
+    }
   }
 }
 
-// Float64 cycles are bound by the float64 pipe (two lanes per SM and clock), so
-// nothing is evaluated twice that costs more than a pointwise product: the legs
-// are split into passes with a halo of one cell.
+// Float64 cycles are bound by the float64 pipe (1.6 lanes per SM and clock
+// measured), so nothing is evaluated twice that costs more than a pointwise
+// product: the legs are split into passes with a halo of one cell.
 enum TilePass : int { kSmoothZero = 0, kSweep = 1, kUpSweep = 2, kRestrict = 3 };
 
 // kSmoothZero: out = two sweeps from zero.  kSweep: out = one sweep of phi.
@@ -454,31 +509,45 @@ tile_pass_kernel(TileLevel L, const T* __restrict__ f, const T* __restrict__ phi
   extern __shared__ __align__(16) unsigned char tile_raw[];
   T* sP = reinterpret_cast<T*>(tile_raw);          // the field being swept, halo 1
   T* sC = sP + kCube<E, 1>;                         // kUpSweep: the coarse error; kRestrict: the residuals
-  T* sX = sC + kCube<E / 2, 2>;                     // kUpSweep: its interpolation along x, and along x and y
-  T* sXY = sX + kInterpX<E, 1>;
+  T* sX = sC + kCube<E / 2, 2>;                     // kUpSweep: its interpolation along x
   __shared__ int s_nb[27];
   const Tile<E> w = tile_of<E>(L, s_nb);
-  int x, y, z;
+  constexpr int W1 = E + 2;
+  int x, y;
   if (PASS == kUpSweep) {
     load_coarse<T, E>(L, w, s_nb, other, ec, sC);
     __syncthreads();
-    interpolate_xy<T, E, 1>(sC, sX, sXY);
+    interpolate_x<T, E, 1>(sC, sX);
+    __syncthreads();
   }
-  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
-    cube_cell<E, 1>(i, x, y, z);
-    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
-    if (PASS == kSmoothZero) sP[i] = relax_zero(f[o], h2);
-    else if (PASS == kUpSweep) sP[i] = phi[o] + interpolate_z<T, E, 1>(sXY, x, y, z);
-    else sP[i] = phi[o];
+  for (int c = threadIdx.x; c < kColumns<E, 1>; c += kTileThreads<E>) {
+    column_xy<E, 1>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    T* q = sP + c + W1 * W1;
+    if constexpr (PASS == kUpSweep) {
+      interpolate_column<T, E, 1>(sX, x, y, [&](int z, T e) { q[z * W1 * W1] = phi[col.at(z)] + e; });
+    } else {
+#pragma unroll
+      for (int z = -1; z < E + 1; ++z)
+        q[z * W1 * W1] = PASS == kSmoothZero ? relax_zero(f[col.at(z)], h2) : phi[col.at(z)];
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
-    cube_cell<E, 0>(i, x, y, z);
-    const T* p = sP + cube_at<E, 1>(x, y, z);
-    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
-    const T s = cube_sum<T, E + 2>(p);
-    if (PASS == kRestrict) sC[i] = residual_of(p[0], s, f[o], ih2);
-    else out[o] = relax(p[0], s, f[o], h2);
+  for (int c = threadIdx.x; c < kColumns<E, 0>; c += kTileThreads<E>) {
+    column_xy<E, 0>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    const T* p = sP + cube_at<E, 1>(x, y, 0);
+    T below = p[-W1 * W1], own = p[0];
+#pragma unroll
+    for (int z = 0; z < E; ++z, p += W1 * W1) {
+      const T above = p[W1 * W1];
+      const long o = col.at(z);
+      const T s = cross_sum<T, W1>(p, below, above);
+      if (PASS == kRestrict) sC[z * E * E + c] = residual_of(own, s, f[o], ih2);
+      else out[o] = relax(own, s, f[o], h2);
+      below = own;
+      own = above;
+    }
   }
   if (PASS == kRestrict) {
     __syncthreads();
@@ -496,20 +565,31 @@ tile_residual_kernel(TileLevel L, const double* __restrict__ f, const double* __
   double* sP = reinterpret_cast<double*>(tile_raw);
   __shared__ int s_nb[27];
   const Tile<E> w = tile_of<E>(L, s_nb);
-  int x, y, z;
-  for (int i = threadIdx.x; i < kCube<E, 1>; i += blockDim.x) {
-    cube_cell<E, 1>(i, x, y, z);
-    sP[i] = phi[cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z)];
+  constexpr int W1 = E + 2;
+  int x, y;
+  for (int c = threadIdx.x; c < kColumns<E, 1>; c += kTileThreads<E>) {
+    column_xy<E, 1>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+#pragma unroll
+    for (int z = -1; z < E + 1; ++z) sP[(z + 1) * W1 * W1 + c] = phi[col.at(z)];
   }
   __syncthreads();
   double worst = 0.0;
-  for (int i = threadIdx.x; i < E * E * E; i += blockDim.x) {
-    cube_cell<E, 0>(i, x, y, z);
-    const double* p = sP + cube_at<E, 1>(x, y, z);
-    const long o = cell_at(L.n, s_nb, w.x + x, w.y + y, w.z + z);
-    const double v = residual_of(p[0], cube_sum<double, E + 2>(p), f[o], ih2);
-    if (MAX) worst = fabs(v) > worst ? fabs(v) : worst;
-    else r[o] = (float)v;
+  for (int c = threadIdx.x; c < kColumns<E, 0>; c += kTileThreads<E>) {
+    column_xy<E, 0>(c, x, y);
+    const Column<E> col(L.n, s_nb, w, x, y);
+    const double* p = sP + cube_at<E, 1>(x, y, 0);
+    double below = p[-W1 * W1], own = p[0];
+#pragma unroll
+    for (int z = 0; z < E; ++z, p += W1 * W1) {
+      const double above = p[W1 * W1];
+      const long o = col.at(z);
+      const double v = residual_of(own, cross_sum<double, W1>(p, below, above), f[o], ih2);
+      if (MAX) worst = fabs(v) > worst ? fabs(v) : worst;
+      else r[o] = (float)v;
+      below = own;
+      own = above;
+    }
   }
   if (MAX) {
     for (int k = 16; k > 0; k >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, k));
@@ -517,7 +597,7 @@ tile_residual_kernel(TileLevel L, const double* __restrict__ f, const double* __
     if ((threadIdx.x & 31) == 0) sP[threadIdx.x >> 5] = worst;
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int k = 1; k < (int)(blockDim.x >> 5); ++k) worst = fmax(worst, sP[k]);
+      for (int k = 1; k < kTileThreads<E> / 32; ++k) worst = fmax(worst, sP[k]);
       partial[blockIdx.x] = worst;
     }
   }
@@ -668,9 +748,9 @@ inline int tile_edge(int n, int blocks) {
 template <typename T, int E>
 constexpr size_t up_smem() {
   constexpr int H = sizeof(T) == 4 ? 2 : 1;
-  constexpr int interp = kInterpX<E, H> + kInterpXY<E, H>;
+  constexpr int interp = kCube<E / 2, 2> + kInterpX<E, H>;
   constexpr int second = sizeof(T) == 4 ? kCube<E, 1> : 0;
-  return sizeof(T) * (kCube<E, H> + kCube<E / 2, 2> + (interp > second ? interp : second));
+  return sizeof(T) * (kCube<E, H> + (interp > second ? interp : second));
 }
 
 template <typename T>
