@@ -113,7 +113,7 @@ static void refresh_nf(const DevMesh& m, T* U, int leaf0, int nleaf, const int* 
   constexpr int G = kGhosts, N = NB + 2 * G;
   auto blocks = [](long threads, int per) { return (unsigned)((threads + per - 1) / per); };
   if ((phases & kRefreshSlow) && nslow > 0)
-    refresh_slow_kernel<T, NB, NF, false><<<nslow, 128, 0, s>>>(m, U, slow, nslow);
+    refresh_slow_kernel<T, NB, NF, false><<<nslow, kSlowThreads, 0, s>>>(m, U, slow, nslow);
   if (nleaf <= 0) return;
   if (phases & kRefreshX)   // float32: one thread per row pair (see refresh_x_kernel)
     refresh_x_kernel<T, NB, NF><<<blocks((long)nleaf * NB * (sizeof(T) == 4 ? NB / 2 : NB), 256), 256, 0, s>>>(
@@ -129,7 +129,7 @@ static void refresh_nf(const DevMesh& m, T* U, int leaf0, int nleaf, const int* 
     refresh_z_kernel<T, NB, NF, true><<<blocks((long)nleaf * 2 * NF * (G * NB * N / S), 256), 256, 0, s>>>(
         m, U, leaf0, nleaf);
   if ((phases & kRefreshSlowZFirst) && nslow > 0)
-    refresh_slow_kernel<T, NB, NF, true><<<nslow, 128, 0, s>>>(m, U, slow, nslow);
+    refresh_slow_kernel<T, NB, NF, true><<<nslow, kSlowThreads, 0, s>>>(m, U, slow, nslow);
 }
 
 template <typename T, int NB>
