@@ -186,8 +186,12 @@ sweep_kernel(DevMesh m, SweepParams prm) {
     if (j >= 2 && j <= N - 3) {
       const T* pr = sW + 4 * A + p;
       const T* un = sW + 1 * A + p;
-      sFT[j * S + p] = flatten_tilde(pr[(j - 2) * S], pr[(j - 1) * S], pr[(j + 1) * S], pr[(j + 2) * S],
-                                     un[(j - 1) * S], un[(j + 1) * S]);
+      if constexpr (kPacked)
+        sFT[j * S + p] = px::detector(pr[(j - 2) * S], pr[(j - 1) * S], pr[(j + 1) * S], pr[(j + 2) * S],
+                                      un[(j - 1) * S], un[(j + 1) * S]);
+      else
+        sFT[j * S + p] = flatten_tilde(pr[(j - 2) * S], pr[(j - 1) * S], pr[(j + 1) * S], pr[(j + 2) * S],
+                                       un[(j - 1) * S], un[(j + 1) * S]);
     }
     __syncthreads();
     // ---- phase 3 (interfaces j+1/2 read by cells 3..N-4)
@@ -220,7 +224,9 @@ sweep_kernel(DevMesh m, SweepParams prm) {
       const T* pr = sW + 4 * A + p;
       const T s = pr[(j + 1) * S] - pr[(j - 1) * S];
       const T fj = sFT[j * S + p], fm = sFT[(j - 1) * S + p], fpp = sFT[(j + 1) * S + p];
-      const T f = (s > T(0)) ? vmax(fj, fm) : ((s < T(0)) ? vmax(fj, fpp) : fj);
+      T f;
+      if constexpr (kPacked) f = px::flattening(s, fj, fm, fpp);
+      else f = (s > T(0)) ? vmax(fj, fm) : ((s < T(0)) ? vmax(fj, fpp) : fj);
       T W[NQ], aL[NQ], aR[NQ], Wm[NQ], Wp[NQ];
 #pragma unroll
       for (int k = 0; k < NQ; ++k) {
@@ -493,7 +499,7 @@ __device__ __forceinline__ void stream_step(px::Window<(RS & 4) ? 6 : 5>& S, int
   if (k >= 3 && k <= N - 2)
     S.dm[1] = px::each([](auto am, auto a0, auto ap) { return px::slope(am, a0, ap); }, S.w[2], S.w[3], S.w[4]);
   if (k >= 4) {
-    S.ft[2] = flatten_tilde(S.w[0].a.y, S.w[1].a.y, S.w[3].a.y, S.w[4].a.y, S.w[1].a.x, S.w[3].a.x);
+    S.ft[2] = px::detector(S.w[0].a.y, S.w[1].a.y, S.w[3].a.y, S.w[4].a.y, S.w[1].a.x, S.w[3].a.x);
     if (RS & 2)
       S.eta[2] = px::steepening(px::lo(S.w[0].c), px::lo(S.w[1].c), px::lo(S.w[2].c), px::lo(S.w[3].c),
                                 px::lo(S.w[4].c), S.w[1].a.y, S.w[3].a.y, gs.gamma);
@@ -504,7 +510,7 @@ __device__ __forceinline__ void stream_step(px::Window<(RS & 4) ? 6 : 5>& S, int
   if (k >= 6) {
     // cell j = k-3: W = w[1], aL = ai[0], aR = ai[1], shock detectors ft[0..2]
     const float s = S.w[2].a.y - S.w[0].a.y;
-    const float f = (s > 0.0f) ? vmax(S.ft[1], S.ft[0]) : ((s < 0.0f) ? vmax(S.ft[1], S.ft[2]) : S.ft[1]);
+    const float f = px::flattening(s, S.ft[1], S.ft[0], S.ft[2]);
     C aL = S.ai[0], aR = S.ai[1];
     if (RS & 2) {   // density of cell k-3: neighbours k-4 (slope dr[0]) and k-2 (slope dm[0])
       const float e = S.eta[1], ome = px::sub(1.0f, e);

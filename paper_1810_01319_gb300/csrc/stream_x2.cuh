@@ -120,12 +120,10 @@ template <class V>
 __device__ __forceinline__ V slope(V am, V a0, V ap) {
   const V dl = sub(a0, am), dr = sub(ap, a0);
   const V da = mul(splat<V>(0.5f), sub(ap, am));
-  const V pr = mul(dl, dr);
-  (void)pr;
   // with s = sign(da): s dl and s dr are both positive exactly where dl dr > 0
   const V sg = lanes([](float d) { return copysignf(1.0f, d); }, da);
-  const V mn = mul(splat<V>(2.0f), lanes([](float x, float y) { return vmin(x, y); }, mul(sg, dl), mul(sg, dr)));
-  return mul(sg, lanes([](float d, float m) { return vmax(vmin(fabsf(d), m), 0.0f); }, da, mn));
+  const V mn = mul(splat<V>(2.0f), lanes([](float x, float y) { return fminf(x, y); }, mul(sg, dl), mul(sg, dr)));
+  return mul(sg, lanes([](float d, float m) { return fmaxf(fminf(fabsf(d), m), 0.0f); }, da, mn));
 }
 
 // Interface value (a0 + a1)/2 - (dm1 - dm0)/6.
@@ -188,32 +186,11 @@ template <class V> __device__ __forceinline__ V pick(const float2& x);
 template <> __device__ __forceinline__ float pick<float>(const float2& x) { return x.x; }
 template <> __device__ __forceinline__ float2 pick<float2>(const float2& x) { return x; }
 
-template <int NQ>
-__device__ __forceinline__ Cell<NQ> avg_right(const Cell<NQ>& aR, const Cell<NQ>& da, const Cell<NQ>& a6,
-                                              const Wave& w) {
-  using CT = typename Cell<NQ>::CT;
-  Cell<NQ> r;
-  r.a = avg_r(aR.a, da.a, a6.a, w.nk, w.nh);
-  r.b = avg_r(aR.b, da.b, a6.b, w.nk, w.nh);
-  r.c = avg_r(aR.c, da.c, a6.c, pick<CT>(w.nk), pick<CT>(w.nh));
-  return r;
-}
-template <int NQ>
-__device__ __forceinline__ Cell<NQ> avg_left(const Cell<NQ>& aL, const Cell<NQ>& da, const Cell<NQ>& a6,
-                                             const Wave& w) {
-  using CT = typename Cell<NQ>::CT;
-  Cell<NQ> r;
-  r.a = avg_l(aL.a, da.a, a6.a, w.kp, w.nh);
-  r.b = avg_l(aL.b, da.b, a6.b, w.kp, w.nh);
-  r.c = avg_l(aL.c, da.c, a6.c, pick<CT>(w.kp), pick<CT>(w.nh));
-  return r;
-}
-
 // Conserved -> primitive in groups (sweep-local conserved order in U).
 template <int NQ>
 __device__ __forceinline__ Cell<NQ> primitives(const float* U, const Gas<float>& gs) {
   Cell<NQ> W;
-  const float rho = vmax(U[0], float(kRhoFloor));
+  const float rho = fmaxf(U[0], float(kRhoFloor));
   const float ir = __fdividef(1.0f, rho);
   const float un = mul(U[1], ir);
   W.b = mul(make_float2(U[2], U[3]), splat<float2>(ir));
@@ -223,10 +200,10 @@ __device__ __forceinline__ Cell<NQ> primitives(const float* U, const Gas<float>&
   if constexpr (NQ == 6) {
     const float eint = sub(U[4], ke);
     const float src = (eint > mul(float(kDualEta1), U[4])) ? eint : U[5];
-    p = vmax(mul(gs.gm1, src), float(kPFloor));
+    p = fmaxf(mul(gs.gm1, src), float(kPFloor));
     W.c = make_float2(rho, mul(U[5], ir));
   } else {
-    p = vmax(mul(gs.gm1, sub(U[4], ke)), float(kPFloor));
+    p = fmaxf(mul(gs.gm1, sub(U[4], ke)), float(kPFloor));
     W.c = rho;
   }
   W.a = make_float2(un, p);
@@ -237,6 +214,7 @@ __device__ __forceinline__ Cell<NQ> primitives(const float* U, const Gas<float>&
 template <int NQ>
 __device__ __forceinline__ void trace_cell(const Cell<NQ>& W, const Cell<NQ>& aL, const Cell<NQ>& aR, float2 dtdx2,
                                            const Gas<float>& gs, Cell<NQ>& Wm, Cell<NQ>& Wp) {
+  using CT = typename Cell<NQ>::CT;
   const float rho = lo(W.c), un = W.a.x, p = W.a.y;
   const float csq = __fdividef(mul(gs.gamma, p), rho);
   const float c = sqrtf(csq);
@@ -254,46 +232,76 @@ __device__ __forceinline__ void trace_cell(const Cell<NQ>& W, const Cell<NQ>& aL
   const Wave W0_ = wave(mul(un2, dtdx2));             // lambda0 = u
   const Wave Wm_ = wave(mul(sub(un2, c2), dtdx2));   // lambda- = u - c
 
+  // The reference state of an edge is the average under the fastest wave towards
+  // it, or the edge value if none moves that way: a zero weight gives exactly that,
+  // one select instead of one per field.  The transverse velocities ride the
+  // entropy wave where it moves towards the edge, and the reference wave else: one
+  // average with the weights of the one that applies.
   {  // right edge: waves moving right
-    const Cell<NQ> avp = avg_right(aR, da, a6, Wp_);
-    const Cell<NQ> ref = (lp > 0.0f) ? avp : aR;
+    const float2 nh = splat<float2>((lp > 0.0f) ? Wp_.nh.x : 0.0f);
+    const float2 nkb = splat<float2>((l0 > 0.0f) ? W0_.nk.x : Wp_.nk.x);
+    const float2 nhb = splat<float2>((l0 > 0.0f) ? W0_.nh.x : nh.x);
+    const float2 refa = avg_r(aR.a, da.a, a6.a, Wp_.nk, nh);
+    const CT refc = avg_r(aR.c, da.c, a6.c, pick<CT>(Wp_.nk), pick<CT>(nh));
     float bm = 0.0f, b0 = 0.0f;
     if (lm > 0.0f) {
-      const float2 d = sub(ref.a, avg_r(aR.a, da.a, a6.a, Wm_.nk, Wm_.nh));
+      const float2 d = sub(refa, avg_r(aR.a, da.a, a6.a, Wm_.nk, Wm_.nh));
       bm = fma(d.y, half_inv_csq, -mul(d.x, half_rho_c));
     }
-    const Cell<NQ> av0 = avg_right(aR, da, a6, W0_);
-    if (l0 > 0.0f) b0 = sub(sub(lo(ref.c), lo(av0.c)), __fdividef(sub(ref.a.y, av0.a.y), csq));
-    Wp.a.x = fma(c_rho, bm, ref.a.x);
-    Wp.a.y = vmax(fma(-csq, bm, ref.a.y), float(kPFloor));
-    Wp.b = (l0 > 0.0f) ? av0.b : ref.b;
+    const float2 av0a = avg_r(aR.a, da.a, a6.a, W0_.nk, W0_.nh);
+    const CT av0c = avg_r(aR.c, da.c, a6.c, pick<CT>(W0_.nk), pick<CT>(W0_.nh));
+    if (l0 > 0.0f) b0 = sub(sub(lo(refc), lo(av0c)), __fdividef(sub(refa.y, av0a.y), csq));
+    Wp.a.x = fma(c_rho, bm, refa.x);
+    Wp.a.y = fmaxf(fma(-csq, bm, refa.y), float(kPFloor));
+    Wp.b = avg_r(aR.b, da.b, a6.b, nkb, nhb);
     if constexpr (NQ == 6) {
-      Wp.c.x = vmax(sub(ref.c.x, add(b0, bm)), float(kRhoFloor));
-      Wp.c.y = (l0 > 0.0f) ? av0.c.y : ref.c.y;
+      Wp.c.x = fmaxf(sub(refc.x, add(b0, bm)), float(kRhoFloor));
+      Wp.c.y = (l0 > 0.0f) ? av0c.y : refc.y;
     } else {
-      Wp.c = vmax(sub(ref.c, add(b0, bm)), float(kRhoFloor));
+      Wp.c = fmaxf(sub(refc, add(b0, bm)), float(kRhoFloor));
     }
   }
   {  // left edge: waves moving left
-    const Cell<NQ> avm = avg_left(aL, da, a6, Wm_);
-    const Cell<NQ> ref = (lm < 0.0f) ? avm : aL;
+    const float2 nh = splat<float2>((lm < 0.0f) ? Wm_.nh.x : 0.0f);
+    const float2 kpb = splat<float2>((l0 < 0.0f) ? W0_.kp.x : Wm_.kp.x);
+    const float2 nhb = splat<float2>((l0 < 0.0f) ? W0_.nh.x : nh.x);
+    const float2 refa = avg_l(aL.a, da.a, a6.a, Wm_.kp, nh);
+    const CT refc = avg_l(aL.c, da.c, a6.c, pick<CT>(Wm_.kp), pick<CT>(nh));
     float bp = 0.0f, b0 = 0.0f;
     if (lp < 0.0f) {
-      const float2 d = sub(ref.a, avg_l(aL.a, da.a, a6.a, Wp_.kp, Wp_.nh));
+      const float2 d = sub(refa, avg_l(aL.a, da.a, a6.a, Wp_.kp, Wp_.nh));
       bp = fma(d.y, half_inv_csq, mul(d.x, half_rho_c));
     }
-    const Cell<NQ> av0 = avg_left(aL, da, a6, W0_);
-    if (l0 < 0.0f) b0 = sub(sub(lo(ref.c), lo(av0.c)), __fdividef(sub(ref.a.y, av0.a.y), csq));
-    Wm.a.x = fma(-c_rho, bp, ref.a.x);
-    Wm.a.y = vmax(fma(-csq, bp, ref.a.y), float(kPFloor));
-    Wm.b = (l0 < 0.0f) ? av0.b : ref.b;
+    const float2 av0a = avg_l(aL.a, da.a, a6.a, W0_.kp, W0_.nh);
+    const CT av0c = avg_l(aL.c, da.c, a6.c, pick<CT>(W0_.kp), pick<CT>(W0_.nh));
+    if (l0 < 0.0f) b0 = sub(sub(lo(refc), lo(av0c)), __fdividef(sub(refa.y, av0a.y), csq));
+    Wm.a.x = fma(-c_rho, bp, refa.x);
+    Wm.a.y = fmaxf(fma(-csq, bp, refa.y), float(kPFloor));
+    Wm.b = avg_l(aL.b, da.b, a6.b, kpb, nhb);
     if constexpr (NQ == 6) {
-      Wm.c.x = vmax(sub(ref.c.x, add(b0, bp)), float(kRhoFloor));
-      Wm.c.y = (l0 < 0.0f) ? av0.c.y : ref.c.y;
+      Wm.c.x = fmaxf(sub(refc.x, add(b0, bp)), float(kRhoFloor));
+      Wm.c.y = (l0 < 0.0f) ? av0c.y : refc.y;
     } else {
-      Wm.c = vmax(sub(ref.c, add(b0, bp)), float(kRhoFloor));
+      Wm.c = fmaxf(sub(refc, add(b0, bp)), float(kRhoFloor));
     }
   }
+}
+
+// Shock detector of the flattening coefficient (ppm.cuh: flatten_tilde); the
+// ratio only where there is a shock, which whole warps mostly skip, and its clamp
+// to [0, 1] in the multiply-add.
+__device__ __forceinline__ float detector(float pm2, float pm1, float pp1, float pp2, float um1, float up1) {
+  const float dp1 = sub(pp1, pm1), dp2 = sub(pp2, pm2);
+  float ft = 0.0f;
+  if (fabsf(dp1) > mul(float(kEpsShock), fminf(pp1, pm1)) && um1 > up1 && dp2 != 0.0f)
+    ft = __saturatef(fma(float(kOmega2), __fdividef(dp1, dp2), float(-kOmega2 * kOmega1)));
+  return ft;
+}
+
+// The flattening coefficient of a cell from its detector and its neighbours'
+// (all >= 0), s the pressure difference across it.
+__device__ __forceinline__ float flattening(float s, float fj, float fm, float fp) {
+  return fmaxf(fj, (s > 0.0f) ? fm : ((s < 0.0f) ? fp : 0.0f));
 }
 
 // Contact-steepening weight (ppm.cuh: steepening_eta), explicitly rounded.
@@ -303,17 +311,17 @@ __device__ __forceinline__ float steepening(float rm2, float rm1, float r0, floa
   const float Dp = add(sub(rp2, mul(2.0f, rp1)), r0);
   const float drho = sub(rp1, rm1);
   const bool off = (mul(Dp, Dm) > 0.0f) ||
-                   (sub(fabsf(drho), mul(float(kEpsSteep), vmin(fabsf(rp1), fabsf(rm1)))) < 0.0f) ||
-                   (__fdividef(mul(mul(gamma, float(kK0Steep)), fabsf(drho)), vmin(rp1, rm1)) <
-                    __fdividef(fabsf(sub(pp1, pm1)), vmin(pp1, pm1)));
+                   (sub(fabsf(drho), mul(float(kEpsSteep), fminf(fabsf(rp1), fabsf(rm1)))) < 0.0f) ||
+                   (__fdividef(mul(mul(gamma, float(kK0Steep)), fabsf(drho)), fminf(rp1, rm1)) <
+                    __fdividef(fabsf(sub(pp1, pm1)), fminf(pp1, pm1)));
   const float eta_t = off ? 0.0f : __fdividef(-sub(Dp, Dm), mul(6.0f, drho));
-  return vmax(vmin(mul(float(kEta1), sub(eta_t, float(kEta2))), 1.0f), 0.0f);
+  return fmaxf(fminf(mul(float(kEta1), sub(eta_t, float(kEta2))), 1.0f), 0.0f);
 }
 
 // Synchronised rho e of an updated cell (ppm.cuh: dual_sync), explicitly
 // rounded; the kinetic energy as in primitives().
 __device__ __forceinline__ float dual_sync6(const float v[6]) {
-  const float rho = vmax(v[0], float(kRhoFloor));
+  const float rho = fmaxf(v[0], float(kRhoFloor));
   const float ir = __fdividef(1.0f, rho);
   const float un = mul(v[1], ir);
   const float2 t = mul(make_float2(v[2], v[3]), splat<float2>(ir));
@@ -353,7 +361,7 @@ __device__ __forceinline__ void two_shock(const Cell<NQ>& Lc, const Cell<NQ>& Rc
   const float2 iC = make_float2(rsqrtf(q.x), rsqrtf(q.y));
   const float2 C = mul(q, iC);
   float ps = __fdividef(fma(mul(C.x, C.y), sub(uL, uR), fma(C.y, pL, mul(C.x, pR))), add(C.x, C.y));
-  ps = vmax(ps, float(kPFloor));
+  ps = fmaxf(ps, float(kPFloor));
   const float2 a = make_float2(__fdividef(gs.g1, pL), __fdividef(gs.g1, pR));
   const float2 b = splat<float2>(1.0f - gs.g1);
   const float2 niC = mul(iC, make_float2(-1.0f, 1.0f));   // (-1/C_L, 1/C_R)
@@ -370,7 +378,7 @@ __device__ __forceinline__ void two_shock(const Cell<NQ>& Lc, const Cell<NQ>& Rc
     Z = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
     if (it == kRiemannIters) break;
     const float pn =
-        vmax(sub(ps, __fdividef(mul(mul(Z.x, Z.y), sub(us.y, us.x)), add(Z.x, Z.y))), float(kPFloor));
+        fmaxf(sub(ps, __fdividef(mul(mul(Z.x, Z.y), sub(us.y, us.x)), add(Z.x, Z.y))), float(kPFloor));
     if (pn == ps) break;   // fixed point (see riemann_flux)
     ps = pn;
   }
@@ -386,7 +394,7 @@ __device__ __forceinline__ void two_shock(const Cell<NQ>& Lc, const Cell<NQ>& Rc
   const float irs = __fdividef(1.0f, rs);
   const float tau = sub(irs, __fdividef(sub(ps, p_s), mul(W_s, W_s)));
   float rstar = (tau > 0.0f) ? __fdividef(1.0f, tau) : float(kRhoFloor);
-  rstar = vmax(rstar, float(kRhoFloor));
+  rstar = fmaxf(rstar, float(kRhoFloor));
   const float c_s = sqrtf(mul(mul(gs.gamma, p_s), irs));
   const float c_star = sqrtf(__fdividef(mul(gs.gamma, ps), rstar));
   const bool shock = ps > p_s;
@@ -421,8 +429,8 @@ __device__ __forceinline__ void hllc(const Cell<NQ>& Lc, const Cell<NQ>& Rc, con
   const float rR = lo(Rc.c), uR = Rc.a.x, pR = Rc.a.y;
   const float cL = sqrtf(__fdividef(mul(gs.gamma, pL), rL));
   const float cR = sqrtf(__fdividef(mul(gs.gamma, pR), rR));
-  const float SL = vmin(sub(uL, cL), sub(uR, cR));
-  const float SR = vmax(add(uL, cL), add(uR, cR));
+  const float SL = fminf(sub(uL, cL), sub(uR, cR));
+  const float SR = fmaxf(add(uL, cL), add(uR, cR));
   const float mL = mul(rL, sub(SL, uL));
   const float mR = mul(rR, sub(SR, uR));
   const float Ss = __fdividef(add(sub(pR, pL), fma(mL, uL, -mul(mR, uR))), sub(mL, mR));
