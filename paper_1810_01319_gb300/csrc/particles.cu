@@ -22,6 +22,7 @@
 #include "cello_internal.h"
 #include "morton.h"
 #include "ppm.cuh"
+#include "widen.cuh"
 
 namespace cello {
 namespace {
@@ -35,16 +36,23 @@ struct PartMesh {
   bool pow2;               // both widths powers of two
 };
 
+// floor(v) of |v| < 2^31 from the low word of v + 1.5 2^52 rounded down: one
+// float64 instruction, where floor and a conversion are two of the same pipe.
+__device__ __forceinline__ int floor_int(double v) {
+  const int big = __double2hiint(v) & 0x7fffffff;   // exponent and top of the fraction
+  if (big < 0x41e00000) return __double2loint(__dadd_rd(v, 6755399441055744.0));
+  return __double2int_rd(v);   // saturates
+}
+
 __device__ __forceinline__ double over_w(const PartMesh& P, double d) { return P.pow2 ? d * P.inv_w : d / P.w; }
 
 __device__ __forceinline__ int locate_point(const PartMesh& P, const double x[3]) {
   unsigned b[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const long nb = (long)P.m.root[a] << P.m.max_level;
-    long v = (long)floor(over_w(P, x[a] - P.lo[a]));
-    v = v < 0 ? 0 : (v > nb - 1 ? nb - 1 : v);
-    b[a] = (unsigned)v;
+    const int nb = P.m.root[a] << P.m.max_level;   // at most 2^20
+    const int v = floor_int(over_w(P, x[a] - P.lo[a]));
+    b[a] = (unsigned)(v < 0 ? 0 : (v > nb - 1 ? nb - 1 : v));
   }
   const unsigned long long k = morton3(b[0], b[1], b[2]);
   int lo = 0, hi = P.m.B;   // first key > k
@@ -56,22 +64,35 @@ __device__ __forceinline__ int locate_point(const PartMesh& P, const double x[3]
   return lo - 1;
 }
 
-// 1/rho: the correctly rounded float32 reciprocal of float32(rho) refined by
-// two float64 Newton steps (within 2 ulp), a handful of float64 operations
-// where a float64 division costs many on this part's slow float64 pipe.
-__device__ __forceinline__ double reciprocal(double rho) {
-  double r = (double)__frcp_rn((float)rho);
-  r = r * (2.0 - rho * r);
-  return r * (2.0 - rho * r);
+// Velocity (3 components) of the cell at offset o of a padded block: momentum
+// times 1/rho, the reciprocal a float32 seed refined in float64 by r (1 + e +
+// e^2), e = 1 - rho r, |e| < 2^-22 (within 1 ulp; a float64 division costs ten
+// instructions of the float64 pipe, which bounds the push).
+__device__ __forceinline__ void cell_velocity(const double* blk, long SLAB, long o, double v[3]) {
+  const double r = blk[o];
+  const double rho = r > kRhoFloor ? r : kRhoFloor;
+  const double s = (double)__frcp_rn((float)rho);
+  const double e = fma(-rho, s, 1.0);
+  const double ir = fma(s, fma(e, e, e), s);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) v[c] = blk[(1 + c) * SLAB + o] * ir;
 }
 
-// Velocity (3 components) of the cell at offset o of a padded block.
-template <typename T>
-__device__ __forceinline__ void cell_velocity(const T* blk, long SLAB, long o, double v[3]) {
-  const double r = (double)blk[o];
-  const double ir = reciprocal(r > kRhoFloor ? r : kRhoFloor);
+// Float32 state: e = 1 - rho r is exact in float32, e^2 needs no more, and the
+// values reach float64 by integer instructions (widen): 5 float64 instructions a
+// corner instead of 16 with the conversions.
+__device__ __forceinline__ void cell_velocity(const float* blk, long SLAB, long o, double v[3]) {
+  const float rho = blk[o];
+  double ir;
+  if (rho > 1e-9f && rho < 1e30f) {   // seed and remainder are normal numbers
+    const float s = __frcp_rn(rho), e = __fmaf_rn(-rho, s, 1.0f);
+    const double sd = widen(s);
+    ir = fma(sd, widen(e) + widen(__fmul_rn(e, e)), sd);
+  } else {
+    ir = 1.0 / ((double)rho > kRhoFloor ? (double)rho : kRhoFloor);
+  }
 #pragma unroll
-  for (int c = 0; c < 3; ++c) v[c] = (double)blk[(1 + c) * SLAB + o] * ir;
+  for (int c = 0; c < 3; ++c) v[c] = widen(blk[(1 + c) * SLAB + o]) * ir;
 }
 
 // Three CTAs of 256 per SM (80 registers, a few spilled to L1): the corner
@@ -99,7 +120,7 @@ __global__ void __launch_bounds__(256, 3) particles_push_kernel(PartMesh P, cons
     const double d = x[a] - (P.lo[a] + (double)(lidx[a] * n) * dx);
     const double s = (P.pow2 ? d * inv_dx : d / dx) - 0.5;
     const double c = floor(s);
-    i0[a] = (int)c + g;
+    i0[a] = floor_int(c) + g;
     f[a] = s - c;
   }
   const T* blk = U + (long)b * m.nf * SLAB;
