@@ -257,6 +257,7 @@ struct cello_mesh {
   unsigned* d_err = nullptr;       // error word set by the reduction
   int* d_flag = nullptr;           // result word of the table and remap-map kernels
   RemapEntry* d_map = nullptr;     // remap entries of this mesh as the new one
+  mutable std::mutex remap_lock;   // d_flag and d_map: one remap into this mesh at a time
   PoissonScratch* poisson = nullptr;   // multigrid levels, allocated by the first Poisson solve
   double* d_zero = nullptr;        // dt = 0, for timing sweeps without changing the state
   void* adj_scratch = nullptr;   // three states for the adjoint's forward recomputation
@@ -897,10 +898,23 @@ cello_status cello_mesh_leaves(const cello_mesh* M, int32_t* out) {
 
 cello_status cello_neighbour_table(const cello_mesh* M, int8_t* kind, int32_t* idx, int32_t* fine8) {
   if (!M) return fail(CELLO_EINVAL, "mesh is NULL");
+  // the table stays on the device; a stream of its own in the relaxed capture
+  // mode, so that a query during a graph capture neither joins nor breaks it
   const size_t entries = (size_t)M->B * 27;
-  if (kind) CELLO_CUDA(cudaMemcpy(kind, M->d_kind, entries, cudaMemcpyDeviceToHost));
-  if (idx) CELLO_CUDA(cudaMemcpy(idx, M->d_idx, entries * sizeof(int), cudaMemcpyDeviceToHost));
-  if (fine8) CELLO_CUDA(cudaMemcpy(fine8, M->d_fine8, entries * 8 * sizeof(int), cudaMemcpyDeviceToHost));
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CELLO_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+  cudaStream_t s = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  auto get = [&](void* to, const void* from, size_t bytes) {
+    if (to && e == cudaSuccess) e = cudaMemcpyAsync(to, from, bytes, cudaMemcpyDeviceToHost, s);
+  };
+  get(kind, M->d_kind, entries);
+  get(idx, M->d_idx, entries * sizeof(int));
+  get(fine8, M->d_fine8, entries * 8 * sizeof(int));
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (s) cudaStreamDestroy(s);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  CELLO_CUDA(e);
   return CELLO_OK;
 }
 
@@ -1138,7 +1152,9 @@ cello_status cello_remap(const cello_mesh* old, const void* U_old, const cello_m
   if (std::memcmp(&old->desc, &neu->desc, sizeof(cello_mesh_desc)) != 0)
     return fail(CELLO_EINVAL, "meshes built from different descriptions");
   // the entries by binary search of the sorted keys on the device; if a new leaf
-  // has no source there, nothing is written and the call says so
+  // has no source there, nothing is written and the call says so.  The call ends
+  // with its work, so calls from several threads take turns with the entries.
+  const std::lock_guard<std::mutex> turn(neu->remap_lock);
   cudaStream_t s = (cudaStream_t)stream;
   CELLO_CUDA(cudaMemsetAsync(neu->d_flag, 0, sizeof(int), s));
   launch_remap(neu->dev(), neu->d_keys, old->dev(), old->d_keys, U_old, U_new, neu->d_map, neu->d_flag,

@@ -58,6 +58,51 @@ def test_remap_refuses_unrelated_meshes():
     assert bool((V == 3.0).all())
 
 
+def test_remap_from_several_threads():
+    """Two old meshes and two states each, remapped into one new mesh at the same time."""
+    import threading
+    from paper_1810_01319_gb300 import Mesh
+    od = H.oracle_desc(root=(3, 2, 2), n=8, lmax=2)
+    d = H.gpu_desc(od, 8)
+    root = Mesh(d)
+    neu = Mesh(d, root, np.array([1] * 3 + [0] * 9, np.int8))
+    jobs = []
+    for old in (root, Mesh(d, neu, np.ones(neu.n_leaves, np.int8))):
+        for k in range(2):
+            U = torch.rand(old.n_leaves, 5, 16, 16, 16, dtype=torch.float64, device="cuda") + 0.5
+            old.ghost_refresh(U)
+            jobs.append((old, U, neu.remap_from(old, U), torch.zeros_like(neu.empty_state()), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def work(old, U, want, got, stream):
+        for _ in range(50):
+            neu.remap_from(old, U, got, stream=stream)
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for old, U, want, got, stream in jobs:
+        assert torch.equal(got, want)
+
+
+def test_neighbour_table_during_a_capture():
+    from paper_1810_01319_gb300 import Mesh
+    od = H.oracle_desc(root=(2, 2, 1), n=8, lmax=1)
+    gm = Mesh(H.gpu_desc(od, 8))
+    want = gm.neighbour_table()
+    x, g = torch.zeros(4, device="cuda"), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        x += 1
+        got = gm.neighbour_table()
+        x += 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert all(np.array_equal(a, b) for a, b in zip(got, want)) and bool((x == 2).all())
+
+
 @pytest.mark.parametrize("dual", [False, True])
 @pytest.mark.parametrize("field", [0, 4])
 @pytest.mark.parametrize("tau, tau_c", [(0.3, 0.075), (0.3, 0.3), (0.0, 0.0), (1e-30, 1e-30), (0.25, -0.5)])
