@@ -288,13 +288,13 @@ __device__ __forceinline__ void trace_cell(const Cell<NQ>& W, const Cell<NQ>& aL
 }
 
 // Shock detector of the flattening coefficient (ppm.cuh: flatten_tilde); the
-// ratio only where there is a shock, which whole warps mostly skip, and its clamp
-// to [0, 1] in the multiply-add.
+// ratio only where there is a shock, which whole warps mostly skip, and its offset
+// in one fused multiply-add with the reciprocal.
 __device__ __forceinline__ float detector(float pm2, float pm1, float pp1, float pp2, float um1, float up1) {
   const float dp1 = sub(pp1, pm1), dp2 = sub(pp2, pm2);
   float ft = 0.0f;
   if (fabsf(dp1) > mul(float(kEpsShock), fminf(pp1, pm1)) && um1 > up1 && dp2 != 0.0f)
-    ft = __saturatef(fma(float(kOmega2), __fdividef(dp1, dp2), float(-kOmega2 * kOmega1)));
+    ft = fmaxf(fminf(mul(float(kOmega2), fma(dp1, __fdividef(1.0f, dp2), float(-kOmega1))), 1.0f), 0.0f);
   return ft;
 }
 
