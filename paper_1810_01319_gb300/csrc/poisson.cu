@@ -26,7 +26,7 @@
 // 50 sweeps.  Mean of f removed first, mean of phi removed last.  Every value
 // is the plain expression in its order on the same grid values (the block
 // layout only changes where they are stored), with 1/h^2 and 1/6 as
-// multiplications by reciprocals computed once and the multiply-adds fused.
+// multiplications by reciprocals computed once (float64: and multiply-adds fused).
 #include <mutex>
 #include <vector>
 
@@ -48,30 +48,30 @@ __device__ __forceinline__ unsigned gidx(int x, int y, int z, int M) {
 }
 __device__ __forceinline__ int wrapm(int v, int M) { return v < 0 ? v + M : (v >= M ? v - M : v); }
 
-__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
-
+// The cycle's formulas.  Float64, bound by the float64 pipe, fuses multiplies with
+// adds.  Float32 rounds term by term: after a few cycles of a mixed-precision
+// solve its rounding is what is left of the error, and fused values would differ
+// there by 1e-9 of the potential and more.
+//
 // Damped Jacobi value of a cell from its value c, neighbour sum s and
-// right-hand side f: (1 - w) c + (w / 6) (s - h^2 f), 3 instructions.
-template <typename T>
-__device__ __forceinline__ T relax(T c, T s, T f, T h2) {
-  return mad(T(kOmega / 6.0), mad(-h2, f, s), T(1.0 - kOmega) * c);
+// right-hand side f.
+__device__ __forceinline__ double relax(double c, double s, double f, double h2) {   // 3 instructions
+  return fma(kOmega / 6.0, fma(-h2, f, s), (1.0 - kOmega) * c);
+}
+__device__ __forceinline__ float relax(float c, float s, float f, float h2) {
+  return float(1.0 - kOmega) * c + float(kOmega) * ((s - h2 * f) * float(1.0 / 6.0));
 }
 // The same from a zero field (neighbour sum and cell 0).
-template <typename T>
-__device__ __forceinline__ T relax_zero(T f, T h2) {
-  return T(kOmega / 6.0) * (-h2 * f);
-}
+__device__ __forceinline__ double relax_zero(double f, double h2) { return (kOmega / 6.0) * (-h2 * f); }
+__device__ __forceinline__ float relax_zero(float f, float h2) { return float(kOmega) * ((-h2 * f) * float(1.0 / 6.0)); }
 // f - lap(phi).
-template <typename T>
-__device__ __forceinline__ T residual_of(T c, T s, T f, T ih2) {
-  return mad(-ih2, mad(T(-6), c, s), f);
+__device__ __forceinline__ double residual_of(double c, double s, double f, double ih2) {
+  return fma(-ih2, fma(-6.0, c, s), f);
 }
-// Linear interpolation a quarter of the way from p to q.
-template <typename T>
-__device__ __forceinline__ T quarter(T p, T q) {
-  return mad(T(0.75), p, T(0.25) * q);
-}
+__device__ __forceinline__ float residual_of(float c, float s, float f, float ih2) { return f - (s - 6.0f * c) * ih2; }
+// Linear interpolation a quarter of the way from p to q (q / 4 is exact).
+__device__ __forceinline__ double quarter(double p, double q) { return fma(0.25, q, 0.75 * p); }
+__device__ __forceinline__ float quarter(float p, float q) { return fmaf(0.25f, q, 0.75f * p); }
 
 template <typename T>
 __device__ __forceinline__ T nbsum(const T* p, int x, int y, int z, int M) {
