@@ -9,18 +9,25 @@
 // divisor, fused multiply-adds.
 #pragma once
 
+#include <type_traits>
+
 #include "ppm.cuh"
+#include "ppm64.cuh"
 
 namespace cello {
 
 CELLO_HD float vfma(float a, float b, float c) { return fmaf(a, b, c); }
 CELLO_HD double vfma(double a, double b, double c) { return fma(a, b, c); }
 
+// Reciprocal of what only scales an adjoint.
+CELLO_HD float inverse(float a) { return 1.0f / a; }
+CELLO_HD double inverse(double a) { return q64::inverse(a); }
+
 // W = to_primitive(U); rho = max(U_0, floor) and p = max(p of U, floor).
 template <typename T>
 CELLO_HD void to_primitive_bwd(const T W[5], const Gas<T>& gs, const T Wb[5], T Ub[5]) {
   const T rho = W[0], un = W[1], ut1 = W[2], ut2 = W[3];
-  const T ir = T(1) / rho;
+  const T ir = inverse(rho);
   const T s = vfma(un, un, vfma(ut1, ut1, ut2 * ut2));
   const T prawb = (W[4] > T(kPFloor)) ? Wb[4] : T(0);
   const T keb = -gs.gm1 * prawb;
@@ -149,7 +156,7 @@ CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, cons
     a6b[q] = T(0);
   }
   const T lm = un - c, l0 = un, lp = un + c;
-  const T ic = T(1) / c, ir = T(1) / rho, icsq = ic * ic;
+  const T ic = inverse(c), ir = inverse(rho), icsq = ic * ic;
   const T hrc = (T(0.5) * rho) * ic;
   const T hic = T(0.5) * icsq;
   const T cr = c * ir;
@@ -326,11 +333,10 @@ struct ShockSide {
 
 // Adjoints of (us, Z, W) of the shock curve at pressure ps -> (ps, p, C, u):
 // x = 1 + g1 (ps/p - 1), W = C sqrt(x), us = u -/+ (ps - p)/W,
-// Z = 2 W^3/(W^2 + C^2).  Returns the adjoint of ps.
+// Z = 2 W^3/(W^2 + C^2).  Returns the adjoint of ps.  iW = 1/W, iden = 1/(W^2 + C^2).
 template <typename T>
-CELLO_HD T shock_side_bwd(ShockSide<T>& k, T ps, T W, T usb, T Zb, T Wb, const Gas<T>& gs) {
+CELLO_HD T shock_side_bwd(ShockSide<T>& k, T ps, T W, T iW, T iden, T usb, T Zb, T Wb, const Gas<T>& gs) {
   const T W2 = W * W, C2 = k.C * k.C;
-  const T iW = T(1) / W, iden = T(1) / (W2 + C2);
   const T z = T(2) * W2 * (iden * iden) * Zb;
   const T q = (ps - k.p) * iW, qb = k.sgn * usb * iW;
   const T Wbar = vfma(-qb, q, vfma(z, vfma(T(3), C2, W2), Wb));
@@ -346,35 +352,47 @@ template <typename T>
 CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, const T Fb[5], T Lb[5], T Rb[5]) {
   const T rL = L[0], uL = L[1], pL = L[4];
   const T rR = R[0], uR = R[1], pR = R[4];
-  const T CL = vsqrt((gs.gamma * pL) * rL);
-  const T CR = vsqrt((gs.gamma * pR) * rR);
   // the forward iteration with its exit at a fixed point; pressures and W kept
   T hp[kRiemannIters + 1], hL[kRiemannIters + 1], hR[kRiemannIters + 1];
   unsigned floored = 0;   // bit k: the pressure of evaluation k was floored
-  const T ps_raw0 = ((CR * pL + CL * pR) + (CL * CR) * (uL - uR)) / (CL + CR);
-  T ps = vmax(ps_raw0, T(kPFloor));
-  if (!(ps_raw0 > T(kPFloor))) floored |= 1u;
-  T WLs, WRs, uLs, uRs, ZL, ZR;
   int last = 0;
-#pragma unroll 1
-  for (;; ++last) {
-    WLs = CL * vsqrt(T(1) + gs.g1 * (ps / pL - T(1)));
-    WRs = CR * vsqrt(T(1) + gs.g1 * (ps / pR - T(1)));
-    uLs = uL - (ps - pL) / WLs;
-    uRs = uR + (ps - pR) / WRs;
-    ZL = ((T(2) * WLs) * WLs) * WLs / (WLs * WLs + CL * CL);
-    ZR = ((T(2) * WRs) * WRs) * WRs / (WRs * WRs + CR * CR);
-    hp[last] = ps;
-    hL[last] = WLs;
-    hR[last] = WRs;
-    if (last == kRiemannIters) break;
-    const T raw = ps - ((ZL * ZR) * (uRs - uLs)) / (ZL + ZR);
-    const T pn = vmax(raw, T(kPFloor));
-    if (!(raw > T(kPFloor))) floored |= 2u << last;
-    if (pn == ps) break;
-    ps = pn;
+  T CL, CR, ps_raw0, ps, WLs, WRs, uLs, uRs, ZL, ZR;
+  bool solved = false;
+  if constexpr (std::is_same<T, double>::value) {
+    q64::Side l, r;
+    solved = q64::shock_history(L, R, gs, hp, hL, hR, floored, last, ps_raw0, l, r);
+    if (solved) {
+      ps = hp[last];
+      CL = l.C; WLs = l.W; uLs = l.us; ZL = T(2) * l.z;
+      CR = r.C; WRs = r.W; uRs = r.us; ZR = T(2) * r.z;
+    }
   }
-  const T iD = T(1) / (ZL + ZR);
+  if (!solved) {
+    CL = vsqrt((gs.gamma * pL) * rL);
+    CR = vsqrt((gs.gamma * pR) * rR);
+    ps_raw0 = ((CR * pL + CL * pR) + (CL * CR) * (uL - uR)) / (CL + CR);
+    ps = vmax(ps_raw0, T(kPFloor));
+    floored = (ps_raw0 > T(kPFloor)) ? 0u : 1u;
+#pragma unroll 1
+    for (last = 0;; ++last) {
+      WLs = CL * vsqrt(T(1) + gs.g1 * (ps / pL - T(1)));
+      WRs = CR * vsqrt(T(1) + gs.g1 * (ps / pR - T(1)));
+      uLs = uL - (ps - pL) / WLs;
+      uRs = uR + (ps - pR) / WRs;
+      ZL = ((T(2) * WLs) * WLs) * WLs / (WLs * WLs + CL * CL);
+      ZR = ((T(2) * WRs) * WRs) * WRs / (WRs * WRs + CR * CR);
+      hp[last] = ps;
+      hL[last] = WLs;
+      hR[last] = WRs;
+      if (last == kRiemannIters) break;
+      const T raw = ps - ((ZL * ZR) * (uRs - uLs)) / (ZL + ZR);
+      const T pn = vmax(raw, T(kPFloor));
+      if (!(raw > T(kPFloor))) floored |= 2u << last;
+      if (pn == ps) break;
+      ps = pn;
+    }
+  }
+  const T iD = inverse(ZL + ZR);
   const T us = (ZL * uLs + ZR * uRs) / (ZL + ZR);
   const bool left = us >= T(0);
   const T rs = left ? rL : rR, u_s = left ? uL : uR, p_s = left ? pL : pR, W_s = left ? WLs : WRs;
@@ -428,7 +446,7 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
   } else if (star) {
     rstarb = rb; usb = ub; psb = pb;
   }
-  const T irs = T(1) / rs;
+  const T irs = inverse(rs);
   if (fan) {   // rarefaction: head = v_s + c_s, tail = v* + c*, c = sqrt(gamma p / rho)
     const T wb = vfma(rb, rstar - rs, vfma(ub, us - u_s, pb * (ps - p_s)));
     rstarb = rb * w; rsb = rb - rstarb;
@@ -436,7 +454,7 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
     psb = pb * w; p_sb = pb - psb;
     v_sb = -wb * tail * (iht * iht);
     v_starb = wb * w * iht;
-    const T sb = T(0.5) * v_sb / c_s, xb = T(0.5) * v_starb / c_star, irst = T(1) / rstar;
+    const T sb = T(0.5) * v_sb / c_s, xb = T(0.5) * v_starb / c_star, irst = inverse(rstar);
     p_sb = vfma(sb * gs.gamma, irs, p_sb);
     rsb = vfma(-sb * gs.gamma * p_s, irs * irs, rsb);
     psb = vfma(xb * gs.gamma, irst, psb);
@@ -445,19 +463,19 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
   if (rstar_raw > T(kRhoFloor) && tau > T(0)) {  // rstar = 1/tau
     const T taub = -rstarb * rstar * rstar;
     rsb = vfma(-taub, irs * irs, rsb);
-    const T iW = T(1) / W_s, tw = taub * iW * iW;
+    const T iW = inverse(W_s), tw = taub * iW * iW;
     psb -= tw;
     p_sb += tw;
     W_sb = T(2) * tw * (ps - p_s) * iW;
   }
   usb += left ? -v_starb : v_starb;
   ShockSide<T> a, b;
-  a.p = pL; a.C = CL; a.ip = T(1) / pL; a.iC = T(1) / CL; a.sgn = T(-1);
-  b.p = pR; b.C = CR; b.ip = T(1) / pR; b.iC = T(1) / CR; b.sgn = T(1);
+  a.p = pL; a.C = CL; a.ip = inverse(pL); a.iC = inverse(CL); a.sgn = T(-1);
+  b.p = pR; b.C = CR; b.ip = inverse(pR); b.iC = inverse(CR); b.sgn = T(1);
   a.pb = a.Cb = a.ub = b.pb = b.Cb = b.ub = T(0);
   // us = (ZL*usL + ZR*usR)/D
-  psb += shock_side_bwd(a, ps, WLs, usb * ZL * iD, usb * (uLs - us) * iD, left ? W_sb : T(0), gs);
-  psb += shock_side_bwd(b, ps, WRs, usb * ZR * iD, usb * (uRs - us) * iD, left ? T(0) : W_sb, gs);
+  psb += shock_side_bwd(a, ps, WLs, inverse(WLs), inverse(vfma(WLs, WLs, CL * CL)), usb * ZL * iD, usb * (uLs - us) * iD, left ? W_sb : T(0), gs);
+  psb += shock_side_bwd(b, ps, WRs, inverse(WRs), inverse(vfma(WRs, WRs, CR * CR)), usb * ZR * iD, usb * (uRs - us) * iD, left ? T(0) : W_sb, gs);
   // Newton iterations in reverse, p_{k+1} = max(p_k - q(p_k), floor): those
   // after a fixed point all have its derivative m = 1 - q', so n of them pass
   // psb m^n on and add (1 + m + ... + m^(n-1)) times one iteration's adjoints
@@ -470,15 +488,17 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
       continue;
     }
     const T pk = hp[it], WA = hL[it], WB = hR[it];
-    const T ZA = T(2) * WA * WA * WA / vfma(WA, WA, CL * CL), ZB = T(2) * WB * WB * WB / vfma(WB, WB, CR * CR);
-    const T iZ = T(1) / (ZA + ZB);
-    const T du = (uR + (pk - pR) / WB) - (uL - (pk - pL) / WA);
+    const T iA = inverse(WA), dA = inverse(vfma(WA, WA, CL * CL));
+    const T iB = inverse(WB), dB = inverse(vfma(WB, WB, CR * CR));
+    const T ZA = T(2) * WA * WA * WA * dA, ZB = T(2) * WB * WB * WB * dB;
+    const T iZ = inverse(ZA + ZB);
+    const T du = vfma(pk - pR, iB, uR) - vfma(pL - pk, iA, uL);
     const T zz = ZA * ZB * iZ, q = zz * du;
     ShockSide<T> x = a, y = b;   // one iteration's adjoints for psb = 1
     x.pb = x.Cb = x.ub = y.pb = y.Cb = y.ub = T(0);
     T m = T(1);
-    m += shock_side_bwd(x, pk, WA, zz, -vfma(ZB, du, -q) * iZ, T(0), gs);
-    m += shock_side_bwd(y, pk, WB, -zz, -vfma(ZA, du, -q) * iZ, T(0), gs);
+    m += shock_side_bwd(x, pk, WA, iA, dA, zz, -vfma(ZB, du, -q) * iZ, T(0), gs);
+    m += shock_side_bwd(y, pk, WB, iB, dB, -zz, -vfma(ZA, du, -q) * iZ, T(0), gs);
     T sum = T(0);
     for (int k = 0; k < reps; ++k) {
       sum += psb;
@@ -488,7 +508,7 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
     b.pb = vfma(sum, y.pb, b.pb); b.Cb = vfma(sum, y.Cb, b.Cb); b.ub = vfma(sum, y.ub, b.ub);
   }
   if (!(floored & 1u)) {  // p_0 = ((CR pL + CL pR) + (CL CR)(uL - uR)) / (CL + CR)
-    const T nb = psb / (CL + CR), du = uL - uR, cc = nb * CL * CR;
+    const T nb = psb * inverse(CL + CR), du = uL - uR, cc = nb * CL * CR;
     a.pb = vfma(nb, CR, a.pb);
     b.pb = vfma(nb, CL, b.pb);
     a.Cb = vfma(nb, vfma(CR, du, pR) - ps_raw0, a.Cb);

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__((NB + 8) * adj_pencils(NB))
 adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
   constexpr int G = kGhosts, N = NB + 2 * G, P = adj_pencils(NB), A = N * P;
   constexpr long SLAB = (long)N * N * N;
+  constexpr bool k64 = std::is_same<T, double>::value;   // ppm64.cuh: the same values
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sW = reinterpret_cast<T*>(smem_raw);   // primitives
   T* sLam = sW + 5 * A;                      // lam', then lam
@@ -84,7 +85,8 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
       T Us[5], W[5];
 #pragma unroll
       for (int k = 0; k < 5; ++k) Us[k] = moves ? U[off + comp[k] * SLAB] : T(1);
-      to_primitive(Us, gs, W);
+      if constexpr (k64) q64::primitives<5>(Us, gs, W);
+      else to_primitive(Us, gs, W);
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         sW[k * A + mc * P + mp] = W[k];
@@ -98,17 +100,22 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         const T* a = sW + k * A + at;
-        sD[k * A + at] = limited_slope(a[-P], a[0], a[P]);
+        if constexpr (k64) sD[k * A + at] = q64::slope(a[-P], a[0], a[P]);
+        else sD[k * A + at] = limited_slope(a[-P], a[0], a[P]);
       }
       const T *pr = sW + 4 * A + at, *un = sW + A + at;
-      ft = flatten_tilde(pr[-2 * P], pr[-P], pr[P], pr[2 * P], un[-P], un[P]);
+      if constexpr (k64) ft = q64::detector(pr[-2 * P], pr[-P], pr[P], pr[2 * P], un[-P], un[P]);
+      else ft = flatten_tilde(pr[-2 * P], pr[-P], pr[P], pr[2 * P], un[-P], un[P]);
     }
     sFT[at] = ft;
     __syncthreads();
     if (j >= 2 && j <= N - 4) {
 #pragma unroll
-      for (int k = 0; k < 5; ++k)
-        sI[k * A + at] = interface_value(sW[k * A + at], sW[k * A + at + P], sD[k * A + at], sD[k * A + at + P]);
+      for (int k = 0; k < 5; ++k) {
+        const T a0 = sW[k * A + at], a1 = sW[k * A + at + P], d0 = sD[k * A + at], d1 = sD[k * A + at + P];
+        if constexpr (k64) sI[k * A + at] = q64::interface_val(a0, a1, d0, d1);
+        else sI[k * A + at] = interface_value(a0, a1, d0, d1);
+      }
     }
     __syncthreads();
     const bool traced = j >= 3 && j <= N - 4;
@@ -130,9 +137,10 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
         W[k] = sW[k * A + at];
         aL[k] = sI[k * A + at - P];
         aR[k] = sI[k * A + at];
-        flatten_monotone(W[k], f, aL[k], aR[k]);
+        if constexpr (!k64) flatten_monotone(W[k], f, aL[k], aR[k]);
       }
-      trace(W, aL, aR, dtdx, gs, Wm, Wp);
+      if constexpr (k64) q64::edge_states<5>(W, f, aL, aR, dtdx, gs, Wm, Wp);
+      else trace(W, aL, aR, dtdx, gs, Wm, Wp);
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         sL[k * A + at] = Wm[k];

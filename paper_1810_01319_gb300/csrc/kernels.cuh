@@ -4,6 +4,7 @@
 
 #include "cello_internal.h"
 #include "ppm.cuh"
+#include "ppm64.cuh"
 #include "stream_x2.cuh"
 
 namespace cello {
@@ -44,13 +45,15 @@ __host__ __device__ constexpr int sweep_arrays(int RS) {
 
 template <int RS, typename T>
 __device__ __forceinline__ void interface_flux(const T L[5], const T R[5], const Gas<T>& gs, T F[5]) {
-  if (RS & 1) hllc_flux(L, R, gs, F);
+  if constexpr ((RS & 1) != 0) hllc_flux(L, R, gs, F);
+  else if constexpr (std::is_same<T, double>::value) q64::two_shock_flux<5>(L, R, gs, F);
   else riemann_flux_bulk(L, R, gs, F);
 }
 
 template <int RS, typename T>
 __device__ __forceinline__ void interface_flux6(const T L[6], const T R[6], const Gas<T>& gs, T F[6], T* uf) {
-  if (RS & 1) hllc_flux<T, 6>(L, R, gs, F, uf);
+  if constexpr ((RS & 1) != 0) hllc_flux<T, 6>(L, R, gs, F, uf);
+  else if constexpr (std::is_same<T, double>::value) q64::two_shock_flux<6>(L, R, gs, F, uf);
   else riemann_flux_bulk6(L, R, gs, F, uf);
 }
 
@@ -163,10 +166,8 @@ sweep_kernel(DevMesh m, SweepParams prm) {
         const px::Cell<NQ> Wc = px::primitives<NQ>(Us, gs);
 #pragma unroll
         for (int k = 0; k < NQ; ++k) W[k] = Wc.get(k);
-      } else if constexpr (DE) {
-        to_primitive_de(Us, gs, W);
       } else {
-        to_primitive(Us, gs, W);
+        q64::primitives<NQ>(Us, gs, W);
       }
 #pragma unroll
       for (int k = 0; k < NQ; ++k) sW[k * A + lc * S + lp] = W[k];
@@ -180,7 +181,7 @@ sweep_kernel(DevMesh m, SweepParams prm) {
       for (int k = 0; k < NQ; ++k) {
         const T* a = sW + k * A + p;
         if constexpr (kPacked) sA[k * A + j * S + p] = px::slope(a[(j - 1) * S], a[j * S], a[(j + 1) * S]);
-        else sA[k * A + j * S + p] = limited_slope(a[(j - 1) * S], a[j * S], a[(j + 1) * S]);
+        else sA[k * A + j * S + p] = q64::slope(a[(j - 1) * S], a[j * S], a[(j + 1) * S]);
       }
     }
     if (j >= 2 && j <= N - 3) {
@@ -190,7 +191,7 @@ sweep_kernel(DevMesh m, SweepParams prm) {
         sFT[j * S + p] = px::detector(pr[(j - 2) * S], pr[(j - 1) * S], pr[(j + 1) * S], pr[(j + 2) * S],
                                       un[(j - 1) * S], un[(j + 1) * S]);
       else
-        sFT[j * S + p] = flatten_tilde(pr[(j - 2) * S], pr[(j - 1) * S], pr[(j + 1) * S], pr[(j + 2) * S],
+        sFT[j * S + p] = q64::detector(pr[(j - 2) * S], pr[(j - 1) * S], pr[(j + 1) * S], pr[(j + 2) * S],
                                        un[(j - 1) * S], un[(j + 1) * S]);
     }
     __syncthreads();
@@ -202,8 +203,8 @@ sweep_kernel(DevMesh m, SweepParams prm) {
           sB[k * A + j * S + p] = px::interface_val(sW[k * A + j * S + p], sW[k * A + (j + 1) * S + p],
                                                     sA[k * A + j * S + p], sA[k * A + (j + 1) * S + p]);
         else
-          sB[k * A + j * S + p] = interface_value(sW[k * A + j * S + p], sW[k * A + (j + 1) * S + p],
-                                                  sA[k * A + j * S + p], sA[k * A + (j + 1) * S + p]);
+          sB[k * A + j * S + p] = q64::interface_val(sW[k * A + j * S + p], sW[k * A + (j + 1) * S + p],
+                                                     sA[k * A + j * S + p], sA[k * A + (j + 1) * S + p]);
       }
     }
     if ((RS & 2) && j >= 3 && j <= N - 4) {   // contact steepening of cell j (density)
@@ -222,11 +223,10 @@ sweep_kernel(DevMesh m, SweepParams prm) {
     // ---- phase 4
     if (j >= 3 && j <= N - 4) {
       const T* pr = sW + 4 * A + p;
-      const T s = pr[(j + 1) * S] - pr[(j - 1) * S];
       const T fj = sFT[j * S + p], fm = sFT[(j - 1) * S + p], fpp = sFT[(j + 1) * S + p];
       T f;
-      if constexpr (kPacked) f = px::flattening(s, fj, fm, fpp);
-      else f = (s > T(0)) ? vmax(fj, fm) : ((s < T(0)) ? vmax(fj, fpp) : fj);
+      if constexpr (kPacked) f = px::flattening(pr[(j + 1) * S] - pr[(j - 1) * S], fj, fm, fpp);
+      else f = q64::flattening(pr[(j - 1) * S], pr[(j + 1) * S], fj, fm, fpp);
       T W[NQ], aL[NQ], aR[NQ], Wm[NQ], Wp[NQ];
 #pragma unroll
       for (int k = 0; k < NQ; ++k) {
@@ -245,7 +245,6 @@ sweep_kernel(DevMesh m, SweepParams prm) {
           }
         }
         if constexpr (kPacked) px::flatten_mono(W[k], f, px::sub(1.0f, f), aL[k], aR[k]);
-        else flatten_monotone(W[k], f, aL[k], aR[k]);
       }
       if constexpr (kPacked) {
         px::Cell<NQ> Wc, aLc, aRc, Wmc, Wpc;
@@ -262,7 +261,7 @@ sweep_kernel(DevMesh m, SweepParams prm) {
           Wp[k] = Wpc.get(k);
         }
       } else {
-        trace<T, NQ>(W, aL, aR, dtdx, gs, Wm, Wp);
+        q64::edge_states<NQ>(W, f, aL, aR, dtdx, gs, Wm, Wp);
       }
 #pragma unroll
       for (int k = 0; k < NQ; ++k) {
