@@ -46,7 +46,7 @@ __device__ __forceinline__ int floor_int(double v) {
 
 __device__ __forceinline__ double over_w(const PartMesh& P, double d) { return P.pow2 ? d * P.inv_w : d / P.w; }
 
-__device__ __forceinline__ int locate_point(const PartMesh& P, const double x[3]) {
+__device__ __forceinline__ unsigned long long point_key(const PartMesh& P, const double x[3]) {
   unsigned b[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -54,7 +54,10 @@ __device__ __forceinline__ int locate_point(const PartMesh& P, const double x[3]
     const int v = floor_int(over_w(P, x[a] - P.lo[a]));
     b[a] = (unsigned)(v < 0 ? 0 : (v > nb - 1 ? nb - 1 : v));
   }
-  const unsigned long long k = morton3(b[0], b[1], b[2]);
+  return morton3(b[0], b[1], b[2]);
+}
+
+__device__ __forceinline__ int locate_key(const PartMesh& P, unsigned long long k) {
   int lo = 0, hi = P.m.B;   // first key > k
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -81,18 +84,37 @@ __device__ __forceinline__ void cell_velocity(const double* blk, long SLAB, long
 // Float32 state: e = 1 - rho r is exact in float32, e^2 needs no more, and the
 // values reach float64 by integer instructions (widen): 5 float64 instructions a
 // corner instead of 16 with the conversions.
-__device__ __forceinline__ void cell_velocity(const float* blk, long SLAB, long o, double v[3]) {
-  const float rho = blk[o];
-  double ir;
+__device__ __forceinline__ double density_reciprocal(float rho) {
   if (rho > 1e-9f && rho < 1e30f) {   // seed and remainder are normal numbers
     const float s = __frcp_rn(rho), e = __fmaf_rn(-rho, s, 1.0f);
     const double sd = widen(s);
-    ir = fma(sd, widen(e) + widen(__fmul_rn(e, e)), sd);
-  } else {
-    ir = 1.0 / ((double)rho > kRhoFloor ? (double)rho : kRhoFloor);
+    return fma(sd, widen(e) + widen(__fmul_rn(e, e)), sd);
   }
+  return 1.0 / ((double)rho > kRhoFloor ? (double)rho : kRhoFloor);
+}
+
+// The eight corner velocities, x fastest: corner (dz, dy, dx) at 4 dz + 2 dy + dx.
+__device__ __forceinline__ void corner_velocities(const double* blk, long SLAB, long o, long sy, long sz,
+                                                  double cv[8][3]) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c) v[c] = widen(blk[(1 + c) * SLAB + o]) * ir;
+  for (int q = 0; q < 8; ++q) cell_velocity(blk, SLAB, o + (q >> 2) * sz + ((q >> 1) & 1) * sy + (q & 1), cv[q]);
+}
+
+// Float32: every value is asked for before the first is used (the branches between
+// the corners kept the loads apart, and randomly placed tracers wait on them).
+__device__ __forceinline__ void corner_velocities(const float* blk, long SLAB, long o, long sy, long sz,
+                                                  double cv[8][3]) {
+  float u[4][8];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) u[c][q] = __ldg(blk + c * SLAB + o + (q >> 2) * sz + ((q >> 1) & 1) * sy + (q & 1));
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const double ir = density_reciprocal(u[0][q]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) cv[q][c] = widen(u[1 + c][q]) * ir;
+  }
 }
 
 // Three CTAs of 256 per SM (80 registers, a few spilled to L1): the corner
@@ -125,12 +147,10 @@ __global__ void __launch_bounds__(256, 3) particles_push_kernel(PartMesh P, cons
   }
   const T* blk = U + (long)b * m.nf * SLAB;
   const long o000 = ((long)i0[2] * N + i0[1]) * N + i0[0];
-  const long sx = 1, sy = N, sz = (long)N * N;
   const double dt = *dt_dev;
-  // the eight corner velocities, x fastest: corner (dz, dy, dx) at index 4 dz + 2 dy + dx
+  const unsigned long long here = P.keys[b], beyond = b + 1 < m.B ? P.keys[b + 1] : ~0ull;
   double cv[8][3];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) cell_velocity(blk, SLAB, o000 + (q >> 2) * sz + ((q >> 1) & 1) * sy + (q & 1) * sx, cv[q]);
+  corner_velocities(blk, SLAB, o000, N, (long)N * N, cv);
   bool lost = false;
 #pragma unroll
   for (int comp = 0; comp < 3; ++comp) {
@@ -153,14 +173,21 @@ __global__ void __launch_bounds__(256, 3) particles_push_kernel(PartMesh P, cons
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) pos[a * count + i] = x[a];
-  leaf[i] = lost ? -1 : locate_point(P, x);
+  // most tracers stay in their leaf, whose keys are at hand: the search is a chain
+  // of loads
+  if (lost) {
+    leaf[i] = -1;
+  } else {
+    const unsigned long long k = point_key(P, x);
+    if (k < here || k >= beyond) leaf[i] = locate_key(P, k);
+  }
 }
 
 __global__ void particles_locate_kernel(PartMesh P, const double* pos, int* leaf, long count) {
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const double x[3] = {pos[i], pos[count + i], pos[2 * count + i]};
-  leaf[i] = locate_point(P, x);
+  leaf[i] = locate_key(P, point_key(P, x));
 }
 
 bool is_pow2(double v) {
