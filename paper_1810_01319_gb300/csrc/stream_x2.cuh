@@ -366,8 +366,9 @@ __device__ __forceinline__ void two_shock(const Cell<NQ>& Lc, const Cell<NQ>& Rc
   const float2 b = splat<float2>(1.0f - gs.g1);
   const float2 niC = mul(iC, make_float2(-1.0f, 1.0f));   // (-1/C_L, 1/C_R)
   float2 W, us, Z;
+  float before = -1.0f;   // the pressure two steps before the next one
 #pragma unroll 1
-  for (int it = 0; it <= kRiemannIters; ++it) {
+  for (int it = 0;; ++it) {
     const float2 ps2 = splat<float2>(ps);
     const float2 x = fma(a, ps2, b);                        // 1 + g1 (p*/p - 1)
     const float2 rx = make_float2(rsqrtf(x.x), rsqrtf(x.y));
@@ -376,10 +377,15 @@ __device__ __forceinline__ void two_shock(const Cell<NQ>& Lc, const Cell<NQ>& Rc
     const float2 num = mul(mul(splat<float2>(2.0f), W), x);
     const float2 den = add(x, splat<float2>(1.0f));
     Z = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
-    if (it == kRiemannIters) break;
+    if (it >= kRiemannIters) break;
     const float pn =
         fmaxf(sub(ps, __fdividef(mul(mul(Z.x, Z.y), sub(us.y, us.x)), add(Z.x, Z.y))), float(kPFloor));
     if (pn == ps) break;   // fixed point (see riemann_flux)
+    if (pn == before) {    // two pressures in turn: the last step's is this one, or takes one evaluation
+      if (((kRiemannIters - it) & 1) == 0) break;
+      it = kRiemannIters - 1;
+    }
+    before = ps;
     ps = pn;
   }
   const float ust = __fdividef(fma(Z.x, us.x, mul(Z.y, us.y)), add(Z.x, Z.y));
