@@ -43,25 +43,35 @@ CELLO_HD void to_primitive_bwd(const T W[5], const Gas<T>& gs, const T Wb[5], T 
   }
 }
 
+// The slope is 1/2 (ap - am), 2 (a0 - am) or 2 (ap - a0), the smallest of the three,
+// where the last two have one sign.
 template <typename T>
 CELLO_HD void limited_slope_bwd(T am, T a0, T ap, T ob, T& amb, T& a0b, T& apb) {
-  const T dl = a0 - am, dr = ap - a0, da = T(0.5) * (ap - am);
-  if (!(dl * dr > T(0))) return;
-  const T mb = (da < T(0)) ? -ob : ob;
-  const T adl = T(2) * vabs(dl), adr = T(2) * vabs(dr);
-  const T inner = vmin(adl, adr);
-  if (vabs(da) < inner) {
-    const T dab = (da < T(0)) ? -mb : mb;
-    apb += T(0.5) * dab;
-    amb -= T(0.5) * dab;
-  } else if (adl < adr) {
-    const T dlb = T(2) * ((dl < T(0)) ? -mb : mb);
-    a0b += dlb;
-    amb -= dlb;
+  const T dl = a0 - am, dr = ap - a0;
+  bool centred, left;
+  if (std::is_same<T, double>::value && q64::within<-500, 500>(q64::mag(dl)) &&
+      q64::within<-500, 500>(q64::mag(dr))) {   // on their bits: see q64::slope
+    if ((int)(q64::high(dl) ^ q64::high(dr)) < 0) return;
+    constexpr long long kTwo = 0x0010000000000000ll;
+    const long long l = q64::bits(q64::absval(dl)), r = q64::bits(q64::absval(dr));
+    const long long d = q64::bits(q64::absval(ap - am)) - kTwo;
+    centred = d < (l < r ? l : r) + kTwo;
+    left = l < r;
   } else {
-    const T drb = T(2) * ((dr < T(0)) ? -mb : mb);
-    apb += drb;
-    a0b -= drb;
+    if (!(dl * dr > T(0))) return;
+    const T adl = T(2) * vabs(dl), adr = T(2) * vabs(dr);
+    centred = vabs(T(0.5) * (ap - am)) < vmin(adl, adr);
+    left = adl < adr;
+  }
+  if (centred) {
+    apb = vfma(T(0.5), ob, apb);
+    amb = vfma(T(-0.5), ob, amb);
+  } else if (left) {
+    a0b = vfma(T(2), ob, a0b);
+    amb = vfma(T(-2), ob, amb);
+  } else {
+    apb = vfma(T(2), ob, apb);
+    a0b = vfma(T(-2), ob, a0b);
   }
 }
 
@@ -76,9 +86,9 @@ CELLO_HD void interface_value_bwd(T ob, T& a0b, T& a1b, T& dm0b, T& dm1b) {
 template <typename T>
 CELLO_HD void flatten_tilde_bwd(T pm2, T pm1, T pp1, T pp2, T um1, T up1, T ob, T& pm2b, T& pm1b, T& pp1b,
                                 T& pp2b) {
+  if (!(um1 - up1 > T(0))) return;
   const T dp1 = pp1 - pm1, dp2 = pp2 - pm2;
-  const bool shock = (vabs(dp1) > T(kEpsShock) * vmin(pp1, pm1)) && (um1 - up1 > T(0)) && (dp2 != T(0));
-  if (!shock) return;
+  if (!(vabs(dp1) > T(kEpsShock) * vmin(pp1, pm1)) || !(dp2 != T(0))) return;
   const T ratio = dp1 / dp2;
   const T x = T(kOmega2) * (ratio - T(kOmega1));
   if (!(x < T(1)) || !(x > T(0))) return;
@@ -90,56 +100,68 @@ CELLO_HD void flatten_tilde_bwd(T pm2, T pm1, T pp1, T pp2, T um1, T up1, T ob, 
   pm2b -= dp2b;
 }
 
+// Where f is 0 the detector it came from is 0 and passes nothing on: fb is left
+// out there, as are the products with f.
 template <typename T>
 CELLO_HD void flatten_monotone_bwd(T a, T f, T aL, T aR, T oLb, T oRb, T& ab, T& fb, T& aLb, T& aRb) {
-  const T l = f * a + (T(1) - f) * aL;
-  const T r = f * a + (T(1) - f) * aR;
-  const bool ext = (r - a) * (a - l) <= T(0);
-  T lb = T(0), rb = T(0);
+  const bool flat = f != T(0);
+  T l = aL, r = aR;
+  if (flat) {
+    l = f * a + (T(1) - f) * aL;
+    r = f * a + (T(1) - f) * aR;
+  }
+  const T d1 = r - a, d2 = a - l;
+  bool ext;
+  if (std::is_same<T, double>::value && q64::within<-500, 500>(q64::mag(d1)) &&
+      q64::within<-500, 500>(q64::mag(d2)))
+    ext = (int)(q64::high(d1) ^ q64::high(d2)) < 0;
+  else
+    ext = d1 * d2 <= T(0);
   if (ext) {
     ab += oLb + oRb;
-  } else {
-    const T da = r - l, dm = a - T(0.5) * (l + r);
-    const T t1 = da * dm, t2 = (da * da) * T(1.0 / 6.0);
-    if (t1 > t2) {
-      ab += T(3) * oLb;
-      rb -= T(2) * oLb;
-    } else {
-      lb += oLb;
-    }
-    if (-t2 > t1) {
-      ab += T(3) * oRb;
-      lb -= T(2) * oRb;
-    } else {
-      rb += oRb;
-    }
+    return;
   }
-  fb += lb * (a - aL) + rb * (a - aR);
-  ab += (lb + rb) * f;
-  aLb += lb * (T(1) - f);
-  aRb += rb * (T(1) - f);
+  T lb = oLb, rb = oRb;
+  const T da = r - l, dm = a - T(0.5) * (l + r);
+  const T t1 = da * dm, t2 = (da * da) * T(1.0 / 6.0);
+  if (t1 > t2) {
+    ab = vfma(T(3), oLb, ab);
+    rb = vfma(T(-2), oLb, rb);
+    lb = T(0);
+  }
+  if (-t2 > t1) {   // not both
+    ab = vfma(T(3), oRb, ab);
+    lb = vfma(T(-2), oRb, lb);
+    rb = T(0);
+  }
+  if (flat) {
+    fb += lb * (a - aL) + rb * (a - aR);
+    ab += (lb + rb) * f;
+    lb *= T(1) - f;
+    rb *= T(1) - f;
+  }
+  aLb += lb;
+  aRb += rb;
 }
 
 template <typename T>
 CELLO_HD void avg_right_bwd(T aL, T aR, T a6, T s, T ob, T& aLb, T& aRb, T& a6b, T& sb) {
   const T h = T(0.5) * s, g = T(1) - T(2.0 / 3.0) * s;
-  const T inner = vfma(-g, a6, aR - aL);
   const T oh = ob * h;
   aRb += ob - oh;
   aLb += oh;
   a6b = vfma(oh, g, a6b);
-  sb = vfma(-ob, vfma(h * T(2.0 / 3.0), a6, T(0.5) * inner), sb);
+  sb = vfma(-ob, vfma(T(2.0 / 3.0) * s - T(0.5), a6, T(0.5) * (aR - aL)), sb);   // h 2/3 - g/2 = 2/3 s - 1/2
 }
 
 template <typename T>
 CELLO_HD void avg_left_bwd(T aL, T aR, T a6, T s, T ob, T& aLb, T& aRb, T& a6b, T& sb) {
   const T h = T(0.5) * s, g = T(1) - T(2.0 / 3.0) * s;
-  const T inner = vfma(g, a6, aR - aL);
   const T oh = ob * h;
   aLb += ob - oh;
   aRb += oh;
   a6b = vfma(oh, g, a6b);
-  sb = vfma(ob, vfma(-h * T(2.0 / 3.0), a6, T(0.5) * inner), sb);
+  sb = vfma(ob, vfma(T(0.5) - T(2.0 / 3.0) * s, a6, T(0.5) * (aR - aL)), sb);
 }
 
 // Reverse of trace(): adjoints of the two edge states -> adjoints of the
@@ -148,15 +170,29 @@ template <typename T>
 CELLO_HD void trace_bwd(const T W[5], const T aL[5], const T aR[5], T dtdx, const Gas<T>& gs, const T Wmb[5],
                         const T Wpb[5], T Wb[5], T aLb[5], T aRb[5]) {
   const T rho = W[0], un = W[1], p = W[4];
-  const T csq = (gs.gamma * p) / rho;
-  const T c = vsqrt(csq);
+  T csq, c, ic, ir;
+  bool fast = false;
+  if constexpr (std::is_same<T, double>::value) {   // the ranges of q64::edge_states
+    fast = q64::within<-34, 50>(q64::high(rho)) && q64::within<-68, 50>(q64::high(p)) && gs.gamma < 16.0;
+    if (fast) {
+      ir = q64::rcp(rho);
+      csq = q64::quot(gs.gamma * p, rho, ir);
+      c = q64::root(csq, ic);
+    }
+  }
+  if (!fast) {
+    csq = (gs.gamma * p) / rho;
+    c = vsqrt(csq);
+    ic = inverse(c);
+    ir = inverse(rho);
+  }
   T a6[5], a6b[5];
   for (int q = 0; q < 5; ++q) {
-    a6[q] = T(6) * (W[q] - T(0.5) * (aL[q] + aR[q]));
+    a6[q] = T(6) * vfma(T(-0.5), aL[q] + aR[q], W[q]);
     a6b[q] = T(0);
   }
   const T lm = un - c, l0 = un, lp = un + c;
-  const T ic = inverse(c), ir = inverse(rho), icsq = ic * ic;
+  const T icsq = ic * ic;
   const T hrc = (T(0.5) * rho) * ic;
   const T hic = T(0.5) * icsq;
   const T cr = c * ir;
@@ -355,12 +391,12 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
   // the forward iteration with its exit at a fixed point; pressures and W kept
   T hp[kRiemannIters + 1], hL[kRiemannIters + 1], hR[kRiemannIters + 1];
   unsigned floored = 0;   // bit k: the pressure of evaluation k was floored
-  int last = 0;
+  int last = 0, turn = -1;
   T CL, CR, ps_raw0, ps, WLs, WRs, uLs, uRs, ZL, ZR;
   bool solved = false;
   if constexpr (std::is_same<T, double>::value) {
     q64::Side l, r;
-    solved = q64::shock_history(L, R, gs, hp, hL, hR, floored, last, ps_raw0, l, r);
+    solved = q64::shock_history(L, R, gs, hp, hL, hR, floored, last, turn, ps_raw0, l, r);
     if (solved) {
       ps = hp[last];
       CL = l.C; WLs = l.W; uLs = l.us; ZL = T(2) * l.z;
@@ -478,15 +514,9 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
   psb += shock_side_bwd(b, ps, WRs, inverse(WRs), inverse(vfma(WRs, WRs, CR * CR)), usb * ZR * iD, usb * (uRs - us) * iD, left ? T(0) : W_sb, gs);
   // Newton iterations in reverse, p_{k+1} = max(p_k - q(p_k), floor): those
   // after a fixed point all have its derivative m = 1 - q', so n of them pass
-  // psb m^n on and add (1 + m + ... + m^(n-1)) times one iteration's adjoints
-  int reps = kRiemannIters - last;
-#pragma unroll 1
-  for (int it = reps > 0 ? last : last - 1; it >= 0; --it, reps = 1) {
-    if (reps == 0) reps = 1;
-    if (floored & (2u << it)) {
-      psb = T(0);
-      continue;
-    }
+  // psb m^n on and add (1 + m + ... + m^(n-1)) times one iteration's adjoints;
+  // two pressures in turn likewise, with one evaluation of each
+  auto iteration = [&](int it, T adj[6]) {   // for psb = 1: (p, C, u) of both sides; returns m
     const T pk = hp[it], WA = hL[it], WB = hR[it];
     const T iA = inverse(WA), dA = inverse(vfma(WA, WA, CL * CL));
     const T iB = inverse(WB), dB = inverse(vfma(WB, WB, CR * CR));
@@ -494,18 +524,46 @@ CELLO_HD void riemann_flux_bwd(const T L[5], const T R[5], const Gas<T>& gs, con
     const T iZ = inverse(ZA + ZB);
     const T du = vfma(pk - pR, iB, uR) - vfma(pL - pk, iA, uL);
     const T zz = ZA * ZB * iZ, q = zz * du;
-    ShockSide<T> x = a, y = b;   // one iteration's adjoints for psb = 1
+    ShockSide<T> x = a, y = b;
     x.pb = x.Cb = x.ub = y.pb = y.Cb = y.ub = T(0);
     T m = T(1);
     m += shock_side_bwd(x, pk, WA, iA, dA, zz, -vfma(ZB, du, -q) * iZ, T(0), gs);
     m += shock_side_bwd(y, pk, WB, iB, dB, -zz, -vfma(ZA, du, -q) * iZ, T(0), gs);
+    adj[0] = x.pb; adj[1] = x.Cb; adj[2] = x.ub;
+    adj[3] = y.pb; adj[4] = y.Cb; adj[5] = y.ub;
+    return m;
+  };
+  auto add = [&](T sum, const T adj[6]) {
+    a.pb = vfma(sum, adj[0], a.pb); a.Cb = vfma(sum, adj[1], a.Cb); a.ub = vfma(sum, adj[2], a.ub);
+    b.pb = vfma(sum, adj[3], b.pb); b.Cb = vfma(sum, adj[4], b.Cb); b.ub = vfma(sum, adj[5], b.ub);
+  };
+  int reps = kRiemannIters - last, it = reps > 0 ? last : last - 1;
+  if (turn >= 0 && last - turn > 2 && floored == 0) {
+    T adj[2][6], m[2], sum[2] = {T(0), T(0)};
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) m[k] = iteration(turn + k, adj[k]);
+    for (; it >= turn; --it) {
+      sum[(it - turn) & 1] += psb;
+      psb *= m[(it - turn) & 1];
+    }
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) add(sum[k], adj[k]);
+  }
+#pragma unroll 1
+  for (; it >= 0; --it, reps = 1) {
+    if (reps == 0) reps = 1;
+    if (floored & (2u << it)) {
+      psb = T(0);
+      continue;
+    }
+    T adj[6];
+    const T m = iteration(it, adj);
     T sum = T(0);
     for (int k = 0; k < reps; ++k) {
       sum += psb;
       psb *= m;
     }
-    a.pb = vfma(sum, x.pb, a.pb); a.Cb = vfma(sum, x.Cb, a.Cb); a.ub = vfma(sum, x.ub, a.ub);
-    b.pb = vfma(sum, y.pb, b.pb); b.Cb = vfma(sum, y.Cb, b.Cb); b.ub = vfma(sum, y.ub, b.ub);
+    add(sum, adj);
   }
   if (!(floored & 1u)) {  // p_0 = ((CR pL + CL pR) + (CL CR)(uL - uR)) / (CL + CR)
     const T nb = psb * inverse(CL + CR), du = uL - uR, cc = nb * CL * CR;

@@ -471,9 +471,11 @@ CELLO_HD void two_shock_flux(const double L[NQ], const double R[NQ], const Gas<d
 // The iteration of two_shock with every pressure and both W of it kept (hp, hL,
 // hR; entry `last` is the final one) and bit k of floored set where pressure k
 // came from the floor; raw0 is pressure 0 before its floor.  A pressure that
-// returns after two steps fills the rest from the two before.
+// returns after two steps fills the rest from the two before, the first of which
+// is entry `turn` (-1: none does).
 CELLO_HD bool shock_history(const double L[5], const double R[5], const Gas<double>& gs, double hp[], double hL[],
-                            double hR[], unsigned& floored, int& last, double& raw0, Side& l, Side& r) {
+                            double hR[], unsigned& floored, int& last, int& turn, double& raw0, Side& l, Side& r) {
+  turn = -1;
   if (!ordinary<5>(L, R, gs)) return false;
   l.set(L, gs);
   r.set(R, gs);
@@ -497,6 +499,7 @@ CELLO_HD bool shock_history(const double L[5], const double R[5], const Gas<doub
     ps = pn;
     if (last == 0 || bits(pn) != bits(hp[last - 1])) continue;
     const bool here = ((kRiemannIters - last) & 1) == 0;   // the last pressure is this one
+    turn = last - 1;
     while (last < kRiemannIters) {
       ++last;
       hp[last] = hp[last - 2];
