@@ -131,7 +131,12 @@ sweep_kernel(DevMesh m, SweepParams prm) {
 
   const int t = threadIdx.x;
   const int lc = t / P, lp = t % P;           // this thread's cell and pencil
-  const int cp = lp, cj = lc;
+  // Phases 2 to 5 leave out two or three cells at each end of a pencil: their
+  // threads start at the first cell they have, so that the idle ones are whole
+  // warps at the end (16^3 blocks: 5 warps of 6 work in phases 2 to 4; idle lanes
+  // at both ends kept all 6 on the arithmetic pipes).  Float64, two steps of 939
+  // 16^3 leaves: 37.4 -> 34.7 ms; 4 pencils a CTA fill fewer lanes (40.3 ms), 16 or
+  // three CTAs per SM measure the same.
   __shared__ int s_item;
   __shared__ T s_dtdx[16];
   // dt/dx per level, once per CTA (a float64 division per thread and item
@@ -174,9 +179,10 @@ sweep_kernel(DevMesh m, SweepParams prm) {
     }
     __syncthreads();
 
-    const int j = cj, p = cp;
+    const int p = lp;
+    int j = 2 + lc;
     // ---- phase 2 (slopes of cells 2..N-3: the interfaces used below are 2..N-4)
-    if (j >= 2 && j <= N - 3) {
+    if (j <= N - 3) {
 #pragma unroll
       for (int k = 0; k < NQ; ++k) {
         const T* a = sW + k * A + p;
@@ -184,7 +190,7 @@ sweep_kernel(DevMesh m, SweepParams prm) {
         else sA[k * A + j * S + p] = q64::slope(a[(j - 1) * S], a[j * S], a[(j + 1) * S]);
       }
     }
-    if (j >= 2 && j <= N - 3) {
+    if (j <= N - 3) {
       const T* pr = sW + 4 * A + p;
       const T* un = sW + 1 * A + p;
       if constexpr (kPacked)
@@ -196,7 +202,7 @@ sweep_kernel(DevMesh m, SweepParams prm) {
     }
     __syncthreads();
     // ---- phase 3 (interfaces j+1/2 read by cells 3..N-4)
-    if (j >= 2 && j <= N - 4) {
+    if (j <= N - 4) {
 #pragma unroll
       for (int k = 0; k < NQ; ++k) {
         if constexpr (kPacked)
@@ -221,7 +227,8 @@ sweep_kernel(DevMesh m, SweepParams prm) {
     }
     __syncthreads();
     // ---- phase 4
-    if (j >= 3 && j <= N - 4) {
+    j = 3 + lc;
+    if (j <= N - 4) {
       const T* pr = sW + 4 * A + p;
       const T fj = sFT[j * S + p], fm = sFT[(j - 1) * S + p], fpp = sFT[(j + 1) * S + p];
       T f;
@@ -271,7 +278,7 @@ sweep_kernel(DevMesh m, SweepParams prm) {
     }
     __syncthreads();
     // ---- phase 5
-    if (j >= 3 && j <= N - 5) {
+    if (j <= N - 5) {
       T L[NQ], R[NQ], F[NQ];
 #pragma unroll
       for (int k = 0; k < NQ; ++k) {
