@@ -25,20 +25,22 @@ namespace cello {
 // thread ran every primitive, slope and edge value up to eight times: three
 // steps of a gradient on 64 leaves of 16^3 took 99.9 ms; with reciprocals shared
 // per divisor and the Newton reverse from the stored history 69.1 ms; each
-// quantity once, as here, 38.2 ms.
-// P: enough pencils that the cells without an edge state (three at each end)
-// leave whole warps idle rather than lanes, within the registers of one CTA.
+// quantity once, as here, 38.2 ms; with the short float64 forms of ppm64.cuh 28.0 ms,
+// of which the float64 forward sweeps then lost another 1.3 ms.
+// The cells without an edge state (three at each end) come last in the CTA, so
+// that they leave whole warps idle rather than lanes (26.7 -> 26.4 ms; 8^3 blocks 7.3 ->
+// 7.15 ms); P: see adj_pencils.
 // ---------------------------------------------------------------------
 template <typename T, int NB>
 constexpr size_t adjoint_smem() {
-  constexpr int A = (NB + 2 * kGhosts) * adj_pencils(NB);
+  constexpr int A = (NB + 2 * kGhosts) * adj_pencils(NB, (int)sizeof(T));
   return (sizeof(T) * 33 + sizeof(int)) * A;
 }
 
 template <typename T, int NB>
-__global__ void __launch_bounds__((NB + 8) * adj_pencils(NB))
+__global__ void __launch_bounds__((NB + 8) * adj_pencils(NB, (int)sizeof(T)))
 adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
-  constexpr int G = kGhosts, N = NB + 2 * G, P = adj_pencils(NB), A = N * P;
+  constexpr int G = kGhosts, N = NB + 2 * G, P = adj_pencils(NB, (int)sizeof(T)), A = N * P;
   constexpr long SLAB = (long)N * N * N;
   constexpr bool k64 = std::is_same<T, double>::value;   // ppm64.cuh: the same values
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -68,7 +70,9 @@ adjoint_sweep_kernel(DevMesh m, AdjSweepParams prm) {
   const int t = threadIdx.x;
   // cell and pencil moved to and from memory (along x first on the x sweep), and computed
   const int mc = axis == 0 ? t % N : t / P, mp = axis == 0 ? t / N : t % P;
-  const int j = t / P, at = t, p = t % P;
+  // cells from the first one with an edge state on, the three before it last: those
+  // without one (three at each end) are whole warps
+  const int j = t / P + 3 < N ? t / P + 3 : t / P + 3 - N, p = t % P, at = j * P + p;
   __shared__ T s_dtdx[16];
   if (t <= m.max_level) s_dtdx[t] = T(*prm.dt / ldexp(m.dx0, -t));
   __syncthreads();

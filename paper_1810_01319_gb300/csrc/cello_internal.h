@@ -11,8 +11,11 @@ namespace cello {
 
 constexpr int kGhosts = 4;
 constexpr int kFields = 5;
-// Pencils per adjoint-sweep CTA for blocks of n cells per edge.
-constexpr int adj_pencils(int n) { return n == 32 ? 8 : 16; }
+// Pencils per adjoint-sweep CTA for blocks of n cells per edge and values of elem
+// bytes: 16 fill whole warps (float64, gradient on 64 leaves of 16^3: 26.4 ms against 28.3
+// with 8) as far as one CTA's registers go; float32 waits for latency instead, and two
+// smaller CTAs per SM hide it (2.16 -> 1.83 ms).
+constexpr int adj_pencils(int n, int elem) { return n == 32 || (n == 16 && elem == 4) ? 8 : 16; }
 
 // Launch variants of the PPM sweep: pencils per CTA, the minimum number of
 // resident CTAs per SM the register allocation is bounded for, and the

@@ -40,7 +40,7 @@ static void prepare_adj() {
 
 template <int NB>
 static void adj_sweep_n(const DevMesh& m, const AdjSweepParams& p, cudaStream_t s) {
-  constexpr int threads = (NB + 2 * kGhosts) * adj_pencils(NB);
+  constexpr int threads = (NB + 2 * kGhosts) * adj_pencils(NB, 4);
   adjoint_sweep_kernel<float, NB><<<p.n_items, threads, adjoint_smem<float, NB>(), s>>>(m, p);
 }
 

@@ -80,7 +80,7 @@ static void prepare_adj() {
 
 template <int NB>
 static void adj_sweep_n(const DevMesh& m, const AdjSweepParams& p, cudaStream_t s) {
-  constexpr int threads = (NB + 2 * kGhosts) * adj_pencils(NB);
+  constexpr int threads = (NB + 2 * kGhosts) * adj_pencils(NB, 8);
   adjoint_sweep_kernel<double, NB><<<p.n_items, threads, adjoint_smem<double, NB>(), s>>>(m, p);
 }
 

@@ -760,7 +760,7 @@ cello_status adjoint_step(cello_mesh* M, const void* Un, void* lam, const double
     p.axis = order[oi];
     p.a0 = rng[oi][0]; p.a1 = rng[oi][1]; p.b0 = rng[oi][2]; p.b1 = rng[oi][3];
     const int pencils = (p.a1 - p.a0) * (p.b1 - p.b0);
-    p.tiles_per_leaf = (pencils + adj_pencils(d.n) - 1) / adj_pencils(d.n);
+    p.tiles_per_leaf = (pencils + adj_pencils(d.n, d.precision) - 1) / adj_pencils(d.n, d.precision);
     p.dt = dt;
     p.leaf0 = 0;
     p.nleaf = B;
