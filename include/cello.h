@@ -291,8 +291,9 @@ cello_status cello_poisson_solve(cello_mesh* mesh, const double* f_dev, double* 
  * II.C), the numerator of the sweep kernel's ALU roofline.  Host only, no
  * device work: the sweep's formulas run in float32 through a counting
  * scalar (one operation per add, subtract, multiply, divide, square root,
- * comparison, absolute value or copysign) over the pencils the sweep kernel
- * covers, on `count` leaves whose slabs the caller copied (ghosts refreshed)
+ * comparison, absolute value or copysign) over the interior and ghost rows a
+ * leaf needs when it is swept alone (a whole step sweeps each row once, in the
+ * leaf that owns it), on `count` leaves whose slabs the caller copied (ghosts refreshed)
  * into U_host (float32, [count][fields][(n+2g)^3] with 5 or, with dual
  * energy, 6 fields, overwritten with the swept
  * state); leaf_ids are those leaves' indices in the mesh; dt and cycle as in
