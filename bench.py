@@ -34,15 +34,6 @@ WORKLOAD = dict(workload="blob-amr-large", root=[16, 16, 16], n=32, max_level=2,
                 exec="graph", l2="inputs larger than L2 (state tens of GB)")
 
 
-# DRAM bytes (read + written) per 32^3 leaf of one sweep launch, measured by
-# ncu on the 4^3-root blob box (3,970 leaves) for the same kernel form and
-# position in the sweep order, keyed "axis-form-position"; the roofline's
-# traffic is this times the leaves of the launch.
-SWEEP_DRAM_BYTES_PER_LEAF = {"x-streaming-staged-sweep_1": 2.573e6,
-                             "y-streaming-staged-sweep_2": 2.290e6, "y-streaming-sweep_2": 2.290e6,
-                             "z-streaming-staged-sweep_3": 1.830e6, "z-streaming-sweep_3": 1.830e6}
-
-
 def alu_peak(log=print):
     """The FP32 ALU roofline's denominator: measured FFMA lane instructions
     per second (cello_fp32_ffma_rate), and the nominal figure from the
@@ -630,13 +621,15 @@ def main():
     value, ms = combine_ranks(ms, cells, args.steps)
     if world > 1:
         torch.distributed.barrier()
-    # kernels per step: reduction partials + finish, refresh phases X, Y, Z
-    # (+ the slow faces), three sweeps, flux correction (with coarse-fine faces)
-    launches_per_step = 2 + 3 + 3 + (2 if mesh.n_coarse_fine else 0)
+    # kernels per step: reduction partials + finish, the first sweep's margins,
+    # three sweeps, with coarse-fine faces the slow faces and the flux correction
+    launches_per_step = 2 + 1 + 3 + (2 if mesh.n_coarse_fine else 0)
 
     # algorithmic operations of the step's sweeps, counted by the library on a
-    # sample of leaves (their slabs copied to the host, ghosts refreshed) and
-    # scaled to the launch; then per-phase times of one batched step on the
+    # sample of leaves (their slabs copied to the host, ghosts refreshed), per
+    # updated cell over the interior and ghost rows of those leaves, and scaled to
+    # the interior cells of the mesh: a step sweeps each row once, and the ghost rows
+    # behind coarse-fine faces and boundaries, swept in addition, are left out; then per-phase times of one batched step on the
     # same state and cycle (events between the library's launches)
     cycle += cycle % 2          # an even cycle: the sweeps run x, y, z
     sample_ids = np.unique(np.linspace(0, mesh.n_leaves - 1, 32).round().astype(np.int64))
@@ -644,17 +637,16 @@ def main():
     t_ops = time.time()
     ops, pencils, swept_cells, _ = mesh.sweep_opcount(U, sample_ids, float(dt.item()), cycle)
     log(f"[bench] operation count on {len(sample_ids)} leaves in {time.time() - t_ops:.1f}s")
-    scale = mesh.n_leaves / len(sample_ids)
     prof = mesh.profile_step(U, dt, cycle, cfg["cfl"])
     names = ["ghost_refresh", "sweep_1", "sweep_2", "sweep_3", "flux_correct", "reduce"]
     top = max(range(len(prof)), key=lambda i: prof[i])
     hbm, src = peaks()
     elem = 4
-    N = cfg["n"] + 8
-    ghost_cells = mesh.n_leaves * (N ** 3 - cfg["n"] ** 3)
+    ghost_cells = mesh.n_leaves * 8 * cfg["n"] ** 2
     # algorithmic bytes per launch: each sweep reads and writes the nf (five,
     # six with dual energy) fields of every leaf interior cell once; the
-    # refresh writes every ghost cell and reads one source value for it; the
+    # refresh of an even step writes the x margins of the interior rows (and the
+    # slow faces, not counted) and reads one source value per cell; the
     # reduction reads the interior
     nf = mesh.nf
     alg_bytes = {"ghost_refresh": ghost_cells * 2 * nf * elem, "sweep_1": cells * 2 * nf * elem,
@@ -673,7 +665,7 @@ def main():
             else "shared-memory",
             "ms": prof[1 + k], "hbm_gbs_algorithmic": alg_bytes[f"sweep_{k + 1}"] / t / 1e9}
         if ops is not None:
-            ops_launch = float(ops[k].sum()) * scale
+            ops_launch = float(ops[k].sum() / swept_cells[k]) * cells
             sweeps[f"sweep_{k + 1}"].update({
                 "ops_per_launch": ops_launch, "ops_per_updated_cell": float(ops[k].sum() / swept_cells[k]),
                 "ops_by_phase_per_updated_cell": {p: float(ops[k][i] / swept_cells[k])
@@ -682,12 +674,6 @@ def main():
     kname = names[top]
     if kname.startswith("sweep") and ops is not None:
         sw = sweeps[kname]
-        traffic, tsrc = None, None
-        key = f"{sw['axis']}-{sw['form']}-{kname}"
-        if key in SWEEP_DRAM_BYTES_PER_LEAF and cfg["n"] == 32 and mesh.nf == 5:   # measured on five fields
-            traffic = SWEEP_DRAM_BYTES_PER_LEAF[key] * mesh.n_leaves
-            tsrc = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per leaf of the same kernel and sweep "
-                    "position on the 4^3-root blob box, times the leaves of this launch")
         roofline = {"bound": "alu", "kernel": kname, "achieved": sw["achieved_tops"], "peak": alu_tops,
                     "unit": "T FP32 lane-op/s", "frac": sw["achieved_tops"] / alu_tops,
                     "peak_source": "measured: cello_fp32_ffma_rate, FP32 fused multiply-add lane instructions "
@@ -699,10 +685,10 @@ def main():
                                   "operation, so a fused multiply-add counts two, while the peak counts one "
                                   "FFMA instruction per lane per clock; against the flop convention (an FFMA = "
                                   "2 flops, peak x 2) the same count gives half this frac",
-                    "traffic": traffic, "traffic_source": tsrc,
+                    "traffic": None,
                     "algorithmic_ops_per_launch": sw["ops_per_launch"],
-                    "ops_sample": f"{len(sample_ids)} leaves evenly spaced in Morton order, scaled by "
-                                  f"{mesh.n_leaves}/{len(sample_ids)}",
+                    "ops_sample": f"operations per updated cell of {len(sample_ids)} leaves evenly spaced in "
+                                  "Morton order, times the interior cells",
                     "hbm": {"achieved": sw["hbm_gbs_algorithmic"], "peak": hbm, "unit": "GB/s",
                             "frac": sw["hbm_gbs_algorithmic"] / hbm, "peak_source": src,
                             "algorithmic_bytes_per_launch": alg_bytes[kname]},
@@ -714,8 +700,8 @@ def main():
                     "algorithmic_bytes_per_launch": alg_bytes[kname], "sweeps": sweeps,
                     "phase_ms": dict(zip(names, prof))}
     # the memory-bound phases against the HBM roofline on their algorithmic
-    # bytes (the refresh: every ghost cell written once and its source read
-    # once; the reduction: the interior read once)
+    # bytes (the refresh: every x margin of an interior row written once and its
+    # source read once; the reduction: the interior read once)
     roofline["memory_phases"] = {
         k: {"ms": prof[names.index(k)], "algorithmic_bytes": alg_bytes[k],
             "achieved_gbs": alg_bytes[k] / (prof[names.index(k)] / 1e3) / 1e9,
