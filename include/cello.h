@@ -110,8 +110,10 @@ cello_status cello_mesh_from_leaves(const cello_mesh_desc* desc, const int32_t* 
 /* Failure detection: every reduction (cello_reduce, or a step asked for dt
  * or totals) sets bit 0 of the mesh's device error word when a leaf interior
  * holds a non-finite value or a non-positive density or pressure (before
- * the floors).  This call waits for the device, returns the word in *word
- * (nullable), clears it, and returns CELLO_ENONFINITE if bit 0 was set. */
+ * the floors).  Bit 1: a sweep gave up waiting for the device to hand it its
+ * next work item, so that the state is incomplete.  This call waits for the
+ * device, returns the word in *word (nullable), clears it, and returns
+ * CELLO_EINTERNAL if bit 1 was set, else CELLO_ENONFINITE if bit 0 was. */
 cello_status cello_check(cello_mesh* mesh, uint32_t* word);
 
 /* Sizes: leaves, elements per leaf (fields * N^3: 5, or 6 with dual energy),
@@ -218,8 +220,8 @@ cello_status cello_set_exec(cello_mesh* mesh, int mode);
  * adjoint, for all three sweep axes: the form (shared-memory phases with
  * one thread per cell, or register streaming with one thread per pencil),
  * pencils per CTA, register bound (minimum resident CTAs per SM) and
- * schedule (one CTA per work item, or one resident wave pulling items from
- * a device counter).  Float32 has 24 variants (12 shared-memory, 12
+ * schedule (one CTA per work item, or resident CTAs that take over the items
+ * that have not started).  Float32 has 24 variants (12 shared-memory, 12
  * streaming, of which 4 read x pencils as 16-byte vectors), float64 2, the
  * same for dual-energy meshes.  The variants of one form compute the same values;
  * the two float32 forms agree to float32 rounding (a multiply and an add

@@ -19,12 +19,12 @@ constexpr int adj_pencils(int n, int elem) { return n == 32 || (n == 16 && elem 
 
 // Launch variants of the PPM sweep: pencils per CTA, the minimum number of
 // resident CTAs per SM the register allocation is bounded for, and the
-// schedule (static: one CTA per item; persistent: one resident wave of CTAs
-// pulling items from a device counter).  The autotuner times them.
+// schedule (static: one CTA per item; persistent: resident CTAs take over the
+// items that have not started, ItemQueue in kernels.cuh).  The autotuner times them.
 struct SweepVariant {
   int pencils;       // pencils per CTA (the CTA size of the streaming form)
   int min_blocks;    // resident CTAs per SM the register bound is set for
-  bool persistent;   // work-counter schedule over a resident grid
+  bool persistent;
   bool stream;       // register-streaming form (sweep_stream_kernel)
   int vec;           // streaming form moving x pencils four cells at a time, staged by cp.async (3), or not (0)
 };
@@ -114,8 +114,8 @@ struct SweepParams {
   int push;                // transverse axis across whose same-level faces the updated rows are also stored, or -1
   const double* dt;        // device scalar
   double* reg;             // flux registers (may be null)
-  unsigned* work;          // work counter for persistent variants (device, 4 bytes)
-  int n_items;             // set by the launcher
+  int n_items;             // set by the launcher: the grid, one CTA per item
+  bool persistent;         // set by the launcher: CTAs take over items that have not started
   int variant;             // index into the sweep variants of the precision; -1: the launcher's rule
 
   // The items of the three regions for per_cta pencils per item.
@@ -231,23 +231,21 @@ void launch_refresh_f64(const DevMesh& m, double* U, int leaf0, int nleaf, const
 void launch_sweep_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s);
 void launch_sweep_f64(const DevMesh& m, const SweepParams& p, cudaStream_t s);
 template <int NB>
-void prepare_sweep_f32(int sms);
+void prepare_sweep_f32();
 template <int NB>
 void launch_sweep_f32_nb(const DevMesh& m, const SweepParams& p, cudaStream_t s);
 // Dual-energy sweeps (both float32 forms, sweep_de_f32.cuh; float64, k_de_f64.cu),
-// launched by the planners above with the grid they computed.
+// launched by the planners above with the items they planned.
 template <int NB, int P, int MINB>
-void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
+void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s);
 template <int NB, int CT, int VEC>
-void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
+void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s);
 template <int NB>
-void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s);
-constexpr int kSweepKernels = 12;   // float32 sweep kernel instantiations per method code
-// Attributes of the dual-energy kernels and their resident CTAs, rows 4 to 7 of the table.
+void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, cudaStream_t s);
+// Attributes of the dual-energy kernels.
 template <int NB>
-void prepare_sweep_de_f32(int (*resident)[kSweepKernels], int sms);
-// Attributes of the float64 dual-energy kernels and their resident CTAs, by block size and method code.
-void prepare_kernels_de_f64(int (*resident)[8], int sms);
+void prepare_sweep_de_f32();
+void prepare_kernels_de_f64();
 void launch_fluxcorr(const DevMesh& m, void* U, int precision, const CoarseFace* faces,
                      const int* group_start, int ngroups, const double* reg, const double* dt,
                      cudaStream_t s);

@@ -11,8 +11,9 @@ static constexpr size_t de_smem64() {
 }
 
 template <int NB>
-void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s) {
+void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
   constexpr int T = (NB + 2 * kGhosts) * 8;
+  const int grid = p.n_items;
   switch (method_code(m.riemann, m.steepen)) {
     case 0: sweep_kernel<double, NB, 8, 2, 4><<<grid, T, de_smem64<NB, 4>(), s>>>(m, p); break;
     case 1: sweep_kernel<double, NB, 8, 2, 5><<<grid, T, de_smem64<NB, 5>(), s>>>(m, p); break;
@@ -21,32 +22,26 @@ void launch_sweep_de_f64(const DevMesh& m, const SweepParams& p, int grid, cudaS
   }
 }
 
-template void launch_sweep_de_f64<8>(const DevMesh&, const SweepParams&, int, cudaStream_t);
-template void launch_sweep_de_f64<16>(const DevMesh&, const SweepParams&, int, cudaStream_t);
-template void launch_sweep_de_f64<32>(const DevMesh&, const SweepParams&, int, cudaStream_t);
-
-template <int NB, int RS>
-static void prepare_de64(int (*resident)[8], int nbi, int sms) {
-  constexpr int T = (NB + 2 * kGhosts) * 8;
-  constexpr size_t sh = de_smem64<NB, RS>();
-  int nb = 0;
-  cudaFuncSetAttribute(sweep_kernel<double, NB, 8, 2, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<double, NB, 8, 2, RS>, T, sh);
-  resident[nbi][RS] = (nb > 0 ? nb : 1) * sms;
-}
+template void launch_sweep_de_f64<8>(const DevMesh&, const SweepParams&, cudaStream_t);
+template void launch_sweep_de_f64<16>(const DevMesh&, const SweepParams&, cudaStream_t);
+template void launch_sweep_de_f64<32>(const DevMesh&, const SweepParams&, cudaStream_t);
 
 template <int NB>
-static void prepare_de64_nb(int (*resident)[8], int nbi, int sms) {
-  prepare_de64<NB, 4>(resident, nbi, sms);
-  prepare_de64<NB, 5>(resident, nbi, sms);
-  prepare_de64<NB, 6>(resident, nbi, sms);
-  prepare_de64<NB, 7>(resident, nbi, sms);
+static void prepare_de64() {
+#define CELLO_DE_ATTR(RS)                                                                               \
+  cudaFuncSetAttribute(sweep_kernel<double, NB, 8, 2, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       (int)de_smem64<NB, RS>())
+  CELLO_DE_ATTR(4);
+  CELLO_DE_ATTR(5);
+  CELLO_DE_ATTR(6);
+  CELLO_DE_ATTR(7);
+#undef CELLO_DE_ATTR
 }
 
-void prepare_kernels_de_f64(int (*resident)[8], int sms) {
-  prepare_de64_nb<8>(resident, 0, sms);
-  prepare_de64_nb<16>(resident, 1, sms);
-  prepare_de64_nb<32>(resident, 2, sms);
+void prepare_kernels_de_f64() {
+  prepare_de64<8>();
+  prepare_de64<16>();
+  prepare_de64<32>();
 }
 
 }  // namespace cello

@@ -54,12 +54,9 @@ void launch_adjoint_sweep_f32(const DevMesh& m, const AdjSweepParams& p, cudaStr
 }
 
 void prepare_kernels_f32() {
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  prepare_sweep_f32<8>(sms);
-  prepare_sweep_f32<16>(sms);
-  prepare_sweep_f32<32>(sms);
+  prepare_sweep_f32<8>();
+  prepare_sweep_f32<16>();
+  prepare_sweep_f32<32>();
   prepare_adj<8>();
   prepare_adj<16>();
   prepare_adj<32>();

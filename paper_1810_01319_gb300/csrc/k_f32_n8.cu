@@ -2,7 +2,7 @@
 #include "sweep_f32.cuh"
 
 namespace cello {
-template void prepare_sweep_f32<8>(int sms);
+template void prepare_sweep_f32<8>();
 template void launch_sweep_f32_nb<8>(const DevMesh& m, const SweepParams& p, cudaStream_t s);
 
 int sweep_variant_count_f32() { return kNV; }

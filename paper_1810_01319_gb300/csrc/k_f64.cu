@@ -10,9 +10,6 @@ namespace cello {
 // Float64 sweep variants: {pencils per CTA, min resident CTAs per SM, persistent}.
 static const SweepVariant kVariants64[] = {{8, 2, false}, {8, 2, true}};
 constexpr int kNV64 = 2;
-static int g_resident64[3][8];   // resident CTAs per GPU by block size and method code
-
-static int nb_index64(int n) { return n == 8 ? 0 : (n == 16 ? 1 : 2); }
 
 template <int NB, int RS>
 static constexpr size_t sweep_smem64() {
@@ -20,22 +17,16 @@ static constexpr size_t sweep_smem64() {
   return sizeof(double) * sweep_arrays(RS) * N * 8;
 }
 
-template <int NB, int RS>
-static void prepare_method64(int sms) {
-  constexpr int T = (NB + 2 * kGhosts) * 8;
-  constexpr size_t sh = sweep_smem64<NB, RS>();
-  int nb = 0;
-  cudaFuncSetAttribute(sweep_kernel<double, NB, 8, 2, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sweep_kernel<double, NB, 8, 2, RS>, T, sh);
-  g_resident64[nb_index64(NB)][RS] = (nb > 0 ? nb : 1) * sms;
-}
-
 template <int NB>
-static void prepare_nb64(int sms) {
-  prepare_method64<NB, 0>(sms);
-  prepare_method64<NB, 1>(sms);
-  prepare_method64<NB, 2>(sms);
-  prepare_method64<NB, 3>(sms);
+static void prepare_nb64() {
+#define CELLO_ATTR64(RS)                                                                                \
+  cudaFuncSetAttribute(sweep_kernel<double, NB, 8, 2, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       (int)sweep_smem64<NB, RS>())
+  CELLO_ATTR64(0);
+  CELLO_ATTR64(1);
+  CELLO_ATTR64(2);
+  CELLO_ATTR64(3);
+#undef CELLO_ATTR64
 }
 
 template <int NB>
@@ -46,19 +37,14 @@ static void launch_nb64(const DevMesh& m, SweepParams p, cudaStream_t s) {
   const int v = (p.variant >= 0 && p.variant < kNV64) ? p.variant : 1;
   p.plan(8);
   if (p.n_items <= 0) return;
-  int grid = p.n_items;
-  if (kVariants64[v].persistent && p.work) {
-    const int resident = g_resident64[nb_index64(NB)][method_code(m.riemann, m.steepen, m.nf == 6)];
-    grid = resident < grid ? resident : grid;
-  } else {
-    p.work = nullptr;
-  }
+  const int grid = p.n_items;
+  p.persistent = kVariants64[v].persistent;
   switch (method_code(m.riemann, m.steepen, m.nf == 6)) {
     case 0: sweep_kernel<double, NB, 8, 2, 0><<<grid, N * 8, sweep_smem64<NB, 0>(), s>>>(m, p); break;
     case 1: sweep_kernel<double, NB, 8, 2, 1><<<grid, N * 8, sweep_smem64<NB, 1>(), s>>>(m, p); break;
     case 2: sweep_kernel<double, NB, 8, 2, 2><<<grid, N * 8, sweep_smem64<NB, 2>(), s>>>(m, p); break;
     case 3: sweep_kernel<double, NB, 8, 2, 3><<<grid, N * 8, sweep_smem64<NB, 3>(), s>>>(m, p); break;
-    default: launch_sweep_de_f64<NB>(m, p, grid, s); break;   // dual energy (k_de_f64.cu)
+    default: launch_sweep_de_f64<NB>(m, p, s); break;   // dual energy (k_de_f64.cu)
   }
 }
 
@@ -95,13 +81,10 @@ void launch_adjoint_sweep_f64(const DevMesh& m, const AdjSweepParams& p, cudaStr
 
 
 void prepare_kernels_f64() {
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  prepare_nb64<8>(sms);
-  prepare_nb64<16>(sms);
-  prepare_nb64<32>(sms);
-  prepare_kernels_de_f64(g_resident64, sms);
+  prepare_nb64<8>();
+  prepare_nb64<16>();
+  prepare_nb64<32>();
+  prepare_kernels_de_f64();
   prepare_adj<8>();
   prepare_adj<16>();
   prepare_adj<32>();

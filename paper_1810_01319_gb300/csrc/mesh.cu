@@ -253,8 +253,7 @@ struct cello_mesh {
   std::vector<int> slow_ax_start[3];
   int exec_mode = CELLO_EXEC_BATCHED;
   int sweep_variant[3] = {-1, -1, -1};   // per sweep axis; chosen by cello_autotune or set by the caller, -1: by rule
-  unsigned* d_work = nullptr;      // work counter of the persistent sweep variants
-  unsigned* d_err = nullptr;       // error word set by the reduction
+  unsigned* d_err = nullptr;       // error word: bit 0 set by the reduction, bit 1 by a sweep (ItemQueue)
   int* d_flag = nullptr;           // result word of the table and remap-map kernels
   RemapEntry* d_map = nullptr;     // remap entries of this mesh as the new one
   mutable std::mutex remap_lock;   // d_flag and d_map: one remap into this mesh at a time
@@ -457,7 +456,6 @@ cello_status finish_build(cello_mesh* M) {
   M->d_leaf = part<int4>(M->d_table, o_leaf);
   M->d_keys = part<unsigned long long>(M->d_table, o_keys);
   M->d_err = part<unsigned>(M->d_table, o_word);
-  M->d_work = M->d_err + 8;
   M->d_zero = part<double>(M->d_table, o_word) + 16;
   M->d_flag = part<int>(M->d_table, o_flag);
   M->d_kind = part<int8_t>(M->d_table, o_kind);
@@ -631,7 +629,6 @@ void enqueue_sweeps(const cello_mesh* M, const DevMesh& dm, void* U, const doubl
     p.U = U;
     p.dt = dt;
     p.reg = M->d_reg;
-    p.work = M->d_work;
     p.variant = M->sweep_variant[order[oi]];
     if (plain) {
       for (int b = leaf0; b < leaf0 + nleaf; ++b) {
@@ -737,7 +734,6 @@ cello_status adjoint_step(cello_mesh* M, const void* Un, void* lam, const double
       p.U = entry[oi + 1];
       p.dt = dt;
       p.reg = nullptr;
-      p.work = M->d_work;
       p.variant = M->sweep_variant[axis];
       set_regions(M, p, order, oi, 0, B, false);   // the adjoint sweeps read every ghost row
       launch_sweep(M, dm, p, s);
@@ -871,6 +867,7 @@ cello_status cello_check(cello_mesh* M, uint32_t* word) {
   CELLO_CUDA(cudaMemcpy(&w, M->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost));
   CELLO_CUDA(cudaMemset(M->d_err, 0, sizeof(unsigned)));
   if (word) *word = w;
+  if (w & 2u) return fail(CELLO_EINTERNAL, "a sweep gave up waiting for its next work item: the state is incomplete");
   if (w & 1u) return fail(CELLO_ENONFINITE, "a reduction saw a non-finite value or a non-positive density or pressure");
   return CELLO_OK;
 }
@@ -1222,7 +1219,6 @@ cello_status cello_autotune(cello_mesh* M, void* U, int* variants_out, float* ms
           p.U = U;
           p.dt = M->d_zero;
           p.reg = nullptr;
-          p.work = M->d_work;
           p.variant = v;
           set_regions(M, p, order, oi, 0, nleaf, true);
           p.push = -1;   // the sample's neighbours keep their ghost rows

@@ -1,7 +1,7 @@
 // Float32 dual-energy sweeps (both forms with a sixth field rho e; method
 // code RS | 4) for blocks of CELLO_DE_NB cells per edge, one translation unit
 // per block size.  Compiled with the float32 sweep's flags; the planners in
-// sweep_f32.cuh compute the grid and call launch_sweep_de_f32 (shared-memory
+// sweep_f32.cuh count the items and call launch_sweep_de_f32 (shared-memory
 // form) or launch_stream_de_f32 (register streaming).
 #pragma once
 
@@ -15,8 +15,9 @@ static constexpr size_t de_smem() {
 }
 
 template <int NB, int P, int MINB>
-void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s) {
+void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
   constexpr int T = (NB + 2 * kGhosts) * P;
+  const int grid = p.n_items;
   switch (method_code(m.riemann, m.steepen)) {
     case 0: sweep_kernel<float, NB, P, MINB, 4><<<grid, T, de_smem<NB, P, 4>(), s>>>(m, p); break;
     case 1: sweep_kernel<float, NB, P, MINB, 5><<<grid, T, de_smem<NB, P, 5>(), s>>>(m, p); break;
@@ -33,9 +34,10 @@ void launch_sweep_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaS
 // bytes a thread) cost more than the extra warps give: 183 leaves of 32^3 with
 // HLLC and steepening, two steps of variants 22, 21, 21, 2.06 -> 1.72 ms.
 template <int NB, int CT, int VEC>
-void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cudaStream_t s) {
+void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
   constexpr int MINB = 384 / CT;
   constexpr size_t sh = VEC == 3 ? sizeof(float4) * 4 * 6 * CT : 0;
+  const int grid = p.n_items;
   switch (method_code(m.riemann, m.steepen)) {
     case 0: sweep_stream_kernel<float, NB, CT, MINB, VEC, 4><<<grid, CT, sh, s>>>(m, p); break;
     case 1: sweep_stream_kernel<float, NB, CT, MINB, VEC, 5><<<grid, CT, sh, s>>>(m, p); break;
@@ -47,62 +49,36 @@ void launch_stream_de_f32(const DevMesh& m, const SweepParams& p, int grid, cuda
 // The streaming variants of the float32 table: {CTA size, vector I/O}.
 #define CELLO_DE_STREAM(X, NB) X(NB, 64, 0) X(NB, 128, 0) X(NB, 32, 0) X(NB, 64, 3)
 #define CELLO_DE_SINST(NB, CT, VEC) \
-  template void launch_stream_de_f32<NB, CT, VEC>(const DevMesh&, const SweepParams&, int, cudaStream_t);
+  template void launch_stream_de_f32<NB, CT, VEC>(const DevMesh&, const SweepParams&, cudaStream_t);
 CELLO_DE_STREAM(CELLO_DE_SINST, CELLO_DE_NB)
 #undef CELLO_DE_SINST
 #undef CELLO_DE_STREAM
 
-template <typename K>
-static int resident_de(K kernel, int threads, size_t smem, int sms) {
-  int nb = 0;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem);
-  return (nb > 0 ? nb : 1) * sms;
-}
-
 template <int NB, int P, int MINB>
-static void prepare_de(int (*resident)[kSweepKernels], int v, int sms) {
-  constexpr int T = (NB + 2 * kGhosts) * P;
-  resident[4][v] = resident_de(sweep_kernel<float, NB, P, MINB, 4>, T, de_smem<NB, P, 4>(), sms);
-  resident[5][v] = resident_de(sweep_kernel<float, NB, P, MINB, 5>, T, de_smem<NB, P, 5>(), sms);
-  resident[6][v] = resident_de(sweep_kernel<float, NB, P, MINB, 6>, T, de_smem<NB, P, 6>(), sms);
-  resident[7][v] = resident_de(sweep_kernel<float, NB, P, MINB, 7>, T, de_smem<NB, P, 7>(), sms);
-}
-
-template <int NB, int CT, int VEC>
-static void prepare_stream_de(int (*resident)[kSweepKernels], int v, int sms) {
-  constexpr int MINB = 384 / CT;
-  constexpr size_t sh = VEC == 3 ? sizeof(float4) * 4 * 6 * CT : 0;
-  resident[4][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 4>, CT, sh, sms);
-  resident[5][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 5>, CT, sh, sms);
-  resident[6][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 6>, CT, sh, sms);
-  resident[7][v] = resident_de(sweep_stream_kernel<float, NB, CT, MINB, VEC, 7>, CT, sh, sms);
+static void prepare_de() {
+#define CELLO_DE_ATTR(RS)                                                                                 \
+  cudaFuncSetAttribute(sweep_kernel<float, NB, P, MINB, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       (int)de_smem<NB, P, RS>())
+  CELLO_DE_ATTR(4);
+  CELLO_DE_ATTR(5);
+  CELLO_DE_ATTR(6);
+  CELLO_DE_ATTR(7);
+#undef CELLO_DE_ATTR
 }
 
 // The shared-memory variants of the float32 table: {pencils, min CTAs per SM}.
 #define CELLO_DE_VARIANTS(X, NB) X(NB, 8, 3) X(NB, 8, 4) X(NB, 4, 6) X(NB, 16, 1) X(NB, 4, 8) X(NB, 16, 2)
 #define CELLO_DE_INST(NB, P, MINB) \
-  template void launch_sweep_de_f32<NB, P, MINB>(const DevMesh&, const SweepParams&, int, cudaStream_t);
+  template void launch_sweep_de_f32<NB, P, MINB>(const DevMesh&, const SweepParams&, cudaStream_t);
 CELLO_DE_VARIANTS(CELLO_DE_INST, CELLO_DE_NB)
 #undef CELLO_DE_INST
 
-#undef CELLO_DE_VARIANTS
-
 template <>
-void prepare_sweep_de_f32<CELLO_DE_NB>(int (*resident)[kSweepKernels], int sms) {
-  constexpr int NB = CELLO_DE_NB;
-  prepare_de<NB, 8, 3>(resident, 0, sms);
-  prepare_de<NB, 8, 4>(resident, 1, sms);
-  prepare_de<NB, 4, 6>(resident, 2, sms);
-  prepare_de<NB, 16, 1>(resident, 3, sms);
-  prepare_de<NB, 4, 8>(resident, 4, sms);
-  prepare_de<NB, 16, 2>(resident, 5, sms);
-  prepare_stream_de<NB, 64, 0>(resident, 6, sms);
-  prepare_stream_de<NB, 128, 0>(resident, 7, sms);
-  prepare_stream_de<NB, 64, 0>(resident, 8, sms);
-  prepare_stream_de<NB, 32, 0>(resident, 9, sms);
-  prepare_stream_de<NB, 64, 3>(resident, 10, sms);
-  prepare_stream_de<NB, 64, 3>(resident, 11, sms);
+void prepare_sweep_de_f32<CELLO_DE_NB>() {
+#define CELLO_DE_PREP(NB, P, MINB) prepare_de<NB, P, MINB>();
+  CELLO_DE_VARIANTS(CELLO_DE_PREP, CELLO_DE_NB)
+#undef CELLO_DE_PREP
 }
+#undef CELLO_DE_VARIANTS
 
 }  // namespace cello

@@ -10,7 +10,7 @@ namespace cello {
 // Float32 sweep variants.  Shared-memory form: {pencils per CTA, min
 // resident CTAs per SM}; register-streaming form: {CTA size = pencils per
 // CTA, min resident CTAs per SM}; each without and with the persistent
-// work-counter schedule.
+// schedule (ItemQueue).
 static const SweepVariant kVariants[] = {
     {8, 3, false, false},  {8, 4, false, false},  {4, 6, false, false}, {16, 1, false, false},
     {4, 8, false, false},  {16, 2, false, false}, {64, 8, false, true}, {128, 4, false, true},
@@ -19,20 +19,8 @@ static const SweepVariant kVariants[] = {
     {4, 8, true, false},   {16, 2, true, false},  {64, 8, true, true},  {128, 4, true, true},
     {64, 6, true, true},   {32, 16, true, true},  {64, 8, true, true, 3},  {64, 6, true, true, 3},
 };
-constexpr int kNT = kSweepKernels;  // variant v uses template v % kNT
+constexpr int kNT = 12;  // distinct kernel instantiations; variant v uses template v % kNT
 constexpr int kNV = sizeof(kVariants) / sizeof(kVariants[0]);
-// Resident CTAs per GPU by method code and kernel instantiation, from the
-// occupancy API: a persistent launch of more would leave the rest waiting with
-// their first items.
-template <int NB> inline int g_resident[8][kNT];
-
-template <int NB, typename K>
-static void set_resident(int rs, int v, K kernel, int threads, size_t smem, int sms) {
-  int nb = 0;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem);
-  g_resident<NB>[rs][v] = (nb > 0 ? nb : 1) * sms;
-}
 
 // Shared memory of the shared-memory form: sweep_arrays(RS) arrays of N x P
 // values (21; 24 with contact steepening).
@@ -43,12 +31,15 @@ static constexpr size_t sweep_smem() {
 }
 
 template <int NB, int P, int MINB>
-static void prepare_variant(int v, int sms) {
-  constexpr int T = (NB + 2 * kGhosts) * P;
-  set_resident<NB>(0, v, sweep_kernel<float, NB, P, MINB, 0>, T, sweep_smem<NB, P, 0>(), sms);
-  set_resident<NB>(1, v, sweep_kernel<float, NB, P, MINB, 1>, T, sweep_smem<NB, P, 1>(), sms);
-  set_resident<NB>(2, v, sweep_kernel<float, NB, P, MINB, 2>, T, sweep_smem<NB, P, 2>(), sms);
-  set_resident<NB>(3, v, sweep_kernel<float, NB, P, MINB, 3>, T, sweep_smem<NB, P, 3>(), sms);
+static void prepare_variant() {
+#define CELLO_ATTR(RS)                                                                                    \
+  cudaFuncSetAttribute(sweep_kernel<float, NB, P, MINB, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       (int)sweep_smem<NB, P, RS>())
+  CELLO_ATTR(0);
+  CELLO_ATTR(1);
+  CELLO_ATTR(2);
+  CELLO_ATTR(3);
+#undef CELLO_ATTR
 }
 
 // Dynamic shared memory of the streaming form: the staged form keeps three
@@ -58,51 +49,34 @@ static constexpr size_t stream_smem() {
   return VEC == 3 ? sizeof(float4) * 4 * 5 * CT : 0;
 }
 
-template <int NB, int CT, int MINB, int VEC>
-static void prepare_stream_variant(int v, int sms) {
-  constexpr size_t sh = stream_smem<CT, VEC>();
-  set_resident<NB>(0, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 0>, CT, sh, sms);
-  set_resident<NB>(1, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 1>, CT, sh, sms);
-  set_resident<NB>(2, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 2>, CT, sh, sms);
-  set_resident<NB>(3, v, sweep_stream_kernel<float, NB, CT, MINB, VEC, 3>, CT, sh, sms);
-}
-
-// Work items, grid and schedule of one launch; false if there is no work.
-template <int NB>
-static bool plan_launch(const DevMesh& m, SweepParams& p, int per_cta, int v, int& grid) {
+// Work items and schedule of one launch; false if there is no work.
+static bool plan_launch(SweepParams& p, int per_cta, int v) {
   p.plan(per_cta);
-  if (p.n_items <= 0) return false;
-  grid = p.n_items;
-  if (kVariants[v].persistent && p.work) {
-    const int resident = g_resident<NB>[method_code(m.riemann, m.steepen, m.nf == 6)][v % kNT];
-    grid = resident < grid ? resident : grid;
-  } else {
-    p.work = nullptr;
-  }
-  return true;
+  p.persistent = kVariants[v].persistent;
+  return p.n_items > 0;
 }
 
 template <int NB, int P, int MINB>
 static void launch_variant(const DevMesh& m, SweepParams p, int v, cudaStream_t s) {
   constexpr int N = NB + 2 * kGhosts;
-  int grid = 0;
-  if (!plan_launch<NB>(m, p, P, v, grid)) return;
+  if (!plan_launch(p, P, v)) return;
+  const int grid = p.n_items;
   switch (method_code(m.riemann, m.steepen, m.nf == 6)) {
     case 0: sweep_kernel<float, NB, P, MINB, 0><<<grid, N * P, sweep_smem<NB, P, 0>(), s>>>(m, p); break;
     case 1: sweep_kernel<float, NB, P, MINB, 1><<<grid, N * P, sweep_smem<NB, P, 1>(), s>>>(m, p); break;
     case 2: sweep_kernel<float, NB, P, MINB, 2><<<grid, N * P, sweep_smem<NB, P, 2>(), s>>>(m, p); break;
     case 3: sweep_kernel<float, NB, P, MINB, 3><<<grid, N * P, sweep_smem<NB, P, 3>(), s>>>(m, p); break;
-    default: launch_sweep_de_f32<NB, P, MINB>(m, p, grid, s); break;   // dual energy (sweep_de_f32.cuh)
+    default: launch_sweep_de_f32<NB, P, MINB>(m, p, s); break;   // dual energy (sweep_de_f32.cuh)
   }
 }
 
 template <int NB, int CT, int MINB, int VEC>
 static void launch_stream_variant(const DevMesh& m, SweepParams p, int v, cudaStream_t s) {
-  int grid = 0;
-  if (!plan_launch<NB>(m, p, CT, v, grid)) return;
+  if (!plan_launch(p, CT, v)) return;
+  const int grid = p.n_items;
   constexpr size_t sh = stream_smem<CT, VEC>();
   if (m.nf == 6) {   // dual energy (sweep_de_f32.cuh)
-    launch_stream_de_f32<NB, CT, VEC>(m, p, grid, s);
+    launch_stream_de_f32<NB, CT, VEC>(m, p, s);
     return;
   }
   switch (method_code(m.riemann, m.steepen)) {
@@ -114,20 +88,14 @@ static void launch_stream_variant(const DevMesh& m, SweepParams p, int v, cudaSt
 }
 
 template <int NB>
-void prepare_sweep_f32(int sms) {
-  prepare_variant<NB, 8, 3>(0, sms);
-  prepare_variant<NB, 8, 4>(1, sms);
-  prepare_variant<NB, 4, 6>(2, sms);
-  prepare_variant<NB, 16, 1>(3, sms);
-  prepare_variant<NB, 4, 8>(4, sms);
-  prepare_variant<NB, 16, 2>(5, sms);
-  prepare_stream_variant<NB, 64, 8, 0>(6, sms);
-  prepare_stream_variant<NB, 128, 4, 0>(7, sms);
-  prepare_stream_variant<NB, 64, 6, 0>(8, sms);
-  prepare_stream_variant<NB, 32, 16, 0>(9, sms);
-  prepare_stream_variant<NB, 64, 8, 3>(10, sms);
-  prepare_stream_variant<NB, 64, 6, 3>(11, sms);
-  prepare_sweep_de_f32<NB>(g_resident<NB>, sms);
+void prepare_sweep_f32() {
+  prepare_variant<NB, 8, 3>();
+  prepare_variant<NB, 8, 4>();
+  prepare_variant<NB, 4, 6>();
+  prepare_variant<NB, 16, 1>();
+  prepare_variant<NB, 4, 8>();
+  prepare_variant<NB, 16, 2>();
+  prepare_sweep_de_f32<NB>();
 }
 
 // The variant of a sweep that the caller has not chosen one for.  The streaming
