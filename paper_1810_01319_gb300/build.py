@@ -100,7 +100,8 @@ def build_hostcheck() -> str:
     (csrc/hostcheck.cu), used only by the CPU unit tests."""
     os.makedirs(BUILD, exist_ok=True)
     src = os.path.join(CSRC, "hostcheck.cu")
-    deps = [src] + [os.path.join(CSRC, f) for f in ("ppm.cuh", "ppm64.cuh", "adjoint.cuh", "opcount.cu", "cello_internal.h")]
+    deps = [src] + [os.path.join(CSRC, f) for f in ("ppm.cuh", "ppm64.cuh", "adjoint.cuh", "opcount.cu", "cello_internal.h",
+                                                        "per_device.h")]
     if _stale(HOSTCHECK, deps):
         cmd = [nvcc(), *ARCH, "-O2", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=off", "-I", CSRC,
                "-I", INCLUDE, "-shared", src, "-o", HOSTCHECK]

@@ -194,8 +194,8 @@ DevMesh mesh_dev(const cello_mesh* mesh);
 int mesh_precision(const cello_mesh* mesh);
 cello_status set_error(cello_status status, const char* message);
 
-// One-time kernel attribute set-up (dynamic shared memory limits), done
-// outside any stream capture.
+// Kernel attributes (dynamic shared memory limits) for the current device, set
+// once per device, outside any stream capture.
 void prepare_kernels();
 void prepare_kernels_f32();
 void prepare_kernels_f64();

@@ -3,8 +3,11 @@
 // for CPU unit tests of the device math (the same CELLO_HD functions the
 // kernels run).  Built into a separate test library; the product library
 // does not contain it.
+#include <thread>
+
 #include "adjoint.cuh"
 #include "opcount.cu"
+#include "per_device.h"
 #include "ppm64.cuh"
 
 using namespace cello;
@@ -41,6 +44,18 @@ void cello_hc_window_flux_vjp(const double* U, double dtdx, double gamma, int pr
                               double* Ub) {
   if (precision == 4) vjp_t<float>(U, dtdx, gamma, Fb, Ub);
   else vjp_t<double>(U, dtdx, gamma, Fb, Ub);
+}
+// One set-up asked for on each of the listed devices in turn, each by two threads at
+// once; calls[d] counts its runs on device d.
+void cello_hc_once_per_device(const int* devices, int count, int* calls) {
+  OncePerDevice once;
+  for (int i = 0; i < count; ++i) {
+    const int d = devices[i];
+    auto ask = [&] { once.run(d, [&] { ++calls[d]; }); };
+    std::thread other(ask);
+    ask();
+    other.join();
+  }
 }
 // One leaf's sweep through the counting scalar (float32 arithmetic), its
 // update written back into slab [fields][N^3]; counts[6] per phase.

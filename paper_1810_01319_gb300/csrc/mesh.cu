@@ -13,6 +13,7 @@
 #include "cello.h"
 #include "cello_internal.h"
 #include "morton.h"
+#include "per_device.h"
 
 using namespace cello;
 
@@ -189,27 +190,19 @@ unsigned long long leaf_key(const cello_mesh_desc& d, const Node& t) {
 
 namespace cello {
 void prepare_kernels() {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static OncePerDevice once;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  once.run(dev, [] {
     prepare_kernels_f32();
     prepare_kernels_f64();
+    // L2 fetch granularity of this process's context on the device: 64 bytes.
+    // The ghost refresh reads 32-byte margin sectors of 160-byte rows; with the
+    // limit left unset, misses fetched 128-byte lines (phase X: 3.2x its requested
+    // sectors read from DRAM).  A hint of this context only, not a device setting.
+    if (cudaDeviceSetLimit(cudaLimitMaxL2FetchGranularity, 64) != cudaSuccess)
+      cudaGetLastError();   // a device that does not take the hint keeps its default
   });
-  // L2 fetch granularity of this process's context on the current device, set
-  // once per device: 64 bytes.  The ghost refresh reads 32-byte margin
-  // sectors of 160-byte rows; with the limit left unset, misses fetched
-  // 128-byte lines (phase X: 3.2x its requested sectors read from DRAM).  A
-  // hint of this context only, not a device setting.
-  static std::mutex mu;
-  static unsigned long long done = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
-    std::lock_guard<std::mutex> lock(mu);
-    if (!(done >> dev & 1ull)) {
-      if (cudaDeviceSetLimit(cudaLimitMaxL2FetchGranularity, 64) != cudaSuccess)
-        cudaGetLastError();   // a device that does not take the hint keeps its default
-      done |= 1ull << dev;
-    }
-  }
 }
 }  // namespace cello
 

@@ -27,10 +27,10 @@
 // is the plain expression in its order on the same grid values (the block
 // layout only changes where they are stored), with 1/h^2 and 1/6 as
 // multiplications by reciprocals computed once (float64: and multiply-adds fused).
-#include <mutex>
 #include <vector>
 
 #include "cello_internal.h"
+#include "per_device.h"
 #include "widen.cuh"
 
 namespace cello {
@@ -972,8 +972,11 @@ void residual(const DevMesh& m, const double* f, const double* phi, float* r, do
 cudaError_t poisson_solve(PoissonScratch** scratch, const DevMesh& m, int M, double h, const double* f_leaves,
                           double* phi_leaves, int cycles, int inner, double* resid_host, cudaStream_t s) {
   const int n = m.n, B = m.B;
-  static std::once_flag once;
-  std::call_once(once, prepare_poisson);
+  static OncePerDevice once;
+  int dev = 0;
+  const cudaError_t found = cudaGetDevice(&dev);
+  if (found != cudaSuccess) return found;
+  once.run(dev, prepare_poisson);
   if (!*scratch) *scratch = new PoissonScratch();
   PoissonScratch* S = *scratch;
   const long nl = (long)B * n * n * n;
