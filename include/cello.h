@@ -235,9 +235,10 @@ cello_status cello_set_sweep_variants(cello_mesh* mesh, const int* variants);
 
 /* Autotuner (Sec. IV: agglomerated work units on accelerators): times the
  * sweeps of an even and an odd step (each axis in both of its positions)
- * for every sweep variant on up to 4096 leaves of U with dt = 0 (U is left
- * bit-for-bit unchanged), keeps the fastest variant of each axis for this
- * mesh and returns them in variants_out[3] (nullable); ms_out (host,
+ * for every sweep variant with dt = 0 on a copy of up to 4096 leaves of U (U
+ * is left bit-for-bit unchanged; where the device has no room for the copy,
+ * the sweeps run in place, and with dual energy rho e may be synchronised),
+ * keeps the fastest variant of each axis for this mesh and returns them in variants_out[3] (nullable); ms_out (host,
  * nullable, ms_len entries) receives at [3 v + axis] the best time of
  * variant v on that axis.  Blocks until done; call it outside any stream
  * capture. */

@@ -81,9 +81,10 @@ __device__ __forceinline__ long push_offset(const DevMesh& m, const SweepParams&
   const int side = c < 2 * G ? -1 : (c >= NB ? 1 : 0);
   if (side == 0) return 0;
   const int e = at.leaf * 27 + face_dir(prm.push, side);
-  if (m.kind[e] != kSame) return 0;
+  const int to = m.idx[e];
+  if (m.kind[e] != kSame || to >= m.B) return 0;   // beyond B: outside the autotuner's sample
   const long stride = prm.push == 0 ? 1 : (prm.push == 1 ? N : (long)N * N);
-  return ((long)m.idx[e] - at.leaf) * NQ * SLAB - side * NB * stride;
+  return ((long)to - at.leaf) * NQ * SLAB - side * NB * stride;
 }
 
 // The persistent schedule: one CTA per item is launched, and a resident CTA that

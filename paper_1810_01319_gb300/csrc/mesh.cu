@@ -1190,16 +1190,28 @@ cello_status cello_autotune(cello_mesh* M, void* U, int* variants_out, float* ms
   CELLO_REQUIRE_ALIGNED(U);
   cudaStream_t s = (cudaStream_t)stream;
   const cello_mesh_desc& d = M->desc;
-  const DevMesh dm = M->dev();
   const int nv = d.precision == 4 ? sweep_variant_count_f32() : sweep_variant_count_f64();
   const int nleaf = std::min(M->B, 4096);   // per-leaf cost is uniform: a sample of leaves suffices
+  DevMesh dm = M->dev();
+  dm.B = nleaf;
+  // The sweeps of a whole step, stores into the neighbours' ghost rows included, on
+  // a copy of the sample.  Where there is no room for one they run in place and
+  // leave the neighbours' ghost rows alone (dt = 0: the interiors stay as they are,
+  // but for a rho e that the dual-energy synchronisation resets).
+  const size_t bytes = (size_t)nleaf * nfields(d) * M->N * M->N * M->N * d.precision;
+  void* copy = nullptr;
+  if (cudaMalloc(&copy, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    copy = nullptr;
+  }
   cudaEvent_t ev[4];
   for (int i = 0; i < 4; ++i) CELLO_CUDA(cudaEventCreate(&ev[i]));
   int best[3] = {0, 0, 0};
   float best_ms[3] = {1e30f, 1e30f, 1e30f};
-  cudaError_t err = cudaSuccess;
+  cudaError_t err = copy ? cudaMemcpyAsync(copy, U, bytes, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
+  std::vector<float> times(3 * (size_t)nv, 1e30f);
   for (int v = 0; v < nv && err == cudaSuccess; ++v) {
-    float vbest[3] = {1e30f, 1e30f, 1e30f};
+    float* vbest = &times[3 * v];
     for (int rep = 0; rep < 4 && err == cudaSuccess; ++rep) {
       float axis_ms[3] = {0, 0, 0};
       // the sweeps of an even (x, y, z) and an odd (z, y, x) cycle, dt = 0 (state unchanged):
@@ -1209,12 +1221,12 @@ cello_status cello_autotune(cello_mesh* M, void* U, int* variants_out, float* ms
         cudaEventRecord(ev[0], s);
         for (int oi = 0; oi < 3; ++oi) {
           SweepParams p{};
-          p.U = U;
+          p.U = copy ? copy : U;
           p.dt = M->d_zero;
           p.reg = nullptr;
           p.variant = v;
           set_regions(M, p, order, oi, 0, nleaf, true);
-          p.push = -1;   // the sample's neighbours keep their ghost rows
+          if (!copy) p.push = -1;
           launch_sweep(M, dm, p, s);
           cudaEventRecord(ev[oi + 1], s);
         }
@@ -1237,6 +1249,7 @@ cello_status cello_autotune(cello_mesh* M, void* U, int* variants_out, float* ms
     }
   }
   for (int i = 0; i < 4; ++i) cudaEventDestroy(ev[i]);
+  if (copy) cudaFree(copy);
   CELLO_CUDA(err);
   CELLO_CUDA(cudaGetLastError());
   if (variants_out)
