@@ -223,7 +223,8 @@ cello_status cello_set_exec(cello_mesh* mesh, int mode);
  * schedule (one CTA per work item, or resident CTAs that take over the items
  * that have not started).  Float32 has 24 variants (12 shared-memory, 12
  * streaming, of which 4 read x pencils as 16-byte vectors), float64 2, the
- * same for dual-energy meshes.  The variants of one form compute the same values;
+ * same for dual-energy meshes (there the streaming variants that differ in
+ * the register bound alone are one kernel).  The variants of one form compute the same values;
  * the two float32 forms agree to float32 rounding (a multiply and an add
  * may be fused across what is a register in one form and shared memory in
  * the other).  Cached graphs are dropped. */

@@ -29,6 +29,9 @@ struct SweepVariant {
   int vec;           // streaming form moving x pencils four cells at a time, staged by cp.async (3), or not (0)
 };
 int sweep_variant_count_f32();
+// The first variant with the kernel and schedule of variant v: v itself, but for
+// dual-energy meshes, whose streaming kernels all have one register bound.
+int sweep_variant_twin_f32(int v, bool dual);
 int sweep_variant_count_f64();
 
 // Neighbour kinds of the 27-entry table.
