@@ -224,10 +224,9 @@ cello_status cello_set_exec(cello_mesh* mesh, int mode);
  * that have not started).  Float32 has 24 variants (12 shared-memory, 12
  * streaming, of which 4 read x pencils as 16-byte vectors), float64 2, the
  * same for dual-energy meshes (there the streaming variants that differ in
- * the register bound alone are one kernel).  The variants of one form compute the same values;
- * the two float32 forms agree to float32 rounding (a multiply and an add
- * may be fused across what is a register in one form and shared memory in
- * the other).  Cached graphs are dropped. */
+ * the register bound alone are one kernel).  Every variant of a precision computes
+ * the same values, bit for bit.  -1, which a new mesh starts with: a variant by
+ * the number of pencils of the sweep.  Cached graphs are dropped. */
 cello_status cello_set_sweep_variant(cello_mesh* mesh, int variant);
 
 /* The same with one variant per sweep axis: variants[3] for the x, y and z

@@ -333,7 +333,8 @@ class Mesh:
         return list(v), [list(x) for x in t if any(x)]
 
     def set_sweep_variants(self, variants):
-        """One sweep variant per axis (x, y, z)."""
+        """One sweep variant per axis (x, y, z); -1: by the size of the sweep, as on
+        a new mesh."""
         arr = (ctypes.c_int * 3)(*[int(x) for x in variants])
         _lib.check(_lib.lib().cello_set_sweep_variants(self.handle, ctypes.cast(arr, ctypes.c_void_p)),
                    "cello_set_sweep_variants")

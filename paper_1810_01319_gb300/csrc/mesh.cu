@@ -1173,7 +1173,7 @@ cello_status cello_set_sweep_variants(cello_mesh* M, const int* variants) {
   if (!M || !variants) return fail(CELLO_EINVAL, "NULL argument");
   const int nv = M->desc.precision == 4 ? sweep_variant_count_f32() : sweep_variant_count_f64();
   for (int a = 0; a < 3; ++a)
-    if (variants[a] < 0 || variants[a] >= nv) return fail(CELLO_EINVAL, "sweep variant out of range");
+    if (variants[a] < -1 || variants[a] >= nv) return fail(CELLO_EINVAL, "sweep variant out of range");
   for (int a = 0; a < 3; ++a) M->sweep_variant[a] = variants[a];
   for (auto& g : M->graphs) cudaGraphExecDestroy(g.exec);
   M->graphs.clear();

@@ -1,6 +1,8 @@
-"""Sweep variants chosen by rule, by the caller and by the autotuner: the autotuner
-leaves every bit of the state, takes variants that are one kernel as one, and times
-on a sample inside a larger mesh."""
+"""Sweep variants chosen by rule, by the caller and by the autotuner: -1 gives a
+mesh its rule back; the autotuner leaves every bit of the state, takes variants that
+are one kernel as one, and times them on a sample inside a larger mesh; and leaf
+ranges whose size makes the rule take the shared-memory form give the bits of whole
+steps in the streaming form."""
 import numpy as np
 import pytest
 import torch
@@ -42,3 +44,40 @@ def test_autotuner_on_more_leaves_than_its_sample():
     mesh.autotune(U)
     torch.cuda.synchronize()
     assert torch.equal(U, before)
+
+
+def test_rule_given_back():
+    from paper_1810_01319_gb300 import CelloError
+    mesh, U = _mesh(2, 16, 0, precision=4)
+    dt = torch.zeros(1, dtype=torch.float64, device="cuda")
+    mesh.reduce(U, 0.4, dt_next=dt)
+    want = U.clone()
+    mesh.hydro_step(want, dt, 0)
+    mesh.set_sweep_variants([3, 21, 7])
+    mesh.set_sweep_variant(-1)
+    mesh.set_sweep_variants([-1, 20, -1])
+    for bad in ([-2, 0, 0], [0, 24, 0]):
+        with pytest.raises(CelloError):
+            mesh.set_sweep_variants(bad)
+    mesh.hydro_step(U, dt, 0)
+    assert torch.equal(U, want)
+
+
+@pytest.mark.parametrize("kw", [{}, dict(riemann=1, steepening=1), dict(dual_energy=1)])
+def test_small_ranges_equal_the_whole_step(kw):
+    mesh, V = _mesh(4, 32, 1, precision=4, **kw)     # the whole: 70,000 pencils and more; a range of 8 leaves: 12,800
+    dt = torch.zeros(1, dtype=torch.float64, device="cuda")
+    mesh.reduce(V, 0.4, dt_next=dt)
+    inner = (slice(None),) + (slice(4, 36),) * 3
+    for cycle in (0, 1):
+        parts = [(b, min(8, mesh.n_leaves - b)) for b in range(0, mesh.n_leaves, 8)]
+        want = V.clone()
+        mesh.hydro_step(want, dt, cycle)
+        pools = [V.clone() for _ in parts]
+        for part in (0, 1):                          # every range's face fluxes before any correction
+            for W, (b, nb) in zip(pools, parts):
+                mesh.hydro_step_part(W, dt, cycle, b, nb, part)
+        for W, (b, nb) in zip(pools, parts):
+            for leaf in range(b, b + nb):
+                assert torch.equal(W[leaf][inner], want[leaf][inner]), (cycle, leaf)
+        V = want
