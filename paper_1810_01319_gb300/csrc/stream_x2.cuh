@@ -23,6 +23,13 @@
 // same rho, and the streaming and shared-memory forms of the sweep, which
 // both call these functions, compute the same bits.  The expressions follow
 // the formulas of ppm.cuh term by term.
+//
+// Beside a value that is not finite the limited slope is 0, as in ppm.cuh.  Other
+// minima and maxima take the operand that is a number, and an average of weight
+// zero still takes in a difference that is not finite, so that within the stencil
+// a NaN may spread to other cells than in float64.  The cell that holds it keeps it
+// (but for a rho e that is synchronised), every reduction reports it, and cells
+// beyond the stencil are what they are without it.
 #pragma once
 
 #include <type_traits>
@@ -48,6 +55,13 @@ __device__ __forceinline__ float2 sub(float2 a, float2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
   float2 r;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+  return r;
+}
+
+// Minimum that is NaN where an operand is.
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
 
@@ -115,15 +129,16 @@ __device__ __forceinline__ Cell<NQ> each(Fn f, const Cell<NQ>& x, const Cell<NQ>
 
 // Limited slope: dl = a0 - am, dr = ap - a0, da = (ap - am)/2; min(|da|,
 // 2|dl|, 2|dr|) with the sign of da where dl dr > 0, else 0 (doubling is
-// exact, so 2 min(|dl|, |dr|) equals min(2|dl|, 2|dr|)).
+// exact, so 2 min(|dl|, |dr|) equals min(2|dl|, 2|dr|)).  A NaN among the
+// differences passes both minima and ends as 0.
 template <class V>
 __device__ __forceinline__ V slope(V am, V a0, V ap) {
   const V dl = sub(a0, am), dr = sub(ap, a0);
   const V da = mul(splat<V>(0.5f), sub(ap, am));
   // with s = sign(da): s dl and s dr are both positive exactly where dl dr > 0
   const V sg = lanes([](float d) { return copysignf(1.0f, d); }, da);
-  const V mn = mul(splat<V>(2.0f), lanes([](float x, float y) { return fminf(x, y); }, mul(sg, dl), mul(sg, dr)));
-  return mul(sg, lanes([](float d, float m) { return fmaxf(fminf(fabsf(d), m), 0.0f); }, da, mn));
+  const V mn = mul(splat<V>(2.0f), lanes([](float x, float y) { return min_nan(x, y); }, mul(sg, dl), mul(sg, dr)));
+  return mul(sg, lanes([](float d, float m) { return fmaxf(min_nan(fabsf(d), m), 0.0f); }, da, mn));
 }
 
 // Interface value (a0 + a1)/2 - (dm1 - dm0)/6.
