@@ -1696,7 +1696,10 @@ __device__ __forceinline__ float flag_value_f32(const float* b, long o, int fiel
   if constexpr (NF == 6) {
     const float cut = float(kDualEta1) * E;
     if (fabsf(src - cut) <= slack) err = INFINITY;
-    if (!(src > cut)) src = b[5 * SLAB + o];
+    if (!(src > cut)) {
+      src = b[5 * SLAB + o];
+      err += 5e-7f * fabsf(gm1 * src);   // however large beside E
+    }
   }
   return fmaxf(gm1 * src, float(kPFloor));
 }
