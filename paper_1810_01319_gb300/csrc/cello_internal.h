@@ -87,6 +87,15 @@ struct FastDiv {
   __device__ __forceinline__ unsigned div(unsigned x) const { return (__umulhi(x, m) + x) >> s; }
 };
 
+// Padded index of the lower corner of a tracer, v cells from its leaf's first cell.
+// A tracer inside its leaf has v in [-1, n); one that is not (a NaN, a step across
+// the box, a leaf index that is not the position's) reads the block's outermost
+// cells instead of memory outside it.
+__host__ __device__ __forceinline__ int corner_index(int v, int g, int N) {
+  const int lo = -g, hi = N - 2 - g;
+  return (v < lo ? lo : (v > hi ? hi : v)) + g;
+}
+
 // Transverse pencils of one work item's leaf: cb pencils along transverse axis
 // B times count / cb along A, from (a0, b0).  Region 0 of a sweep is a
 // rectangle of every leaf; regions 1 and 2 belong to listed faces (leaf * 6 +

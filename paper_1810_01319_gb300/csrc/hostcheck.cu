@@ -57,6 +57,7 @@ void cello_hc_once_per_device(const int* devices, int count, int* calls) {
     other.join();
   }
 }
+int cello_hc_corner_index(int v, int g, int N) { return corner_index(v, g, N); }
 // One leaf's sweep through the counting scalar (float32 arithmetic), its
 // update written back into slab [fields][N^3]; counts[6] per phase.
 void cello_hc_opcount_leaf(float* slab, int n, int g, int axis, int a0, int a1, int b0, int b1, double dtdx,

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256, 3) particles_push_kernel(PartMesh P, cons
     const double d = x[a] - (P.lo[a] + (double)(lidx[a] * n) * dx);
     const double s = (P.pow2 ? d * inv_dx : d / dx) - 0.5;
     const double c = floor(s);
-    i0[a] = floor_int(c) + g;
+    i0[a] = corner_index(floor_int(c), g, N);
     f[a] = s - c;
   }
   const T* blk = U + (long)b * m.nf * SLAB;
