@@ -12,6 +12,111 @@
 
 using namespace cello;
 
+// The flux at the interface between cells 3 and 4 of an 8-cell window of
+// conserved states (sweep component order), and its vector-Jacobian
+// product: Ub[c][k] += sum_q Fb[q] dF_q/dU[c][k].  The pieces are those of the
+// kernels, put together here interface by interface; the kernels evaluate each once
+// per cell and hand it to the neighbours through shared memory.
+template <typename T>
+CELLO_HD void window_flux(const T U[8][5], T dtdx, const Gas<T>& gs, T F[5]) {
+  T W[8][5];
+  for (int c = 0; c < 8; ++c) to_primitive(U[c], gs, W[c]);
+  T dm[8][5];
+  for (int c = 1; c < 7; ++c)
+    for (int q = 0; q < 5; ++q) dm[c][q] = limited_slope(W[c - 1][q], W[c][q], W[c + 1][q]);
+  T ai[8][5];  // ai[c] = interface c|c+1, c = 2, 3, 4
+  for (int c = 2; c < 5; ++c)
+    for (int q = 0; q < 5; ++q) ai[c][q] = interface_value(W[c][q], W[c + 1][q], dm[c][q], dm[c + 1][q]);
+  T ft[8];
+  for (int c = 2; c < 6; ++c)
+    ft[c] = flatten_tilde(W[c - 2][4], W[c - 1][4], W[c + 1][4], W[c + 2][4], W[c - 1][1], W[c + 1][1]);
+  T edge[2][5];
+  for (int side = 0; side < 2; ++side) {
+    const int j = 3 + side;
+    const T s = W[j + 1][4] - W[j - 1][4];
+    const T f = (s > T(0)) ? vmax(ft[j], ft[j - 1]) : ((s < T(0)) ? vmax(ft[j], ft[j + 1]) : ft[j]);
+    T aL[5], aR[5], Wm[5], Wp[5];
+    for (int q = 0; q < 5; ++q) {
+      aL[q] = ai[j - 1][q];
+      aR[q] = ai[j][q];
+      flatten_monotone(W[j][q], f, aL[q], aR[q]);
+    }
+    trace(W[j], aL, aR, dtdx, gs, Wm, Wp);
+    for (int q = 0; q < 5; ++q) edge[side][q] = side == 0 ? Wp[q] : Wm[q];
+  }
+  riemann_flux(edge[0], edge[1], gs, F);
+}
+
+template <typename T>
+CELLO_HD void window_flux_vjp(const T U[8][5], T dtdx, const Gas<T>& gs, const T Fb[5], T Ub[8][5]) {
+  T W[8][5];
+  for (int c = 0; c < 8; ++c) to_primitive(U[c], gs, W[c]);
+  T dm[8][5];
+  for (int c = 1; c < 7; ++c)
+    for (int q = 0; q < 5; ++q) dm[c][q] = limited_slope(W[c - 1][q], W[c][q], W[c + 1][q]);
+  T ai[8][5];
+  for (int c = 2; c < 5; ++c)
+    for (int q = 0; q < 5; ++q) ai[c][q] = interface_value(W[c][q], W[c + 1][q], dm[c][q], dm[c + 1][q]);
+  T ft[8];
+  for (int c = 2; c < 6; ++c)
+    ft[c] = flatten_tilde(W[c - 2][4], W[c - 1][4], W[c + 1][4], W[c + 2][4], W[c - 1][1], W[c + 1][1]);
+  T fval[2], aLm[2][5], aRm[2][5], edge[2][5];
+  int fsel[2];  // -1: f = ft[j-1], 0: ft[j], +1: ft[j+1]
+  for (int side = 0; side < 2; ++side) {
+    const int j = 3 + side;
+    const T s = W[j + 1][4] - W[j - 1][4];
+    T f;
+    if (s > T(0)) {
+      f = vmax(ft[j], ft[j - 1]);
+      fsel[side] = (ft[j] > ft[j - 1]) ? 0 : -1;
+    } else if (s < T(0)) {
+      f = vmax(ft[j], ft[j + 1]);
+      fsel[side] = (ft[j] > ft[j + 1]) ? 0 : 1;
+    } else {
+      f = ft[j];
+      fsel[side] = 0;
+    }
+    fval[side] = f;
+    T Wm[5], Wp[5];
+    for (int q = 0; q < 5; ++q) {
+      aLm[side][q] = ai[j - 1][q];
+      aRm[side][q] = ai[j][q];
+      flatten_monotone(W[j][q], f, aLm[side][q], aRm[side][q]);
+    }
+    trace(W[j], aLm[side], aRm[side], dtdx, gs, Wm, Wp);
+    for (int q = 0; q < 5; ++q) edge[side][q] = side == 0 ? Wp[q] : Wm[q];
+  }
+  // ---- reverse
+  T eb[2][5] = {{0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}};
+  riemann_flux_bwd(edge[0], edge[1], gs, Fb, eb[0], eb[1]);
+  T Wb[8][5], aib[8][5], dmb[8][5], ftb[8];
+  for (int c = 0; c < 8; ++c) {
+    ftb[c] = T(0);
+    for (int q = 0; q < 5; ++q) Wb[c][q] = aib[c][q] = dmb[c][q] = T(0);
+  }
+  for (int side = 0; side < 2; ++side) {
+    const int j = 3 + side;
+    const T zero5[5] = {0, 0, 0, 0, 0};
+    T aLb[5] = {0, 0, 0, 0, 0}, aRb[5] = {0, 0, 0, 0, 0};
+    trace_bwd(W[j], aLm[side], aRm[side], dtdx, gs, side == 0 ? zero5 : eb[1], side == 0 ? eb[0] : zero5, Wb[j],
+              aLb, aRb);
+    T fb = T(0);
+    for (int q = 0; q < 5; ++q)
+      flatten_monotone_bwd(W[j][q], fval[side], ai[j - 1][q], ai[j][q], aLb[q], aRb[q], Wb[j][q], fb, aib[j - 1][q],
+                           aib[j][q]);
+    ftb[j + fsel[side]] += fb;
+  }
+  for (int c = 5; c >= 2; --c)
+    flatten_tilde_bwd(W[c - 2][4], W[c - 1][4], W[c + 1][4], W[c + 2][4], W[c - 1][1], W[c + 1][1], ftb[c], Wb[c - 2][4],
+                      Wb[c - 1][4], Wb[c + 1][4], Wb[c + 2][4]);
+  for (int c = 4; c >= 2; --c)
+    for (int q = 0; q < 5; ++q) interface_value_bwd(aib[c][q], Wb[c][q], Wb[c + 1][q], dmb[c][q], dmb[c + 1][q]);
+  for (int c = 6; c >= 1; --c)
+    for (int q = 0; q < 5; ++q) limited_slope_bwd(W[c - 1][q], W[c][q], W[c + 1][q], dmb[c][q], Wb[c - 1][q], Wb[c][q],
+                                                  Wb[c + 1][q]);
+  for (int c = 0; c < 8; ++c) to_primitive_bwd(W[c], gs, Wb[c], Ub[c]);
+}
+
 template <typename T>
 static void flux_t(const double* U, double dtdx, double gamma, double* F) {
   T u[8][5], f[5];

@@ -418,126 +418,12 @@ sweep_kernel(DevMesh m, SweepParams prm) {
 // index ranges of every quantity are those of sweep_kernel, so the two
 // forms evaluate the same expressions on the same values.
 // =====================================================================
-// The sliding window of one pencil.
-// NQ = 6 with the dual-energy formalism (e as a sixth primitive).
-template <typename T, int NQ = 5>
-struct PencilWindow {
-  T w[5][NQ];   // primitives of cells k-4 .. k (sweep-local components)
-  T dm[2][NQ];  // slopes of cells k-2, k-1
-  T ft[3];      // shock detectors of cells k-4 .. k-2
-  T ai[3][NQ];  // interface values k-4+1/2 .. k-2+1/2
-  T wp[NQ];     // right-edge state of cell k-4 (left state of interface k-4+1/2)
-  T fl[NQ];     // flux at interface k-5+1/2
-  T eta[3];     // contact-steepening weights of cells k-4 .. k-2 (RS & 2)
-  T dr[2];      // density slopes of cells k-4, k-3 (RS & 2)
-  T ufl;        // interface-state velocity at k-5+1/2 (dual energy)
-};
-
 // One step of the walk: cell k enters as conserved values Us (sweep-local
 // components); old holds cell k-4 as stored (component order), read
 // before it is overwritten here.
 // DEFER: the updated cell is returned in upd[NQ] (component order) instead
 // of being stored.  RS & 4 (dual energy): six fields, rho e taking the
 // compression term with the pressure of its cell and the synchronisation.
-template <typename T, int NB, int RS, bool DEFER = false>
-__device__ __forceinline__ void stream_step(PencilWindow<T, (RS & 4) ? 6 : 5>& S, int k, const T* Us, const T* old,
-                                            T* base, long sAx, const int* comp, T dtdx, const Gas<T>& gs,
-                                            const DevMesh& m, const SweepParams& prm, int leaf, int axis,
-                                            bool face_row, int pa, int pb, long push, T* upd = nullptr) {
-  constexpr int G = kGhosts, N = NB + 2 * G;
-  constexpr long SLAB = (long)N * N * N;
-  constexpr int NQ = (RS & 4) ? 6 : 5;
-  if constexpr (NQ == 6) to_primitive_de(Us, gs, S.w[4]);
-  else to_primitive(Us, gs, S.w[4]);
-  if (k >= 3 && k <= N - 2) {
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) S.dm[1][c] = limited_slope(S.w[2][c], S.w[3][c], S.w[4][c]);
-  }
-  if (k >= 4) {
-    S.ft[2] = flatten_tilde(S.w[0][4], S.w[1][4], S.w[3][4], S.w[4][4], S.w[1][1], S.w[3][1]);
-    if (RS & 2)
-      S.eta[2] = steepening_eta(S.w[0][0], S.w[1][0], S.w[2][0], S.w[3][0], S.w[4][0], S.w[1][4], S.w[3][4], gs.gamma);
-    if (k <= N - 2) {
-#pragma unroll
-      for (int c = 0; c < NQ; ++c)
-        S.ai[2][c] = interface_value(S.w[2][c], S.w[3][c], S.dm[0][c], S.dm[1][c]);
-    }
-  }
-  if (k >= 6) {
-    // cell j = k-3: W = w[1], aL = ai[0], aR = ai[1], shock detectors ft[0..2]
-    const T s = S.w[2][4] - S.w[0][4];
-    const T f = (s > T(0)) ? vmax(S.ft[1], S.ft[0]) : ((s < T(0)) ? vmax(S.ft[1], S.ft[2]) : S.ft[1]);
-    T aL[NQ], aR[NQ], Wm[NQ], Wp[NQ];
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) {
-      aL[c] = S.ai[0][c];
-      aR[c] = S.ai[1][c];
-      if ((RS & 2) && c == 0) {   // density of cell k-3: neighbours k-4 (slope dr[0]) and k-2 (slope dm[0])
-        const T e = S.eta[1];
-        aL[0] = aL[0] * (T(1) - e) + (S.w[0][0] + T(0.5) * S.dr[0]) * e;
-        aR[0] = aR[0] * (T(1) - e) + (S.w[2][0] - T(0.5) * S.dm[0][0]) * e;
-      }
-      flatten_monotone(S.w[1][c], f, aL[c], aR[c]);
-    }
-    trace<T, NQ>(S.w[1], aL, aR, dtdx, gs, Wm, Wp);
-    if (k >= 7) {
-      // interface j = k-4 (+1/2): left state wp (cell k-4), right state Wm (cell k-3)
-      T F[NQ];
-      T uf = T(0);
-      if constexpr (NQ == 6) interface_flux6<RS>(S.wp, Wm, gs, F, &uf);
-      else interface_flux<RS>(S.wp, Wm, gs, F);
-      const int j = k - 4;
-      if (face_row && (j == G - 1 || j == G + NB - 1)) {
-        const int face = 2 * axis + (j == G - 1 ? 0 : 1);
-        const int slot = m.face_slot[leaf * 6 + face];
-        if (slot >= 0) {
-          double* r = prm.reg + (long)slot * NQ * NB * NB + (pa - G) * NB + (pb - G);
-#pragma unroll
-          for (int c = 0; c < NQ; ++c) r[(long)comp[c] * NB * NB] = double(F[c]);
-        }
-      }
-      if (k >= 8) {
-        // cell j = k-4 (window slot w[0]) between interfaces j-1/2 (fl) and j+1/2 (F)
-        T v[NQ];
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) v[c] = old[c] - dtdx * sub_rn(F[c], S.fl[c]);
-        if constexpr (NQ == 6) {
-          v[5] = v[5] - (dtdx * S.w[0][4]) * sub_rn(uf, S.ufl);
-          v[5] = dual_sync(v);
-        }
-#pragma unroll
-        for (int c = 0; c < NQ; ++c) {
-          if (DEFER) upd[c] = v[c];
-          else base[comp[c] * SLAB + (long)j * sAx] = v[c];
-        }
-        if (!DEFER && push) {
-#pragma unroll
-          for (int c = 0; c < NQ; ++c) base[push + comp[c] * SLAB + (long)j * sAx] = v[c];
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < NQ; ++c) S.fl[c] = F[c];
-      if constexpr (NQ == 6) S.ufl = uf;
-    }
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) S.wp[c] = Wp[c];
-  }
-  // slide the windows
-  if (RS & 2) {
-    S.eta[0] = S.eta[1]; S.eta[1] = S.eta[2];
-    S.dr[0] = S.dr[1]; S.dr[1] = S.dm[0][0];
-  }
-#pragma unroll
-  for (int c = 0; c < NQ; ++c) {
-    S.w[0][c] = S.w[1][c]; S.w[1][c] = S.w[2][c]; S.w[2][c] = S.w[3][c]; S.w[3][c] = S.w[4][c];
-    S.dm[0][c] = S.dm[1][c];
-    S.ai[0][c] = S.ai[1][c]; S.ai[1][c] = S.ai[2][c];
-  }
-  S.ft[0] = S.ft[1]; S.ft[1] = S.ft[2];
-}
-
-// Float32 form of stream_step: the same quantities at the same cells, the
-// fields of each in lane-pair groups (stream_x2.cuh).
 template <typename T, int NB, int RS, bool DEFER = false>
 __device__ __forceinline__ void stream_step(px::Window<(RS & 4) ? 6 : 5>& S, int k, const float* Us,
                                             const float* old, float* base, long sAx, const int* comp, float dtdx,
@@ -636,11 +522,6 @@ __device__ __forceinline__ void stream_step(px::Window<(RS & 4) ? 6 : 5>& S, int
   S.ft[0] = S.ft[1]; S.ft[1] = S.ft[2];
 }
 
-// The window type of the streaming sweep: float32 keeps its fields in lane
-// pairs.
-template <typename T, int NQ> struct WindowOf { using type = PencilWindow<T, NQ>; };
-template <int NQ> struct WindowOf<float, NQ> { using type = px::Window<NQ>; };
-
 __device__ __forceinline__ float lane4(const float4& v, int i) {
   return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
@@ -692,7 +573,7 @@ sweep_stream_kernel(DevMesh m, SweepParams prm) {
       T* base = U + (long)leaf * NQ * SLAB + pa * sTA + pb * sTB;
       const long push = push_offset<NB, NQ>(m, prm, axis, at, pa, pb);
       const bool face_row = prm.reg && pa >= G && pa < G + NB && pb >= G && pb < G + NB;
-      typename WindowOf<T, NQ>::type S;
+      px::Window<NQ> S;
       T old[NQ];
       if (VEC == 3 && axis == 0) {
         // the groups of four cells are copied HBM -> shared memory by cp.async, one group

@@ -64,7 +64,7 @@ CELLO_HD float from_fbits(unsigned v) {
 CELLO_HD unsigned high(double a) { return (unsigned)((unsigned long long)bits(a) >> 32); }
 CELLO_HD unsigned mag(double a) { return high(a) & 0x7fffffffu; }   // high word without the sign
 
-constexpr unsigned exp_word(int e) { return (unsigned)(e + 1023) << 20; }   // high word of 2^e
+CELLO_HD constexpr unsigned exp_word(int e) { return (unsigned)(e + 1023) << 20; }   // high word of 2^e
 // The high word lies in that of [2^lo, 2^hi): false for negative numbers, zero, NaN.
 template <int LO, int HI>
 CELLO_HD bool within(unsigned h) { return h - exp_word(LO) < exp_word(HI) - exp_word(LO); }

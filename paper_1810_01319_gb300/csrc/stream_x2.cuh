@@ -489,7 +489,7 @@ __device__ __forceinline__ void flux(const Cell<NQ>& L, const Cell<NQ>& R, const
   else two_shock<NQ>(L, R, gs, F, uf);
 }
 
-// Sliding window of one pencil (see PencilWindow), fields in groups.
+// Sliding window of one pencil, fields in groups.
 template <int NQ>
 struct Window {
   Cell<NQ> w[5];    // primitives of cells k-4 .. k

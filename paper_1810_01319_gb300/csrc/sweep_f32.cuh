@@ -107,7 +107,6 @@ void prepare_sweep_f32() {
 // 23 against 39 us).  On x the staged form bounded for 6 CTAs per SM is ahead up
 // to some hundred thousand pencils (512 leaves of 16^3: 73 against 80 us), for 8
 // beyond (4,096 leaves of 32^3: 3.7 against 4.0 ms).
-template <int NB>
 static int default_variant(const SweepParams& p) {
   long pencils = (long)p.nleaf * p.reg3[0].count;
   for (int r = 1; r < 3; ++r) pencils += (long)p.reg3[r].nfaces * p.reg3[r].count;
@@ -117,7 +116,7 @@ static int default_variant(const SweepParams& p) {
 
 template <int NB>
 void launch_sweep_f32_nb(const DevMesh& m, const SweepParams& p, cudaStream_t s) {
-  const int v = (p.variant >= 0 && p.variant < kNV) ? p.variant : default_variant<NB>(p);
+  const int v = (p.variant >= 0 && p.variant < kNV) ? p.variant : default_variant(p);
   switch (v % kNT) {
     case 0: launch_variant<NB, 8, 3>(m, p, v, s); break;
     case 1: launch_variant<NB, 8, 4>(m, p, v, s); break;
