@@ -34,6 +34,15 @@ WORKLOAD = dict(workload="blob-amr-large", root=[16, 16, 16], n=32, max_level=2,
                 exec="graph", l2="inputs larger than L2 (state tens of GB)")
 
 
+# DRAM bytes (read + written) per 32^3 leaf of one sweep launch, measured by
+# ncu on the 4^3-root blob box (3,970 leaves) for the same kernel form and
+# position in the sweep order (profiles/float32_kernels.md), keyed
+# "axis-form-position"; the roofline's traffic is this times the leaves of the
+# launch.
+SWEEP_DRAM_BYTES_PER_LEAF = {"x-streaming-staged-sweep_1": 1.994e6, "y-streaming-sweep_2": 2.121e6,
+                             "z-streaming-sweep_3": 1.830e6}
+
+
 def alu_peak(log=print):
     """The FP32 ALU roofline's denominator: measured FFMA lane instructions
     per second (cello_fp32_ffma_rate), and the nominal figure from the
@@ -674,6 +683,12 @@ def main():
     kname = names[top]
     if kname.startswith("sweep") and ops is not None:
         sw = sweeps[kname]
+        traffic, tsrc = None, None
+        key = f"{sw['axis']}-{sw['form']}-{kname}"
+        if key in SWEEP_DRAM_BYTES_PER_LEAF and cfg["n"] == 32 and mesh.nf == 5:   # measured on five fields
+            traffic = SWEEP_DRAM_BYTES_PER_LEAF[key] * mesh.n_leaves
+            tsrc = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per leaf of the same kernel and sweep "
+                    "position on the 4^3-root blob box, times the leaves of this launch")
         roofline = {"bound": "alu", "kernel": kname, "achieved": sw["achieved_tops"], "peak": alu_tops,
                     "unit": "T FP32 lane-op/s", "frac": sw["achieved_tops"] / alu_tops,
                     "peak_source": "measured: cello_fp32_ffma_rate, FP32 fused multiply-add lane instructions "
@@ -685,7 +700,7 @@ def main():
                                   "operation, so a fused multiply-add counts two, while the peak counts one "
                                   "FFMA instruction per lane per clock; against the flop convention (an FFMA = "
                                   "2 flops, peak x 2) the same count gives half this frac",
-                    "traffic": None,
+                    "traffic": traffic, "traffic_source": tsrc,
                     "algorithmic_ops_per_launch": sw["ops_per_launch"],
                     "ops_sample": f"operations per updated cell of {len(sample_ids)} leaves evenly spaced in "
                                   "Morton order, times the interior cells",

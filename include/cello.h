@@ -184,7 +184,8 @@ cello_status cello_ghost_refresh(cello_mesh* mesh, void* U, void* stream);
  * the step's dt.  Afterwards dt_next_dev (device double, may be NULL) =
  * cfl * min over leaf cells of dx/(max|u_d| + c), and totals_dev (device
  * double[5], may be NULL) = float64 sums of each conserved field times cell
- * volume over leaf interiors. */
+ * volume over leaf interiors.  U's ghost cells are the step's scratch: it reads
+ * none that it has not written, and leaves no particular values in them. */
 cello_status cello_hydro_step(cello_mesh* mesh, void* U, const double* dt_dev, int cycle, double cfl,
                               double* dt_next_dev, double* totals_dev, void* stream);
 
@@ -269,9 +270,9 @@ cello_status cello_particles_push(cello_mesh* mesh, const void* U, double* pos_d
  * V-cycle, the self-gravity solver of the paper's uniform-grid runs), on a
  * uniform mesh (every leaf at one level), periodic on every axis, cubic
  * root array, at most 512 blocks per axis.  The V-cycle runs on the leaf
- * blocks while they have at least 4 cells per edge, each block with a
- * one-cell ghost layer refreshed from its neighbours through the mesh's
- * neighbour table, and on single arrays below that.  f_dev and phi_dev: device
+ * blocks while they have at least 4 cells per edge (stored without ghost
+ * layers: a kernel reads a tile's halo from the neighbour blocks through the
+ * mesh's neighbour table), and on single arrays below that.  f_dev and phi_dev: device
  * float64 leaf interiors [B][n^3] (no ghosts; x fastest) in leaf order.
  * The 7-point cell-centred Laplacian; the mean of f is removed first and
  * the mean of phi last.  cycles V-cycles from phi = 0, each two damped
@@ -284,8 +285,8 @@ cello_status cello_particles_push(cello_mesh* mesh, const void* U, double* pos_d
  * cost).  resid_host (nullable, host,
  * `cycles` doubles) receives the max-norm of the residual after each cycle,
  * and then the call waits for the stream.  The first solve on a mesh
- * allocates the level arrays (padded blocks: about 3 x 8 x 1.3 bytes per
- * cell for n = 32, more for smaller blocks), freed with the mesh.
+ * allocates the level arrays (about 3 x 8 x 8/7 bytes per cell for float64
+ * cycles, 8 + 3 x 4 x 8/7 for mixed precision), freed with the mesh.
  * CELLO_EINVAL on a mesh it does not support. */
 cello_status cello_poisson_solve(cello_mesh* mesh, const double* f_dev, double* phi_dev, int cycles, int inner,
                                  double* resid_host, void* stream);
