@@ -20,7 +20,10 @@
  *    never frees it.
  *  - Streams: every device call is enqueued on the given cudaStream_t
  *    (passed as void*, NULL = legacy default stream) and returns without
- *    synchronising.  dt, totals and flags stay on the device.
+ *    synchronising.  dt, totals and flags stay on the device.  Calls on one
+ *    mesh may overlap on several streams unless both use the mesh's scratch:
+ *    the reduction (dt or totals asked for), the flux registers (steps of a
+ *    mesh with coarse-fine faces), the adjoint step, the Poisson solver.
  *  - Errors: every call returns a cello_status and never aborts; the text of
  *    the last error of the calling thread is in cello_last_error().
  *  - A cello_mesh is not thread-safe; use one per host thread.

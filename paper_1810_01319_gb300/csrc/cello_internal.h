@@ -28,6 +28,7 @@ struct SweepVariant {
   bool stream;       // register-streaming form (sweep_stream_kernel)
   int vec;           // streaming form moving x pencils four cells at a time, staged by cp.async (3), or not (0)
 };
+constexpr int kMaxSweepVariants = 24;   // of a precision
 int sweep_variant_count_f32();
 // The first variant with the kernel and schedule of variant v: v itself, but for
 // dual-energy meshes, whose streaming kernels all have one register bound.

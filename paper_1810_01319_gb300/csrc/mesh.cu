@@ -1199,22 +1199,23 @@ cello_status cello_autotune(cello_mesh* M, void* U, int* variants_out, float* ms
   // leave the neighbours' ghost rows alone (dt = 0: the interiors stay as they are,
   // but for a rho e that the dual-energy synchronisation resets).
   const size_t bytes = (size_t)nleaf * nfields(d) * M->N * M->N * M->N * d.precision;
+  cudaEvent_t ev[4];
+  for (int i = 0; i < 4; ++i) CELLO_CUDA(cudaEventCreate(&ev[i]));
   void* copy = nullptr;
   if (cudaMalloc(&copy, bytes) != cudaSuccess) {
     cudaGetLastError();
     copy = nullptr;
   }
-  cudaEvent_t ev[4];
-  for (int i = 0; i < 4; ++i) CELLO_CUDA(cudaEventCreate(&ev[i]));
   int best[3] = {0, 0, 0};
   float best_ms[3] = {1e30f, 1e30f, 1e30f};
   cudaError_t err = copy ? cudaMemcpyAsync(copy, U, bytes, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
-  std::vector<float> times(3 * (size_t)nv, 1e30f);
+  float times[kMaxSweepVariants][3];
   for (int v = 0; v < nv && err == cudaSuccess; ++v) {
-    float* vbest = &times[3 * v];
+    float* vbest = times[v];
+    std::fill(vbest, vbest + 3, 1e30f);
     const int twin = d.precision == 4 ? sweep_variant_twin_f32(v, d.dual_energy != 0) : v;
     if (twin != v)   // the same kernel and schedule: timed already
-      std::copy(&times[3 * twin], &times[3 * twin] + 3, vbest);
+      std::copy(times[twin], times[twin] + 3, vbest);
     for (int rep = 0; rep < 4 && twin == v && err == cudaSuccess; ++rep) {
       float axis_ms[3] = {0, 0, 0};
       // the sweeps of an even (x, y, z) and an odd (z, y, x) cycle, dt = 0 (state unchanged):

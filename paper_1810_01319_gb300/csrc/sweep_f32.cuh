@@ -21,6 +21,7 @@ static const SweepVariant kVariants[] = {
 };
 constexpr int kNT = 12;  // distinct kernel instantiations; variant v uses template v % kNT
 constexpr int kNV = sizeof(kVariants) / sizeof(kVariants[0]);
+static_assert(kNV <= kMaxSweepVariants, "the autotuner keeps a time for each");
 
 // Shared memory of the shared-memory form: sweep_arrays(RS) arrays of N x P
 // values (21; 24 with contact steepening).
