@@ -94,8 +94,8 @@ __device__ __forceinline__ long push_offset(const DevMesh& m, const SweepParams&
 // launch: sweeps that overlap, on two streams or in replayed graphs, cannot take
 // each other's items, and there is nothing to reset, which a counter of the mesh
 // does not give.  Two steps of 23,897 leaves of 32^3: 125.1 ms, with
-// that counter 125.2, with a fixed stride of a resident grid 133.7 (its CTAs drift
-// apart, and the rows they share leave the L2).
+// that counter 125.2, with a fixed stride of a resident grid 133.7 (neither the
+// balance nor the order of the items is kept there).
 // Thread 0 of the CTA makes every call; one request is in flight at most.
 struct ItemQueue {
   alignas(16) uint4 answer;
